@@ -5,12 +5,14 @@ import os
 import shutil
 import subprocess
 import sys
+import tempfile
+from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "librdk_b200.so")
-SOURCES = ["rdk_api.cu", "rdk_ids.cu", "rdk_row.cu", "rdk_row_stream.cu", "rdk_emit.cu", "rdk_affinity.cu", "rdk_affinity_tc.cu", "rdk_exact.cu", "rdk_exact_tc.cu"]
+SOURCES = ["rdk_api.cu", "rdk_ids.cu", "rdk_row.cu", "rdk_row_cluster.cu", "rdk_row_stream.cu", "rdk_emit.cu", "rdk_affinity.cu", "rdk_affinity_tc.cu", "rdk_exact.cu", "rdk_exact_tc.cu"]
 
 
 def _nvcc() -> str:
@@ -32,17 +34,25 @@ def build(force: bool = False, verbose: bool = False) -> str:
     """Build the shared library if it is missing or older than a source; return its path."""
     if not force and not _stale():
         return LIB
-    cmd = [_nvcc(), "-shared", "-Xcompiler", "-fPIC", "-std=c++17", "-O3", "-lineinfo",
-           "-gencode", "arch=compute_100a,code=sm_100a",
-           "-I", os.path.join(ROOT, "include"), "-I", CSRC]
+    flags = ["-Xcompiler", "-fPIC", "-std=c++17", "-O3", "-lineinfo", "-gencode", "arch=compute_100a,code=sm_100a",
+             "-I", os.path.join(ROOT, "include"), "-I", CSRC]
     if verbose:
-        cmd += ["-Xptxas", "-v"]
-    cmd += [os.path.join(CSRC, s) for s in SOURCES] + ["-o", LIB]
-    res = subprocess.run(cmd, capture_output=True, text=True)
-    if res.returncode != 0:
-        raise RuntimeError("nvcc failed:\n" + res.stdout + res.stderr)
+        flags += ["-Xptxas", "-v"]
+    nvcc = _nvcc()
+
+    def run(cmd):
+        res = subprocess.run(cmd, capture_output=True, text=True)
+        if res.returncode != 0:
+            raise RuntimeError("nvcc failed:\n" + res.stdout + res.stderr)
+        return res.stdout + res.stderr
+
+    with tempfile.TemporaryDirectory() as tmp:      # one compiler process per source file, side by side
+        objs = [os.path.join(tmp, s + ".o") for s in SOURCES]
+        with ThreadPoolExecutor(max_workers=min(len(SOURCES), os.cpu_count() or 1)) as pool:
+            logs = list(pool.map(lambda so: run([nvcc, "-c", *flags, os.path.join(CSRC, so[0]), "-o", so[1]]), zip(SOURCES, objs)))
+        logs.append(run([nvcc, "-shared", *flags, *objs, "-o", LIB]))
     if verbose:
-        print(res.stdout + res.stderr)
+        print("".join(logs))
     return LIB
 
 

@@ -52,7 +52,6 @@ __device__ __forceinline__ void load_pw(const RowParams& P, const RowCtx& c, con
             }
         }
     }
-#pragma unroll
     if (P.prior) {    // Eq. rdk-taylor with the prior's distribution pi in place of p
         const TZ* prow = static_cast<const TZ*>(P.prior) + (long long)blockIdx.x * P.prior_stride;
         float pr[kVec];
@@ -467,6 +466,17 @@ static int run_rows(const rdk_problem* pb, int mode, const void* target, const v
     if (mode == RDK_MODE_LINEAR && trials > 0 && !prior && !(pb->flags & RDK_FLAG_ROW_KERNEL)) {
         e = launch_stream_linear(P, pb->target_dtype, pb->drafter_dtype, pb->drafter_kind, pb->batch, ws, ws_bytes, s);
         if (e == cudaSuccess) return RDK_OK;          // the streaming kernel also wrote accepted_len
+    }
+    if (e == cudaErrorNotSupported && !(pb->flags & RDK_FLAG_ROW_KERNEL)) {
+        RowParams Q = P;
+        uint32_t tag = 0;
+        if (Q.accepted_len && Q.accepted && ws && ws_bytes >= stream_workspace_bytes(P.rows, pb->batch, trials)) {
+            Q.arrivals = stream_workspace_arrivals(ws, P.rows);     // accepted_len is counted inside the kernel
+            tag = next_tag();
+        }
+        e = launch_cluster_rows(Q, mode, pb->target_dtype, pb->drafter_dtype, pb->drafter_kind, tag, stream_spin_limit(), s);
+        if (e == cudaSuccess && Q.arrivals) return RDK_OK;
+        if (e == cudaErrorNotSupported) (void)cudaGetLastError();
     }
     if (e == cudaErrorNotSupported)
         e = (mode == RDK_MODE_LINEAR)

@@ -25,6 +25,7 @@ struct RowParams {
     int32_t* accepted_len;
     float* rec;            // per-row records in the workspace
     int32_t* counters;     // per (sequence, trial) arrival counters in the workspace
+    unsigned long long* arrivals;   // the cluster kernel's: (tag, arrivals) words; NULL: accepted_len is counted by a kernel of its own
     unsigned char* xrec;   // per (row, CTA of the group) published partial records and flags in the workspace
 };
 
@@ -123,9 +124,17 @@ __device__ __forceinline__ int pick_in_segment(const float (&x)[kVec], float rem
 // cudaErrorNotSupported (and launches nothing) when the one-CTA-per-row kernel has to be used.
 cudaError_t launch_stream_linear(RowParams P, int tz, int ty, int kind, int batch, void* ws, size_t ws_bytes, cudaStream_t s);
 size_t stream_workspace_bytes(int rows, int batch, int trials);
+unsigned long long* stream_workspace_arrivals(void* ws, int rows);     // one word per (sequence, trial) in that workspace
 // Why a problem cannot take the streaming kernel (a static string), or NULL when it can.  Host only.
 const char* stream_ineligible(const RowParams& P, int tz, int ty, int kind, int batch, const void* ws, size_t ws_bytes);
-// Failed tries after which a device-side wait of the streaming kernel gives up (0: the default).
+// A value that differs from the one of every recent call of this process: marks the words a call leaves in the workspace.
+uint32_t next_tag();
+// Failed tries after which a device-side wait gives up (0: the default), and the value that was set.
 void set_stream_spin_limit(unsigned limit);
+unsigned stream_spin_limit();
+
+// Launches the cluster kernel (rdk_row_cluster.cu) in either mode; cudaErrorNotSupported (nothing launched) when a row does
+// not fit the shared memory of a cluster.
+cudaError_t launch_cluster_rows(RowParams P, int mode, int tz, int ty, int kind, uint32_t tag, unsigned spin_limit, cudaStream_t s);
 
 }  // namespace rdk

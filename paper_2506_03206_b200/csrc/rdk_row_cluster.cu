@@ -1,0 +1,798 @@
+// Cluster row kernel: one thread-block cluster takes one row (sequence, draft position) from its logits to its
+// draws in one launch, the row held once in the cluster's shared memory.
+//   soft-max statistics, Token-Level Intersection     (Eq. tli-drafter)
+//   first-order redistribution                        (Eq. rdk-taylor), with p or a separate prior inside it,
+//     or a given w = M^T q'                           (Algorithm 1 step 2)
+//   acceptance rate, draft draw, rejection test, residual draw, or q~ written out   (Algorithm 4 steps 4-8)
+//
+// The row's 16-byte aligned positions are dealt out to the cluster's CTAs and inside a CTA to its warps, each warp
+// a contiguous run ("segment").  Up to the first exchange everything is a warp's own affair: a warp copies its
+// segment (cp.async.bulk on a barrier of its own, the few elements a 16-byte copy cannot cover by plain loads, so
+// any row alignment will do), takes its own maximum as the scale of its exponentials, and leaves one record.  The
+// CTAs then exchange one record each through distributed shared memory (theta, 1/Z_p, 1/Z_q), the warps finish
+// their segment sums of w, min(p, q~), max(0, p - q~) and p, and a second exchange hands every CTA the sums of all
+// segments.  The warp whose segment a draw falls into makes the draw from shared memory; CTA 0 collects the draws
+// of a row and writes the outputs.  Two exchanges and one collection: three cluster barriers per row.
+//
+// Four variants:
+//   kVarSparse  N >= 4096, Eq. rdk-taylor with p itself.  A token that is not kept has q~ = theta x < p, x = p / N, so such
+//               tokens enter through the segment's sum of p only; only the kept tokens are visited a second time,
+//               from registers (kRegSlots x 32 per warp; the rest, where kept ids crowd together, is evaluated anew).
+//   kVarPrior   N >= 4096, Eq. rdk-taylor with a prior pi.  Here a token that is not kept needs its own min(p, theta pi / N),
+//               so the second visit runs over all tokens; the first one takes the kept tokens out of shared memory
+//               (into registers, or to be read again), so that they weigh nothing in it.
+//   kVarDense   any N, q~ output and small vocabularies, with or without a prior: a fp32 array of q' for all tokens of
+//               the segment beside the logits.
+//   kVarGiven   w in place of q'.
+#include <atomic>
+#ifdef RDK_TUNE
+#include <stdlib.h>
+#endif
+
+#include "rdk_device.cuh"
+#include "rdk_row.cuh"
+
+namespace rdk {
+
+enum { kVarSparse = 0, kVarPrior = 1, kVarDense = 2, kVarGiven = 3 };
+
+constexpr int kCluMaxCtas = 16;                     // CTAs per cluster (above 8: non-portable)
+constexpr int kCluMaxWarps = 16;
+constexpr int kCluMaxSeg = kCluMaxCtas * kCluMaxWarps;
+constexpr int kCluRound = 32;                       // trials settled between two collections
+constexpr int kRegSlots = 8;                        // kept tokens per lane held in registers
+constexpr unsigned kCluSpinDefault = 1u << 22;
+
+struct CluGeo {
+    int per;                 // vectors of 8 positions per warp
+    uint32_t zoff_p, zoff_q; // byte offsets of the prior and of the q' array in dynamic shared memory
+    uint32_t tag;            // marks this call's arrival counters
+    unsigned spin_limit;
+};
+
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void st_cluster4(uint32_t local, uint32_t cta, float a, float b, float c, float d) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local), "r"(cta));
+    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(r), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+}
+
+// One segment's share of the row, on the scales m (target), my (drafter), mp (prior)
+struct SegRec { float E, Zq, th, m, my, Ep, mp, W; };
+
+// Folds the records of the warp's lanes into one (lanes without a record hold m = my = mp = -inf and zeros); the
+// scale of th is that of the target (or the prior) times that of the drafter.
+template <bool PRIOR>
+__device__ __forceinline__ SegRec fold_records(const SegRec& r, int lane) {
+    SegRec o;
+    o.m = warp_max_redux(r.m); o.my = warp_max_redux(r.my);
+    const float f = r.m > -INFINITY ? ex2((r.m - o.m) * kLog2e) : 0.f;
+    const float g = r.my > -INFINITY ? ex2((r.my - o.my) * kLog2e) : 0.f;
+    float fp = f;
+    o.mp = 0.f; o.Ep = 0.f;
+    if (PRIOR) {
+        o.mp = warp_max_redux(r.mp);
+        fp = r.mp > -INFINITY ? ex2((r.mp - o.mp) * kLog2e) : 0.f;
+    }
+    const float t = warp_sum4(r.E * f, r.Zq * g, r.th * (fp * g), PRIOR ? r.Ep * fp : r.W, lane);
+    o.E = __shfl_sync(0xffffffffu, t, 0); o.Zq = __shfl_sync(0xffffffffu, t, 8); o.th = __shfl_sync(0xffffffffu, t, 16);
+    const float last = __shfl_sync(0xffffffffu, t, 24);
+    if (PRIOR) { o.Ep = last; o.W = 0.f; } else o.W = last;
+    return o;
+}
+
+// 8 consecutive values at a 16-byte aligned shared address, as fp32
+template <typename T> __device__ __forceinline__ void lds8(uint32_t a, float (&v)[kVec]);
+template <> __device__ __forceinline__ void lds8<__nv_bfloat16>(uint32_t a, float (&v)[kVec]) {
+    const uint4 q = lds128(a);
+    v[0] = bf16_lo(q.x); v[1] = bf16_hi(q.x); v[2] = bf16_lo(q.y); v[3] = bf16_hi(q.y);
+    v[4] = bf16_lo(q.z); v[5] = bf16_hi(q.z); v[6] = bf16_lo(q.w); v[7] = bf16_hi(q.w);
+}
+template <> __device__ __forceinline__ void lds8<float>(uint32_t a, float (&v)[kVec]) {
+    const uint4 q = lds128(a), r = lds128(a + 16u);
+    v[0] = __uint_as_float(q.x); v[1] = __uint_as_float(q.y); v[2] = __uint_as_float(q.z); v[3] = __uint_as_float(q.w);
+    v[4] = __uint_as_float(r.x); v[5] = __uint_as_float(r.y); v[6] = __uint_as_float(r.z); v[7] = __uint_as_float(r.w);
+}
+template <typename T> __device__ __forceinline__ void sts_elem(uint32_t a, T v);
+template <> __device__ __forceinline__ void sts_elem<float>(uint32_t a, float v) { sts32(a, __float_as_uint(v)); }
+template <> __device__ __forceinline__ void sts_elem<__nv_bfloat16>(uint32_t a, __nv_bfloat16 v) {
+    asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"(__bfloat16_as_ushort(v)) : "memory");
+}
+template <typename T> __device__ __forceinline__ T minus_inf();
+template <> __device__ __forceinline__ float minus_inf<float>() { return -INFINITY; }
+template <> __device__ __forceinline__ __nv_bfloat16 minus_inf<__nv_bfloat16>() { return __ushort_as_bfloat16((unsigned short)0xff80u); }
+
+// How elements [0, cnt) of src get to shared address dst: when the two share their phase (mod 16 bytes), `body` elements
+// behind the first `head` go by one bulk copy and the rest by plain loads; else all by plain loads.  Returns the bytes
+// the barrier has to expect.
+template <typename T>
+__device__ __forceinline__ uint32_t copy_in_plan(const T* src, int cnt, uint32_t dst, int& head, int& body) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(src);
+    head = cnt; body = 0;
+    if (((a ^ dst) & 15u) == 0) {
+        const int h = min(cnt, (int)(((16u - (unsigned)(a & 15u)) & 15u) / sizeof(T)));
+        const int b = (cnt - h) / (int)(16 / sizeof(T)) * (int)(16 / sizeof(T));
+        if (b > 0) { head = h; body = b; }
+    }
+    return (uint32_t)body * (uint32_t)sizeof(T);
+}
+template <typename T>
+__device__ __forceinline__ void copy_in_issue(const T* src, int cnt, uint32_t dst, int head, int body, uint32_t bar, int lane) {
+    if (lane == 0 && body)
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                     ::"r"(dst + (uint32_t)(head * sizeof(T))), "l"(src + head), "r"((uint32_t)(body * sizeof(T))), "r"(bar) : "memory");
+#pragma unroll 8
+    for (int i = lane; i < head; i += 32) sts_elem<T>(dst + (uint32_t)(i * sizeof(T)), src[i]);
+    for (int i = head + body + lane; i < cnt; i += 32) sts_elem<T>(dst + (uint32_t)(i * sizeof(T)), src[i]);
+}
+
+// Bounded wait for phase 0 of `bar` by one warp; false when the limit is reached.  A try may park the warp for a
+// while, except under the small limits of the failure-path tests, whose tries must be able to run out.
+__device__ __forceinline__ bool clu_wait(uint32_t bar, unsigned limit) {
+    uint32_t done = 0;
+    for (unsigned spins = 0; !done && spins < limit; ++spins) {
+        if (limit < 64)
+            asm volatile("{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], 0;\n selp.u32 %0, 1, 0, p;\n}"
+                         : "=r"(done) : "r"(bar) : "memory");
+        else
+            asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n selp.u32 %0, 1, 0, p;\n}"
+                         : "=r"(done) : "r"(bar) : "memory");
+    }
+    return __all_sync(0xffffffffu, done != 0);
+}
+
+// w_j = (N q'_j + theta p_j) / (N + p_j) = q'_j + x (theta - q'_j) / (1 + x) for 8 tokens, x = p_j / N (p the prior's where there
+// is one).  From N = 4096 on 1 / (1 + x) = 1 - x up to x^2 <= 2^-24 of the correction term, which itself is x times a probability.
+__device__ __forceinline__ void redistribute8(const float (&x)[kVec], const float (&qp)[kVec], float theta, bool small, float (&w)[kVec]) {
+    if (small) {
+#pragma unroll
+        for (int k = 0; k < kVec; ++k) w[k] = fmaf(x[k] * (theta - qp[k]), __frcp_rn(1.f + x[k]), qp[k]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < kVec; ++k) w[k] = fmaf(x[k] * (theta - qp[k]), 1.f - x[k], qp[k]);
+    }
+}
+__device__ __forceinline__ float redistribute1(float x, float qp, float theta) { return fmaf(x * (theta - qp), 1.f - x, qp); }
+
+template <typename TZ, typename TY, int KIND, int VAR, bool kPrior>
+__global__ void __launch_bounds__(512, 2)
+rdk_cluster_kernel(const RowParams P, const CluGeo g) {
+    constexpr bool kLinear = VAR != kVarGiven, kDense = VAR == kVarDense || VAR == kVarGiven;
+    constexpr uint32_t es = (uint32_t)sizeof(TZ);
+    extern __shared__ __align__(128) unsigned char csm[];
+    __shared__ __align__(16) float4 segs[kCluMaxSeg];            // per segment: sums of w, min(p, q~), max(0, p - q~), p
+    __shared__ __align__(16) double cdf[3][kCluMaxSeg];          // their prefix sums (w, residual, p)
+    __shared__ __align__(16) float4 xrec[kCluMaxCtas][2];        // one record per CTA of the cluster
+    __shared__ __align__(16) float wrec[kCluMaxWarps][8];
+    __shared__ __align__(16) float4 resD[kCluRound], resR[kCluRound];   // CTA 0: draft and residual draws of a round
+    __shared__ __align__(8) unsigned long long wbar[kCluMaxWarps];
+    __shared__ float alpha_s, part_s[kCluMaxWarps];
+
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0), nw = blockDim.x >> 5;
+    uint32_t rank, C;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(C));
+    const int row = (int)(blockIdx.x / C);
+    const bool small = P.N < kStreamMinN;
+
+    bool identity = true;
+    int nvalid = 0;
+    if (kLinear) {
+        const int4 h0 = __ldg(reinterpret_cast<const int4*>(P.header)), h1 = __ldg(reinterpret_cast<const int4*>(P.header) + 1);
+        if (h0.x != kIdxMagic || h0.y != P.N || h0.z != P.n) {      // not an index of this problem: the same decision everywhere
+            if (tid == 0 && rank == 0 && P.status_word) atomicCAS(P.status_word, 0, (int)RDK_ERR_INVALID_ARG);
+            return;
+        }
+        nvalid = h0.w; identity = h1.y != 0;
+    }
+    const uint32_t bar = smem_u32(&wbar[warp]);
+    if (lane == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar));
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    __syncwarp();
+
+    // ---- this warp's segment: positions [seg_pos, seg_pos + len) of the row, position = token + phase -------------
+    const TZ* zrow = static_cast<const TZ*>(P.target) + (long long)row * P.target_stride;
+    const TZ* prow = kPrior ? static_cast<const TZ*>(P.prior) + (long long)row * P.prior_stride : nullptr;
+    const int phase = (int)((reinterpret_cast<uintptr_t>(zrow) & 15u) / es);
+    const int len = g.per * kVec;
+    const int sg = (int)rank * nw + warp, nseg = (int)C * nw;
+    const int seg_tok = sg * len - phase;                        // token at the segment's first position (may be negative)
+    const int t0 = min(max(seg_tok, 0), P.N), t1 = max(t0, min(P.N, seg_tok + len));
+    const uint32_t zb = smem_u32(csm) + (uint32_t)(warp * len) * es;
+    const uint32_t pb = smem_u32(csm) + g.zoff_p + (uint32_t)(warp * len) * es;
+    const uint32_t qb = smem_u32(csm) + g.zoff_q + (uint32_t)(warp * len) * 4u;
+
+    // kept tokens of the segment: ranks [r0, r0 + cnt)
+    int r0 = 0, cnt = 0;
+    if (kLinear) {
+        const int tok = lane == 0 ? t0 : t1;
+        int r = nvalid;
+        if (tok < P.N && lane < 2) {
+            const uint32_t word = __ldg(P.mask + (tok >> 5));
+            r = __ldg(P.rank + (tok >> 5)) + __popc(word & ((1u << (tok & 31)) - 1u));
+        }
+        r0 = __shfl_sync(0xffffffffu, r, 0);
+        cnt = __shfl_sync(0xffffffffu, r, 1) - r0;
+    }
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");       // inputs may be the previous kernel's outputs
+
+    {   // start the copies; positions without a token weigh nothing
+        int zh, zl, ph = 0, pl = 0, qh = 0, ql = 0;
+        const int n_tok = t1 - t0;
+        const uint32_t lead = (uint32_t)(t0 - seg_tok);          // positions before the first token
+        uint32_t total = copy_in_plan<TZ>(zrow + t0, n_tok, zb + lead * es, zh, zl);
+        const float* wrow = VAR == kVarGiven ? P.w + (long long)row * P.w_stride : nullptr;
+        if (kPrior) total += copy_in_plan<TZ>(prow + t0, n_tok, pb + lead * es, ph, pl);
+        if (VAR == kVarGiven) total += copy_in_plan<float>(wrow + t0, n_tok, qb + lead * 4u, qh, ql);
+        if (lane == 0) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(total) : "memory");
+        __syncwarp();
+        copy_in_issue<TZ>(zrow + t0, n_tok, zb + lead * es, zh, zl, bar, lane);
+        if (kPrior) copy_in_issue<TZ>(prow + t0, n_tok, pb + lead * es, ph, pl, bar, lane);
+        if (VAR == kVarGiven) copy_in_issue<float>(wrow + t0, n_tok, qb + lead * 4u, qh, ql, bar, lane);
+        for (int i = lane; i < len - n_tok; i += 32) {
+            const uint32_t o = (uint32_t)(i < (int)lead ? i : i + n_tok);
+            sts_elem<TZ>(zb + o * es, minus_inf<TZ>());
+            if (kPrior) sts_elem<TZ>(pb + o * es, minus_inf<TZ>());
+            if (VAR == kVarGiven) sts32(qb + o * 4u, 0u);
+        }
+        if (kDense && kLinear)
+            for (int i = lane; i < len / 4; i += 32) sts128(qb + (uint32_t)i * 16u, 0.f, 0.f, 0.f, 0.f);
+    }
+
+    // ---- kept tokens: drafter values and positions of the first kRegSlots x 32, and the largest value -------------
+    const TY* yrow = kLinear ? static_cast<const TY*>(P.drafter) + (long long)row * P.drafter_stride : nullptr;
+    auto kept_at = [&](int il, int& pos) -> float {              // drafter value of the il-th kept token of the segment, its position
+        int i = r0 + il;
+        if (!identity) i = __ldg(P.slot + i);
+        pos = __ldg(P.ids + i) - seg_tok;
+        return to_float<TY>(yrow[i]);
+    };
+    float ky[kRegSlots];
+    int kpos[kRegSlots];
+    float my_w = KIND == RDK_LOGITS ? -INFINITY : 0.f;
+    if (kLinear) {
+#pragma unroll
+        for (int k = 0; k < kRegSlots; ++k) {
+            ky[k] = KIND == RDK_LOGITS ? -INFINITY : 0.f; kpos[k] = -1;
+            if (k * 32 + lane < cnt) ky[k] = kept_at(k * 32 + lane, kpos[k]);
+        }
+        if (KIND == RDK_LOGITS) {
+#pragma unroll
+            for (int k = 0; k < kRegSlots; ++k) my_w = fmaxf(my_w, ky[k]);
+            for (int il = kRegSlots * 32 + lane; il < cnt; il += 32) { int pos; my_w = fmaxf(my_w, kept_at(il, pos)); }
+            my_w = warp_max_redux(my_w);
+        }
+    }
+    const float yoff = my_w > -INFINITY ? -my_w * kLog2e : 0.f;
+
+    if (!clu_wait(bar, g.spin_limit)) {      // the copies must land before the CTA leaves all the same (bounded as well)
+        for (unsigned spins = 0; spins < (1u << 16); ++spins) {
+            uint32_t done;
+            asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n selp.u32 %0, 1, 0, p;\n}"
+                         : "=r"(done) : "r"(bar) : "memory");
+            if (done) break;
+            __nanosleep(100);
+        }
+        if (lane == 0 && P.status_word) atomicCAS(P.status_word, 0, (int)RDK_ERR_TIMEOUT);
+    }
+    __syncwarp();
+
+    // ---- first visit ------------------------------------------------------------------------------------------------
+    const int nv16 = len * (int)es / 16;
+    auto seg_max = [&](uint32_t base) -> float {
+        MaxAcc<TZ> a;
+#pragma unroll 4
+        for (int v = lane; v < nv16; v += 32) a.push(lds128(base + (uint32_t)v * 16u));
+        return warp_max_redux(a.result());
+    };
+    auto seg_sum = [&](uint32_t base, float off) -> float {
+        float2 Ea = splat(0.f), Eb = splat(0.f);
+        const float2 l2 = splat(kLog2e), of = splat(off);
+#pragma unroll 4
+        for (int v = lane; v < nv16; v += 32) exp_sum_vec<TZ>(lds128(base + (uint32_t)v * 16u), l2, of, Ea, Eb);
+        return (Ea.x + Ea.y) + (Eb.x + Eb.y);
+    };
+    const float m_w = seg_max(zb);
+    const float zoff = m_w > -INFINITY ? -m_w * kLog2e : 0.f;
+    const float mp_w = kPrior ? seg_max(pb) : -INFINITY;
+    const float poff = kPrior && mp_w > -INFINITY ? -mp_w * kLog2e : 0.f;
+    float E = seg_sum(zb, zoff), Ep = kPrior ? seg_sum(pb, poff) : 0.f;
+    float K = 0.f, Zq = 0.f, th = 0.f, W = 0.f;
+    if (VAR == kVarGiven) {
+#pragma unroll 4
+        for (int v = lane; v < len / 4; v += 32) {
+            const uint4 q = lds128(qb + (uint32_t)v * 16u);
+            W += (__uint_as_float(q.x) + __uint_as_float(q.y)) + (__uint_as_float(q.z) + __uint_as_float(q.w));
+        }
+    }
+    float kz[kRegSlots], kp[VAR == kVarPrior ? kRegSlots : 1];       // e of the kept tokens (kp: of their prior logits)
+    if (kLinear) {
+        const uint32_t db = kPrior ? pb : zb;                        // the distribution that enters theta
+        const float doff = kPrior ? poff : zoff;
+        auto kept_visit = [&](int pos, float y, float& ez, float& ep, float& ey) {
+            ep = ex2(fmaf(lds_z<TZ>(db + (uint32_t)pos * es), kLog2e, doff));
+            ez = VAR == kVarPrior ? ex2(fmaf(lds_z<TZ>(zb + (uint32_t)pos * es), kLog2e, zoff)) : ep;
+            ey = KIND == RDK_LOGITS ? ex2(fmaf(y, kLog2e, yoff)) : y;
+            if (kDense) sts32(qb + (uint32_t)pos * 4u, __float_as_uint(ey));
+            if (VAR == kVarPrior) { sts_elem<TZ>(zb + (uint32_t)pos * es, minus_inf<TZ>()); sts_elem<TZ>(pb + (uint32_t)pos * es, minus_inf<TZ>()); }
+        };
+#pragma unroll
+        for (int k = 0; k < kRegSlots; ++k) {
+            float ez = 0.f, ep = 0.f, ey = 0.f;
+            if (kpos[k] >= 0) kept_visit(kpos[k], ky[k], ez, ep, ey);
+            ky[k] = ey; kz[k] = ez;
+            if (VAR == kVarPrior) kp[k] = ep;
+            K += ez; Zq += ey; th = fmaf(ep, ey, th);
+        }
+        for (int il = kRegSlots * 32 + lane; il < cnt; il += 32) {
+            int pos;
+            float ez, ep, ey;
+            const float y = kept_at(il, pos);
+            kept_visit(pos, y, ez, ep, ey);
+            K += ez; Zq += ey; th = fmaf(ep, ey, th);
+        }
+    }
+    {   // warp totals
+        const float t = warp_sum4(E, K, Zq, th, lane);
+        E = __shfl_sync(0xffffffffu, t, 0); K = __shfl_sync(0xffffffffu, t, 8);
+        Zq = __shfl_sync(0xffffffffu, t, 16); th = __shfl_sync(0xffffffffu, t, 24);
+        if (kPrior) Ep = warp_sum(Ep);
+        if (VAR == kVarGiven) W = warp_sum(W);
+    }
+    if (lane == 0) {
+        reinterpret_cast<float4*>(wrec[warp])[0] = make_float4(E, Zq, th, m_w);
+        reinterpret_cast<float4*>(wrec[warp])[1] = make_float4(my_w, Ep, mp_w, W);
+    }
+    __syncthreads();
+
+    // ---- first exchange: the row's soft-max sums and theta ------------------------------------------------------------
+    if (warp == 0) {
+        SegRec r{0.f, 0.f, 0.f, -INFINITY, -INFINITY, 0.f, -INFINITY, 0.f};
+        if (lane < nw) {
+            const float4 a = reinterpret_cast<const float4*>(wrec[lane])[0], b = reinterpret_cast<const float4*>(wrec[lane])[1];
+            r = SegRec{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+        }
+        r = fold_records<kPrior>(r, lane);
+        if (lane < (int)C) {
+            st_cluster4(smem_u32(&xrec[rank][0]), (uint32_t)lane, r.E, r.Zq, r.th, r.m);
+            st_cluster4(smem_u32(&xrec[rank][1]), (uint32_t)lane, r.my, r.Ep, r.mp, r.W);
+        }
+    }
+    cluster_sync();
+    SegRec tot{0.f, 0.f, 0.f, -INFINITY, -INFINITY, 0.f, -INFINITY, 0.f};
+    if (lane < (int)C) {
+        const float4 a = xrec[lane][0], b = xrec[lane][1];
+        tot = SegRec{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    }
+    tot = fold_records<kPrior>(tot, lane);
+    const float inv_zp = 1.f / tot.E, inv_zq = kLinear ? 1.f / tot.Zq : 1.f, inv_zpi = kPrior ? 1.f / tot.Ep : inv_zp;
+    const float theta = kLinear ? tot.th * inv_zpi * inv_zq : 0.f;
+    const float inv_n = 1.f / (float)P.N;
+    const float offg = -tot.m * kLog2e, poffg = kPrior ? -tot.mp * kLog2e : 0.f;
+    const float yoffg = KIND == RDK_LOGITS ? -tot.my * kLog2e : 0.f;
+    // factor that turns the e_y of this segment into q' (e_y on the segment's scale), 1 for a given w
+    const float fy = !kLinear ? 1.f : (KIND == RDK_LOGITS ? (my_w > -INFINITY ? ex2((my_w - tot.my) * kLog2e) : 0.f) : 1.f) * inv_zq;
+    float inv_s = 1.f;
+
+    // p and w of the 8 positions of vector v of this segment, from the array of q' (or of w)
+    auto dense_pw = [&](int v, float (&p)[kVec], float (&w)[kVec]) {
+        float z[kVec], q[kVec];
+        lds8<TZ>(zb + (uint32_t)v * kVec * es, z);
+        lds8<float>(qb + (uint32_t)v * kVec * 4u, q);
+#pragma unroll
+        for (int k = 0; k < kVec; ++k) p[k] = ex2(fmaf(z[k], kLog2e, offg)) * inv_zp;
+        if (VAR == kVarGiven) {
+#pragma unroll
+            for (int k = 0; k < kVec; ++k) w[k] = q[k];
+            return;
+        }
+        if (kPrior) {
+            lds8<TZ>(pb + (uint32_t)v * kVec * es, z);
+#pragma unroll
+            for (int k = 0; k < kVec; ++k) z[k] = ex2(fmaf(z[k], kLog2e, poffg)) * inv_zpi * inv_n;
+        } else {
+#pragma unroll
+            for (int k = 0; k < kVec; ++k) z[k] = p[k] * inv_n;
+        }
+#pragma unroll
+        for (int k = 0; k < kVec; ++k) q[k] *= fy;
+        redistribute8(z, q, theta, small, w);
+    };
+    // the same where q' is not at hand as an array: the kept tokens among the 8 are looked up in the index (and, with a
+    // prior, their logits in global memory again, because the first visit took them out of shared memory)
+    auto sparse_pw = [&](int v, float (&p)[kVec], float (&w)[kVec]) {
+        float z[kVec], pr[kVec], y[kVec];
+        lds8<TZ>(zb + (uint32_t)v * kVec * es, z);
+        if (kPrior) lds8<TZ>(pb + (uint32_t)v * kVec * es, pr);
+        const int jb = seg_tok + v * kVec, wi = jb >> 5, sh = jb & 31;
+        const bool in = jb < P.N;
+        const uint32_t lo = wi >= 0 && in ? __ldg(P.mask + wi) : 0u;
+        const uint32_t hi = in && (wi + 1) * 32 < P.N ? __ldg(P.mask + wi + 1) : 0u;
+        const uint32_t mb = __funnelshift_r(lo, hi, sh) & 0xffu;
+        const int rb = wi >= 0 && in ? __ldg(P.rank + wi) + __popc(lo & ((1u << sh) - 1u)) : 0;
+#pragma unroll
+        for (int k = 0; k < kVec; ++k) {
+            y[k] = 0.f;
+            if ((mb >> k) & 1u) {
+                int i = rb + __popc(mb & ((1u << k) - 1u));
+                if (!identity) i = __ldg(P.slot + i);
+                y[k] = to_float<TY>(yrow[i]);
+                if (kPrior) { z[k] = to_float<TZ>(zrow[jb + k]); pr[k] = to_float<TZ>(prow[jb + k]); }
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < kVec; ++k) {
+            p[k] = ex2(fmaf(z[k], kLog2e, offg)) * inv_zp;
+            const float x = kPrior ? ex2(fmaf(pr[k], kLog2e, poffg)) * inv_zpi * inv_n : p[k] * inv_n;
+            const float qp = (mb >> k) & 1u ? (KIND == RDK_LOGITS ? ex2(fmaf(y[k], kLog2e, yoffg)) : y[k]) * inv_zq : 0.f;
+            w[k] = redistribute1(x, qp, theta);
+        }
+    };
+
+    // ---- S.  Sum w = 1 + O(N^-2), because sum q' = 1 and the first-order terms cancel: taken as 1 from N = 4096 on -----
+    if (VAR == kVarGiven) {
+        inv_s = P.w_as_given ? 1.f : 1.f / tot.W;
+    } else if (kDense && small) {                       // a small vocabulary: one CTA has the whole row
+        float s = 0.f;
+        for (int v = lane; v < g.per; v += 32) {
+            float p[kVec], w[kVec];
+            dense_pw(v, p, w);
+#pragma unroll
+            for (int k = 0; k < kVec; ++k) s += w[k];
+        }
+        s = warp_sum(s);
+        if (lane == 0) part_s[warp] = s;
+        __syncthreads();
+        s = lane < nw ? part_s[lane] : 0.f;
+        inv_s = 1.f / warp_sum(s);
+    }
+
+    // ---- second visit: the segment's sums of w, min(p, q~), max(0, p - q~), p -----------------------------------------
+    float4 sums;
+    const float fz = (m_w > -INFINITY ? ex2((m_w - tot.m) * kLog2e) : 0.f) * inv_zp;      // e on the segment's scale -> p
+    if (VAR == kVarSparse) {
+        const float xs = fz * inv_n;
+        float ak = 0.f;
+#pragma unroll
+        for (int k = 0; k < kRegSlots; ++k) {
+            const float qp = ky[k] * fy;
+            ak += fminf(kz[k] * fz, fmaf(kz[k] * xs, theta - qp, qp));
+        }
+        for (int il = kRegSlots * 32 + lane; il < cnt; il += 32) {
+            int pos;
+            const float y = kept_at(il, pos);
+            const float ez = ex2(fmaf(lds_z<TZ>(zb + (uint32_t)pos * es), kLog2e, zoff));
+            const float qp = (KIND == RDK_LOGITS ? ex2(fmaf(y, kLog2e, yoff)) : y) * fy;
+            ak += fminf(ez * fz, fmaf(ez * xs, theta - qp, qp));
+        }
+        ak = warp_sum(ak);
+        const float segP = E * fz;
+        const float oov = theta * xs * fmaxf(0.f, E - K);
+        const float Kw = fy * Zq - fy * xs * th + theta * xs * K;
+        sums = make_float4(oov + Kw, oov + ak, fmaxf(0.f, segP - (oov + ak)), segP);
+    } else if (VAR == kVarPrior) {
+        const float xs = (mp_w > -INFINITY ? ex2((mp_w - tot.mp) * kLog2e) : 0.f) * inv_zpi * inv_n;
+        // tokens that are not kept: w = theta x (1 - x)
+        float2 sw2 = splat(0.f), sa2 = splat(0.f), sr2 = splat(0.f);
+        const float2 l2 = splat(kLog2e), zo = splat(zoff), po = splat(poff), f2 = splat(fz), x2 = splat(xs), t2 = splat(theta), m1 = splat(-1.f), p1 = splat(1.f);
+        auto pair = [&](float2 z, float2 pr) {
+            const float2 p = fmul2(ex2_2(ffma2(z, l2, zo)), f2), x = fmul2(ex2_2(ffma2(pr, l2, po)), x2);
+            const float2 w = fmul2(fmul2(t2, x), ffma2(x, m1, p1));
+            const float2 a = make_float2(fminf(p.x, w.x), fminf(p.y, w.y));
+            sw2 = fadd2(sw2, w); sa2 = fadd2(sa2, a); sr2 = fadd2(sr2, ffma2(a, m1, p));
+        };
+#pragma unroll 2
+        for (int v = lane; v < nv16; v += 32) {
+            const uint4 qz = lds128(zb + (uint32_t)v * 16u), qp = lds128(pb + (uint32_t)v * 16u);
+            if (sizeof(TZ) == 2) {
+                pair(make_float2(bf16_lo(qz.x), bf16_hi(qz.x)), make_float2(bf16_lo(qp.x), bf16_hi(qp.x)));
+                pair(make_float2(bf16_lo(qz.y), bf16_hi(qz.y)), make_float2(bf16_lo(qp.y), bf16_hi(qp.y)));
+                pair(make_float2(bf16_lo(qz.z), bf16_hi(qz.z)), make_float2(bf16_lo(qp.z), bf16_hi(qp.z)));
+                pair(make_float2(bf16_lo(qz.w), bf16_hi(qz.w)), make_float2(bf16_lo(qp.w), bf16_hi(qp.w)));
+            } else {
+                pair(make_float2(__uint_as_float(qz.x), __uint_as_float(qz.y)), make_float2(__uint_as_float(qp.x), __uint_as_float(qp.y)));
+                pair(make_float2(__uint_as_float(qz.z), __uint_as_float(qz.w)), make_float2(__uint_as_float(qp.z), __uint_as_float(qp.w)));
+            }
+        }
+        float sw = sw2.x + sw2.y, sa = sa2.x + sa2.y, sr = sr2.x + sr2.y;
+        auto kept_again = [&](float ez, float ep, float ey) {
+            const float p = ez * fz, w = redistribute1(ep * xs, ey * fy, theta), a = fminf(p, w);
+            sw += w; sa += a; sr += p - a;
+        };
+#pragma unroll
+        for (int k = 0; k < kRegSlots; ++k) kept_again(kz[k], kp[k], ky[k]);
+        for (int il = kRegSlots * 32 + lane; il < cnt; il += 32) {
+            int pos;
+            const float y = kept_at(il, pos);
+            const float z = to_float<TZ>(zrow[seg_tok + pos]), pr = to_float<TZ>(prow[seg_tok + pos]);
+            kept_again(ex2(fmaf(z, kLog2e, zoff)), ex2(fmaf(pr, kLog2e, poff)), KIND == RDK_LOGITS ? ex2(fmaf(y, kLog2e, yoff)) : y);
+        }
+        const float t = warp_sum4(sw, sa, sr, 0.f, lane);
+        sums = make_float4(__shfl_sync(0xffffffffu, t, 0), __shfl_sync(0xffffffffu, t, 8), __shfl_sync(0xffffffffu, t, 16), E * fz);
+    } else {
+        float sw = 0.f, sa = 0.f, sr = 0.f, sp = 0.f;
+        float* qrow = P.qtilde ? P.qtilde + (long long)row * P.N : nullptr;
+        // the row of q~ and the positions share their 16-byte phase: store vectors straight away, else by way of shared memory
+        const bool straight = qrow && ((reinterpret_cast<uintptr_t>(qrow) - 4u * (unsigned)phase) & 15u) == 0;
+        for (int v = lane; v < g.per; v += 32) {
+            float p[kVec], w[kVec];
+            dense_pw(v, p, w);
+#pragma unroll
+            for (int k = 0; k < kVec; ++k) {
+                const float qt = w[k] * inv_s;
+                sw += w[k]; sp += p[k];
+                sa += fminf(p[k], qt); sr += fmaxf(0.f, p[k] - qt);
+                w[k] = qt;
+            }
+            if (kLinear && qrow) {
+                const int tok = seg_tok + v * kVec;
+                if (straight && tok >= 0 && tok + kVec <= P.N) {
+                    reinterpret_cast<float4*>(qrow + tok)[0] = make_float4(w[0], w[1], w[2], w[3]);
+                    reinterpret_cast<float4*>(qrow + tok)[1] = make_float4(w[4], w[5], w[6], w[7]);
+                } else if (straight) {
+#pragma unroll
+                    for (int k = 0; k < kVec; ++k) if (tok + k >= 0 && tok + k < P.N) qrow[tok + k] = w[k];
+                } else {
+                    sts128(qb + (uint32_t)v * 32u, w[0], w[1], w[2], w[3]);
+                    sts128(qb + (uint32_t)v * 32u + 16u, w[4], w[5], w[6], w[7]);
+                }
+            }
+        }
+        if (kLinear && qrow && !straight) {
+            __syncwarp();
+            for (int t = t0 + lane; t < t1; t += 32) qrow[t] = __uint_as_float(lds32(qb + (uint32_t)(t - seg_tok) * 4u));
+        }
+        const float t = warp_sum4(sw, sa, sr, sp, lane);
+        sums = make_float4(__shfl_sync(0xffffffffu, t, 0), __shfl_sync(0xffffffffu, t, 8), __shfl_sync(0xffffffffu, t, 16), __shfl_sync(0xffffffffu, t, 24));
+    }
+
+    // ---- second exchange: every CTA gets the sums of all segments -------------------------------------------------------
+    if (lane < (int)C) st_cluster4(smem_u32(&segs[sg]), (uint32_t)lane, sums.x, sums.y, sums.z, sums.w);
+    cluster_sync();
+    if (P.trials == 0 && rank != 0) return;              // nobody reads or writes another CTA's memory from here on
+    for (int job = warp; job < 4; job += nw) {
+        constexpr int kPerLane = kCluMaxSeg / 32;
+        const int per_lane = (nseg + 31) >> 5, s0 = lane * per_lane;
+        double run[kPerLane], x = 0.0;
+#pragma unroll
+        for (int k = 0; k < kPerLane; ++k) {
+            if (k < per_lane && s0 + k < nseg) {
+                const float4 s = segs[s0 + k];
+                x += (double)(job == 0 ? s.x : (job == 1 ? s.z : (job == 2 ? s.w : s.y)));
+            }
+            run[k] = x;
+        }
+        if (job == 3) {
+            x = warp_sum_d(x);
+            if (lane == 0) alpha_s = (float)x;
+        } else {
+            double incl = x;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const double a = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += a;
+            }
+            double before = __shfl_up_sync(0xffffffffu, incl, 1);
+            if (lane == 0) before = 0.0;
+#pragma unroll
+            for (int k = 0; k < kPerLane; ++k)
+                if (k < per_lane && s0 + k < nseg) cdf[job][s0 + k] = before + run[k];
+        }
+    }
+    __syncthreads();
+    const double S_d = cdf[0][nseg - 1], R_d = cdf[1][nseg - 1], Pt_d = cdf[2][nseg - 1];
+    if (rank == 0 && tid == 0) {
+        if (P.alpha) P.alpha[row] = alpha_s;
+        if (P.theta) P.theta[row] = theta;
+        if (P.S) P.S[row] = (float)S_d;
+        if (P.residual_mass) P.residual_mass[row] = (float)R_d;
+    }
+
+    // ---- draws: the warp whose segment holds the threshold makes the draw -----------------------------------------------
+    const bool from_p = !(R_d > 0.0);                    // p and q~ coincide: the replacement comes from p itself
+    const double* cdf_r = from_p ? cdf[2] : cdf[1];
+    // first segment whose prefix sum exceeds the threshold; the last one if rounding leaves none
+    auto mine = [&](const double* c, double thr) {
+        return (c[sg] > thr || sg == nseg - 1) && (sg == 0 || !(c[sg - 1] > thr));
+    };
+    // token of this segment where the running sum of x passes rem: what = 0: x = w, 1: x = max(0, p - q~), 2: x = p
+    auto seg_draw = [&](int what, float rem, float& pd, float& wd) -> int {
+        int tok = -1;
+        float cum = 0.f;
+        pd = 0.f; wd = 0.f;
+        for (int pass = 0; pass < 2 && tok < 0; ++pass) {        // second pass: rounding left no token, take the last positive one
+            for (int v0 = 0; v0 < g.per; v0 += 32) {
+                float p[kVec], w[kVec], x[kVec];
+#pragma unroll
+                for (int k = 0; k < kVec; ++k) { p[k] = 0.f; w[k] = 0.f; }
+                if (v0 + lane < g.per) {
+                    if (kDense) dense_pw(v0 + lane, p, w); else sparse_pw(v0 + lane, p, w);
+                }
+                float s = 0.f;
+#pragma unroll
+                for (int k = 0; k < kVec; ++k) {
+                    x[k] = what == 0 ? w[k] : (what == 1 ? fmaxf(0.f, p[k] - w[k] * inv_s) : p[k]);
+                    s += x[k];
+                }
+                s = warp_sum(s);
+                if (!(s > 0.f)) continue;
+                if (pass == 0 && !(cum + s > rem)) { cum += s; continue; }
+                const int sel = max(pick_in_segment(x, pass == 0 ? rem - cum : INFINITY, lane), 0);
+#pragma unroll
+                for (int k = 0; k < kVec; ++k) if (k == (sel & (kVec - 1))) { pd = p[k]; wd = w[k]; }
+                pd = __shfl_sync(0xffffffffu, pd, sel / kVec);
+                wd = __shfl_sync(0xffffffffu, wd, sel / kVec);
+                tok = seg_tok + v0 * kVec + sel;
+                if (pass == 0) break;
+            }
+        }
+        return tok < 0 ? t0 : tok;
+    };
+    for (int base = 0; base < P.trials; base += kCluRound) {
+        const int nt = min(kCluRound, P.trials - base);
+        const float* u = P.uniforms + ((long long)row * P.trials + base + lane) * 4;
+        double thr_d = 0.0, thr_r = 0.0;
+        bool md = false, mr = false;
+        if (lane < nt) {
+            thr_d = (double)__ldg(u) * S_d;
+            thr_r = (double)__ldg(u + 2) * (from_p ? Pt_d : R_d);
+            md = mine(cdf[0], thr_d); mr = mine(cdf_r, thr_r);
+        }
+        const float rem_d = (float)(thr_d - (sg ? cdf[0][sg - 1] : 0.0)), rem_r = (float)(thr_r - (sg ? cdf_r[sg - 1] : 0.0));
+        // both kinds of draw through one piece of code (it is long): bit t of `todo` and then of `todo_r`
+        uint32_t todo = __ballot_sync(0xffffffffu, md), todo_r = __ballot_sync(0xffffffffu, mr);
+        while (todo | todo_r) {
+            const bool draft = todo != 0;
+            const int t = __ffs(draft ? todo : todo_r) - 1;
+            if (draft) todo &= todo - 1u; else todo_r &= todo_r - 1u;
+            float pd, wd;
+            const int tok = seg_draw(draft ? 0 : (from_p ? 2 : 1), __shfl_sync(0xffffffffu, draft ? rem_d : rem_r, t), pd, wd);
+            if (lane == 0) st_cluster4(smem_u32(draft ? &resD[t] : &resR[t]), 0u, __int_as_float(tok), pd, wd, 0.f);
+        }
+        cluster_sync();
+        if (rank == 0 && tid < nt) {
+            const int dtok = __float_as_int(resD[tid].x);
+            const float pd = resD[tid].y, qd = resD[tid].z * inv_s;
+            const bool acc = __ldg(u + 1) * qd < pd;
+            const long long o = (long long)row * P.trials + base + tid;
+            if (P.draft_token) P.draft_token[o] = dtok;
+            if (P.accepted) P.accepted[o] = acc ? 1 : 0;
+            if (P.accept_prob) P.accept_prob[o] = (pd >= qd) ? 1.f : pd / qd;
+            if (P.out_token) P.out_token[o] = acc ? dtok : __float_as_int(resR[tid].x);
+            if (P.arrivals && P.accepted_len) {
+                // the last position of a sequence to arrive counts the accepted prefix (Algorithm 4 step 7).  The word
+                // holds (tag of the call, arrivals), so it needs no initialisation; the last one clears it for a replay.
+                const int b = row / P.positions;
+                unsigned long long* word = P.arrivals + (long long)b * P.trials + base + tid;
+                __threadfence();
+                unsigned long long old = *reinterpret_cast<volatile unsigned long long*>(word), want;
+                unsigned n_arrived;
+                for (;;) {
+                    n_arrived = ((uint32_t)(old >> 32) == g.tag ? (unsigned)old : 0u) + 1u;
+                    want = n_arrived == (unsigned)P.positions ? 0ull : ((unsigned long long)g.tag << 32) | n_arrived;
+                    const unsigned long long seen = atomicCAS(word, old, want);
+                    if (seen == old) break;              // at most `positions` CTAs contend for a word
+                    old = seen;
+                }
+                if (n_arrived == (unsigned)P.positions) {
+                    __threadfence();
+                    int k = 0;
+                    const volatile uint8_t* af = P.accepted;
+                    while (k < P.positions && af[((long long)b * P.positions + k) * P.trials + base + tid]) ++k;
+                    P.accepted_len[(long long)b * P.trials + base + tid] = k;
+                }
+            }
+        }
+        if (base + kCluRound < P.trials) cluster_sync();         // CTA 0 has read the round's draws
+    }
+}
+
+// ------------------------------------------------------------------------------------------------
+// host side
+// ------------------------------------------------------------------------------------------------
+constexpr int kCluStatic = 14 * 1024;                            // static shared memory of the kernel, rounded up
+constexpr int kCluDynamic = 227 * 1024 - kCluStatic;
+
+struct CluShape { int C, nw, per; size_t smem; };
+
+// CTAs per row, warps per CTA and vectors per warp; false when a row does not fit a cluster's shared memory.
+static bool plan_cluster(int N, int rows, size_t es, int variant, bool prior, CluShape& s) {
+    const size_t bytes = es * (prior ? 2 : 1) + (variant == kVarDense || variant == kVarGiven ? 4 : 0);    // per position
+    const long long positions = (long long)N + 8;
+    int C = 1, nw;
+    if (N >= kStreamMinN) {
+        while (C < kCluMaxCtas && (long long)C * 8192 < positions) C *= 2;
+        while (C < kCluMaxCtas && rows * C < 148 && positions / C > 2048) C *= 2;
+    }
+    nw = (int)((positions / C + 1023) / 1024);
+    nw = nw < 4 ? 4 : (nw > kCluMaxWarps ? kCluMaxWarps : nw);
+#ifdef RDK_TUNE
+    if (getenv("RDK_C") && N >= kStreamMinN) { C = atoi(getenv("RDK_C")); nw = atoi(getenv("RDK_NW")); }
+#endif
+    s.C = C; s.nw = nw;
+    s.per = (int)((positions + (long long)C * nw * kVec - 1) / ((long long)C * nw * kVec));
+    s.smem = (size_t)nw * s.per * kVec * bytes;
+    return s.smem <= (size_t)kCluDynamic;
+}
+
+template <typename TZ, typename TY, int KIND, int VAR, bool PRIOR>
+static cudaError_t launch_cluster(const RowParams& P, CluGeo g, const CluShape& sh, cudaStream_t s) {
+    auto kern = rdk_cluster_kernel<TZ, TY, KIND, VAR, PRIOR>;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorNotSupported;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)P.rows * (unsigned)sh.C, 1, 1);
+    cfg.blockDim = dim3((unsigned)sh.nw * 32, 1, 1);
+    cfg.dynamicSmemBytes = sh.smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)sh.C; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // may set itself up while the previous kernel drains
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    // once per kernel, device and cluster size: the limits raised, and whether such a cluster can be resident at all
+    static std::atomic<uint32_t> known[64];                       // bit log2(C): asked; bit 8 + log2(C): fits
+    const uint32_t bit = (uint32_t)__builtin_ctz((unsigned)sh.C);
+    uint32_t k = known[dev].load(std::memory_order_acquire);
+    if (!(k >> bit & 1u)) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kCluDynamic);
+        if (e != cudaSuccess) return e;
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) return e;
+        cudaLaunchConfig_t q = cfg;
+        q.dynamicSmemBytes = kCluDynamic;
+        q.numAttrs = 1;
+        int fit = 0;
+        e = cudaOccupancyMaxActiveClusters(&fit, kern, &q);
+        if (e != cudaSuccess) { (void)cudaGetLastError(); fit = 0; }
+        k = (1u << bit) | (fit > 0 ? 256u << bit : 0u);
+        k |= known[dev].fetch_or(k, std::memory_order_acq_rel);
+    }
+    if (!(k >> (8 + bit) & 1u)) return cudaErrorNotSupported;
+    return cudaLaunchKernelEx(&cfg, kern, P, g);
+}
+
+template <typename TZ, typename TY, int KIND>
+static cudaError_t launch_variant(const RowParams& P, const CluGeo& g, const CluShape& sh, int variant, cudaStream_t s) {
+    if (variant == kVarSparse) return launch_cluster<TZ, TY, KIND, kVarSparse, false>(P, g, sh, s);
+    if (variant == kVarPrior) return launch_cluster<TZ, TY, KIND, kVarPrior, true>(P, g, sh, s);
+    return P.prior ? launch_cluster<TZ, TY, KIND, kVarDense, true>(P, g, sh, s) : launch_cluster<TZ, TY, KIND, kVarDense, false>(P, g, sh, s);
+}
+
+template <typename TZ, typename TY>
+static cudaError_t launch_kind_c(const RowParams& P, const CluGeo& g, const CluShape& sh, int variant, int kind, cudaStream_t s) {
+    return kind == RDK_LOGITS ? launch_variant<TZ, TY, RDK_LOGITS>(P, g, sh, variant, s) : launch_variant<TZ, TY, RDK_PROBS>(P, g, sh, variant, s);
+}
+
+cudaError_t launch_cluster_rows(RowParams P, int mode, int tz, int ty, int kind, uint32_t tag, unsigned spin_limit, cudaStream_t s) {
+    using B = __nv_bfloat16;
+    const size_t es = tz == RDK_F32 ? 4 : 2;
+    const int variant = mode == RDK_MODE_PRECOMPUTED_W ? kVarGiven
+                        : (P.qtilde || P.N < kStreamMinN ? kVarDense : (P.prior ? kVarPrior : kVarSparse));
+    CluShape sh;
+    if (!plan_cluster(P.N, P.rows, es, variant, P.prior != nullptr, sh)) return cudaErrorNotSupported;
+    if ((long long)P.rows * sh.C > 0x7fffffffLL) return cudaErrorNotSupported;
+    CluGeo g;
+    g.per = sh.per;
+    const size_t zbytes = (size_t)sh.nw * sh.per * kVec * es;
+    g.zoff_p = (uint32_t)zbytes;
+    g.zoff_q = (uint32_t)(P.prior ? 2 * zbytes : zbytes);
+    g.tag = tag; g.spin_limit = spin_limit ? spin_limit : kCluSpinDefault;
+    if (variant == kVarGiven)
+        return tz == RDK_F32 ? launch_cluster<float, float, RDK_LOGITS, kVarGiven, false>(P, g, sh, s) : launch_cluster<B, float, RDK_LOGITS, kVarGiven, false>(P, g, sh, s);
+    if (tz == RDK_F32) return ty == RDK_F32 ? launch_kind_c<float, float>(P, g, sh, variant, kind, s) : launch_kind_c<float, B>(P, g, sh, variant, kind, s);
+    return ty == RDK_F32 ? launch_kind_c<B, float>(P, g, sh, variant, kind, s) : launch_kind_c<B, B>(P, g, sh, variant, kind, s);
+}
+
+}  // namespace rdk
