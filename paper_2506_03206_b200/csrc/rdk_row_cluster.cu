@@ -11,8 +11,8 @@
 // any row alignment will do), takes its own maximum as the scale of its exponentials, and leaves one record.  The
 // CTAs then exchange one record each through distributed shared memory (theta, 1/Z_p, 1/Z_q), the warps finish
 // their segment sums of w, min(p, q~), max(0, p - q~) and p, and a second exchange hands every CTA the sums of all
-// segments.  The warp whose segment a draw falls into makes the draw from shared memory; CTA 0 collects the draws
-// of a row and writes the outputs.  Two exchanges and one collection: three cluster barriers per row.
+// segments.  The CTA whose segment a draw falls into makes the draw from shared memory, its warps sharing the
+// segment's 256-position chunks; CTA 0 collects the draws of a row and writes the outputs.  Two exchanges and one collection: three cluster barriers per row.
 //
 // Four variants:
 //   kVarSparse  N >= 4096, Eq. rdk-taylor with p itself.  A token that is not kept has q~ = theta x < p, x = p / N, so such
@@ -39,7 +39,8 @@ enum { kVarSparse = 0, kVarPrior = 1, kVarDense = 2, kVarGiven = 3 };
 constexpr int kCluMaxCtas = 16;                     // CTAs per cluster (above 8: non-portable)
 constexpr int kCluMaxWarps = 16;
 constexpr int kCluMaxSeg = kCluMaxCtas * kCluMaxWarps;
-constexpr int kCluRound = 32;                       // trials settled between two collections
+constexpr int kCluRound = 16;                       // trials settled between two collections
+constexpr int kCluMaxChunks = 32;                   // 256-position chunks of a segment
 constexpr int kRegSlots = 8;                        // kept tokens per lane held in registers
 constexpr unsigned kCluSpinDefault = 1u << 22;
 
@@ -166,7 +167,8 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     __shared__ __align__(16) double cdf[3][kCluMaxSeg];          // their prefix sums (w, residual, p)
     __shared__ __align__(16) float4 xrec[kCluMaxCtas][2];        // one record per CTA of the cluster
     __shared__ __align__(16) float wrec[kCluMaxWarps][8];
-    __shared__ __align__(16) float4 resD[kCluRound], resR[kCluRound];   // CTA 0: draft and residual draws of a round
+    __shared__ __align__(16) float4 res[2 * kCluRound];          // CTA 0: draft (first half) and residual draws of a round
+    __shared__ float dsum[2 * kCluRound][kCluMaxChunks];         // a draw's sums over the chunks of its segment
     __shared__ __align__(8) unsigned long long wbar[kCluMaxWarps];
     __shared__ float alpha_s, part_s[kCluMaxWarps];
 
@@ -254,14 +256,31 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
         pos = __ldg(P.ids + i) - seg_tok;
         return to_float<TY>(yrow[i]);
     };
+    // (loads without branches, four slots at a time, so that a lane's loads travel together)
     float ky[kRegSlots];
     int kpos[kRegSlots];
     float my_w = KIND == RDK_LOGITS ? -INFINITY : 0.f;
     if (kLinear) {
 #pragma unroll
-        for (int k = 0; k < kRegSlots; ++k) {
-            ky[k] = KIND == RDK_LOGITS ? -INFINITY : 0.f; kpos[k] = -1;
-            if (k * 32 + lane < cnt) ky[k] = kept_at(k * 32 + lane, kpos[k]);
+        for (int h = 0; h < kRegSlots; h += 4) {
+            int i[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) { ky[h + k] = KIND == RDK_LOGITS ? -INFINITY : 0.f; kpos[h + k] = -1; }
+            if (h * 32 < cnt) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) i[k] = r0 + min((h + k) * 32 + lane, cnt - 1);
+                if (!identity) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) i[k] = __ldg(P.slot + i[k]);
+                }
+                float y[4];
+                int id[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) { y[k] = to_float<TY>(yrow[i[k]]); id[k] = __ldg(P.ids + i[k]); }
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if ((h + k) * 32 + lane < cnt) { ky[h + k] = y[k]; kpos[h + k] = id[k] - seg_tok; }
+            }
         }
         if (KIND == RDK_LOGITS) {
 #pragma unroll
@@ -316,26 +335,34 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     if (kLinear) {
         const uint32_t db = kPrior ? pb : zb;                        // the distribution that enters theta
         const float doff = kPrior ? poff : zoff;
-        auto kept_visit = [&](int pos, float y, float& ez, float& ep, float& ey) {
+        auto kept_visit = [&](int pos, bool valid, float y, float& ez, float& ep, float& ey) {
             ep = ex2(fmaf(lds_z<TZ>(db + (uint32_t)pos * es), kLog2e, doff));
             ez = VAR == kVarPrior ? ex2(fmaf(lds_z<TZ>(zb + (uint32_t)pos * es), kLog2e, zoff)) : ep;
             ey = KIND == RDK_LOGITS ? ex2(fmaf(y, kLog2e, yoff)) : y;
-            if (kDense) sts32(qb + (uint32_t)pos * 4u, __float_as_uint(ey));
-            if (VAR == kVarPrior) { sts_elem<TZ>(zb + (uint32_t)pos * es, minus_inf<TZ>()); sts_elem<TZ>(pb + (uint32_t)pos * es, minus_inf<TZ>()); }
+            if (kDense && valid) sts32(qb + (uint32_t)pos * 4u, __float_as_uint(ey));
+            if (VAR == kVarPrior && valid) { sts_elem<TZ>(zb + (uint32_t)pos * es, minus_inf<TZ>()); sts_elem<TZ>(pb + (uint32_t)pos * es, minus_inf<TZ>()); }
         };
 #pragma unroll
         for (int k = 0; k < kRegSlots; ++k) {
-            float ez = 0.f, ep = 0.f, ey = 0.f;
-            if (kpos[k] >= 0) kept_visit(kpos[k], ky[k], ez, ep, ey);
-            ky[k] = ey; kz[k] = ez;
-            if (VAR == kVarPrior) kp[k] = ep;
-            K += ez; Zq += ey; th = fmaf(ep, ey, th);
+            kz[k] = 0.f;
+            if (VAR == kVarPrior) kp[k] = 0.f;
+            if ((k & ~3) * 32 < cnt) {
+                float ez, ep, ey;
+                kept_visit(max(kpos[k], 0), kpos[k] >= 0, ky[k], ez, ep, ey);
+                if (kpos[k] < 0) { ez = 0.f; ep = 0.f; }           // (e_y is 0 already)
+                kz[k] = ez;
+                if (VAR == kVarPrior) kp[k] = ep;
+                K += ez; Zq += ey; th = fmaf(ep, ey, th);
+                ky[k] = ey;
+            } else {
+                ky[k] = 0.f;
+            }
         }
         for (int il = kRegSlots * 32 + lane; il < cnt; il += 32) {
             int pos;
             float ez, ep, ey;
             const float y = kept_at(il, pos);
-            kept_visit(pos, y, ez, ep, ey);
+            kept_visit(pos, true, y, ez, ep, ey);
             K += ez; Zq += ey; th = fmaf(ep, ey, th);
         }
     }
@@ -381,11 +408,13 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     const float fy = !kLinear ? 1.f : (KIND == RDK_LOGITS ? (my_w > -INFINITY ? ex2((my_w - tot.my) * kLog2e) : 0.f) : 1.f) * inv_zq;
     float inv_s = 1.f;
 
-    // p and w of the 8 positions of vector v of this segment, from the array of q' (or of w)
-    auto dense_pw = [&](int v, float (&p)[kVec], float (&w)[kVec]) {
+    // p and w of the 8 positions of vector v (counted over the CTA's segments), from the array of q' (or of w); fyv is the
+    // factor of the segment
+    const uint32_t zb0 = smem_u32(csm), pb0 = zb0 + g.zoff_p, qb0 = zb0 + g.zoff_q;
+    auto dense_pw = [&](int v, float fyv, float (&p)[kVec], float (&w)[kVec]) {
         float z[kVec], q[kVec];
-        lds8<TZ>(zb + (uint32_t)v * kVec * es, z);
-        lds8<float>(qb + (uint32_t)v * kVec * 4u, q);
+        lds8<TZ>(zb0 + (uint32_t)v * kVec * es, z);
+        lds8<float>(qb0 + (uint32_t)v * kVec * 4u, q);
 #pragma unroll
         for (int k = 0; k < kVec; ++k) p[k] = ex2(fmaf(z[k], kLog2e, offg)) * inv_zp;
         if (VAR == kVarGiven) {
@@ -394,7 +423,7 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
             return;
         }
         if (kPrior) {
-            lds8<TZ>(pb + (uint32_t)v * kVec * es, z);
+            lds8<TZ>(pb0 + (uint32_t)v * kVec * es, z);
 #pragma unroll
             for (int k = 0; k < kVec; ++k) z[k] = ex2(fmaf(z[k], kLog2e, poffg)) * inv_zpi * inv_n;
         } else {
@@ -402,30 +431,42 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
             for (int k = 0; k < kVec; ++k) z[k] = p[k] * inv_n;
         }
 #pragma unroll
-        for (int k = 0; k < kVec; ++k) q[k] *= fy;
+        for (int k = 0; k < kVec; ++k) q[k] *= fyv;
         redistribute8(z, q, theta, small, w);
     };
     // the same where q' is not at hand as an array: the kept tokens among the 8 are looked up in the index (and, with a
     // prior, their logits in global memory again, because the first visit took them out of shared memory)
     auto sparse_pw = [&](int v, float (&p)[kVec], float (&w)[kVec]) {
         float z[kVec], pr[kVec], y[kVec];
-        lds8<TZ>(zb + (uint32_t)v * kVec * es, z);
-        if (kPrior) lds8<TZ>(pb + (uint32_t)v * kVec * es, pr);
-        const int jb = seg_tok + v * kVec, wi = jb >> 5, sh = jb & 31;
+        lds8<TZ>(zb0 + (uint32_t)v * kVec * es, z);
+        if (kPrior) lds8<TZ>(pb0 + (uint32_t)v * kVec * es, pr);
+        const int jb = (int)rank * nw * len - phase + v * kVec, wi = jb >> 5, sh = jb & 31;
         const bool in = jb < P.N;
         const uint32_t lo = wi >= 0 && in ? __ldg(P.mask + wi) : 0u;
         const uint32_t hi = in && (wi + 1) * 32 < P.N ? __ldg(P.mask + wi + 1) : 0u;
+        const int rw = wi >= 0 && in ? __ldg(P.rank + wi) : 0;
         const uint32_t mb = __funnelshift_r(lo, hi, sh) & 0xffu;
-        const int rb = wi >= 0 && in ? __ldg(P.rank + wi) + __popc(lo & ((1u << sh) - 1u)) : 0;
+        const int rb = wi >= 0 ? rw + __popc(lo & ((1u << sh) - 1u)) : 0;
+        // independent loads: a token that is not kept reads what the first kept one does (or entry 0)
+        int i[kVec];
 #pragma unroll
-        for (int k = 0; k < kVec; ++k) {
-            y[k] = 0.f;
-            if ((mb >> k) & 1u) {
-                int i = rb + __popc(mb & ((1u << k) - 1u));
-                if (!identity) i = __ldg(P.slot + i);
-                y[k] = to_float<TY>(yrow[i]);
-                if (kPrior) { z[k] = to_float<TZ>(zrow[jb + k]); pr[k] = to_float<TZ>(prow[jb + k]); }
+        for (int k = 0; k < kVec; ++k) i[k] = (mb >> k) & 1u ? rb + __popc(mb & ((1u << k) - 1u)) : (mb ? rb : 0);
+        if (!identity) {
+#pragma unroll
+            for (int k = 0; k < kVec; ++k) i[k] = __ldg(P.slot + i[k]);
+        }
+#pragma unroll
+        for (int k = 0; k < kVec; ++k) y[k] = to_float<TY>(yrow[i[k]]);
+        if (kPrior) {
+            const int first = mb ? jb + __ffs(mb) - 1 : 0;
+            float zk[kVec], pk[kVec];
+#pragma unroll
+            for (int k = 0; k < kVec; ++k) {
+                const int j = (mb >> k) & 1u ? jb + k : first;
+                zk[k] = to_float<TZ>(zrow[j]); pk[k] = to_float<TZ>(prow[j]);
             }
+#pragma unroll
+            for (int k = 0; k < kVec; ++k) if ((mb >> k) & 1u) { z[k] = zk[k]; pr[k] = pk[k]; }
         }
 #pragma unroll
         for (int k = 0; k < kVec; ++k) {
@@ -443,7 +484,7 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
         float s = 0.f;
         for (int v = lane; v < g.per; v += 32) {
             float p[kVec], w[kVec];
-            dense_pw(v, p, w);
+            dense_pw(warp * g.per + v, fy, p, w);
 #pragma unroll
             for (int k = 0; k < kVec; ++k) s += w[k];
         }
@@ -523,7 +564,7 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
         const bool straight = qrow && ((reinterpret_cast<uintptr_t>(qrow) - 4u * (unsigned)phase) & 15u) == 0;
         for (int v = lane; v < g.per; v += 32) {
             float p[kVec], w[kVec];
-            dense_pw(v, p, w);
+            dense_pw(warp * g.per + v, fy, p, w);
 #pragma unroll
             for (int k = 0; k < kVec; ++k) {
                 const float qt = w[k] * inv_s;
@@ -598,74 +639,91 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     // ---- draws: the warp whose segment holds the threshold makes the draw -----------------------------------------------
     const bool from_p = !(R_d > 0.0);                    // p and q~ coincide: the replacement comes from p itself
     const double* cdf_r = from_p ? cdf[2] : cdf[1];
-    // first segment whose prefix sum exceeds the threshold; the last one if rounding leaves none
-    auto mine = [&](const double* c, double thr) {
-        return (c[sg] > thr || sg == nseg - 1) && (sg == 0 || !(c[sg - 1] > thr));
-    };
-    // token of this segment where the running sum of x passes rem: what = 0: x = w, 1: x = max(0, p - q~), 2: x = p
-    auto seg_draw = [&](int what, float rem, float& pd, float& wd) -> int {
-        int tok = -1;
-        float cum = 0.f;
-        pd = 0.f; wd = 0.f;
-        for (int pass = 0; pass < 2 && tok < 0; ++pass) {        // second pass: rounding left no token, take the last positive one
-            for (int v0 = 0; v0 < g.per; v0 += 32) {
-                float p[kVec], w[kVec], x[kVec];
+    const int nch = (g.per + 31) / 32;
+    // x of the 8 positions of this lane in chunk ch of the CTA's segment ws: what = 0: w, 1: max(0, p - q~), 2: p
+    auto chunk_x = [&](int ws, int ch, int what, float (&p)[kVec], float (&w)[kVec], float (&x)[kVec]) -> float {
+        const int v = ch * 32 + lane;
 #pragma unroll
-                for (int k = 0; k < kVec; ++k) { p[k] = 0.f; w[k] = 0.f; }
-                if (v0 + lane < g.per) {
-                    if (kDense) dense_pw(v0 + lane, p, w); else sparse_pw(v0 + lane, p, w);
-                }
-                float s = 0.f;
-#pragma unroll
-                for (int k = 0; k < kVec; ++k) {
-                    x[k] = what == 0 ? w[k] : (what == 1 ? fmaxf(0.f, p[k] - w[k] * inv_s) : p[k]);
-                    s += x[k];
-                }
-                s = warp_sum(s);
-                if (!(s > 0.f)) continue;
-                if (pass == 0 && !(cum + s > rem)) { cum += s; continue; }
-                const int sel = max(pick_in_segment(x, pass == 0 ? rem - cum : INFINITY, lane), 0);
-#pragma unroll
-                for (int k = 0; k < kVec; ++k) if (k == (sel & (kVec - 1))) { pd = p[k]; wd = w[k]; }
-                pd = __shfl_sync(0xffffffffu, pd, sel / kVec);
-                wd = __shfl_sync(0xffffffffu, wd, sel / kVec);
-                tok = seg_tok + v0 * kVec + sel;
-                if (pass == 0) break;
+        for (int k = 0; k < kVec; ++k) { p[k] = 0.f; w[k] = 0.f; }
+        if (v < g.per) {
+            if (kDense) {
+                float fyv = 1.f;
+                if (kLinear && KIND == RDK_LOGITS) { const float my = wrec[ws][4]; fyv = my > -INFINITY ? ex2((my - tot.my) * kLog2e) : 0.f; }
+                dense_pw(ws * g.per + v, fyv * inv_zq, p, w);
+            } else {
+                sparse_pw(ws * g.per + v, p, w);
             }
         }
-        return tok < 0 ? t0 : tok;
+        float s = 0.f;
+#pragma unroll
+        for (int k = 0; k < kVec; ++k) {
+            x[k] = what == 0 ? w[k] : (what == 1 ? fmaxf(0.f, p[k] - w[k] * inv_s) : p[k]);
+            s += x[k];
+        }
+        return s;
     };
     for (int base = 0; base < P.trials; base += kCluRound) {
         const int nt = min(kCluRound, P.trials - base);
-        const float* u = P.uniforms + ((long long)row * P.trials + base + lane) * 4;
-        double thr_d = 0.0, thr_r = 0.0;
-        bool md = false, mr = false;
-        if (lane < nt) {
-            thr_d = (double)__ldg(u) * S_d;
-            thr_r = (double)__ldg(u + 2) * (from_p ? Pt_d : R_d);
-            md = mine(cdf[0], thr_d); mr = mine(cdf_r, thr_r);
+        // lane t < 16: the draft draw of trial base + t; lane 16 + t: its residual draw (needed only if the draft is rejected)
+        const int trial = lane & (kCluRound - 1), kind = lane / kCluRound;
+        const float* u = P.uniforms + ((long long)row * P.trials + base + trial) * 4;
+        const bool on = trial < nt;
+        const float uu = on ? __ldg(u + 2 * kind) : 0.f;
+        const float u1 = on ? __ldg(u + 1) : 0.f;
+        const double* c = kind == 0 ? cdf[0] : cdf_r;
+        const double thr = (double)uu * c[nseg - 1];
+        const int seg = min(first_above(c, nseg, thr), nseg - 1);
+        const float rem = (float)(thr - (seg ? c[seg - 1] : 0.0));
+        const int ws = seg - (int)rank * nw;
+        const uint32_t here = __ballot_sync(0xffffffffu, on && ws >= 0 && ws < nw);
+        float p[kVec], w[kVec], x[kVec];
+        int k_item = 0;
+        for (uint32_t todo = here; todo; todo &= todo - 1u) {        // the chunks' sums, chunks dealt out to the warps
+            const int t = __ffs(todo) - 1, wst = __shfl_sync(0xffffffffu, ws, t), what = t < kCluRound ? 0 : (from_p ? 2 : 1);
+            for (int ch = 0; ch < nch; ++ch) {
+                if (k_item++ % nw != warp) continue;
+                const float s = warp_sum(chunk_x(wst, ch, what, p, w, x));
+                if (lane == 0) dsum[t][ch] = s;
+            }
         }
-        const float rem_d = (float)(thr_d - (sg ? cdf[0][sg - 1] : 0.0)), rem_r = (float)(thr_r - (sg ? cdf_r[sg - 1] : 0.0));
-        // both kinds of draw through one piece of code (it is long): bit t of `todo` and then of `todo_r`
-        uint32_t todo = __ballot_sync(0xffffffffu, md), todo_r = __ballot_sync(0xffffffffu, mr);
-        while (todo | todo_r) {
-            const bool draft = todo != 0;
-            const int t = __ffs(draft ? todo : todo_r) - 1;
-            if (draft) todo &= todo - 1u; else todo_r &= todo_r - 1u;
-            float pd, wd;
-            const int tok = seg_draw(draft ? 0 : (from_p ? 2 : 1), __shfl_sync(0xffffffffu, draft ? rem_d : rem_r, t), pd, wd);
-            if (lane == 0) st_cluster4(smem_u32(draft ? &resD[t] : &resR[t]), 0u, __int_as_float(tok), pd, wd, 0.f);
+        __syncthreads();
+        k_item = 0;
+        for (uint32_t todo = here; todo; todo &= todo - 1u) {        // the token, draws dealt out to the warps
+            const int t = __ffs(todo) - 1, wst = __shfl_sync(0xffffffffu, ws, t), what = t < kCluRound ? 0 : (from_p ? 2 : 1);
+            const float remt = __shfl_sync(0xffffffffu, rem, t);
+            if (k_item++ % nw != warp) continue;
+            float cum = 0.f, before = 0.f;
+            int chosen = -1, last_pos = -1;
+            for (int ch = 0; ch < nch; ++ch) {
+                const float s = dsum[t][ch];
+                if (s > 0.f) {
+                    if (chosen < 0 && cum + s > remt) { chosen = ch; before = cum; }
+                    last_pos = ch;
+                    cum += s;
+                }
+            }
+            const float r_in = chosen < 0 ? INFINITY : remt - before;    // rounding left no token: the last positive one
+            if (chosen < 0) chosen = max(last_pos, 0);
+            (void)chunk_x(wst, chosen, what, p, w, x);
+            const int sel = max(pick_in_segment(x, r_in, lane), 0);
+            float pd = 0.f, wd = 0.f;
+#pragma unroll
+            for (int k = 0; k < kVec; ++k) if (k == (sel & (kVec - 1))) { pd = p[k]; wd = w[k]; }
+            pd = __shfl_sync(0xffffffffu, pd, sel / kVec);
+            wd = __shfl_sync(0xffffffffu, wd, sel / kVec);
+            const int tok = ((int)rank * nw + wst) * len - phase + chosen * 256 + sel;
+            if (lane == 0) st_cluster4(smem_u32(&res[t]), 0u, __int_as_float(min(max(tok, 0), P.N - 1)), pd, wd, 0.f);
         }
         cluster_sync();
         if (rank == 0 && tid < nt) {
-            const int dtok = __float_as_int(resD[tid].x);
-            const float pd = resD[tid].y, qd = resD[tid].z * inv_s;
-            const bool acc = __ldg(u + 1) * qd < pd;
+            const int dtok = __float_as_int(res[tid].x);
+            const float pd = res[tid].y, qd = res[tid].z * inv_s;
+            const bool acc = u1 * qd < pd;
             const long long o = (long long)row * P.trials + base + tid;
             if (P.draft_token) P.draft_token[o] = dtok;
             if (P.accepted) P.accepted[o] = acc ? 1 : 0;
             if (P.accept_prob) P.accept_prob[o] = (pd >= qd) ? 1.f : pd / qd;
-            if (P.out_token) P.out_token[o] = acc ? dtok : __float_as_int(resR[tid].x);
+            if (P.out_token) P.out_token[o] = acc ? dtok : __float_as_int(res[kCluRound + tid].x);
             if (P.arrivals && P.accepted_len) {
                 // the last position of a sequence to arrive counts the accepted prefix (Algorithm 4 step 7).  The word
                 // holds (tag of the call, arrivals), so it needs no initialisation; the last one clears it for a replay.
@@ -697,7 +755,7 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
 // ------------------------------------------------------------------------------------------------
 // host side
 // ------------------------------------------------------------------------------------------------
-constexpr int kCluStatic = 14 * 1024;                            // static shared memory of the kernel, rounded up
+constexpr int kCluStatic = 18 * 1024;                            // static shared memory of the kernel, rounded up
 constexpr int kCluDynamic = 227 * 1024 - kCluStatic;
 
 struct CluShape { int C, nw, per; size_t smem; };
@@ -719,7 +777,7 @@ static bool plan_cluster(int N, int rows, size_t es, int variant, bool prior, Cl
     s.C = C; s.nw = nw;
     s.per = (int)((positions + (long long)C * nw * kVec - 1) / ((long long)C * nw * kVec));
     s.smem = (size_t)nw * s.per * kVec * bytes;
-    return s.smem <= (size_t)kCluDynamic;
+    return s.smem <= (size_t)kCluDynamic && s.per <= 32 * kCluMaxChunks;
 }
 
 template <typename TZ, typename TY, int KIND, int VAR, bool PRIOR>
