@@ -17,10 +17,9 @@
 // Four variants:
 //   kVarSparse  N >= 4096, Eq. rdk-taylor with p itself.  A token that is not kept has q~ = theta x < p, x = p / N, so such
 //               tokens enter through the segment's sum of p only; only the kept tokens are visited a second time,
-//               from registers (kRegSlots x 32 per warp; the rest, where kept ids crowd together, is evaluated anew).
+//               from registers (kRegSlots x 32 per warp; the rest is evaluated anew).
 //   kVarPrior   N >= 4096, Eq. rdk-taylor with a prior pi.  Here a token that is not kept needs its own min(p, theta pi / N),
-//               so the second visit runs over all tokens; the first one takes the kept tokens out of shared memory
-//               (into registers, or to be read again), so that they weigh nothing in it.
+//               so the second visit runs over all tokens.
 //   kVarDense   any N, q~ output and small vocabularies, with or without a prior: a fp32 array of q' for all tokens of
 //               the segment beside the logits.
 //   kVarGiven   w in place of q'.
@@ -170,6 +169,7 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     __shared__ __align__(16) float4 res[2 * kCluRound];          // CTA 0: draft (first half) and residual draws of a round
     __shared__ float dsum[2 * kCluRound][kCluMaxChunks];         // a draw's sums over the chunks of its segment
     __shared__ __align__(8) unsigned long long wbar[kCluMaxWarps];
+    __shared__ __align__(16) float4 tot_s[2];
     __shared__ float alpha_s, part_s[kCluMaxWarps];
 
     const int tid = threadIdx.x, lane = tid & 31;
@@ -180,16 +180,6 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     const int row = (int)(blockIdx.x / C);
     const bool small = P.N < kStreamMinN;
 
-    bool identity = true;
-    int nvalid = 0;
-    if (kLinear) {
-        const int4 h0 = __ldg(reinterpret_cast<const int4*>(P.header)), h1 = __ldg(reinterpret_cast<const int4*>(P.header) + 1);
-        if (h0.x != kIdxMagic || h0.y != P.N || h0.z != P.n) {      // not an index of this problem: the same decision everywhere
-            if (tid == 0 && rank == 0 && P.status_word) atomicCAS(P.status_word, 0, (int)RDK_ERR_INVALID_ARG);
-            return;
-        }
-        nvalid = h0.w; identity = h1.y != 0;
-    }
     const uint32_t bar = smem_u32(&wbar[warp]);
     if (lane == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar));
@@ -198,7 +188,7 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     }
     __syncwarp();
 
-    // ---- this warp's segment: positions [seg_pos, seg_pos + len) of the row, position = token + phase -------------
+    // ---- this warp's segment: positions [sg len, (sg + 1) len) of the row, position = token + phase ----------------
     const TZ* zrow = static_cast<const TZ*>(P.target) + (long long)row * P.target_stride;
     const TZ* prow = kPrior ? static_cast<const TZ*>(P.prior) + (long long)row * P.prior_stride : nullptr;
     const int phase = (int)((reinterpret_cast<uintptr_t>(zrow) & 15u) / es);
@@ -206,22 +196,29 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     const int sg = (int)rank * nw + warp, nseg = (int)C * nw;
     const int seg_tok = sg * len - phase;                        // token at the segment's first position (may be negative)
     const int t0 = min(max(seg_tok, 0), P.N), t1 = max(t0, min(P.N, seg_tok + len));
-    const uint32_t zb = smem_u32(csm) + (uint32_t)(warp * len) * es;
-    const uint32_t pb = smem_u32(csm) + g.zoff_p + (uint32_t)(warp * len) * es;
-    const uint32_t qb = smem_u32(csm) + g.zoff_q + (uint32_t)(warp * len) * 4u;
+    const uint32_t zb0 = smem_u32(csm), pb0 = zb0 + g.zoff_p, qb0 = zb0 + g.zoff_q;
+    const uint32_t zb = zb0 + (uint32_t)(warp * len) * es, pb = pb0 + (uint32_t)(warp * len) * es, qb = qb0 + (uint32_t)(warp * len) * 4u;
 
-    // kept tokens of the segment: ranks [r0, r0 + cnt)
-    int r0 = 0, cnt = 0;
+    // header of the index and the ranks of the segment's ends, requested together
+    bool identity = true;
+    int r0 = 0, cnt = 0;                                         // kept tokens of the segment: ranks [r0, r0 + cnt)
     if (kLinear) {
+        const int4 h0 = __ldg(reinterpret_cast<const int4*>(P.header)), h1 = __ldg(reinterpret_cast<const int4*>(P.header) + 1);
         const int tok = lane == 0 ? t0 : t1;
-        int r = nvalid;
-        if (tok < P.N && lane < 2) {
-            const uint32_t word = __ldg(P.mask + (tok >> 5));
-            r = __ldg(P.rank + (tok >> 5)) + __popc(word & ((1u << (tok & 31)) - 1u));
+        uint32_t word = 0;
+        int r = 0;
+        if (tok < P.N && lane < 2) { word = __ldg(P.mask + (tok >> 5)); r = __ldg(P.rank + (tok >> 5)); }
+        if (h0.x != kIdxMagic || h0.y != P.N || h0.z != P.n) {      // not an index of this problem: the same decision everywhere
+            if (tid == 0 && rank == 0 && P.status_word) atomicCAS(P.status_word, 0, (int)RDK_ERR_INVALID_ARG);
+            return;
         }
+        identity = h1.y != 0;
+        r = tok < P.N ? r + __popc(word & ((1u << (tok & 31)) - 1u)) : h0.w;
         r0 = __shfl_sync(0xffffffffu, r, 0);
         cnt = __shfl_sync(0xffffffffu, r, 1) - r0;
     }
+    // another CTA's shared memory may be touched only once that CTA runs: arrive here, wait before the first exchange
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");       // inputs may be the previous kernel's outputs
 
@@ -247,49 +244,49 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
         if (kDense && kLinear)
             for (int i = lane; i < len / 4; i += 32) sts128(qb + (uint32_t)i * 16u, 0.f, 0.f, 0.f, 0.f);
     }
+    // uniforms of the first round of draws: lane t < 16 has those of the draft draw of trial t, lane 16 + t of its residual draw
+    const int trial = lane & (kCluRound - 1), kind = lane / kCluRound;
+    const float* u_row = P.uniforms + (long long)row * P.trials * 4;
+    float u_draw = 0.f, u_test = 0.f;
+    if (trial < P.trials) { u_draw = __ldg(u_row + trial * 4 + 2 * kind); u_test = __ldg(u_row + trial * 4 + 1); }
 
-    // ---- kept tokens: drafter values and positions of the first kRegSlots x 32, and the largest value -------------
+    // ---- kept tokens: drafter values and positions of the first kRegSlots x 32 ---------------------------------------
     const TY* yrow = kLinear ? static_cast<const TY*>(P.drafter) + (long long)row * P.drafter_stride : nullptr;
-    auto kept_at = [&](int il, int& pos) -> float {              // drafter value of the il-th kept token of the segment, its position
-        int i = r0 + il;
-        if (!identity) i = __ldg(P.slot + i);
-        pos = __ldg(P.ids + i) - seg_tok;
-        return to_float<TY>(yrow[i]);
+    // four kept tokens per lane, the il-th of the segment and the ones 32, 64, 96 later; loads without branches (they travel
+    // together), pos = -1 and a drafter value of no weight beyond the last
+    auto load_kept = [&](int il, float* y, int* pos) {
+        int i[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) i[k] = r0 + min(il + k * 32, cnt - 1);
+        if (!identity) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) i[k] = __ldg(P.slot + i[k]);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) { y[k] = to_float<TY>(yrow[i[k]]); pos[k] = __ldg(P.ids + i[k]) - seg_tok; }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (il + k * 32 >= cnt) { y[k] = KIND == RDK_LOGITS ? -INFINITY : 0.f; pos[k] = -1; }
     };
-    // (loads without branches, four slots at a time, so that a lane's loads travel together)
     float ky[kRegSlots];
     int kpos[kRegSlots];
     float my_w = KIND == RDK_LOGITS ? -INFINITY : 0.f;
     if (kLinear) {
 #pragma unroll
         for (int h = 0; h < kRegSlots; h += 4) {
-            int i[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) { ky[h + k] = KIND == RDK_LOGITS ? -INFINITY : 0.f; kpos[h + k] = -1; }
             if (h * 32 < cnt) {
+                load_kept(h * 32 + lane, ky + h, kpos + h);
+            } else {
 #pragma unroll
-                for (int k = 0; k < 4; ++k) i[k] = r0 + min((h + k) * 32 + lane, cnt - 1);
-                if (!identity) {
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) i[k] = __ldg(P.slot + i[k]);
-                }
-                float y[4];
-                int id[4];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) { y[k] = to_float<TY>(yrow[i[k]]); id[k] = __ldg(P.ids + i[k]); }
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    if ((h + k) * 32 + lane < cnt) { ky[h + k] = y[k]; kpos[h + k] = id[k] - seg_tok; }
+                for (int k = 0; k < 4; ++k) { ky[h + k] = KIND == RDK_LOGITS ? -INFINITY : 0.f; kpos[h + k] = -1; }
             }
         }
         if (KIND == RDK_LOGITS) {
 #pragma unroll
             for (int k = 0; k < kRegSlots; ++k) my_w = fmaxf(my_w, ky[k]);
-            for (int il = kRegSlots * 32 + lane; il < cnt; il += 32) { int pos; my_w = fmaxf(my_w, kept_at(il, pos)); }
             my_w = warp_max_redux(my_w);
         }
     }
-    const float yoff = my_w > -INFINITY ? -my_w * kLog2e : 0.f;
 
     if (!clu_wait(bar, g.spin_limit)) {      // the copies must land before the CTA leaves all the same (bounded as well)
         for (unsigned spins = 0; spins < (1u << 16); ++spins) {
@@ -304,11 +301,14 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     __syncwarp();
 
     // ---- first visit ------------------------------------------------------------------------------------------------
+    // Scale of a segment's exponentials: not their maximum (finding it is a pass of its own) but that of the first vectors;
+    // any scale gives the same result as long as no sum grows beyond 1e18, in which case (or with nothing but -inf among
+    // the first) the visit is repeated with the maximum.
     const int nv16 = len * (int)es / 16;
-    auto seg_max = [&](uint32_t base) -> float {
+    auto seg_max = [&](uint32_t base, int nv) -> float {
         MaxAcc<TZ> a;
 #pragma unroll 4
-        for (int v = lane; v < nv16; v += 32) a.push(lds128(base + (uint32_t)v * 16u));
+        for (int v = lane; v < nv; v += 32) a.push(lds128(base + (uint32_t)v * 16u));
         return warp_max_redux(a.result());
     };
     auto seg_sum = [&](uint32_t base, float off) -> float {
@@ -318,52 +318,65 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
         for (int v = lane; v < nv16; v += 32) exp_sum_vec<TZ>(lds128(base + (uint32_t)v * 16u), l2, of, Ea, Eb);
         return (Ea.x + Ea.y) + (Eb.x + Eb.y);
     };
-    const float m_w = seg_max(zb);
-    const float zoff = m_w > -INFINITY ? -m_w * kLog2e : 0.f;
-    const float mp_w = kPrior ? seg_max(pb) : -INFINITY;
-    const float poff = kPrior && mp_w > -INFINITY ? -mp_w * kLog2e : 0.f;
-    float E = seg_sum(zb, zoff), Ep = kPrior ? seg_sum(pb, poff) : 0.f;
-    float K = 0.f, Zq = 0.f, th = 0.f, W = 0.f;
+    float m_w = -INFINITY, mp_w = -INFINITY, zoff = 0.f, poff = 0.f, yoff = 0.f;
+    float E = 0.f, Ep = 0.f, K = 0.f, Zq = 0.f, th = 0.f, W = 0.f;
+    float kz[kRegSlots], ke[kRegSlots];                              // e_z and e_y of the first kept tokens
+    const uint32_t db = kPrior ? pb : zb;                            // the distribution that enters theta
+    for (int attempt = 0; attempt < 2; ++attempt) {
+        const int nv_max = attempt == 0 ? min(nv16, 32) : nv16;
+        m_w = seg_max(zb, nv_max);
+        if (kPrior) mp_w = seg_max(pb, nv_max);
+        if (attempt == 1 && kLinear && KIND == RDK_LOGITS) {
+            for (int il = kRegSlots * 32 + lane; il < cnt; il += 128) {
+                float y[4];
+                int pos[4];
+                load_kept(il, y, pos);
+                my_w = fmaxf(fmaxf(my_w, fmaxf(y[0], y[1])), fmaxf(y[2], y[3]));
+            }
+            my_w = warp_max_redux(my_w);
+        }
+        zoff = m_w > -INFINITY ? -m_w * kLog2e : 0.f;
+        poff = mp_w > -INFINITY ? -mp_w * kLog2e : 0.f;
+        yoff = my_w > -INFINITY ? -my_w * kLog2e : 0.f;
+        E = seg_sum(zb, zoff);
+        if (kPrior) Ep = seg_sum(pb, poff);
+        K = 0.f; Zq = 0.f; th = 0.f;
+        if (kLinear) {
+            const float doff = kPrior ? poff : zoff;
+            auto visit = [&](int pos, float y, float& ed, float& ey) {
+                ed = ex2(fmaf(lds_z<TZ>(db + (uint32_t)max(pos, 0) * es), kLog2e, doff));
+                if (pos < 0) ed = 0.f;
+                ey = KIND == RDK_LOGITS ? ex2(fmaf(y, kLog2e, yoff)) : y;
+                if (kDense && pos >= 0) sts32(qb + (uint32_t)pos * 4u, __float_as_uint(ey));
+                K += ed; Zq += ey; th = fmaf(ed, ey, th);
+            };
+#pragma unroll
+            for (int h = 0; h < kRegSlots; h += 4) {
+                if (h * 32 < cnt) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) visit(kpos[h + k], ky[h + k], kz[h + k], ke[h + k]);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) { kz[h + k] = 0.f; ke[h + k] = 0.f; }
+                }
+            }
+            for (int il = kRegSlots * 32 + lane; il - lane < cnt; il += 128) {
+                float y[4], ed, ey;
+                int pos[4];
+                load_kept(il, y, pos);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) visit(pos[k], y[k], ed, ey);
+            }
+        }
+        const bool poor = !(fmaxf(E, fmaxf(Ep, KIND == RDK_LOGITS ? Zq : 0.f)) < 1e18f) || !(m_w > -INFINITY) || (kPrior && !(mp_w > -INFINITY)) ||
+                          (kLinear && KIND == RDK_LOGITS && cnt > kRegSlots * 32 && !(my_w > -INFINITY));
+        if (!__any_sync(0xffffffffu, poor)) break;
+    }
     if (VAR == kVarGiven) {
 #pragma unroll 4
         for (int v = lane; v < len / 4; v += 32) {
             const uint4 q = lds128(qb + (uint32_t)v * 16u);
             W += (__uint_as_float(q.x) + __uint_as_float(q.y)) + (__uint_as_float(q.z) + __uint_as_float(q.w));
-        }
-    }
-    float kz[kRegSlots], kp[VAR == kVarPrior ? kRegSlots : 1];       // e of the kept tokens (kp: of their prior logits)
-    if (kLinear) {
-        const uint32_t db = kPrior ? pb : zb;                        // the distribution that enters theta
-        const float doff = kPrior ? poff : zoff;
-        auto kept_visit = [&](int pos, bool valid, float y, float& ez, float& ep, float& ey) {
-            ep = ex2(fmaf(lds_z<TZ>(db + (uint32_t)pos * es), kLog2e, doff));
-            ez = VAR == kVarPrior ? ex2(fmaf(lds_z<TZ>(zb + (uint32_t)pos * es), kLog2e, zoff)) : ep;
-            ey = KIND == RDK_LOGITS ? ex2(fmaf(y, kLog2e, yoff)) : y;
-            if (kDense && valid) sts32(qb + (uint32_t)pos * 4u, __float_as_uint(ey));
-            if (VAR == kVarPrior && valid) { sts_elem<TZ>(zb + (uint32_t)pos * es, minus_inf<TZ>()); sts_elem<TZ>(pb + (uint32_t)pos * es, minus_inf<TZ>()); }
-        };
-#pragma unroll
-        for (int k = 0; k < kRegSlots; ++k) {
-            kz[k] = 0.f;
-            if (VAR == kVarPrior) kp[k] = 0.f;
-            if ((k & ~3) * 32 < cnt) {
-                float ez, ep, ey;
-                kept_visit(max(kpos[k], 0), kpos[k] >= 0, ky[k], ez, ep, ey);
-                if (kpos[k] < 0) { ez = 0.f; ep = 0.f; }           // (e_y is 0 already)
-                kz[k] = ez;
-                if (VAR == kVarPrior) kp[k] = ep;
-                K += ez; Zq += ey; th = fmaf(ep, ey, th);
-                ky[k] = ey;
-            } else {
-                ky[k] = 0.f;
-            }
-        }
-        for (int il = kRegSlots * 32 + lane; il < cnt; il += 32) {
-            int pos;
-            float ez, ep, ey;
-            const float y = kept_at(il, pos);
-            kept_visit(pos, true, y, ez, ep, ey);
-            K += ez; Zq += ey; th = fmaf(ep, ey, th);
         }
     }
     {   // warp totals
@@ -378,6 +391,7 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
         reinterpret_cast<float4*>(wrec[warp])[1] = make_float4(my_w, Ep, mp_w, W);
     }
     __syncthreads();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");      // all CTAs of the cluster run
 
     // ---- first exchange: the row's soft-max sums and theta ------------------------------------------------------------
     if (warp == 0) {
@@ -393,24 +407,32 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
         }
     }
     cluster_sync();
-    SegRec tot{0.f, 0.f, 0.f, -INFINITY, -INFINITY, 0.f, -INFINITY, 0.f};
-    if (lane < (int)C) {
-        const float4 a = xrec[lane][0], b = xrec[lane][1];
-        tot = SegRec{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    if (warp == 0) {                                     // fold the cluster's records, once per CTA
+        SegRec r{0.f, 0.f, 0.f, -INFINITY, -INFINITY, 0.f, -INFINITY, 0.f};
+        if (lane < (int)C) {
+            const float4 a = xrec[lane][0], b = xrec[lane][1];
+            r = SegRec{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+        }
+        r = fold_records<kPrior>(r, lane);
+        if (lane == 0) { tot_s[0] = make_float4(r.m, r.my, r.mp, r.W); tot_s[1] = make_float4(1.f / r.E, kLinear ? 1.f / r.Zq : 1.f, kPrior ? 1.f / r.Ep : 1.f / r.E, r.th); }
     }
-    tot = fold_records<kPrior>(tot, lane);
-    const float inv_zp = 1.f / tot.E, inv_zq = kLinear ? 1.f / tot.Zq : 1.f, inv_zpi = kPrior ? 1.f / tot.Ep : inv_zp;
-    const float theta = kLinear ? tot.th * inv_zpi * inv_zq : 0.f;
+    __syncthreads();
+    const float4 tot_a = tot_s[0], tot_b = tot_s[1];
+    const float tot_m = tot_a.x, tot_my = tot_a.y, tot_mp = tot_a.z;
+    const float inv_zp = tot_b.x, inv_zq = tot_b.y, inv_zpi = tot_b.z;
+    const float theta = kLinear ? tot_b.w * inv_zpi * inv_zq : 0.f;
     const float inv_n = 1.f / (float)P.N;
-    const float offg = -tot.m * kLog2e, poffg = kPrior ? -tot.mp * kLog2e : 0.f;
-    const float yoffg = KIND == RDK_LOGITS ? -tot.my * kLog2e : 0.f;
-    // factor that turns the e_y of this segment into q' (e_y on the segment's scale), 1 for a given w
-    const float fy = !kLinear ? 1.f : (KIND == RDK_LOGITS ? (my_w > -INFINITY ? ex2((my_w - tot.my) * kLog2e) : 0.f) : 1.f) * inv_zq;
+    const float offg = -tot_m * kLog2e, poffg = kPrior ? -tot_mp * kLog2e : 0.f;
+    const float yoffg = KIND == RDK_LOGITS ? -tot_my * kLog2e : 0.f;
+    // factor that turns the e_y of a segment with scale my into q'
+    auto y_factor = [&](float my) -> float {
+        return !kLinear ? 1.f : (KIND == RDK_LOGITS ? (my > -INFINITY ? ex2((my - tot_my) * kLog2e) : 0.f) : 1.f) * inv_zq;
+    };
+    const float fy = y_factor(my_w);
     float inv_s = 1.f;
 
     // p and w of the 8 positions of vector v (counted over the CTA's segments), from the array of q' (or of w); fyv is the
     // factor of the segment
-    const uint32_t zb0 = smem_u32(csm), pb0 = zb0 + g.zoff_p, qb0 = zb0 + g.zoff_q;
     auto dense_pw = [&](int v, float fyv, float (&p)[kVec], float (&w)[kVec]) {
         float z[kVec], q[kVec];
         lds8<TZ>(zb0 + (uint32_t)v * kVec * es, z);
@@ -434,8 +456,7 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
         for (int k = 0; k < kVec; ++k) q[k] *= fyv;
         redistribute8(z, q, theta, small, w);
     };
-    // the same where q' is not at hand as an array: the kept tokens among the 8 are looked up in the index (and, with a
-    // prior, their logits in global memory again, because the first visit took them out of shared memory)
+    // the same where q' is not at hand as an array: the kept tokens among the 8 are looked up in the index
     auto sparse_pw = [&](int v, float (&p)[kVec], float (&w)[kVec]) {
         float z[kVec], pr[kVec], y[kVec];
         lds8<TZ>(zb0 + (uint32_t)v * kVec * es, z);
@@ -457,17 +478,6 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
         }
 #pragma unroll
         for (int k = 0; k < kVec; ++k) y[k] = to_float<TY>(yrow[i[k]]);
-        if (kPrior) {
-            const int first = mb ? jb + __ffs(mb) - 1 : 0;
-            float zk[kVec], pk[kVec];
-#pragma unroll
-            for (int k = 0; k < kVec; ++k) {
-                const int j = (mb >> k) & 1u ? jb + k : first;
-                zk[k] = to_float<TZ>(zrow[j]); pk[k] = to_float<TZ>(prow[j]);
-            }
-#pragma unroll
-            for (int k = 0; k < kVec; ++k) if ((mb >> k) & 1u) { z[k] = zk[k]; pr[k] = pk[k]; }
-        }
 #pragma unroll
         for (int k = 0; k < kVec; ++k) {
             p[k] = ex2(fmaf(z[k], kLog2e, offg)) * inv_zp;
@@ -479,7 +489,7 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
 
     // ---- S.  Sum w = 1 + O(N^-2), because sum q' = 1 and the first-order terms cancel: taken as 1 from N = 4096 on -----
     if (VAR == kVarGiven) {
-        inv_s = P.w_as_given ? 1.f : 1.f / tot.W;
+        inv_s = P.w_as_given ? 1.f : 1.f / tot_a.w;
     } else if (kDense && small) {                       // a small vocabulary: one CTA has the whole row
         float s = 0.f;
         for (int v = lane; v < g.per; v += 32) {
@@ -497,21 +507,28 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
 
     // ---- second visit: the segment's sums of w, min(p, q~), max(0, p - q~), p -----------------------------------------
     float4 sums;
-    const float fz = (m_w > -INFINITY ? ex2((m_w - tot.m) * kLog2e) : 0.f) * inv_zp;      // e on the segment's scale -> p
+    const float fz = (m_w > -INFINITY ? ex2((m_w - tot_m) * kLog2e) : 0.f) * inv_zp;      // e on the segment's scale -> p
     if (VAR == kVarSparse) {
         const float xs = fz * inv_n;
         float ak = 0.f;
 #pragma unroll
         for (int k = 0; k < kRegSlots; ++k) {
-            const float qp = ky[k] * fy;
-            ak += fminf(kz[k] * fz, fmaf(kz[k] * xs, theta - qp, qp));
+            if ((k & ~3) * 32 < cnt) {
+                const float qp = ke[k] * fy;
+                ak += fminf(kz[k] * fz, fmaf(kz[k] * xs, theta - qp, qp));
+            }
         }
-        for (int il = kRegSlots * 32 + lane; il < cnt; il += 32) {
-            int pos;
-            const float y = kept_at(il, pos);
-            const float ez = ex2(fmaf(lds_z<TZ>(zb + (uint32_t)pos * es), kLog2e, zoff));
-            const float qp = (KIND == RDK_LOGITS ? ex2(fmaf(y, kLog2e, yoff)) : y) * fy;
-            ak += fminf(ez * fz, fmaf(ez * xs, theta - qp, qp));
+        for (int il = kRegSlots * 32 + lane; il - lane < cnt; il += 128) {
+            float y[4];
+            int pos[4];
+            load_kept(il, y, pos);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float ez = ex2(fmaf(lds_z<TZ>(zb + (uint32_t)max(pos[k], 0) * es), kLog2e, zoff));
+                const float qp = (KIND == RDK_LOGITS ? ex2(fmaf(y[k], kLog2e, yoff)) : y[k]) * fy;
+                const float a = fminf(ez * fz, fmaf(ez * xs, theta - qp, qp));
+                ak += pos[k] >= 0 ? a : 0.f;
+            }
         }
         ak = warp_sum(ak);
         const float segP = E * fz;
@@ -519,15 +536,15 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
         const float Kw = fy * Zq - fy * xs * th + theta * xs * K;
         sums = make_float4(oov + Kw, oov + ak, fmaxf(0.f, segP - (oov + ak)), segP);
     } else if (VAR == kVarPrior) {
-        const float xs = (mp_w > -INFINITY ? ex2((mp_w - tot.mp) * kLog2e) : 0.f) * inv_zpi * inv_n;
-        // tokens that are not kept: w = theta x (1 - x)
-        float2 sw2 = splat(0.f), sa2 = splat(0.f), sr2 = splat(0.f);
+        const float xs = (mp_w > -INFINITY ? ex2((mp_w - tot_mp) * kLog2e) : 0.f) * inv_zpi * inv_n;
+        // all tokens as if not kept, w = theta x (1 - x); then the kept ones' difference (what they count too much is
+        // theta x, smaller than 1 / N of a probability: nothing cancels)
+        float2 sw2 = splat(0.f), sa2 = splat(0.f);
         const float2 l2 = splat(kLog2e), zo = splat(zoff), po = splat(poff), f2 = splat(fz), x2 = splat(xs), t2 = splat(theta), m1 = splat(-1.f), p1 = splat(1.f);
         auto pair = [&](float2 z, float2 pr) {
             const float2 p = fmul2(ex2_2(ffma2(z, l2, zo)), f2), x = fmul2(ex2_2(ffma2(pr, l2, po)), x2);
             const float2 w = fmul2(fmul2(t2, x), ffma2(x, m1, p1));
-            const float2 a = make_float2(fminf(p.x, w.x), fminf(p.y, w.y));
-            sw2 = fadd2(sw2, w); sa2 = fadd2(sa2, a); sr2 = fadd2(sr2, ffma2(a, m1, p));
+            sw2 = fadd2(sw2, w); sa2 = fadd2(sa2, make_float2(fminf(p.x, w.x), fminf(p.y, w.y)));
         };
 #pragma unroll 2
         for (int v = lane; v < nv16; v += 32) {
@@ -542,21 +559,26 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
                 pair(make_float2(__uint_as_float(qz.z), __uint_as_float(qz.w)), make_float2(__uint_as_float(qp.z), __uint_as_float(qp.w)));
             }
         }
-        float sw = sw2.x + sw2.y, sa = sa2.x + sa2.y, sr = sr2.x + sr2.y;
-        auto kept_again = [&](float ez, float ep, float ey) {
-            const float p = ez * fz, w = redistribute1(ep * xs, ey * fy, theta), a = fminf(p, w);
-            sw += w; sa += a; sr += p - a;
+        float sw = sw2.x + sw2.y, sa = sa2.x + sa2.y, dw = 0.f, da = 0.f;
+        auto again = [&](int pos, float ep, float ey) {
+            const float p = ex2(fmaf(lds_z<TZ>(zb + (uint32_t)max(pos, 0) * es), kLog2e, zoff)) * fz, x = ep * xs;
+            const float w0 = theta * x * (1.f - x), w = redistribute1(x, ey * fy, theta);
+            if (pos >= 0) { dw += w - w0; da += fminf(p, w) - fminf(p, w0); }
         };
 #pragma unroll
-        for (int k = 0; k < kRegSlots; ++k) kept_again(kz[k], kp[k], ky[k]);
-        for (int il = kRegSlots * 32 + lane; il < cnt; il += 32) {
-            int pos;
-            const float y = kept_at(il, pos);
-            const float z = to_float<TZ>(zrow[seg_tok + pos]), pr = to_float<TZ>(prow[seg_tok + pos]);
-            kept_again(ex2(fmaf(z, kLog2e, zoff)), ex2(fmaf(pr, kLog2e, poff)), KIND == RDK_LOGITS ? ex2(fmaf(y, kLog2e, yoff)) : y);
+        for (int k = 0; k < kRegSlots; ++k) if ((k & ~3) * 32 < cnt) again(kpos[k], kz[k], ke[k]);
+        for (int il = kRegSlots * 32 + lane; il - lane < cnt; il += 128) {
+            float y[4];
+            int pos[4];
+            load_kept(il, y, pos);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                again(pos[k], ex2(fmaf(lds_z<TZ>(pb + (uint32_t)max(pos[k], 0) * es), kLog2e, poff)), KIND == RDK_LOGITS ? ex2(fmaf(y[k], kLog2e, yoff)) : y[k]);
         }
-        const float t = warp_sum4(sw, sa, sr, 0.f, lane);
-        sums = make_float4(__shfl_sync(0xffffffffu, t, 0), __shfl_sync(0xffffffffu, t, 8), __shfl_sync(0xffffffffu, t, 16), E * fz);
+        sw += dw; sa += da;
+        const float segP = E * fz;
+        sw = warp_sum(sw); sa = warp_sum(sa);
+        sums = make_float4(sw, sa, fmaxf(0.f, segP - sa), segP);
     } else {
         float sw = 0.f, sa = 0.f, sr = 0.f, sp = 0.f;
         float* qrow = P.qtilde ? P.qtilde + (long long)row * P.N : nullptr;
@@ -628,7 +650,7 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
         }
     }
     __syncthreads();
-    const double S_d = cdf[0][nseg - 1], R_d = cdf[1][nseg - 1], Pt_d = cdf[2][nseg - 1];
+    const double S_d = cdf[0][nseg - 1], R_d = cdf[1][nseg - 1];
     if (rank == 0 && tid == 0) {
         if (P.alpha) P.alpha[row] = alpha_s;
         if (P.theta) P.theta[row] = theta;
@@ -647,9 +669,7 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
         for (int k = 0; k < kVec; ++k) { p[k] = 0.f; w[k] = 0.f; }
         if (v < g.per) {
             if (kDense) {
-                float fyv = 1.f;
-                if (kLinear && KIND == RDK_LOGITS) { const float my = wrec[ws][4]; fyv = my > -INFINITY ? ex2((my - tot.my) * kLog2e) : 0.f; }
-                dense_pw(ws * g.per + v, fyv * inv_zq, p, w);
+                dense_pw(ws * g.per + v, y_factor(wrec[ws][4]), p, w);
             } else {
                 sparse_pw(ws * g.per + v, p, w);
             }
@@ -664,61 +684,65 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     };
     for (int base = 0; base < P.trials; base += kCluRound) {
         const int nt = min(kCluRound, P.trials - base);
-        // lane t < 16: the draft draw of trial base + t; lane 16 + t: its residual draw (needed only if the draft is rejected)
-        const int trial = lane & (kCluRound - 1), kind = lane / kCluRound;
-        const float* u = P.uniforms + ((long long)row * P.trials + base + trial) * 4;
         const bool on = trial < nt;
-        const float uu = on ? __ldg(u + 2 * kind) : 0.f;
-        const float u1 = on ? __ldg(u + 1) : 0.f;
+        if (base && on) { u_draw = __ldg(u_row + (base + trial) * 4 + 2 * kind); u_test = __ldg(u_row + (base + trial) * 4 + 1); }
         const double* c = kind == 0 ? cdf[0] : cdf_r;
-        const double thr = (double)uu * c[nseg - 1];
-        const int seg = min(first_above(c, nseg, thr), nseg - 1);
-        const float rem = (float)(thr - (seg ? c[seg - 1] : 0.0));
-        const int ws = seg - (int)rank * nw;
-        const uint32_t here = __ballot_sync(0xffffffffu, on && ws >= 0 && ws < nw);
-        float p[kVec], w[kVec], x[kVec];
-        int k_item = 0;
-        for (uint32_t todo = here; todo; todo &= todo - 1u) {        // the chunks' sums, chunks dealt out to the warps
-            const int t = __ffs(todo) - 1, wst = __shfl_sync(0xffffffffu, ws, t), what = t < kCluRound ? 0 : (from_p ? 2 : 1);
-            for (int ch = 0; ch < nch; ++ch) {
-                if (k_item++ % nw != warp) continue;
-                const float s = warp_sum(chunk_x(wst, ch, what, p, w, x));
-                if (lane == 0) dsum[t][ch] = s;
-            }
-        }
-        __syncthreads();
-        k_item = 0;
-        for (uint32_t todo = here; todo; todo &= todo - 1u) {        // the token, draws dealt out to the warps
-            const int t = __ffs(todo) - 1, wst = __shfl_sync(0xffffffffu, ws, t), what = t < kCluRound ? 0 : (from_p ? 2 : 1);
-            const float remt = __shfl_sync(0xffffffffu, rem, t);
-            if (k_item++ % nw != warp) continue;
-            float cum = 0.f, before = 0.f;
-            int chosen = -1, last_pos = -1;
-            for (int ch = 0; ch < nch; ++ch) {
-                const float s = dsum[t][ch];
-                if (s > 0.f) {
-                    if (chosen < 0 && cum + s > remt) { chosen = ch; before = cum; }
-                    last_pos = ch;
-                    cum += s;
+        const double thr = (double)u_draw * c[nseg - 1];
+        // the draw's segment is the first whose prefix sum exceeds the threshold (the last one if rounding leaves none): is it here?
+        const int s_lo = (int)rank * nw, s_hi = s_lo + nw;
+        const bool below = s_lo > 0 && c[s_lo - 1] > thr, beyond = s_hi < nseg && !(c[s_hi - 1] > thr);
+        const uint32_t here = __ballot_sync(0xffffffffu, on && !below && !beyond);
+        if (here) {
+            const int ws = min(first_above(c + s_lo, nw, thr), nw - 1);
+            const float rem = (float)(thr - (s_lo + ws ? c[s_lo + ws - 1] : 0.0));
+            float p[kVec], w[kVec], x[kVec];
+            int k_item = 0, held = -1;                               // the chunk (by its number) that p, w, x belong to
+            for (uint32_t todo = here; todo; todo &= todo - 1u) {        // the chunks' sums, chunks dealt out to the warps
+                const int t = __ffs(todo) - 1, wst = __shfl_sync(0xffffffffu, ws, t), what = t < kCluRound ? 0 : (from_p ? 2 : 1);
+                for (int ch = 0; ch < nch; ++ch) {
+                    if (k_item++ % nw != warp) continue;
+                    held = k_item - 1;
+                    const float s = warp_sum(chunk_x(wst, ch, what, p, w, x));
+                    if (lane == 0) dsum[t][ch] = s;
                 }
             }
-            const float r_in = chosen < 0 ? INFINITY : remt - before;    // rounding left no token: the last positive one
-            if (chosen < 0) chosen = max(last_pos, 0);
-            (void)chunk_x(wst, chosen, what, p, w, x);
-            const int sel = max(pick_in_segment(x, r_in, lane), 0);
-            float pd = 0.f, wd = 0.f;
+            __syncthreads();
+            k_item = 0;
+            for (uint32_t todo = here; todo; todo &= todo - 1u, k_item += nch) {
+                const int t = __ffs(todo) - 1, wst = __shfl_sync(0xffffffffu, ws, t), what = t < kCluRound ? 0 : (from_p ? 2 : 1);
+                const float remt = __shfl_sync(0xffffffffu, rem, t);
+                float cum = 0.f, before = 0.f;
+                int chosen = -1, last_pos = -1;
+                for (int ch = 0; ch < nch; ++ch) {
+                    const float s = dsum[t][ch];
+                    if (s > 0.f) {
+                        if (chosen < 0 && cum + s > remt) { chosen = ch; before = cum; }
+                        last_pos = ch;
+                        cum += s;
+                    }
+                }
+                const float r_in = chosen < 0 ? INFINITY : remt - before;    // rounding left no token: the last positive one
+                if (chosen < 0) chosen = max(last_pos, 0);
+                if ((k_item + chosen) % nw != warp) continue;                // the warp that summed the chunk picks the token,
+                if (held != k_item + chosen) {                               // from its registers unless it went on to another chunk
+                    (void)chunk_x(wst, chosen, what, p, w, x);
+                    held = k_item + chosen;
+                }
+                const int sel = max(pick_in_segment(x, r_in, lane), 0);
+                float pd = 0.f, wd = 0.f;
 #pragma unroll
-            for (int k = 0; k < kVec; ++k) if (k == (sel & (kVec - 1))) { pd = p[k]; wd = w[k]; }
-            pd = __shfl_sync(0xffffffffu, pd, sel / kVec);
-            wd = __shfl_sync(0xffffffffu, wd, sel / kVec);
-            const int tok = ((int)rank * nw + wst) * len - phase + chosen * 256 + sel;
-            if (lane == 0) st_cluster4(smem_u32(&res[t]), 0u, __int_as_float(min(max(tok, 0), P.N - 1)), pd, wd, 0.f);
+                for (int k = 0; k < kVec; ++k) if (k == (sel & (kVec - 1))) { pd = p[k]; wd = w[k]; }
+                pd = __shfl_sync(0xffffffffu, pd, sel / kVec);
+                wd = __shfl_sync(0xffffffffu, wd, sel / kVec);
+                const int tok = (s_lo + wst) * len - phase + chosen * 256 + sel;
+                if (lane == 0) st_cluster4(smem_u32(&res[t]), 0u, __int_as_float(min(max(tok, 0), P.N - 1)), pd, wd, 0.f);
+            }
         }
         cluster_sync();
         if (rank == 0 && tid < nt) {
             const int dtok = __float_as_int(res[tid].x);
             const float pd = res[tid].y, qd = res[tid].z * inv_s;
-            const bool acc = u1 * qd < pd;
+            const bool acc = u_test * qd < pd;
             const long long o = (long long)row * P.trials + base + tid;
             if (P.draft_token) P.draft_token[o] = dtok;
             if (P.accepted) P.accepted[o] = acc ? 1 : 0;
