@@ -10,9 +10,10 @@
 // segment (cp.async.bulk on a barrier of its own, the few elements a 16-byte copy cannot cover by plain loads, so
 // any row alignment will do), takes its own maximum as the scale of its exponentials, and leaves one record.  The
 // CTAs then exchange one record each through distributed shared memory (theta, 1/Z_p, 1/Z_q), the warps finish
-// their segment sums of w, min(p, q~), max(0, p - q~) and p, and a second exchange hands every CTA the sums of all
-// segments.  The CTA whose segment a draw falls into makes the draw from shared memory, its warps sharing the
-// segment's 256-position chunks; CTA 0 collects the draws of a row and writes the outputs.  Two exchanges and one collection: three cluster barriers per row.
+// their segment sums of w, min(p, q~), max(0, p - q~) and p and leave them in CTA 0.  The other CTAs are done then and
+// make room for the next rows; CTA 0 draws: prefix sums over the segments, the draw's segment read again (from L2), its
+// 256-position chunks shared by the warps.  (Draws made in place by the CTA that holds the segment kept whole clusters
+// waiting for two chains of dependent loads: 212 instead of XXX us for 320 rows of 128k with a prior.)
 //
 // Four variants:
 //   kVarSparse  N >= 4096, Eq. rdk-taylor with p itself.  A token that is not kept has q~ = theta x < p, x = p / N, so such
@@ -24,6 +25,7 @@
 //               the segment beside the logits.
 //   kVarGiven   w in place of q'.
 #include <atomic>
+#include <type_traits>
 #ifdef RDK_TUNE
 #include <stdlib.h>
 #endif
@@ -44,7 +46,7 @@ constexpr int kRegSlots = 8;                        // kept tokens per lane held
 constexpr unsigned kCluSpinDefault = 1u << 22;
 
 struct CluGeo {
-    int per;                 // vectors of 8 positions per warp
+    int per;                 // vectors of 8 positions per warp, a multiple of 32
     uint32_t zoff_p, zoff_q; // byte offsets of the prior and of the q' array in dynamic shared memory
     uint32_t tag;            // marks this call's arrival counters
     unsigned spin_limit;
@@ -166,7 +168,7 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     __shared__ __align__(16) double cdf[3][kCluMaxSeg];          // their prefix sums (w, residual, p)
     __shared__ __align__(16) float4 xrec[kCluMaxCtas][2];        // one record per CTA of the cluster
     __shared__ __align__(16) float wrec[kCluMaxWarps][8];
-    __shared__ __align__(16) float4 res[2 * kCluRound];          // CTA 0: draft (first half) and residual draws of a round
+    __shared__ __align__(16) float4 res[2 * kCluRound];          // draft (first half) and residual draws of a round
     __shared__ float dsum[2 * kCluRound][kCluMaxChunks];         // a draw's sums over the chunks of its segment
     __shared__ __align__(8) unsigned long long wbar[kCluMaxWarps];
     __shared__ __align__(16) float4 tot_s[2];
@@ -242,7 +244,7 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
             if (VAR == kVarGiven) sts32(qb + o * 4u, 0u);
         }
         if (kDense && kLinear)
-            for (int i = lane; i < len / 4; i += 32) sts128(qb + (uint32_t)i * 16u, 0.f, 0.f, 0.f, 0.f);
+            for (int i = 0; i < len / 128; ++i) sts128(qb + (uint32_t)(i * 32 + lane) * 16u, 0.f, 0.f, 0.f, 0.f);
     }
     // uniforms of the first round of draws: lane t < 16 has those of the draft draw of trial t, lane 16 + t of its residual draw
     const int trial = lane & (kCluRound - 1), kind = lane / kCluRound;
@@ -256,17 +258,24 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     // together), pos = -1 and a drafter value of no weight beyond the last
     auto load_kept = [&](int il, float* y, int* pos) {
         int i[4];
+        const bool full = il - lane + 128 <= cnt;                // (the same in every lane)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) i[k] = r0 + min(il + k * 32, cnt - 1);
+        for (int k = 0; k < 4; ++k) i[k] = r0 + il + k * 32;
+        if (!full) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) i[k] = min(i[k], r0 + cnt - 1);
+        }
         if (!identity) {
 #pragma unroll
             for (int k = 0; k < 4; ++k) i[k] = __ldg(P.slot + i[k]);
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k) { y[k] = to_float<TY>(yrow[i[k]]); pos[k] = __ldg(P.ids + i[k]) - seg_tok; }
+        if (!full) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-            if (il + k * 32 >= cnt) { y[k] = KIND == RDK_LOGITS ? -INFINITY : 0.f; pos[k] = -1; }
+            for (int k = 0; k < 4; ++k)
+                if (il + k * 32 >= cnt) { y[k] = KIND == RDK_LOGITS ? -INFINITY : 0.f; pos[k] = -1; }
+        }
     };
     float ky[kRegSlots];
     int kpos[kRegSlots];
@@ -304,18 +313,18 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     // Scale of a segment's exponentials: not their maximum (finding it is a pass of its own) but that of the first vectors;
     // any scale gives the same result as long as no sum grows beyond 1e18, in which case (or with nothing but -inf among
     // the first) the visit is repeated with the maximum.
-    const int nv16 = len * (int)es / 16;
-    auto seg_max = [&](uint32_t base, int nv) -> float {
+    const int nit16 = g.per * kVec * (int)es / 512;              // 16-byte vectors per lane
+    auto seg_max = [&](uint32_t base, int nit) -> float {
         MaxAcc<TZ> a;
 #pragma unroll 4
-        for (int v = lane; v < nv; v += 32) a.push(lds128(base + (uint32_t)v * 16u));
+        for (int k = 0; k < nit; ++k) a.push(lds128(base + (uint32_t)(k * 32 + lane) * 16u));
         return warp_max_redux(a.result());
     };
     auto seg_sum = [&](uint32_t base, float off) -> float {
         float2 Ea = splat(0.f), Eb = splat(0.f);
         const float2 l2 = splat(kLog2e), of = splat(off);
 #pragma unroll 4
-        for (int v = lane; v < nv16; v += 32) exp_sum_vec<TZ>(lds128(base + (uint32_t)v * 16u), l2, of, Ea, Eb);
+        for (int k = 0; k < nit16; ++k) exp_sum_vec<TZ>(lds128(base + (uint32_t)(k * 32 + lane) * 16u), l2, of, Ea, Eb);
         return (Ea.x + Ea.y) + (Eb.x + Eb.y);
     };
     float m_w = -INFINITY, mp_w = -INFINITY, zoff = 0.f, poff = 0.f, yoff = 0.f;
@@ -323,9 +332,8 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     float kz[kRegSlots], ke[kRegSlots];                              // e_z and e_y of the first kept tokens
     const uint32_t db = kPrior ? pb : zb;                            // the distribution that enters theta
     for (int attempt = 0; attempt < 2; ++attempt) {
-        const int nv_max = attempt == 0 ? min(nv16, 32) : nv16;
-        m_w = seg_max(zb, nv_max);
-        if (kPrior) mp_w = seg_max(pb, nv_max);
+        m_w = seg_max(zb, attempt == 0 ? 1 : nit16);
+        if (kPrior) mp_w = seg_max(pb, attempt == 0 ? 1 : nit16);
         if (attempt == 1 && kLinear && KIND == RDK_LOGITS) {
             for (int il = kRegSlots * 32 + lane; il < cnt; il += 128) {
                 float y[4];
@@ -374,8 +382,8 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     }
     if (VAR == kVarGiven) {
 #pragma unroll 4
-        for (int v = lane; v < len / 4; v += 32) {
-            const uint4 q = lds128(qb + (uint32_t)v * 16u);
+        for (int k = 0; k < len / 128; ++k) {
+            const uint4 q = lds128(qb + (uint32_t)(k * 32 + lane) * 16u);
             W += (__uint_as_float(q.x) + __uint_as_float(q.y)) + (__uint_as_float(q.z) + __uint_as_float(q.w));
         }
     }
@@ -431,74 +439,44 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     const float fy = y_factor(my_w);
     float inv_s = 1.f;
 
-    // p and w of the 8 positions of vector v (counted over the CTA's segments), from the array of q' (or of w); fyv is the
-    // factor of the segment
-    auto dense_pw = [&](int v, float fyv, float (&p)[kVec], float (&w)[kVec]) {
-        float z[kVec], q[kVec];
-        lds8<TZ>(zb0 + (uint32_t)v * kVec * es, z);
-        lds8<float>(qb0 + (uint32_t)v * kVec * 4u, q);
-#pragma unroll
-        for (int k = 0; k < kVec; ++k) p[k] = ex2(fmaf(z[k], kLog2e, offg)) * inv_zp;
-        if (VAR == kVarGiven) {
-#pragma unroll
-            for (int k = 0; k < kVec; ++k) w[k] = q[k];
-            return;
-        }
-        if (kPrior) {
-            lds8<TZ>(pb0 + (uint32_t)v * kVec * es, z);
-#pragma unroll
-            for (int k = 0; k < kVec; ++k) z[k] = ex2(fmaf(z[k], kLog2e, poffg)) * inv_zpi * inv_n;
-        } else {
-#pragma unroll
-            for (int k = 0; k < kVec; ++k) z[k] = p[k] * inv_n;
-        }
-#pragma unroll
-        for (int k = 0; k < kVec; ++k) q[k] *= fyv;
-        redistribute8(z, q, theta, small, w);
+    // p and w of two neighbouring positions, from their logits (pr: prior's) and e_y (or w)
+    const float fz = (m_w > -INFINITY ? ex2((m_w - tot_m) * kLog2e) : 0.f) * inv_zp;      // e on the segment's scale -> p
+    const float xs = kPrior ? (mp_w > -INFINITY ? ex2((mp_w - tot_mp) * kLog2e) : 0.f) * inv_zpi * inv_n : fz * inv_n;    // -> x
+    const float2 l2e2 = splat(kLog2e), zoff2 = splat(zoff), poff2 = splat(poff), fz2 = splat(fz), xs2 = splat(xs), fy2 = splat(fy), th2 = splat(theta), neg2 = splat(-1.f), one2 = splat(1.f);
+    auto dense_pair = [&](float2 z, float2 pr, float2 q, float2& p, float2& w) {
+        const float2 e = ex2_2(ffma2(z, l2e2, zoff2));
+        p = fmul2(e, fz2);
+        if (VAR == kVarGiven) { w = q; return; }
+        const float2 x = fmul2(kPrior ? ex2_2(ffma2(pr, l2e2, poff2)) : e, xs2), qp = fmul2(q, fy2);
+        const float2 t = fmul2(x, ffma2(qp, neg2, th2));                                   // x (theta - q')
+        const float2 r = small ? make_float2(__frcp_rn(1.f + x.x), __frcp_rn(1.f + x.y)) : ffma2(x, neg2, one2);
+        w = ffma2(t, r, qp);
     };
-    // the same where q' is not at hand as an array: the kept tokens among the 8 are looked up in the index
-    auto sparse_pw = [&](int v, float (&p)[kVec], float (&w)[kVec]) {
-        float z[kVec], pr[kVec], y[kVec];
-        lds8<TZ>(zb0 + (uint32_t)v * kVec * es, z);
-        if (kPrior) lds8<TZ>(pb0 + (uint32_t)v * kVec * es, pr);
-        const int jb = (int)rank * nw * len - phase + v * kVec, wi = jb >> 5, sh = jb & 31;
-        const bool in = jb < P.N;
-        const uint32_t lo = wi >= 0 && in ? __ldg(P.mask + wi) : 0u;
-        const uint32_t hi = in && (wi + 1) * 32 < P.N ? __ldg(P.mask + wi + 1) : 0u;
-        const int rw = wi >= 0 && in ? __ldg(P.rank + wi) : 0;
-        const uint32_t mb = __funnelshift_r(lo, hi, sh) & 0xffu;
-        const int rb = wi >= 0 ? rw + __popc(lo & ((1u << sh) - 1u)) : 0;
-        // independent loads: a token that is not kept reads what the first kept one does (or entry 0)
-        int i[kVec];
+    // the four pairs of vector k * 32 + lane of the segment
+    auto dense_vec = [&](int k, float2 (&p)[4], float2 (&w)[4]) {
+        const uint32_t v = (uint32_t)(k * 32 + lane);
+        float z[kVec], pr[kVec], q[kVec];
+        lds8<TZ>(zb + v * kVec * es, z);
+        if (kPrior) lds8<TZ>(pb + v * kVec * es, pr);
+        lds8<float>(qb + v * 32u, q);
 #pragma unroll
-        for (int k = 0; k < kVec; ++k) i[k] = (mb >> k) & 1u ? rb + __popc(mb & ((1u << k) - 1u)) : (mb ? rb : 0);
-        if (!identity) {
-#pragma unroll
-            for (int k = 0; k < kVec; ++k) i[k] = __ldg(P.slot + i[k]);
-        }
-#pragma unroll
-        for (int k = 0; k < kVec; ++k) y[k] = to_float<TY>(yrow[i[k]]);
-#pragma unroll
-        for (int k = 0; k < kVec; ++k) {
-            p[k] = ex2(fmaf(z[k], kLog2e, offg)) * inv_zp;
-            const float x = kPrior ? ex2(fmaf(pr[k], kLog2e, poffg)) * inv_zpi * inv_n : p[k] * inv_n;
-            const float qp = (mb >> k) & 1u ? (KIND == RDK_LOGITS ? ex2(fmaf(y[k], kLog2e, yoffg)) : y[k]) * inv_zq : 0.f;
-            w[k] = redistribute1(x, qp, theta);
-        }
+        for (int h = 0; h < 4; ++h)
+            dense_pair(make_float2(z[2 * h], z[2 * h + 1]), kPrior ? make_float2(pr[2 * h], pr[2 * h + 1]) : splat(0.f), make_float2(q[2 * h], q[2 * h + 1]), p[h], w[h]);
     };
+    const int nit = g.per / 32;                          // vectors of 8 positions per lane
 
     // ---- S.  Sum w = 1 + O(N^-2), because sum q' = 1 and the first-order terms cancel: taken as 1 from N = 4096 on -----
     if (VAR == kVarGiven) {
         inv_s = P.w_as_given ? 1.f : 1.f / tot_a.w;
     } else if (kDense && small) {                       // a small vocabulary: one CTA has the whole row
-        float s = 0.f;
-        for (int v = lane; v < g.per; v += 32) {
-            float p[kVec], w[kVec];
-            dense_pw(warp * g.per + v, fy, p, w);
+        float2 s2 = splat(0.f);
+        for (int k = 0; k < nit; ++k) {
+            float2 p[4], w[4];
+            dense_vec(k, p, w);
 #pragma unroll
-            for (int k = 0; k < kVec; ++k) s += w[k];
+            for (int h = 0; h < 4; ++h) s2 = fadd2(s2, w[h]);
         }
-        s = warp_sum(s);
+        float s = warp_sum(s2.x + s2.y);
         if (lane == 0) part_s[warp] = s;
         __syncthreads();
         s = lane < nw ? part_s[lane] : 0.f;
@@ -507,9 +485,7 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
 
     // ---- second visit: the segment's sums of w, min(p, q~), max(0, p - q~), p -----------------------------------------
     float4 sums;
-    const float fz = (m_w > -INFINITY ? ex2((m_w - tot_m) * kLog2e) : 0.f) * inv_zp;      // e on the segment's scale -> p
     if (VAR == kVarSparse) {
-        const float xs = fz * inv_n;
         float ak = 0.f;
 #pragma unroll
         for (int k = 0; k < kRegSlots; ++k) {
@@ -536,19 +512,17 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
         const float Kw = fy * Zq - fy * xs * th + theta * xs * K;
         sums = make_float4(oov + Kw, oov + ak, fmaxf(0.f, segP - (oov + ak)), segP);
     } else if (VAR == kVarPrior) {
-        const float xs = (mp_w > -INFINITY ? ex2((mp_w - tot_mp) * kLog2e) : 0.f) * inv_zpi * inv_n;
         // all tokens as if not kept, w = theta x (1 - x); then the kept ones' difference (what they count too much is
         // theta x, smaller than 1 / N of a probability: nothing cancels)
         float2 sw2 = splat(0.f), sa2 = splat(0.f);
-        const float2 l2 = splat(kLog2e), zo = splat(zoff), po = splat(poff), f2 = splat(fz), x2 = splat(xs), t2 = splat(theta), m1 = splat(-1.f), p1 = splat(1.f);
         auto pair = [&](float2 z, float2 pr) {
-            const float2 p = fmul2(ex2_2(ffma2(z, l2, zo)), f2), x = fmul2(ex2_2(ffma2(pr, l2, po)), x2);
-            const float2 w = fmul2(fmul2(t2, x), ffma2(x, m1, p1));
+            const float2 p = fmul2(ex2_2(ffma2(z, l2e2, zoff2)), fz2), x = fmul2(ex2_2(ffma2(pr, l2e2, poff2)), xs2);
+            const float2 w = fmul2(fmul2(th2, x), ffma2(x, neg2, one2));
             sw2 = fadd2(sw2, w); sa2 = fadd2(sa2, make_float2(fminf(p.x, w.x), fminf(p.y, w.y)));
         };
 #pragma unroll 2
-        for (int v = lane; v < nv16; v += 32) {
-            const uint4 qz = lds128(zb + (uint32_t)v * 16u), qp = lds128(pb + (uint32_t)v * 16u);
+        for (int k = 0; k < nit16; ++k) {
+            const uint4 qz = lds128(zb + (uint32_t)(k * 32 + lane) * 16u), qp = lds128(pb + (uint32_t)(k * 32 + lane) * 16u);
             if (sizeof(TZ) == 2) {
                 pair(make_float2(bf16_lo(qz.x), bf16_hi(qz.x)), make_float2(bf16_lo(qp.x), bf16_hi(qp.x)));
                 pair(make_float2(bf16_lo(qz.y), bf16_hi(qz.y)), make_float2(bf16_lo(qp.y), bf16_hi(qp.y)));
@@ -580,31 +554,37 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
         sw = warp_sum(sw); sa = warp_sum(sa);
         sums = make_float4(sw, sa, fmaxf(0.f, segP - sa), segP);
     } else {
-        float sw = 0.f, sa = 0.f, sr = 0.f, sp = 0.f;
+        float2 sw2 = splat(0.f), sa2 = splat(0.f), sr2 = splat(0.f);
+        const float2 is2 = splat(inv_s);
         float* qrow = P.qtilde ? P.qtilde + (long long)row * P.N : nullptr;
         // the row of q~ and the positions share their 16-byte phase: store vectors straight away, else by way of shared memory
         const bool straight = qrow && ((reinterpret_cast<uintptr_t>(qrow) - 4u * (unsigned)phase) & 15u) == 0;
-        for (int v = lane; v < g.per; v += 32) {
-            float p[kVec], w[kVec];
-            dense_pw(warp * g.per + v, fy, p, w);
+        for (int k = 0; k < nit; ++k) {
+            float2 p[4], w[4];
+            dense_vec(k, p, w);
 #pragma unroll
-            for (int k = 0; k < kVec; ++k) {
-                const float qt = w[k] * inv_s;
-                sw += w[k]; sp += p[k];
-                sa += fminf(p[k], qt); sr += fmaxf(0.f, p[k] - qt);
-                w[k] = qt;
+            for (int h = 0; h < 4; ++h) {
+                sw2 = fadd2(sw2, w[h]);
+                w[h] = fmul2(w[h], is2);                             // q~
+                const float2 a = make_float2(fminf(p[h].x, w[h].x), fminf(p[h].y, w[h].y));
+                sa2 = fadd2(sa2, a);
+                sr2 = fadd2(sr2, ffma2(a, neg2, p[h]));              // max(0, p - q~)
             }
             if (kLinear && qrow) {
-                const int tok = seg_tok + v * kVec;
+                const int tok = seg_tok + (k * 32 + lane) * kVec;
                 if (straight && tok >= 0 && tok + kVec <= P.N) {
-                    reinterpret_cast<float4*>(qrow + tok)[0] = make_float4(w[0], w[1], w[2], w[3]);
-                    reinterpret_cast<float4*>(qrow + tok)[1] = make_float4(w[4], w[5], w[6], w[7]);
+                    reinterpret_cast<float4*>(qrow + tok)[0] = make_float4(w[0].x, w[0].y, w[1].x, w[1].y);
+                    reinterpret_cast<float4*>(qrow + tok)[1] = make_float4(w[2].x, w[2].y, w[3].x, w[3].y);
                 } else if (straight) {
 #pragma unroll
-                    for (int k = 0; k < kVec; ++k) if (tok + k >= 0 && tok + k < P.N) qrow[tok + k] = w[k];
+                    for (int h = 0; h < 4; ++h) {
+                        if (tok + 2 * h >= 0 && tok + 2 * h < P.N) qrow[tok + 2 * h] = w[h].x;
+                        if (tok + 2 * h + 1 >= 0 && tok + 2 * h + 1 < P.N) qrow[tok + 2 * h + 1] = w[h].y;
+                    }
                 } else {
-                    sts128(qb + (uint32_t)v * 32u, w[0], w[1], w[2], w[3]);
-                    sts128(qb + (uint32_t)v * 32u + 16u, w[4], w[5], w[6], w[7]);
+                    const uint32_t a = qb + (uint32_t)(k * 32 + lane) * 32u;
+                    sts128(a, w[0].x, w[0].y, w[1].x, w[1].y);
+                    sts128(a + 16u, w[2].x, w[2].y, w[3].x, w[3].y);
                 }
             }
         }
@@ -612,14 +592,15 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
             __syncwarp();
             for (int t = t0 + lane; t < t1; t += 32) qrow[t] = __uint_as_float(lds32(qb + (uint32_t)(t - seg_tok) * 4u));
         }
-        const float t = warp_sum4(sw, sa, sr, sp, lane);
-        sums = make_float4(__shfl_sync(0xffffffffu, t, 0), __shfl_sync(0xffffffffu, t, 8), __shfl_sync(0xffffffffu, t, 16), __shfl_sync(0xffffffffu, t, 24));
+        const float t = warp_sum4(sw2.x + sw2.y, sa2.x + sa2.y, sr2.x + sr2.y, 0.f, lane);
+        sums = make_float4(__shfl_sync(0xffffffffu, t, 0), __shfl_sync(0xffffffffu, t, 8), __shfl_sync(0xffffffffu, t, 16), E * fz);
     }
 
-    // ---- second exchange: every CTA gets the sums of all segments -------------------------------------------------------
-    if (lane < (int)C) st_cluster4(smem_u32(&segs[sg]), (uint32_t)lane, sums.x, sums.y, sums.z, sums.w);
-    cluster_sync();
-    if (P.trials == 0 && rank != 0) return;              // nobody reads or writes another CTA's memory from here on
+    // ---- second exchange: CTA 0 gets the sums of all segments; the others are done -----------------------------------------
+    if (lane == 0) st_cluster4(smem_u32(&segs[sg]), 0u, sums.x, sums.y, sums.z, sums.w);
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    if (rank != 0) return;
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     for (int job = warp; job < 4; job += nw) {
         constexpr int kPerLane = kCluMaxSeg / 32;
         const int per_lane = (nseg + 31) >> 5, s0 = lane * per_lane;
@@ -651,28 +632,64 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     }
     __syncthreads();
     const double S_d = cdf[0][nseg - 1], R_d = cdf[1][nseg - 1];
-    if (rank == 0 && tid == 0) {
+    if (tid == 0) {
         if (P.alpha) P.alpha[row] = alpha_s;
         if (P.theta) P.theta[row] = theta;
         if (P.S) P.S[row] = (float)S_d;
         if (P.residual_mass) P.residual_mass[row] = (float)R_d;
     }
 
-    // ---- draws: the warp whose segment holds the threshold makes the draw -----------------------------------------------
+    // ---- draws ------------------------------------------------------------------------------------------------------------
     const bool from_p = !(R_d > 0.0);                    // p and q~ coincide: the replacement comes from p itself
     const double* cdf_r = from_p ? cdf[2] : cdf[1];
-    const int nch = (g.per + 31) / 32;
-    // x of the 8 positions of this lane in chunk ch of the CTA's segment ws: what = 0: w, 1: max(0, p - q~), 2: p
-    auto chunk_x = [&](int ws, int ch, int what, float (&p)[kVec], float (&w)[kVec], float (&x)[kVec]) -> float {
-        const int v = ch * 32 + lane;
+    const int nch = g.per / 32;
+    // x of this lane's 8 positions in chunk ch of segment sgm, read from global memory again: what = 0: w, 1: max(0, p - q~), 2: p
+    auto load_row8 = [&](const auto* src, int jb, float fill, float (&v)[kVec]) {
+        using T = typename std::remove_cv<typename std::remove_pointer<decltype(src)>::type>::type;
+        if (jb >= 0) {
+            load8<T>(src, jb, P.N, (reinterpret_cast<uintptr_t>(src + jb) & 15u) == 0, fill, v);
+        } else {
 #pragma unroll
-        for (int k = 0; k < kVec; ++k) { p[k] = 0.f; w[k] = 0.f; }
-        if (v < g.per) {
-            if (kDense) {
-                dense_pw(ws * g.per + v, y_factor(wrec[ws][4]), p, w);
-            } else {
-                sparse_pw(ws * g.per + v, p, w);
+            for (int k = 0; k < kVec; ++k) v[k] = jb + k >= 0 && jb + k < P.N ? to_float<T>(src[jb + k]) : fill;
+        }
+    };
+    auto chunk_x = [&](int sgm, int ch, int what, float (&p)[kVec], float (&w)[kVec], float (&x)[kVec]) -> float {
+        const int jb = sgm * len - phase + (ch * 32 + lane) * kVec;
+        float z[kVec];
+        load_row8(zrow, jb, -INFINITY, z);
+        if (VAR == kVarGiven) {
+            load_row8(P.w + (long long)row * P.w_stride, jb, 0.f, w);
+#pragma unroll
+            for (int k = 0; k < kVec; ++k) p[k] = ex2(fmaf(z[k], kLog2e, offg)) * inv_zp;
+        } else {
+            // the kept tokens among the 8, looked up in the index
+            const int wi = jb >> 5, sh = jb & 31;
+            const bool in = jb < P.N;
+            const uint32_t lo = wi >= 0 && in ? __ldg(P.mask + wi) : 0u;
+            const uint32_t hi = in && (wi + 1) * 32 < P.N ? __ldg(P.mask + wi + 1) : 0u;
+            const int rw = wi >= 0 && in ? __ldg(P.rank + wi) : 0;
+            float pr[kVec];
+            if (kPrior) load_row8(prow, jb, -INFINITY, pr);
+            const uint32_t mb = __funnelshift_r(lo, hi, sh) & 0xffu;
+            const int rb = wi >= 0 ? rw + __popc(lo & ((1u << sh) - 1u)) : 0;
+            // independent loads: a token that is not kept reads what the first kept one does (or entry 0)
+            int i[kVec];
+#pragma unroll
+            for (int k = 0; k < kVec; ++k) i[k] = (mb >> k) & 1u ? rb + __popc(mb & ((1u << k) - 1u)) : (mb ? rb : 0);
+            if (!identity) {
+#pragma unroll
+                for (int k = 0; k < kVec; ++k) i[k] = __ldg(P.slot + i[k]);
             }
+            float y[kVec];
+#pragma unroll
+            for (int k = 0; k < kVec; ++k) y[k] = to_float<TY>(yrow[i[k]]);
+#pragma unroll
+            for (int k = 0; k < kVec; ++k) {
+                p[k] = ex2(fmaf(z[k], kLog2e, offg)) * inv_zp;
+                pr[k] = kPrior ? ex2(fmaf(pr[k], kLog2e, poffg)) * inv_zpi * inv_n : p[k] * inv_n;
+                y[k] = (mb >> k) & 1u ? (KIND == RDK_LOGITS ? ex2(fmaf(y[k], kLog2e, yoffg)) : y[k]) * inv_zq : 0.f;
+            }
+            redistribute8(pr, y, theta, small, w);
         }
         float s = 0.f;
 #pragma unroll
@@ -688,58 +705,56 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
         if (base && on) { u_draw = __ldg(u_row + (base + trial) * 4 + 2 * kind); u_test = __ldg(u_row + (base + trial) * 4 + 1); }
         const double* c = kind == 0 ? cdf[0] : cdf_r;
         const double thr = (double)u_draw * c[nseg - 1];
-        // the draw's segment is the first whose prefix sum exceeds the threshold (the last one if rounding leaves none): is it here?
-        const int s_lo = (int)rank * nw, s_hi = s_lo + nw;
-        const bool below = s_lo > 0 && c[s_lo - 1] > thr, beyond = s_hi < nseg && !(c[s_hi - 1] > thr);
-        const uint32_t here = __ballot_sync(0xffffffffu, on && !below && !beyond);
-        if (here) {
-            const int ws = min(first_above(c + s_lo, nw, thr), nw - 1);
-            const float rem = (float)(thr - (s_lo + ws ? c[s_lo + ws - 1] : 0.0));
-            float p[kVec], w[kVec], x[kVec];
-            int k_item = 0, held = -1;                               // the chunk (by its number) that p, w, x belong to
-            for (uint32_t todo = here; todo; todo &= todo - 1u) {        // the chunks' sums, chunks dealt out to the warps
-                const int t = __ffs(todo) - 1, wst = __shfl_sync(0xffffffffu, ws, t), what = t < kCluRound ? 0 : (from_p ? 2 : 1);
-                for (int ch = 0; ch < nch; ++ch) {
-                    if (k_item++ % nw != warp) continue;
-                    held = k_item - 1;
-                    const float s = warp_sum(chunk_x(wst, ch, what, p, w, x));
+        // the draw's segment is the first whose prefix sum exceeds the threshold (the last one if rounding leaves none)
+        const int seg = min(first_above(c, nseg, thr), nseg - 1);
+        const float rem = (float)(thr - (seg ? c[seg - 1] : 0.0));
+        const uint32_t all = __ballot_sync(0xffffffffu, on);
+        float p[kVec], w[kVec], x[kVec];
+        int k_item = 0, turn = 0, held = -1;                     // held: the chunk (by its number) that p, w, x belong to
+        for (uint32_t todo = all; todo; todo &= todo - 1u) {     // the chunks' sums, chunks dealt out to the warps
+            const int t = __ffs(todo) - 1, sgm = __shfl_sync(0xffffffffu, seg, t), what = t < kCluRound ? 0 : (from_p ? 2 : 1);
+            for (int ch = 0; ch < nch; ++ch, ++k_item) {
+                if (turn == warp) {
+                    held = k_item;
+                    const float s = warp_sum(chunk_x(sgm, ch, what, p, w, x));
                     if (lane == 0) dsum[t][ch] = s;
                 }
-            }
-            __syncthreads();
-            k_item = 0;
-            for (uint32_t todo = here; todo; todo &= todo - 1u, k_item += nch) {
-                const int t = __ffs(todo) - 1, wst = __shfl_sync(0xffffffffu, ws, t), what = t < kCluRound ? 0 : (from_p ? 2 : 1);
-                const float remt = __shfl_sync(0xffffffffu, rem, t);
-                float cum = 0.f, before = 0.f;
-                int chosen = -1, last_pos = -1;
-                for (int ch = 0; ch < nch; ++ch) {
-                    const float s = dsum[t][ch];
-                    if (s > 0.f) {
-                        if (chosen < 0 && cum + s > remt) { chosen = ch; before = cum; }
-                        last_pos = ch;
-                        cum += s;
-                    }
-                }
-                const float r_in = chosen < 0 ? INFINITY : remt - before;    // rounding left no token: the last positive one
-                if (chosen < 0) chosen = max(last_pos, 0);
-                if ((k_item + chosen) % nw != warp) continue;                // the warp that summed the chunk picks the token,
-                if (held != k_item + chosen) {                               // from its registers unless it went on to another chunk
-                    (void)chunk_x(wst, chosen, what, p, w, x);
-                    held = k_item + chosen;
-                }
-                const int sel = max(pick_in_segment(x, r_in, lane), 0);
-                float pd = 0.f, wd = 0.f;
-#pragma unroll
-                for (int k = 0; k < kVec; ++k) if (k == (sel & (kVec - 1))) { pd = p[k]; wd = w[k]; }
-                pd = __shfl_sync(0xffffffffu, pd, sel / kVec);
-                wd = __shfl_sync(0xffffffffu, wd, sel / kVec);
-                const int tok = (s_lo + wst) * len - phase + chosen * 256 + sel;
-                if (lane == 0) st_cluster4(smem_u32(&res[t]), 0u, __int_as_float(min(max(tok, 0), P.N - 1)), pd, wd, 0.f);
+                if (++turn == nw) turn = 0;
             }
         }
-        cluster_sync();
-        if (rank == 0 && tid < nt) {
+        __syncthreads();
+        k_item = 0;
+        for (uint32_t todo = all; todo; todo &= todo - 1u, k_item += nch) {
+            const int t = __ffs(todo) - 1, sgm = __shfl_sync(0xffffffffu, seg, t), what = t < kCluRound ? 0 : (from_p ? 2 : 1);
+            const float remt = __shfl_sync(0xffffffffu, rem, t);
+            float cum = 0.f, before = 0.f;
+            int chosen = -1, last_pos = -1;
+            for (int ch = 0; ch < nch; ++ch) {
+                const float s = dsum[t][ch];
+                if (s > 0.f) {
+                    if (chosen < 0 && cum + s > remt) { chosen = ch; before = cum; }
+                    last_pos = ch;
+                    cum += s;
+                }
+            }
+            const float r_in = chosen < 0 ? INFINITY : remt - before;    // rounding left no token: the last positive one
+            if (chosen < 0) chosen = max(last_pos, 0);
+            if ((k_item + chosen) % nw != warp) continue;                // the warp that summed the chunk picks the token,
+            if (held != k_item + chosen) {                               // from its registers unless it went on to another chunk
+                (void)chunk_x(sgm, chosen, what, p, w, x);
+                held = k_item + chosen;
+            }
+            const int sel = max(pick_in_segment(x, r_in, lane), 0);
+            float pd = 0.f, wd = 0.f;
+#pragma unroll
+            for (int k = 0; k < kVec; ++k) if (k == (sel & (kVec - 1))) { pd = p[k]; wd = w[k]; }
+            pd = __shfl_sync(0xffffffffu, pd, sel / kVec);
+            wd = __shfl_sync(0xffffffffu, wd, sel / kVec);
+            const int tok = sgm * len - phase + chosen * 256 + sel;
+            if (lane == 0) res[t] = make_float4(__int_as_float(min(max(tok, 0), P.N - 1)), pd, wd, 0.f);
+        }
+        __syncthreads();
+        if (tid < nt) {
             const int dtok = __float_as_int(res[tid].x);
             const float pd = res[tid].y, qd = res[tid].z * inv_s;
             const bool acc = u_test * qd < pd;
@@ -772,7 +787,7 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
                 }
             }
         }
-        if (base + kCluRound < P.trials) cluster_sync();         // CTA 0 has read the round's draws
+        if (base + kCluRound < P.trials) __syncthreads();        // the round's draws have been read
     }
 }
 
@@ -800,6 +815,7 @@ static bool plan_cluster(int N, int rows, size_t es, int variant, bool prior, Cl
 #endif
     s.C = C; s.nw = nw;
     s.per = (int)((positions + (long long)C * nw * kVec - 1) / ((long long)C * nw * kVec));
+    s.per = (s.per + 31) / 32 * 32;
     s.smem = (size_t)nw * s.per * kVec * bytes;
     return s.smem <= (size_t)kCluDynamic && s.per <= 32 * kCluMaxChunks;
 }
