@@ -74,6 +74,9 @@ typedef enum rdk_mode { RDK_MODE_LINEAR = 0, RDK_MODE_PRECOMPUTED_W = 1 } rdk_mo
  * stands; the draft token is still drawn in proportion to w (a draw needs a distribution); the S
  * output remains sum(w).  The caller guarantees 0 <= w_j and sum(w) <= 1.                         */
 #define RDK_FLAG_W_AS_GIVEN 2
+/* RDK_FLAG_PAD_SEQUENCES (rdk_emit_sequences only): entries of seq_tokens beyond seq_len are set to -1
+ * instead of being left untouched.                                                                */
+#define RDK_FLAG_PAD_SEQUENCES 4
 
 /* Which kernel a call of the linear mode takes (see rdk_sample_route).                           */
 typedef enum rdk_route { RDK_ROUTE_ROW_KERNEL = 0, RDK_ROUTE_STREAM_KERNEL = 1 } rdk_route;
@@ -345,9 +348,10 @@ int rdk_stream_geometry(int32_t N, int32_t n, int32_t target_dtype, int32_t draf
  *   bonus_target  device [batch, N] target logits of problem->target_dtype, row stride in elements
  *                 (0 means N)
  *   uniforms, draft_token, accepted, out_token: as given to / produced by rdk_sample_and_verify
- *   seq_tokens    device int32 [batch, trials, positions + 1] (entries beyond seq_len are untouched)
+ *   seq_tokens    device int32 [batch, trials, positions + 1] (entries beyond seq_len are untouched,
+ *                 or -1 with RDK_FLAG_PAD_SEQUENCES)
  *   seq_len       device int32 [batch, trials]
- * Only problem->N, batch, positions and target_dtype are read.
+ * Only problem->N, batch, positions, target_dtype and the flag above are read.
  * ------------------------------------------------------------------------------------------- */
 int rdk_emit_sequences(const rdk_problem* problem, const void* bonus_target, int64_t bonus_row_stride,
                        const float* uniforms, int32_t trials, const int32_t* draft_token,
