@@ -13,7 +13,7 @@
 // their segment sums of w, min(p, q~), max(0, p - q~) and p and leave them in CTA 0.  The other CTAs are done then and
 // make room for the next rows; CTA 0 draws: prefix sums over the segments, the draw's segment read again (from L2), its
 // 256-position chunks shared by the warps.  (Draws made in place by the CTA that holds the segment kept whole clusters
-// waiting for two chains of dependent loads: 212 instead of XXX us for 320 rows of 128k with a prior.)
+// waiting for two chains of dependent loads: 212 instead of 156 us for 320 rows of 128k with a prior.)
 //
 // Four variants:
 //   kVarSparse  N >= 4096, Eq. rdk-taylor with p itself.  A token that is not kept has q~ = theta x < p, x = p / N, so such
@@ -26,9 +26,6 @@
 //   kVarGiven   w in place of q'.
 #include <atomic>
 #include <type_traits>
-#ifdef RDK_TUNE
-#include <stdlib.h>
-#endif
 
 #include "rdk_device.cuh"
 #include "rdk_row.cuh"
@@ -44,6 +41,13 @@ constexpr int kCluRound = 16;                       // trials settled between tw
 constexpr int kCluMaxChunks = 32;                   // 256-position chunks of a segment
 constexpr int kRegSlots = 8;                        // kept tokens per lane held in registers
 constexpr unsigned kCluSpinDefault = 1u << 22;
+
+// What CTA 0 needs for the draws lies where its part of the row was: nobody reads that any more by then.
+struct DrawSmem {
+    double cdf[3][kCluMaxSeg];                      // prefix sums of the segments' w, residual, p
+    float4 res[2 * kCluRound];                      // draft (first half) and residual draws of a round
+    float dsum[2 * kCluRound][kCluMaxChunks];       // a draw's sums over the chunks of its segment
+};
 
 struct CluGeo {
     int per;                 // vectors of 8 positions per warp, a multiple of 32
@@ -165,11 +169,8 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     constexpr uint32_t es = (uint32_t)sizeof(TZ);
     extern __shared__ __align__(128) unsigned char csm[];
     __shared__ __align__(16) float4 segs[kCluMaxSeg];            // per segment: sums of w, min(p, q~), max(0, p - q~), p
-    __shared__ __align__(16) double cdf[3][kCluMaxSeg];          // their prefix sums (w, residual, p)
     __shared__ __align__(16) float4 xrec[kCluMaxCtas][2];        // one record per CTA of the cluster
     __shared__ __align__(16) float wrec[kCluMaxWarps][8];
-    __shared__ __align__(16) float4 res[2 * kCluRound];          // draft (first half) and residual draws of a round
-    __shared__ float dsum[2 * kCluRound][kCluMaxChunks];         // a draw's sums over the chunks of its segment
     __shared__ __align__(8) unsigned long long wbar[kCluMaxWarps];
     __shared__ __align__(16) float4 tot_s[2];
     __shared__ float alpha_s, part_s[kCluMaxWarps];
@@ -601,6 +602,8 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     if (rank != 0) return;
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    DrawSmem& ds = *reinterpret_cast<DrawSmem*>(csm);
+    double (&cdf)[3][kCluMaxSeg] = ds.cdf;
     for (int job = warp; job < 4; job += nw) {
         constexpr int kPerLane = kCluMaxSeg / 32;
         const int per_lane = (nseg + 31) >> 5, s0 = lane * per_lane;
@@ -717,7 +720,7 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
                 if (turn == warp) {
                     held = k_item;
                     const float s = warp_sum(chunk_x(sgm, ch, what, p, w, x));
-                    if (lane == 0) dsum[t][ch] = s;
+                    if (lane == 0) ds.dsum[t][ch] = s;
                 }
                 if (++turn == nw) turn = 0;
             }
@@ -730,7 +733,7 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
             float cum = 0.f, before = 0.f;
             int chosen = -1, last_pos = -1;
             for (int ch = 0; ch < nch; ++ch) {
-                const float s = dsum[t][ch];
+                const float s = ds.dsum[t][ch];
                 if (s > 0.f) {
                     if (chosen < 0 && cum + s > remt) { chosen = ch; before = cum; }
                     last_pos = ch;
@@ -751,18 +754,18 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
             pd = __shfl_sync(0xffffffffu, pd, sel / kVec);
             wd = __shfl_sync(0xffffffffu, wd, sel / kVec);
             const int tok = sgm * len - phase + chosen * 256 + sel;
-            if (lane == 0) res[t] = make_float4(__int_as_float(min(max(tok, 0), P.N - 1)), pd, wd, 0.f);
+            if (lane == 0) ds.res[t] = make_float4(__int_as_float(min(max(tok, 0), P.N - 1)), pd, wd, 0.f);
         }
         __syncthreads();
         if (tid < nt) {
-            const int dtok = __float_as_int(res[tid].x);
-            const float pd = res[tid].y, qd = res[tid].z * inv_s;
+            const int dtok = __float_as_int(ds.res[tid].x);
+            const float pd = ds.res[tid].y, qd = ds.res[tid].z * inv_s;
             const bool acc = u_test * qd < pd;
             const long long o = (long long)row * P.trials + base + tid;
             if (P.draft_token) P.draft_token[o] = dtok;
             if (P.accepted) P.accepted[o] = acc ? 1 : 0;
             if (P.accept_prob) P.accept_prob[o] = (pd >= qd) ? 1.f : pd / qd;
-            if (P.out_token) P.out_token[o] = acc ? dtok : __float_as_int(res[kCluRound + tid].x);
+            if (P.out_token) P.out_token[o] = acc ? dtok : __float_as_int(ds.res[kCluRound + tid].x);
             if (P.arrivals && P.accepted_len) {
                 // the last position of a sequence to arrive counts the accepted prefix (Algorithm 4 step 7).  The word
                 // holds (tag of the call, arrivals), so it needs no initialisation; the last one clears it for a replay.
@@ -794,29 +797,34 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
 // ------------------------------------------------------------------------------------------------
 // host side
 // ------------------------------------------------------------------------------------------------
-constexpr int kCluStatic = 18 * 1024;                            // static shared memory of the kernel, rounded up
+constexpr int kCluStatic = 6 * 1024;                            // static shared memory of the kernel, rounded up
 constexpr int kCluDynamic = 227 * 1024 - kCluStatic;
 
 struct CluShape { int C, nw, per; size_t smem; };
 
-// CTAs per row, warps per CTA and vectors per warp; false when a row does not fit a cluster's shared memory.
-static bool plan_cluster(int N, int rows, size_t es, int variant, bool prior, CluShape& s) {
+// CTAs per row, warps per CTA and vectors per warp; false when a row does not fit a cluster's shared memory.  `lead`: most
+// positions before a row's first token.
+static bool plan_cluster(int N, int rows, size_t es, int variant, bool prior, int lead, CluShape& s) {
     const size_t bytes = es * (prior ? 2 : 1) + (variant == kVarDense || variant == kVarGiven ? 4 : 0);    // per position
-    const long long positions = (long long)N + 8;
-    int C = 1, nw;
+    const long long positions = (long long)N + lead;
+    int C = 1;
     if (N >= kStreamMinN) {
-        while (C < kCluMaxCtas && (long long)C * 8192 < positions) C *= 2;
-        while (C < kCluMaxCtas && rows * C < 148 && positions / C > 2048) C *= 2;
+        // three CTAs to an SM (their phases of copying, exponentials and waiting overlap; with one to an SM a prior of
+        // 128k tokens takes 515 us for 320 rows, with three 147) ...
+        while (C < kCluMaxCtas && (long long)bytes * (positions / C) > 64 * 1024) C *= 2;
+        // ... and, with few rows, enough CTAs to fill the chip four times over, while each has 4096 positions or more (with
+        // less the exchange between the CTAs costs more than the sweep)
+        while (C < kCluMaxCtas && (long long)rows * C < 4 * 148 && positions / C > 4096) C *= 2;
     }
-    nw = (int)((positions / C + 1023) / 1024);
-    nw = nw < 4 ? 4 : (nw > kCluMaxWarps ? kCluMaxWarps : nw);
-#ifdef RDK_TUNE
-    if (getenv("RDK_C") && N >= kStreamMinN) { C = atoi(getenv("RDK_C")); nw = atoi(getenv("RDK_NW")); }
-#endif
-    s.C = C; s.nw = nw;
-    s.per = (int)((positions + (long long)C * nw * kVec - 1) / ((long long)C * nw * kVec));
-    s.per = (s.per + 31) / 32 * 32;
-    s.smem = (size_t)nw * s.per * kVec * bytes;
+    // about eight warps of equally many 256-position chunks each: more warps mean more per-warp overhead, fewer do not
+    // hide each other's latencies (50257 tokens x 160 rows: 8 warps 29 us, 12 35, 16 46)
+    const int chunks = (int)((positions + C * 256 - 1) / (C * 256));
+    const int per_warp = chunks <= 8 ? 1 : (chunks + 7) / 8;
+    const int nw = (chunks + per_warp - 1) / per_warp;
+    s.C = C; s.nw = nw < 4 ? 4 : nw;
+    s.per = per_warp * 32;
+    s.smem = (size_t)s.nw * s.per * kVec * bytes;
+    if (s.smem < sizeof(DrawSmem)) s.smem = sizeof(DrawSmem);
     return s.smem <= (size_t)kCluDynamic && s.per <= 32 * kCluMaxChunks;
 }
 
@@ -879,7 +887,8 @@ cudaError_t launch_cluster_rows(RowParams P, int mode, int tz, int ty, int kind,
     const int variant = mode == RDK_MODE_PRECOMPUTED_W ? kVarGiven
                         : (P.qtilde || P.N < kStreamMinN ? kVarDense : (P.prior ? kVarPrior : kVarSparse));
     CluShape sh;
-    if (!plan_cluster(P.N, P.rows, es, variant, P.prior != nullptr, sh)) return cudaErrorNotSupported;
+    const bool aligned = !(reinterpret_cast<uintptr_t>(P.target) & 15u) && !((P.target_stride * (long long)es) & 15);
+    if (!plan_cluster(P.N, P.rows, es, variant, P.prior != nullptr, aligned ? 0 : (int)(16 / es) - 1, sh)) return cudaErrorNotSupported;
     if ((long long)P.rows * sh.C > 0x7fffffffLL) return cudaErrorNotSupported;
     CluGeo g;
     g.per = sh.per;
