@@ -1,8 +1,9 @@
-"""ctypes binding of librdk_b200.so: argument marshalling only.
+"""Binding of librdk_b200.so: argument marshalling only.
 
 Every function below has the name of the C entry point it calls (see include/rdk.h), takes torch
 tensors for the device buffers, and passes their data pointers and the current CUDA stream through.
-All arithmetic runs in the CUDA kernels of the library.  There is no fallback: if the shared library
+The calls of a decoding loop are marshalled by the native module _rdk_host (csrc/rdk_host.cpp), the
+others by ctypes.  All arithmetic runs in the CUDA kernels of the library.  There is no fallback: if the shared library
 cannot be loaded, or a call returns an error status, an exception is raised.
 """
 from __future__ import annotations
@@ -16,6 +17,7 @@ import torch
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(HERE, "librdk_b200.so")
+HOST_PATH = os.path.join(HERE, "_rdk_host.so")
 
 RDK_OK = 0
 RDK_ERR_INVALID_ARG, RDK_ERR_BAD_IDS, RDK_ERR_EMPTY_INTERSECTION, RDK_ERR_UNSUPPORTED = 1, 2, 3, 4
@@ -26,6 +28,7 @@ RDK_MODE_LINEAR, RDK_MODE_PRECOMPUTED_W = 0, 1
 RDK_AFF_F32_ROWS, RDK_AFF_BF16_COLS = 0, 1
 RDK_FLAG_ROW_KERNEL = 1
 RDK_FLAG_W_AS_GIVEN = 2
+RDK_FLAG_PAD_SEQUENCES = 4
 RDK_ROUTE_ROW_KERNEL, RDK_ROUTE_STREAM_KERNEL = 0, 1
 
 EXPORTS = [
@@ -125,6 +128,21 @@ def lib() -> C.CDLL:
         L.rdk_test_set_spin_limit.argtypes = [C.c_uint32]
         _lib = L
     return _lib
+
+
+_host = None
+
+
+def host():
+    """Load the binding's native part (once), after the library that it calls."""
+    global _host
+    if _host is None:
+        lib()
+        if not os.path.exists(HOST_PATH):
+            raise RuntimeError(f"{HOST_PATH} is missing: build it with `python -m paper_2506_03206_b200.build`")
+        from . import _rdk_host
+        _host = _rdk_host
+    return _host
 
 
 def _check(status: int, where: str) -> None:
@@ -232,19 +250,16 @@ def rdk_redistribute_exact(index: KeptIndex, drafter: torch.Tensor, M: Dict[str,
                            positions: int, drafter_kind: int = RDK_LOGITS,
                            w_out: Optional[torch.Tensor] = None, ws: Optional[torch.Tensor] = None,
                            status_word: Optional[torch.Tensor] = None):
-    _rows2d(drafter, "drafter")
-    rows = batch * positions
-    pb = make_problem(index, None, drafter, batch, positions, drafter_kind)
     if w_out is None:
-        w_out = torch.empty(rows, index.N, dtype=torch.float32, device=drafter.device)
-    S = torch.empty(rows, dtype=torch.float32, device=drafter.device)
-    wsb = lib().rdk_exact_workspace_bytes(C.byref(pb), M["layout"])
+        w_out = torch.empty(batch * positions, index.N, dtype=torch.float32, device=drafter.device)
     if ws is None:
+        pb = make_problem(index, None, drafter, batch, positions, drafter_kind)
+        wsb = lib().rdk_exact_workspace_bytes(C.byref(pb), M["layout"])
         ws = torch.empty(max(wsb, 256), dtype=torch.uint8, device=drafter.device)
-    a = _aff_struct(M)
-    _check(lib().rdk_redistribute_exact(C.byref(pb), drafter.data_ptr(), C.byref(a), w_out.data_ptr(),
-                                        S.data_ptr(), ws.data_ptr(), ws.numel(), _ptr(status_word), _stream()),
-           "rdk_redistribute_exact")
+    status, S = (_host or host()).exact(index.buffer, index.N, index.n, drafter, M["data"], M["layout"], M["ld"], batch,
+                                        positions, drafter_kind, w_out, ws, status_word)
+    if status:
+        _check(status, "rdk_redistribute_exact")
     return w_out, S, ws
 
 
@@ -267,15 +282,10 @@ def rdk_redistribute_exact_static(index: KeptIndex, drafter: torch.Tensor, M: Di
 
 def rdk_redistribute_linear(index: KeptIndex, target: torch.Tensor, drafter: torch.Tensor, batch: int,
                             positions: int, drafter_kind: int = RDK_LOGITS):
-    _rows2d(target, "target")
-    _rows2d(drafter, "drafter")
-    rows = batch * positions
-    pb = make_problem(index, target, drafter, batch, positions, drafter_kind)
-    qt = torch.empty(rows, index.N, dtype=torch.float32, device=target.device)
-    theta = torch.empty(rows, dtype=torch.float32, device=target.device)
-    S = torch.empty(rows, dtype=torch.float32, device=target.device)
-    _check(lib().rdk_redistribute_linear(C.byref(pb), target.data_ptr(), drafter.data_ptr(), qt.data_ptr(),
-                                         theta.data_ptr(), S.data_ptr(), _stream()), "rdk_redistribute_linear")
+    status, qt, theta, S = (_host or host()).linear(index.buffer, index.N, index.n, target, None, drafter, batch, positions,
+                                                    drafter_kind)
+    if status:
+        _check(status, "rdk_redistribute_linear")
     return qt, theta, S
 
 
@@ -313,20 +323,19 @@ def rdk_sample_and_verify(index: KeptIndex, mode: int, target: torch.Tensor,
                           drafter_kind: int = RDK_LOGITS,
                           out: Optional[Dict[str, torch.Tensor]] = None,
                           ws: Optional[torch.Tensor] = None, flags: int = 0) -> Dict[str, torch.Tensor]:
-    _rows2d(target, "target")
-    rows = batch * positions
-    if uniforms.dtype != torch.float32 or not uniforms.is_contiguous() or uniforms.numel() % (rows * 4):
-        raise ValueError("uniforms must be contiguous float32 [rows, trials, 4]")
-    trials = uniforms.numel() // (rows * 4)
-    pb = make_problem(index, target, drafter, batch, positions, drafter_kind, flags=flags)
-    if out is None:
-        out = alloc_outputs(rows, batch, trials, target.device)
-    o = outputs_struct(out)
-    if ws is None:
-        ws = sample_workspace(pb, mode, trials, target.device)
-    _check(lib().rdk_sample_and_verify(C.byref(pb), mode, target.data_ptr(), _ptr(drafter), _ptr(w),
-                                       0 if w is None else w.stride(0), uniforms.data_ptr(), trials,
-                                       C.byref(o), ws.data_ptr(), ws.numel(), _stream()), "rdk_sample_and_verify")
+    if out is None or ws is None:
+        _rows2d(target, "target")
+        rows = batch * positions
+        trials = uniforms.numel() // (rows * 4)
+        if out is None:
+            out = alloc_outputs(rows, batch, trials, target.device)
+        if ws is None:
+            pb = make_problem(index, target, drafter, batch, positions, drafter_kind, flags=flags)
+            ws = sample_workspace(pb, mode, trials, target.device)
+    status = (_host or host()).sample(index.buffer, index.N, index.n, mode, target, drafter, w, uniforms, batch, positions,
+                                      drafter_kind, flags, out, ws)
+    if status:
+        _check(status, "rdk_sample_and_verify")
     out["_ws"] = ws        # keep the workspace alive until the stream has consumed it
     return out
 
@@ -352,16 +361,9 @@ def rdk_test_set_spin_limit(limit: int) -> None:
 def rdk_emit_sequences(N: int, batch: int, positions: int, bonus_target: torch.Tensor, uniforms: torch.Tensor,
                        draft_token: torch.Tensor, accepted: torch.Tensor, out_token: torch.Tensor):
     """Returns (seq_tokens int32 [batch, trials, positions + 1], seq_len int32 [batch, trials])."""
-    _rows2d(bonus_target, "bonus_target")
-    trials = uniforms.numel() // (batch * positions * 4)
-    pb = rdk_problem()
-    pb.N, pb.n, pb.batch, pb.positions = N, 1, batch, positions
-    pb.target_dtype = _dtype_code(bonus_target)
-    seq = torch.full((batch, trials, positions + 1), -1, dtype=torch.int32, device=bonus_target.device)
-    ln = torch.empty(batch, trials, dtype=torch.int32, device=bonus_target.device)
-    _check(lib().rdk_emit_sequences(C.byref(pb), bonus_target.data_ptr(), bonus_target.stride(0), uniforms.data_ptr(),
-                                    trials, draft_token.data_ptr(), accepted.data_ptr(), out_token.data_ptr(),
-                                    seq.data_ptr(), ln.data_ptr(), _stream()), "rdk_emit_sequences")
+    status, seq, ln = (_host or host()).emit(N, batch, positions, bonus_target, uniforms, draft_token, accepted, out_token)
+    if status:
+        _check(status, "rdk_emit_sequences")
     return seq, ln
 
 
@@ -399,57 +401,26 @@ def rdk_stream_geometry(N: int, n: int, target_dtype: int = RDK_BF16, drafter_dt
     return {k: int(getattr(g, k)) for k, _ in rdk_stream_geometry_t._fields_ if k != "reserved"}
 
 
-def _prior_stride(prior: torch.Tensor, N: int) -> int:
-    """A [N] prior is one row shared by all rows (stride 0); a [rows, N] prior has its row stride."""
-    if prior.dim() == 1:
-        if prior.numel() != N or not prior.is_contiguous():
-            raise ValueError("a shared prior must be a contiguous [N] tensor")
-        return 0
-    _rows2d(prior, "prior")
-    return prior.stride(0)
-
-
 def rdk_redistribute_linear_prior(index: KeptIndex, target: torch.Tensor, prior: torch.Tensor, drafter: torch.Tensor,
                                   batch: int, positions: int, drafter_kind: int = RDK_LOGITS):
     """Eq. rdk-taylor with softmax(prior) in place of p, written out: (q~ [rows, N], theta, S)."""
-    _rows2d(target, "target")
-    _rows2d(drafter, "drafter")
-    if prior.dtype != target.dtype:
-        raise ValueError("the prior must have the target's dtype")
-    rows = batch * positions
-    pb = make_problem(index, target, drafter, batch, positions, drafter_kind)
-    qt = torch.empty(rows, index.N, dtype=torch.float32, device=target.device)
-    theta = torch.empty(rows, dtype=torch.float32, device=target.device)
-    S = torch.empty(rows, dtype=torch.float32, device=target.device)
-    L = lib()
-    L.rdk_redistribute_linear_prior.restype = C.c_int
-    L.rdk_redistribute_linear_prior.argtypes = [C.POINTER(rdk_problem), C.c_void_p, C.c_void_p, C.c_int64, C.c_void_p,
-                                                C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]
-    _check(L.rdk_redistribute_linear_prior(C.byref(pb), target.data_ptr(), prior.data_ptr(), _prior_stride(prior, index.N),
-                                           drafter.data_ptr(), qt.data_ptr(), theta.data_ptr(), S.data_ptr(), _stream()),
-           "rdk_redistribute_linear_prior")
+    status, qt, theta, S = (_host or host()).linear(index.buffer, index.N, index.n, target, prior, drafter, batch, positions,
+                                                    drafter_kind)
+    if status:
+        _check(status, "rdk_redistribute_linear_prior")
     return qt, theta, S
 
 
 def rdk_sample_and_verify_prior(index: KeptIndex, target: torch.Tensor, prior: torch.Tensor, drafter: torch.Tensor,
                                 uniforms: torch.Tensor, batch: int, positions: int, drafter_kind: int = RDK_LOGITS,
                                 out: Optional[Dict[str, torch.Tensor]] = None) -> Dict[str, torch.Tensor]:
-    """The linear mode with a separate prior inside Eq. rdk-taylor; verification against softmax(target)."""
-    _rows2d(target, "target")
-    _rows2d(drafter, "drafter")
-    if prior.dtype != target.dtype:
-        raise ValueError("the prior must have the target's dtype")
-    rows = batch * positions
-    trials = uniforms.numel() // (rows * 4)
-    pb = make_problem(index, target, drafter, batch, positions, drafter_kind)
+    """The linear mode with a separate prior inside Eq. rdk-taylor; verification against softmax(target).  A [N]
+    prior is one row shared by all rows, a [rows, N] prior has a row for each."""
     if out is None:
-        out = alloc_outputs(rows, batch, trials, target.device)
-    o = outputs_struct(out)
-    L = lib()
-    L.rdk_sample_and_verify_prior.restype = C.c_int
-    L.rdk_sample_and_verify_prior.argtypes = [C.POINTER(rdk_problem), C.c_void_p, C.c_void_p, C.c_int64, C.c_void_p,
-                                              C.c_void_p, C.c_int32, C.POINTER(rdk_outputs), C.c_void_p]
-    _check(L.rdk_sample_and_verify_prior(C.byref(pb), target.data_ptr(), prior.data_ptr(), _prior_stride(prior, index.N),
-                                         drafter.data_ptr(), uniforms.data_ptr(), trials, C.byref(o), _stream()),
-           "rdk_sample_and_verify_prior")
+        rows = batch * positions
+        out = alloc_outputs(rows, batch, uniforms.numel() // (rows * 4), target.device)
+    status = (_host or host()).sample_prior(index.buffer, index.N, index.n, target, prior, drafter, uniforms, batch, positions,
+                                            drafter_kind, out)
+    if status:
+        _check(status, "rdk_sample_and_verify_prior")
     return out

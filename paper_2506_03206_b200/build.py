@@ -12,6 +12,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "librdk_b200.so")
+HOST = os.path.join(HERE, "_rdk_host.so")        # the binding's native part
 SOURCES = ["rdk_api.cu", "rdk_ids.cu", "rdk_row.cu", "rdk_row_cluster.cu", "rdk_row_stream.cu", "rdk_emit.cu", "rdk_affinity.cu", "rdk_affinity_tc.cu", "rdk_exact.cu", "rdk_exact_tc.cu"]
 
 
@@ -23,11 +24,25 @@ def _nvcc() -> str:
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(HOST):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(HOST))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(ROOT, "include", "rdk.h")]
     return any(os.path.getmtime(d) > t for d in deps)
+
+
+def _host_command():
+    """Compiler command of the binding's native part, against the headers and libraries of the torch in use."""
+    import sysconfig
+
+    import torch
+    from torch.utils import cpp_extension
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(_nvcc())))
+    inc = [os.path.join(ROOT, "include"), sysconfig.get_paths()["include"], os.path.join(cuda, "include"), *cpp_extension.include_paths()]
+    libdir = os.path.join(os.path.dirname(torch.__file__), "lib")
+    return ["g++", "-shared", "-fPIC", "-std=c++17", "-O2", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+            *[f for i in inc for f in ("-isystem" if "torch" in i else "-I", i)], os.path.join(CSRC, "rdk_host.cpp"),
+            "-L" + HERE, "-l:librdk_b200.so", "-Wl,-rpath,$ORIGIN", "-L" + libdir, "-ltorch_python", "-ltorch_cpu", "-ltorch", "-lc10", "-lc10_cuda"]
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -51,6 +66,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         with ThreadPoolExecutor(max_workers=min(len(SOURCES), os.cpu_count() or 1)) as pool:
             logs = list(pool.map(lambda so: run([nvcc, "-c", *flags, os.path.join(CSRC, so[0]), "-o", so[1]]), zip(SOURCES, objs)))
         logs.append(run([nvcc, "-shared", *flags, *objs, "-o", LIB]))
+        logs.append(run([*_host_command(), "-o", HOST]))
     if verbose:
         print("".join(logs))
     return LIB

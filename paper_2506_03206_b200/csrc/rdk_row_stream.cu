@@ -862,10 +862,12 @@ static size_t stream_smem(const StreamGeo& g, size_t es, bool offsets_in_smem) {
     return (size_t)g.NS * stage + (offsets_in_smem ? (size_t)kSW * g.ycap * (8 * g.NB + 2) : 0) + (size_t)g.NS * 16;
 }
 
+constexpr size_t kStreamSmemBudget = 212 * 1024;    // dynamic shared memory a CTA may ask for: 227 KB less the static part (14.2 KB)
+
 // Stage count, live rows and cache capacity for a vocabulary of N tokens with n kept ids; false when
 // the shapes do not fit shared memory.
 static bool plan_stream(int N, int n, size_t es, size_t ys, bool fast_types, StreamGeo& g) {
-    const size_t budget = 212 * 1024;      // dynamic shared memory a CTA may ask for: 227 KB less the static part (14.2 KB)
+    const size_t budget = kStreamSmemBudget;
     StreamSegs sg;
     if (!stream_segments(N, es, sg)) return false;
     g.C = sg.C; g.Lw = sg.Lw; g.nv = sg.nv;
@@ -911,16 +913,16 @@ template <typename TZ, typename TY, int KIND, int NIT, int NST>
 static cudaError_t launch_stream(const RowParams& P, StreamGeo g, cudaStream_t s) {
     auto kern = rdk_stream_kernel<TZ, TY, KIND, NIT, NST>;
     const size_t smem = stream_smem(g, sizeof(TZ), NST == 0);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     // how many CTAs are resident at once (cached per kernel instance, shared-memory size and device)
-    static thread_local int c_dev = -1, c_ctas = 0;
+    static thread_local int c_dev = -1, c_ctas = 0, sms = 0;
     static thread_local size_t c_smem = 0;
     int dev = 0;
-    e = cudaGetDevice(&dev);
+    cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev != c_dev || smem != c_smem) {
-        int sms = 0, per_sm = 0;
+        int per_sm = 0;
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStreamSmemBudget);
+        if (e != cudaSuccess) return e;
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kSThreads, smem);
@@ -973,9 +975,6 @@ static cudaError_t launch_stream(const RowParams& P, StreamGeo g, cudaStream_t s
     if (e != cudaSuccess) return e;
     // small CTAs when the draws of all rows would not be resident at once with large ones (shorter
     // tail), large CTAs otherwise (shorter chain per row)
-    int sms = 0;
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
     const bool small_ctas = (long long)P.rows * P.trials > (long long)sms * 8;
     cudaLaunchConfig_t dcfg = {};
     dcfg.gridDim = dim3((unsigned)(P.rows * P.trials), 1, 1);
