@@ -214,14 +214,15 @@ def make_problem(index: KeptIndex, target: Optional[torch.Tensor], drafter: Opti
     return p
 
 
-def affinity_alloc(N: int, n: int, layout: int, device) -> Dict[str, object]:
+def affinity_alloc(N: int, n: int, layout: int, device, zero: bool = True) -> Dict[str, object]:
     """Allocate an affinity matrix in one of the two layouts of rdk_affinity_layout."""
+    new = torch.zeros if zero else torch.empty
     if layout == RDK_AFF_F32_ROWS:
-        data = torch.zeros(n, N, dtype=torch.float32, device=device)
+        data = new(n, N, dtype=torch.float32, device=device)
         ld = N
     else:
         ld = (n + 7) // 8 * 8
-        data = torch.zeros(N, ld, dtype=torch.bfloat16, device=device)
+        data = new(N, ld, dtype=torch.bfloat16, device=device)
     return {"data": data, "layout": layout, "ld": ld}
 
 
@@ -235,7 +236,9 @@ def rdk_build_affinity(embeddings: torch.Tensor, kept_ids: torch.Tensor, tau: fl
     _rows2d(embeddings, "embeddings")
     N, d = embeddings.shape
     n = kept_ids.numel()
-    M = affinity_alloc(N, n, layout, embeddings.device)
+    M = affinity_alloc(N, n, layout, embeddings.device, zero=False)     # the library writes every element of [n, N] ...
+    if layout == RDK_AFF_BF16_COLS and M["ld"] > n:
+        M["data"][:, n:].zero_()                                        # ... and leaves the padding columns alone
     wsb = lib().rdk_build_affinity_workspace_bytes(N, n, d)
     ws = torch.empty(wsb, dtype=torch.uint8, device=embeddings.device)
     a = _aff_struct(M)

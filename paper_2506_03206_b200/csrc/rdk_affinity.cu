@@ -27,7 +27,7 @@ __global__ void aff_normalise_kernel(const TE* __restrict__ E, long long stride,
 
 template <int LAYOUT>
 __global__ void __launch_bounds__(kAffThreads)
-aff_rows_kernel(const float* __restrict__ Et, const int32_t* __restrict__ ids, int N, int n, int d,
+aff_fma_kernel(const float* __restrict__ Et, const int32_t* __restrict__ ids, int N, int n, int d,
                 float scale /* log2(e) / tau */, void* __restrict__ Mout, long long ld) {
     extern __shared__ __align__(16) float rows_s[];          // [d][kAffRows]
     __shared__ float red_m[kAffThreads / 32][kAffRows], red_s[kAffThreads / 32][kAffRows];
@@ -114,7 +114,7 @@ aff_rows_kernel(const float* __restrict__ Et, const int32_t* __restrict__ ids, i
 
 // the tensor-core route (bf16 embeddings into the bf16 layout)
 size_t affinity_tc_workspace_bytes(int N, int n, int d);
-bool affinity_tc_eligible(const void* embeddings, int emb_dtype, int d, long long estride, int layout);
+bool affinity_tc_eligible(const void* embeddings, int emb_dtype, const void* ws, int layout);
 int build_affinity_tc(const __nv_bfloat16* E, int d, long long estride, const int32_t* ids, int n, int N, float tau,
                       __nv_bfloat16* Mt, long long ld, void* ws, cudaStream_t s);
 
@@ -156,13 +156,13 @@ extern "C" int rdk_build_affinity(const void* embeddings, int32_t emb_dtype, int
         return RDK_ERR_WORKSPACE_TOO_SMALL;
     }
     const size_t smem = (size_t)d * kAffRows * sizeof(float);
-    if (smem > 200 * 1024) { set_error("rdk_build_affinity: embedding dimension %d too large", d); return RDK_ERR_UNSUPPORTED; }
     const int st = check_arch();
     if (st != RDK_OK) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (affinity_tc_eligible(embeddings, emb_dtype, d, estride, M_desc->layout))
+    if (affinity_tc_eligible(embeddings, emb_dtype, ws, M_desc->layout))
         return build_affinity_tc(static_cast<const __nv_bfloat16*>(embeddings), d, estride, kept_ids, n, N, tau,
                                  static_cast<__nv_bfloat16*>(M_out), M_desc->ld, ws, s);
+    if (smem > 200 * 1024) { set_error("rdk_build_affinity: embedding dimension %d too large", d); return RDK_ERR_UNSUPPORTED; }
     float* Et = static_cast<float*>(ws);
     const int wpb = 8;
     if (emb_dtype == RDK_F32)
@@ -173,11 +173,11 @@ extern "C" int rdk_build_affinity(const void* embeddings, int32_t emb_dtype, int
     const float scale = kLog2e / tau;
     const int blocks = (n + kAffRows - 1) / kAffRows;
     if (M_desc->layout == RDK_AFF_F32_ROWS) {
-        RDK_CUDA(cudaFuncSetAttribute(aff_rows_kernel<RDK_AFF_F32_ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        aff_rows_kernel<RDK_AFF_F32_ROWS><<<blocks, kAffThreads, smem, s>>>(Et, kept_ids, N, n, d, scale, M_out, M_desc->ld);
+        RDK_CUDA(cudaFuncSetAttribute(aff_fma_kernel<RDK_AFF_F32_ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        aff_fma_kernel<RDK_AFF_F32_ROWS><<<blocks, kAffThreads, smem, s>>>(Et, kept_ids, N, n, d, scale, M_out, M_desc->ld);
     } else {
-        RDK_CUDA(cudaFuncSetAttribute(aff_rows_kernel<RDK_AFF_BF16_COLS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        aff_rows_kernel<RDK_AFF_BF16_COLS><<<blocks, kAffThreads, smem, s>>>(Et, kept_ids, N, n, d, scale, M_out, M_desc->ld);
+        RDK_CUDA(cudaFuncSetAttribute(aff_fma_kernel<RDK_AFF_BF16_COLS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        aff_fma_kernel<RDK_AFF_BF16_COLS><<<blocks, kAffThreads, smem, s>>>(Et, kept_ids, N, n, d, scale, M_out, M_desc->ld);
     }
     RDK_CUDA(cudaGetLastError());
     return RDK_OK;

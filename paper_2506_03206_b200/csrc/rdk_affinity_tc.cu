@@ -1,113 +1,328 @@
 // Token-affinity matrix (Eq. symbolic-m with Omega = cosine similarity) for bf16 embeddings and the bf16
 // transposed layout, with the dot products on the tensor cores:
-//   G[j, i] = <e_j, e_{kappa_i}>                       (bf16 x bf16 products are exact, fp32 accumulation;
-//                                                       the tcgen05 kernel of the exact redistribution)
+//   G[j, i] = <e_j, e_{kappa_i}>                       (bf16 x bf16 products are exact, fp32 accumulation)
 //   Mt[j, i] = exp((G[j, i] / (|e_j| |e_{kappa_i}|) - 1) / tau) / Z_i,
 //   Z_i = sum_{j in T} exp((G[j, i] / (|e_j| |e_{kappa_i}|) - 1) / tau)
-// (the shift by the largest possible cosine, 1, cancels in the quotient).  The kept rows are taken in chunks
-// of at most kAffChunk; per chunk: gather the kept embeddings, one GEMM into an fp32 scratch [N, chunk],
-// per-column sums in two deterministic steps, one pass that writes the bf16 result.
+// (the shift by the largest possible cosine, 1, cancels in the quotient).
+//
+// G is never stored: the embedding dimension is a few hundred, so computing it twice costs the tensor cores less
+// (2 x 42 us for 32768 x 8192 x 128) than a round trip of fp32 through HBM.  One kernel runs twice over tiles of
+// 128 x 256 dot products, accumulated in tensor memory (two accumulators, so that one is filled while the other is
+// read back):
+//   kAffSums  : rows = kept ids, columns = tokens.  A thread owns a kept id and adds up its exponentials over the
+//               tokens of a work item; a small kernel adds the items' parts in a fixed order.
+//   kAffWrite : rows = tokens, columns = kept ids.  exp(...) / Z_i as one exponential of (cos - 1) / tau - log Z_i,
+//               rounded to bf16, staged in swizzled shared memory and stored by TMA (128-byte rows).
+// Both are bound by the special-function unit (one exponential per element and pass: 2 x 60 us at 16 per clock and SM)
+// and by the write of the matrix (537 MB: 82 us).  The chain that this replaces, with an fp32 scratch between the GEMM
+// and three streaming passes, took 1490 us for that size.
 #include <math.h>
 
-#include "rdk_common.cuh"
+#include "rdk_device.cuh"
+#include "rdk_tc.cuh"
 
 namespace rdk {
 
-int launch_exact_tc(const __nv_bfloat16* A, long long lda, const __nv_bfloat16* Mt, long long ldm, float* w_out,
-                    float* S_out, int rows, int n, int N, int32_t* status_word, cudaStream_t s);
+constexpr int kAffM = 128, kAffN = 256, kAffK = 64;
+constexpr int kAffABytes = kAffM * kAffK * 2, kAffBBytes = kAffN * kAffK * 2;       // 16 KB, 32 KB
+constexpr int kAffStage = kAffABytes + kAffBBytes;
+constexpr int kAffStages = 3;
+constexpr int kAffEpiWarps = 8;                          // two per quarter of the TMEM lanes, each with half of the columns
+constexpr int kAffThreads = 64 + 32 * kAffEpiWarps;
+constexpr int kAffStoreBytes = 32 * 128;                 // a warp's 32 rows x 64 bf16
+constexpr int kAffSmem = kAffStages * kAffStage + kAffEpiWarps * 2 * kAffStoreBytes + 1024;
+constexpr int kAffSpan = 4;                              // column tiles per work item of kAffSums
+constexpr uint32_t kAffIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kAffN >> 3) << 17) | ((uint32_t)(kAffM >> 4) << 24);
 
-constexpr int kAffChunk = 2048;          // kept rows per GEMM (columns of the fp32 scratch)
-constexpr int kAffBlockRows = 64;        // token rows per CTA in the column-sum pass
-constexpr int kAffColThreads = 256;
+enum { kAffSums = 0, kAffWrite = 1 };
 
-// inv[t] = 1 / max(|e_t|, 1e-12), one warp per token
-__global__ void aff_inv_norm_kernel(const __nv_bfloat16* __restrict__ E, long long stride, float* __restrict__ inv, int N, int d) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (warp >= N) return;
-    const __nv_bfloat16* row = E + (long long)warp * stride;
-    float ss = 0.f;
-    for (int k = lane; k < d; k += 32) { const float v = __bfloat162float(row[k]); ss += v * v; }
-    ss = warp_sum(ss);
-    if (lane == 0) inv[warp] = 1.f / fmaxf(sqrtf(ss), 1e-12f);
-}
+struct AffParams {
+    int N, n, num_kb;
+    int tiles_m, tiles_n, num_items;   // row tiles, column tiles (kAffSums: spans of kAffSpan column tiles), work items
+    int cols;                          // columns in all
+    const float* row_inv;              // 1 / |e| of the rows, zero-padded to whole tiles
+    const float* col_inv;              // 1 / |e| of the columns, zero-padded to whole tiles
+    const float* col_off;              // kAffWrite: exponent offset -1 / tau - log2 Z of every column (-inf: weight 0)
+    float scale;                       // log2(e) / tau
+    float* part;                       // kAffSums: [2 tiles_n][row tiles * 128]
+    int32_t* status;
+};
 
-// Ek[c, :] = e_{kappa_{i0 + c}} (zeros for an id outside [0, N)), invk[c] = its inverse norm (0 for such an id)
-__global__ void aff_gather_kernel(const __nv_bfloat16* __restrict__ E, long long stride, const int32_t* __restrict__ ids,
-                                  const float* __restrict__ inv, __nv_bfloat16* __restrict__ Ek, float* __restrict__ invk,
-                                  int i0, int cols, int N, int d, int dpad) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (warp >= cols) return;
-    const int id = ids[i0 + warp];
-    const bool ok = id >= 0 && id < N;
-    for (int k = lane; k < dpad; k += 32)
-        Ek[(long long)warp * dpad + k] = (ok && k < d) ? E[(long long)id * stride + k] : __float2bfloat16_rn(0.f);
-    if (lane == 0) invk[warp] = ok ? inv[id] : 0.f;
-}
-
-// part[b, c] = sum over the token rows j of block b of 2^((G[j, c] inv[j] invk[c] - 1) scale)
-__global__ void __launch_bounds__(kAffColThreads)
-aff_colsum_kernel(const float* __restrict__ G, const float* __restrict__ inv, const float* __restrict__ invk,
-                  float* __restrict__ part, int N, int cols, float scale) {
-    const int j0 = blockIdx.x * kAffBlockRows;
-    const int j1 = min(N, j0 + kAffBlockRows);
-    for (int c = threadIdx.x; c < cols; c += kAffColThreads) {
-        const float ik = invk[c];
-        float s = 0.f;
-        for (int j = j0; j < j1; ++j)
-            s += ex2((G[(long long)j * cols + c] * (__ldg(inv + j) * ik) - 1.f) * scale);
-        part[(long long)blockIdx.x * cols + c] = s;
+template <int MODE>
+__global__ void __launch_bounds__(kAffThreads, 1)
+aff_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__ CUtensorMap tmapB, const __grid_constant__ CUtensorMap tmapC, const AffParams P) {
+    extern __shared__ __align__(1024) unsigned char aff_smem[];
+    unsigned char* tiles = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(aff_smem) + 1023) & ~uintptr_t(1023));
+    __shared__ __align__(8) unsigned long long full_bar[kAffStages], empty_bar[kAffStages], acc_full[2], acc_empty[2];
+    __shared__ uint32_t tmem_base_s;
+    __shared__ int abort_s;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    volatile int* abort = &abort_s;
+    if (threadIdx.x == 0) {
+        abort_s = 0;
+        for (int s = 0; s < kAffStages; ++s) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(s32(&full_bar[s])));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(s32(&empty_bar[s])));
+        }
+        for (int a = 0; a < 2; ++a) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(s32(&acc_full[a])));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(s32(&acc_empty[a])), "r"(kAffEpiWarps));
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(s32(&tmem_base_s)) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem_base = tmem_base_s;
+    constexpr int kSpan = MODE == kAffSums ? kAffSpan : 1;
+    const int col_tiles = (P.cols + kAffN - 1) / kAffN;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+    // every role walks the same sequence: items blockIdx.x, + gridDim.x, ...; in an item up to kSpan column tiles
+    if (warp == 0) {
+        int stage = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        for (int item = blockIdx.x; item < P.num_items && ok; item += gridDim.x) {
+            const int tm = item / P.tiles_n, tn0 = (item % P.tiles_n) * kSpan;
+            for (int tn = tn0; tn < min(tn0 + kSpan, col_tiles) && ok; ++tn)
+                for (int kb = 0; kb < P.num_kb; ++kb) {
+                    if (!tc_wait(&empty_bar[stage], phase ^ 1u, abort)) { ok = false; break; }
+                    if (lane == 0) {
+                        const uint32_t sa = s32(tiles + stage * kAffStage), bar = s32(&full_bar[stage]);
+                        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"((uint32_t)kAffStage) : "memory");
+                        asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+                                     ::"r"(sa), "l"(reinterpret_cast<uint64_t>(&tmapA)), "r"(kb * kAffK), "r"(tm * kAffM), "r"(bar) : "memory");
+                        asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+                                     ::"r"(sa + kAffABytes), "l"(reinterpret_cast<uint64_t>(&tmapB)), "r"(kb * kAffK), "r"(tn * kAffN), "r"(bar) : "memory");
+                    }
+                    __syncwarp();
+                    if (++stage == kAffStages) { stage = 0; phase ^= 1u; }
+                }
+        }
+    } else if (warp == 1) {
+        int stage = 0, acc = 0;
+        uint32_t phase = 0, acc_phase = 0;
+        bool ok = true;
+        for (int item = blockIdx.x; item < P.num_items && ok; item += gridDim.x) {
+            const int tn0 = (item % P.tiles_n) * kSpan;
+            for (int tn = tn0; tn < min(tn0 + kSpan, col_tiles) && ok; ++tn) {
+                if (!tc_wait(&acc_empty[acc], acc_phase ^ 1u, abort)) { ok = false; break; }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                for (int kb = 0; kb < P.num_kb; ++kb) {
+                    if (!tc_wait(&full_bar[stage], phase, abort)) { ok = false; break; }
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    if (lane == 0) {
+                        const uint32_t a_addr = s32(tiles + stage * kAffStage), b_addr = a_addr + kAffABytes;
+#pragma unroll
+                        for (int k = 0; k < kAffK / 16; ++k) {
+                            const uint64_t adesc = smem_desc(a_addr + k * 32), bdesc = smem_desc(b_addr + k * 32);
+                            asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
+                                         ::"r"(tmem_base + (uint32_t)(acc * kAffN)), "l"(adesc), "l"(bdesc), "r"(kAffIdesc), "r"((kb > 0 || k > 0) ? 1u : 0u) : "memory");
+                        }
+                        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(s32(&empty_bar[stage])) : "memory");
+                    }
+                    __syncwarp();
+                    if (++stage == kAffStages) { stage = 0; phase ^= 1u; }
+                }
+                if (!ok) break;
+                if (lane == 0)
+                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(s32(&acc_full[acc])) : "memory");
+                __syncwarp();
+                if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+            }
+        }
+    } else {
+        const int quarter = warp & 3, half = (warp - 2) >> 2;        // TMEM lanes 32 quarter .. + 32, columns 128 half .. + 128
+        const uint32_t taddr0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(half * 128);
+        unsigned char* stage_c = tiles + kAffStages * kAffStage + (warp - 2) * 2 * kAffStoreBytes;
+        int acc = 0, buf = 0;
+        uint32_t acc_phase = 0;
+        bool ok = true;
+        for (int item = blockIdx.x; item < P.num_items && ok; item += gridDim.x) {
+            const int tm = item / P.tiles_n, tn0 = (item % P.tiles_n) * kSpan;
+            const int row = tm * kAffM + quarter * 32 + lane;
+            const float2 rs = splat(__ldg(P.row_inv + row) * P.scale);
+            float2 sum_a = splat(0.f), sum_b = splat(0.f);
+            for (int tn = tn0; tn < min(tn0 + kSpan, col_tiles); ++tn) {
+                const int c0 = tn * kAffN + half * 128;
+                if (!tc_wait(&acc_full[acc], acc_phase, abort)) { ok = false; break; }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                uint32_t v[2][32];
+                tmem_ld32(taddr0 + (uint32_t)(acc * kAffN), v[0]);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    tmem_wait_ld(v[c & 1]);
+                    if (c < 3) tmem_ld32(taddr0 + (uint32_t)(acc * kAffN + (c + 1) * 32), v[(c + 1) & 1]);
+                    uint32_t (&x)[32] = v[c & 1];
+                    if (c == 3) {                                    // the accumulator is in registers: the next tile may have it
+                        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                        __syncwarp();
+                        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(s32(&acc_empty[acc])) : "memory");
+                    }
+                    const int col = c0 + c * 32;
+                    const float4* ci = reinterpret_cast<const float4*>(P.col_inv + col);
+                    if (MODE == kAffSums) {
+                        const float2 off = splat(-P.scale);
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) {
+                            const float4 k4 = __ldg(ci + q);
+                            float2 e0 = ex2_2(ffma2(make_float2(__uint_as_float(x[4 * q]), __uint_as_float(x[4 * q + 1])), fmul2(make_float2(k4.x, k4.y), rs), off));
+                            float2 e1 = ex2_2(ffma2(make_float2(__uint_as_float(x[4 * q + 2]), __uint_as_float(x[4 * q + 3])), fmul2(make_float2(k4.z, k4.w), rs), off));
+                            if (col + 32 > P.cols) {                 // tokens beyond the vocabulary have no weight
+                                const int left = P.cols - col - 4 * q;
+                                if (left < 1) e0.x = 0.f;
+                                if (left < 2) e0.y = 0.f;
+                                if (left < 3) e1.x = 0.f;
+                                if (left < 4) e1.y = 0.f;
+                            }
+                            sum_a = fadd2(sum_a, e0); sum_b = fadd2(sum_b, e1);
+                        }
+                    } else {
+                        const float4* co = reinterpret_cast<const float4*>(P.col_off + col);
+                        if ((c & 1) == 0) {                          // the staging buffer's last store has been read
+                            if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+                            __syncwarp();
+                        }
+                        const uint32_t rowaddr = s32(stage_c + buf * kAffStoreBytes) + (uint32_t)lane * 128u;
+#pragma unroll
+                        for (int q = 0; q < 8; q += 2) {
+                            uint32_t w[4];
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) {
+                                const float4 k4 = __ldg(ci + q + h), o4 = __ldg(co + q + h);
+                                const int i = 4 * (q + h);
+                                const float2 e0 = ex2_2(ffma2(make_float2(__uint_as_float(x[i]), __uint_as_float(x[i + 1])), fmul2(make_float2(k4.x, k4.y), rs), make_float2(o4.x, o4.y)));
+                                const float2 e1 = ex2_2(ffma2(make_float2(__uint_as_float(x[i + 2]), __uint_as_float(x[i + 3])), fmul2(make_float2(k4.z, k4.w), rs), make_float2(o4.z, o4.w)));
+                                asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w[2 * h]) : "f"(e0.y), "f"(e0.x));
+                                asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w[2 * h + 1]) : "f"(e1.y), "f"(e1.x));
+                            }
+                            // 16-byte chunk (c & 1) * 4 + q / 2 of the row, at its place in the 128-byte swizzle
+                            const uint32_t chunk = (uint32_t)((c & 1) * 4 + q / 2) ^ (uint32_t)(lane & 7);
+                            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(rowaddr + chunk * 16u), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]) : "memory");
+                        }
+                        if (c & 1) {                                 // 64 columns are complete
+                            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                            __syncwarp();
+                            if (lane == 0) {
+                                const int x0 = c0 + (c >> 1) * 64, y0 = tm * kAffM + quarter * 32;
+                                if (x0 < P.n && y0 < P.N)
+                                    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];"
+                                                 ::"l"(reinterpret_cast<uint64_t>(&tmapC)), "r"(x0), "r"(y0), "r"(s32(stage_c + buf * kAffStoreBytes)) : "memory");
+                                asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                            }
+                            buf ^= 1;
+                        }
+                    }
+                }
+                if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+            }
+            if (MODE == kAffSums && ok)
+                P.part[(long long)((item % P.tiles_n) * 2 + half) * (P.tiles_m * kAffM) + row] = (sum_a.x + sum_a.y) + (sum_b.x + sum_b.y);
+        }
+        if (MODE == kAffWrite && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    }
+    // after a wait that gave up, copies may still be on their way into shared memory: let them land (bounded as well)
+    if (abort_s && warp == 0)
+        for (int s = 0; s < kAffStages; ++s)
+            for (unsigned spins = 0; spins < (1u << 12); ++spins) __nanosleep(100);
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 1) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem_base) : "memory");
+    }
+    if (threadIdx.x == 0 && abort_s && P.status) atomicCAS(P.status, 0, (int)RDK_ERR_TIMEOUT);
 }
 
-// invZ[c] = 1 / sum_b part[b, c], blocks taken in order
-__global__ void aff_colsum_reduce_kernel(const float* __restrict__ part, float* __restrict__ invZ, int blocks, int cols) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= cols) return;
-    float s = 0.f;
-    for (int b = 0; b < blocks; ++b) s += part[(long long)b * cols + c];
-    invZ[c] = 1.f / s;
+// One warp per row: rows [0, Npad) are tokens, inv[t] = 1 / max(|e_t|, 1e-12) (0 beyond the vocabulary) and, where
+// Epad is given, the embedding copied to rows of dpad elements; rows [Npad, Npad + npad) are kept ids, their embedding
+// gathered into Ek and its inverse norm into invk (zeros for an id outside [0, N) and beyond the last).
+__global__ void __launch_bounds__(256)
+aff_rows_kernel(const __nv_bfloat16* __restrict__ E, long long stride, const int32_t* __restrict__ ids, __nv_bfloat16* __restrict__ Epad,
+                float* __restrict__ inv, __nv_bfloat16* __restrict__ Ek, float* __restrict__ invk, int32_t* status,
+                int N, int Npad, int n, int npad, int d, int dpad, bool vec) {
+    const int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (r == 0 && lane == 0) *status = 0;
+    if (r >= Npad + npad) return;
+    const bool kept = r >= Npad;
+    const int i = kept ? r - Npad : r;
+    int t = kept ? (i < n ? ids[i] : -1) : (i < N ? i : -1);
+    if (t >= N) t = -1;
+    __nv_bfloat16* copy = kept ? (i < n ? Ek + (long long)i * dpad : nullptr) : (Epad && i < N ? Epad + (long long)i * dpad : nullptr);
+    float ss = 0.f;
+    const __nv_bfloat16* row = E + (long long)max(t, 0) * stride;
+    if (vec) {                            // 16-byte aligned rows of a multiple of 8 elements
+        for (int k = lane * 8; k < d; k += 256) {
+            const uint4 q = t >= 0 ? __ldg(reinterpret_cast<const uint4*>(row + k)) : make_uint4(0u, 0u, 0u, 0u);
+            const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+            for (int h = 0; h < 4; ++h) { const float a = bf16_lo(w[h]), b = bf16_hi(w[h]); ss = fmaf(a, a, fmaf(b, b, ss)); }
+            if (copy) *reinterpret_cast<uint4*>(copy + k) = q;
+        }
+    } else {
+        for (int k = lane; k < dpad; k += 32) {
+            const __nv_bfloat16 q = t >= 0 && k < d ? row[k] : __float2bfloat16_rn(0.f);
+            const float a = __bfloat162float(q);
+            ss = fmaf(a, a, ss);
+            if (copy) copy[k] = q;
+        }
+    }
+    ss = warp_sum(ss);
+    if (lane == 0) (kept ? invk : inv)[i] = t >= 0 ? 1.f / fmaxf(sqrtf(ss), 1e-12f) : 0.f;
 }
 
-// Mt[j, i0 + c] = bf16(2^((G[j, c] inv[j] invk[c] - 1) scale) invZ[c]); kept ids outside the vocabulary give 0
-__global__ void __launch_bounds__(kAffColThreads)
-aff_write_kernel(const float* __restrict__ G, const float* __restrict__ inv, const float* __restrict__ invk,
-                 const float* __restrict__ invZ, __nv_bfloat16* __restrict__ Mt, long long ld, int i0, int N, int cols, float scale) {
-    const int j = blockIdx.x;
-    const float ij = __ldg(inv + j);
-    const float* g = G + (long long)j * cols;
-    __nv_bfloat16* out = Mt + (long long)j * ld + i0;
-    for (int c = threadIdx.x; c < cols; c += kAffColThreads) {
-        const float ik = invk[c];
-        const float v = ik > 0.f ? ex2((g[c] * (ij * ik) - 1.f) * scale) * invZ[c] : 0.f;
-        out[c] = __float2bfloat16_rn(v);
+// off[i] = -scale - log2(sum of the parts of i, in order); -inf where the kept id has no token.  One warp per 32 ids and
+// eight warps share their parts.
+__global__ void __launch_bounds__(256)
+aff_offset_kernel(const float* __restrict__ part, const float* __restrict__ invk, float* __restrict__ off, int parts, int npad, float scale) {
+    __shared__ float s[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    float a = 0.f;
+#pragma unroll 4
+    for (int p = warp; p < parts; p += 8) a += part[(long long)p * npad + i];
+    s[warp][lane] = a;
+    __syncthreads();
+    if (warp == 0) {
+        for (int w = 1; w < 8; ++w) a += s[w][lane];
+        off[i] = invk[i] > 0.f ? -scale - log2f(a) : -INFINITY;
     }
 }
 
 // a wait inside the tensor-core kernel ran out: the matrix is incomplete, make that impossible to miss
 __global__ void aff_poison_kernel(const int32_t* status, __nv_bfloat16* Mt) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (*status != 0) Mt[0] = __float2bfloat16_rn(NAN);
 }
 
 // ------------------------------------------------------------------------------------------------
 // host side
 // ------------------------------------------------------------------------------------------------
-static size_t aff_tc_dpad(int d) { return (size_t)((d + 7) & ~7); }
-static int aff_tc_chunk(int n) { return n < kAffChunk ? n : kAffChunk; }
-
-// workspace: inv[N] | invk[chunk] | invZ[chunk] | status | Ek[chunk, dpad] bf16 | part[blocks, chunk] | G[N, chunk]
-struct AffTcLayout { size_t inv, invk, invZ, status, Ek, part, G, total; int chunk, blocks; };
+// workspace: inv[Npad] | invk[npad] | off[npad] | status | Ek[n, dpad] bf16 | part[2 spans, npad] | Epad[N, dpad] bf16
+struct AffTcLayout { size_t inv, invk, off, status, Ek, part, Epad, total; int Npad, npad, dpad, spans; };
 static AffTcLayout aff_tc_layout(int N, int n, int d) {
     AffTcLayout L;
-    L.chunk = aff_tc_chunk(n);
-    L.blocks = (N + kAffBlockRows - 1) / kAffBlockRows;
+    L.Npad = (N + kAffN - 1) / kAffN * kAffN;
+    L.npad = (n + kAffN - 1) / kAffN * kAffN;
+    L.dpad = (d + 7) & ~7;
+    L.spans = (L.Npad / kAffN + kAffSpan - 1) / kAffSpan;
     size_t o = 0;
-    L.inv = o;    o += idx_align((size_t)N * sizeof(float));
-    L.invk = o;   o += idx_align((size_t)L.chunk * sizeof(float));
-    L.invZ = o;   o += idx_align((size_t)L.chunk * sizeof(float));
+    L.inv = o;    o += idx_align((size_t)L.Npad * sizeof(float));
+    L.invk = o;   o += idx_align((size_t)L.npad * sizeof(float));
+    L.off = o;    o += idx_align((size_t)L.npad * sizeof(float));
     L.status = o; o += idx_align(sizeof(int32_t));
-    L.Ek = o;     o += idx_align((size_t)L.chunk * aff_tc_dpad(d) * sizeof(__nv_bfloat16));
-    L.part = o;   o += idx_align((size_t)L.blocks * L.chunk * sizeof(float));
-    L.G = o;      o += idx_align((size_t)N * L.chunk * sizeof(float));
+    L.Ek = o;     o += idx_align((size_t)n * L.dpad * sizeof(__nv_bfloat16));
+    L.part = o;   o += idx_align((size_t)2 * L.spans * L.npad * sizeof(float));
+    L.Epad = o;   o += idx_align((size_t)N * L.dpad * sizeof(__nv_bfloat16));
     L.total = o;
     return L;
 }
@@ -115,9 +330,24 @@ static AffTcLayout aff_tc_layout(int N, int n, int d) {
 size_t affinity_tc_workspace_bytes(int N, int n, int d) { return aff_tc_layout(N, n, d).total; }
 
 // whether the tensor-core route serves this call (the other route serves everything)
-bool affinity_tc_eligible(const void* embeddings, int emb_dtype, int d, long long estride, int layout) {
-    return emb_dtype == RDK_BF16 && layout == RDK_AFF_BF16_COLS && d >= 64 && (estride % 8) == 0 &&
-           (reinterpret_cast<uintptr_t>(embeddings) & 15u) == 0;
+bool affinity_tc_eligible(const void* embeddings, int emb_dtype, const void* ws, int layout) {
+    return emb_dtype == RDK_BF16 && layout == RDK_AFF_BF16_COLS && (reinterpret_cast<uintptr_t>(embeddings) & 1u) == 0 &&
+           (reinterpret_cast<uintptr_t>(ws) & 15u) == 0;
+}
+
+template <typename K, typename... A>
+static cudaError_t launch_pdl(K kern, unsigned grid, unsigned block, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid, 1, 1);
+    cfg.blockDim = dim3(block, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
 int build_affinity_tc(const __nv_bfloat16* E, int d, long long estride, const int32_t* ids, int n, int N, float tau,
@@ -126,34 +356,48 @@ int build_affinity_tc(const __nv_bfloat16* E, int d, long long estride, const in
     unsigned char* base = static_cast<unsigned char*>(ws);
     float* inv = reinterpret_cast<float*>(base + L.inv);
     float* invk = reinterpret_cast<float*>(base + L.invk);
-    float* invZ = reinterpret_cast<float*>(base + L.invZ);
+    float* off = reinterpret_cast<float*>(base + L.off);
     int32_t* status = reinterpret_cast<int32_t*>(base + L.status);
     __nv_bfloat16* Ek = reinterpret_cast<__nv_bfloat16*>(base + L.Ek);
     float* part = reinterpret_cast<float*>(base + L.part);
-    float* G = reinterpret_cast<float*>(base + L.G);
-    const int dpad = (int)aff_tc_dpad(d);
     const float scale = kLog2e / tau;
+    // TMA reads rows of whole 16-byte units: others are copied to padded rows along with the norms
+    const bool rows16 = (estride % 8) == 0 && (reinterpret_cast<uintptr_t>(E) & 15u) == 0;
+    __nv_bfloat16* Epad = rows16 ? nullptr : reinterpret_cast<__nv_bfloat16*>(base + L.Epad);
     const int wpb = 8;
-    RDK_CUDA(cudaMemsetAsync(status, 0, sizeof(int32_t), s));
-    aff_inv_norm_kernel<<<(N + wpb - 1) / wpb, wpb * 32, 0, s>>>(E, estride, inv, N, d);
-    RDK_CUDA(cudaGetLastError());
-    for (int i0 = 0; i0 < n; i0 += L.chunk) {
-        const int cols = n - i0 < L.chunk ? n - i0 : L.chunk;
-        aff_gather_kernel<<<(cols + wpb - 1) / wpb, wpb * 32, 0, s>>>(E, estride, ids, inv, Ek, invk, i0, cols, N, d, dpad);
-        RDK_CUDA(cudaGetLastError());
-        // G[j, c] = sum_k E[j, k] Ek[c, k]: the GEMM of the exact redistribution with the roles
-        // (rows, contraction, columns) = (tokens, embedding dimension, kept rows of the chunk)
-        const int st = launch_exact_tc(E, estride, Ek, dpad, G, nullptr, N, d, cols, status, s);
-        if (st != RDK_OK) return st;
-        aff_colsum_kernel<<<L.blocks, kAffColThreads, 0, s>>>(G, inv, invk, part, N, cols, scale);
-        RDK_CUDA(cudaGetLastError());
-        aff_colsum_reduce_kernel<<<(cols + 127) / 128, 128, 0, s>>>(part, invZ, L.blocks, cols);
-        RDK_CUDA(cudaGetLastError());
-        aff_write_kernel<<<N, kAffColThreads, 0, s>>>(G, inv, invk, invZ, Mt, ld, i0, N, cols, scale);
-        RDK_CUDA(cudaGetLastError());
-    }
-    aff_poison_kernel<<<1, 1, 0, s>>>(status, Mt);
-    RDK_CUDA(cudaGetLastError());
+    RDK_CUDA(launch_pdl(aff_rows_kernel, (unsigned)((L.Npad + L.npad + wpb - 1) / wpb), 256u, 0, s, E, estride, ids, Epad, inv, Ek, invk, status,
+                        N, L.Npad, n, L.npad, d, L.dpad, rows16 && d % 8 == 0));
+    const __nv_bfloat16* Et = rows16 ? E : Epad;
+    const long long et_stride = rows16 ? estride : L.dpad;
+    CUtensorMap tokA, tokB, keptA, keptB, out;
+    int st;
+    if ((st = make_map(&tokA, Et, (uint64_t)d, (uint64_t)N, (uint64_t)et_stride, kAffK, kAffM)) != RDK_OK) return st;
+    if ((st = make_map(&tokB, Et, (uint64_t)d, (uint64_t)N, (uint64_t)et_stride, kAffK, kAffN)) != RDK_OK) return st;
+    if ((st = make_map(&keptA, Ek, (uint64_t)d, (uint64_t)n, (uint64_t)L.dpad, kAffK, kAffM)) != RDK_OK) return st;
+    if ((st = make_map(&keptB, Ek, (uint64_t)d, (uint64_t)n, (uint64_t)L.dpad, kAffK, kAffN)) != RDK_OK) return st;
+    if ((st = make_map(&out, Mt, (uint64_t)n, (uint64_t)N, (uint64_t)ld, 64, 32)) != RDK_OK) return st;
+    int dev = 0, sms = 0;
+    RDK_CUDA(cudaGetDevice(&dev));
+    RDK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    RDK_CUDA(cudaFuncSetAttribute(aff_tc_kernel<kAffSums>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAffSmem));
+    RDK_CUDA(cudaFuncSetAttribute(aff_tc_kernel<kAffWrite>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAffSmem));
+    AffParams P;
+    P.N = N; P.n = n; P.num_kb = (d + kAffK - 1) / kAffK; P.scale = scale; P.status = status; P.part = part;
+    // sums: rows = kept ids, columns = tokens
+    P.tiles_m = L.npad / kAffM; P.tiles_n = L.spans; P.cols = N;
+    P.row_inv = invk; P.col_inv = inv; P.col_off = nullptr;
+    const long long items = (long long)P.tiles_m * P.tiles_n;
+    const long long items_w = (long long)(L.Npad / kAffM) * (L.npad / kAffN);
+    if (items > 0x7fffffffLL || items_w > 0x7fffffffLL) { set_error("rdk_build_affinity: too many tiles"); return RDK_ERR_UNSUPPORTED; }
+    P.num_items = (int)items;
+    RDK_CUDA(launch_pdl(aff_tc_kernel<kAffSums>, (unsigned)(items < sms ? items : sms), (unsigned)kAffThreads, (size_t)kAffSmem, s, keptA, tokB, out, P));
+    RDK_CUDA(launch_pdl(aff_offset_kernel, (unsigned)(L.npad / 32), 256u, 0, s, (const float*)part, (const float*)invk, off, 2 * L.spans, L.npad, scale));
+    // the matrix: rows = tokens, columns = kept ids
+    P.tiles_m = L.Npad / kAffM; P.tiles_n = L.npad / kAffN; P.cols = n;
+    P.row_inv = inv; P.col_inv = invk; P.col_off = off;
+    P.num_items = (int)items_w;
+    RDK_CUDA(launch_pdl(aff_tc_kernel<kAffWrite>, (unsigned)(items_w < sms ? items_w : sms), (unsigned)kAffThreads, (size_t)kAffSmem, s, tokA, keptB, out, P));
+    RDK_CUDA(launch_pdl(aff_poison_kernel, 1u, 1u, 0, s, (const int32_t*)status, Mt));
     return RDK_OK;
 }
 

@@ -11,9 +11,9 @@
 // Items are ordered so that the row tiles of one 256-column panel of Mt run at the same time: the
 // panel is fetched from HBM once and shared through L2.
 // Every wait is bounded; on expiry the CTA flags RDK_ERR_TIMEOUT in the status word and winds down.
-#include <cuda.h>
+#include <atomic>
 
-#include "rdk_common.cuh"
+#include "rdk_tc.cuh"
 
 namespace rdk {
 
@@ -27,7 +27,6 @@ constexpr int kBBytes = kBN * kBK * 2;           // 32 KB
 constexpr int kStageBytes = kABytes + kBBytes;   // 64 KB
 constexpr int kTcThreads = 192;
 constexpr int kTmemCols = 512;
-constexpr unsigned kTcSpin = 1u << 21;
 
 struct TcParams {
     float* w; float* S; int rows, N, K;
@@ -47,37 +46,6 @@ __device__ __forceinline__ void decode_item(const TcParams& P, int item, int& ro
     row0 = tm * kTileM + (half > 0 ? kBM : 0);
     const int left = P.rows - row0;
     mt = left <= 0 ? 0 : ((half < 0 && left > kBM) ? 2 : 1);
-}
-
-__device__ __forceinline__ uint32_t s32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-// Bounded wait on an mbarrier phase; false (and *abort set) when the limit is reached or another
-// role has already given up.
-// Called by all lanes of a warp; the answer is the same in every lane.
-__device__ __forceinline__ bool tc_wait(unsigned long long* bar, uint32_t parity, volatile int* abort) {
-    bool ok = false;
-    for (unsigned spins = 0; spins < kTcSpin; ++spins) {
-        uint32_t done;
-        asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-                     : "=r"(done) : "r"(s32(bar)), "r"(parity) : "memory");
-        if (done) { ok = true; break; }
-        if (*abort) break;
-    }
-    ok = __all_sync(0xffffffffu, ok);
-    if (!ok) *abort = 1;
-    return ok;
-}
-
-// shared-memory matrix descriptor: K-major operand, rows of 128 bytes, 128-byte swizzle, groups of
-// 8 rows 1024 bytes apart
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
-    uint64_t d = 0;
-    d |= (uint64_t)((addr & 0x3FFFFu) >> 4);         // start address
-    d |= (uint64_t)1 << 16;                          // leading byte offset (unused for swizzled K-major)
-    d |= (uint64_t)(1024 >> 4) << 32;                // stride byte offset
-    d |= (uint64_t)1 << 46;                          // descriptor version of this architecture
-    d |= (uint64_t)2 << 61;                          // 128-byte swizzle
-    return d;
 }
 
 // instruction descriptor: D = fp32, A = B = bf16, both K-major, M = 128, N = 256
@@ -245,8 +213,20 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-static int make_map(EncodeTiledFn enc, CUtensorMap* map, const void* base, uint64_t inner, uint64_t outer, uint64_t pitch_elems,
-                    uint32_t box_inner, uint32_t box_outer) {
+int make_map(CUtensorMap* map, const void* base, uint64_t inner, uint64_t outer, uint64_t pitch_elems, uint32_t box_inner, uint32_t box_outer) {
+    static std::atomic<EncodeTiledFn> known{nullptr};
+    EncodeTiledFn enc = known.load();
+    if (!enc) {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult qres;
+        RDK_CUDA(cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres));
+        if (qres != cudaDriverEntryPointSuccess || !fn) {
+            set_error("the driver does not provide cuTensorMapEncodeTiled");
+            return RDK_ERR_CUDA;
+        }
+        enc = reinterpret_cast<EncodeTiledFn>(fn);
+        known.store(enc);
+    }
     const cuuint64_t dims[2] = {inner, outer};
     const cuuint64_t strides[1] = {pitch_elems * 2};
     const cuuint32_t box[2] = {box_inner, box_outer};
@@ -263,25 +243,14 @@ static int make_map(EncodeTiledFn enc, CUtensorMap* map, const void* base, uint6
 
 int launch_exact_tc(const __nv_bfloat16* A, long long lda, const __nv_bfloat16* Mt, long long ldm, float* w_out,
                     float* S_out, int rows, int n, int N, int32_t* status_word, cudaStream_t s) {
-    static EncodeTiledFn enc = nullptr;
-    if (!enc) {
-        void* fn = nullptr;
-        cudaDriverEntryPointQueryResult qres;
-        RDK_CUDA(cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres));
-        if (qres != cudaDriverEntryPointSuccess || !fn) {
-            set_error("rdk_redistribute_exact: the driver does not provide cuTensorMapEncodeTiled");
-            return RDK_ERR_CUDA;
-        }
-        enc = reinterpret_cast<EncodeTiledFn>(fn);
-    }
     if ((reinterpret_cast<uintptr_t>(A) & 15u) || (lda % 8) || (ldm % 8)) {
         set_error("rdk_redistribute_exact: tensor-core operands need 16-byte aligned rows");
         return RDK_ERR_INVALID_ARG;
     }
     CUtensorMap mapA, mapB;
-    int st = make_map(enc, &mapA, A, (uint64_t)n, (uint64_t)rows, (uint64_t)lda, kBK, kTileM);
+    int st = make_map(&mapA, A, (uint64_t)n, (uint64_t)rows, (uint64_t)lda, kBK, kTileM);
     if (st != RDK_OK) return st;
-    st = make_map(enc, &mapB, Mt, (uint64_t)n, (uint64_t)N, (uint64_t)ldm, kBK, kBN);
+    st = make_map(&mapB, Mt, (uint64_t)n, (uint64_t)N, (uint64_t)ldm, kBK, kBN);
     if (st != RDK_OK) return st;
     TcParams P;
     P.w = w_out; P.S = S_out; P.rows = rows; P.N = N; P.K = n;
