@@ -237,7 +237,8 @@ int rdk_redistribute_linear(const rdk_problem* problem, const void* target, cons
  *   trials     >= 1 independent draws per row (each uses its own 4 uniforms)
  *   out        see rdk_outputs
  *   ws         device workspace of rdk_sample_workspace_bytes(problem, mode, trials) bytes, 256-byte
- *              aligned (may be NULL when that size is 0).  The streaming kernels keep there one
+ *              aligned (may be NULL when that size is 0; the precomputed mode counts accepted_len in the
+ *              kernel that draws if given 8 bytes per (sequence, trial), else in one more launch).  The streaming kernels keep there one
  *              record of 4160 bytes per row (row scalars and per-segment sums of w, min(p, q~),
  *              max(0, p - q~), p), one 4-byte counter per (sequence, trial), and 64 bytes per
  *              (row, CTA sharing the row) through which those CTAs exchange their partial

@@ -317,7 +317,7 @@ def outputs_struct(out: Dict[str, torch.Tensor]) -> rdk_outputs:
 
 def sample_workspace(pb: rdk_problem, mode: int, trials: int, device) -> torch.Tensor:
     nbytes = lib().rdk_sample_workspace_bytes(C.byref(pb), mode, trials)
-    return torch.empty(max(nbytes, 256), dtype=torch.uint8, device=device)
+    return torch.empty(max(nbytes, 256, 8 * pb.batch * trials), dtype=torch.uint8, device=device)
 
 
 def rdk_sample_and_verify(index: KeptIndex, mode: int, target: torch.Tensor,

@@ -27,10 +27,12 @@ constexpr int kAffM = 128, kAffN = 256, kAffK = 64;
 constexpr int kAffABytes = kAffM * kAffK * 2, kAffBBytes = kAffN * kAffK * 2;       // 16 KB, 32 KB
 constexpr int kAffStage = kAffABytes + kAffBBytes;
 constexpr int kAffStages = 3;
-constexpr int kAffEpiWarps = 8;                          // two per quarter of the TMEM lanes, each with half of the columns
-constexpr int kAffThreads = 64 + 32 * kAffEpiWarps;
+// Epilogue warps: 16 for the sums, whose exponentials need the latency hidden (101 us instead of 118 with 8), 8 with two
+// store buffers each for the write, which waits for memory (170 us instead of 181 with 16).
+constexpr int kAffSumWarps = 16, kAffWriteWarps = 8;
+constexpr int kAffStoreBuffers = 16;
 constexpr int kAffStoreBytes = 32 * 128;                 // a warp's 32 rows x 64 bf16
-constexpr int kAffSmem = kAffStages * kAffStage + kAffEpiWarps * 2 * kAffStoreBytes + 1024;
+constexpr int kAffSmem = kAffStages * kAffStage + kAffStoreBuffers * kAffStoreBytes + 1024;
 constexpr int kAffSpan = 4;                              // column tiles per work item of kAffSums
 constexpr uint32_t kAffIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kAffN >> 3) << 17) | ((uint32_t)(kAffM >> 4) << 24);
 
@@ -44,13 +46,17 @@ struct AffParams {
     const float* col_inv;              // 1 / |e| of the columns, zero-padded to whole tiles
     const float* col_off;              // kAffWrite: exponent offset -1 / tau - log2 Z of every column (-inf: weight 0)
     float scale;                       // log2(e) / tau
-    float* part;                       // kAffSums: [2 tiles_n][row tiles * 128]
+    float* part;                       // kAffSums: [kAffSumWarps / 4 * tiles_n][row tiles * 128]
     int32_t* status;
 };
 
+constexpr int aff_threads(int mode) { return 64 + 32 * (mode == kAffSums ? kAffSumWarps : kAffWriteWarps); }
+
 template <int MODE>
-__global__ void __launch_bounds__(kAffThreads, 1)
+__global__ void __launch_bounds__(aff_threads(MODE), 1)
 aff_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__ CUtensorMap tmapB, const __grid_constant__ CUtensorMap tmapC, const AffParams P) {
+    constexpr int kEpi = MODE == kAffSums ? kAffSumWarps : kAffWriteWarps, kCols = 4 * kAffN / kEpi;     // columns per epilogue warp
+    constexpr int kBufs = kAffStoreBuffers / kEpi;
     extern __shared__ __align__(1024) unsigned char aff_smem[];
     unsigned char* tiles = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(aff_smem) + 1023) & ~uintptr_t(1023));
     __shared__ __align__(8) unsigned long long full_bar[kAffStages], empty_bar[kAffStages], acc_full[2], acc_empty[2];
@@ -66,7 +72,7 @@ aff_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__
         }
         for (int a = 0; a < 2; ++a) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(s32(&acc_full[a])));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(s32(&acc_empty[a])), "r"(kAffEpiWarps));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(s32(&acc_empty[a])), "r"(kEpi));
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -138,10 +144,11 @@ aff_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__
             }
         }
     } else {
-        const int quarter = warp & 3, half = (warp - 2) >> 2;        // TMEM lanes 32 quarter .. + 32, columns 128 half .. + 128
-        const uint32_t taddr0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(half * 128);
-        unsigned char* stage_c = tiles + kAffStages * kAffStage + (warp - 2) * 2 * kAffStoreBytes;
-        int acc = 0, buf = 0;
+        int buf = 0;
+        const int quarter = warp & 3, share = (warp - 2) >> 2;       // TMEM lanes 32 quarter .. + 32, columns kCols share .. + kCols
+        const uint32_t taddr0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(share * kCols);
+        unsigned char* stage_c = tiles + kAffStages * kAffStage + (warp - 2) * kBufs * kAffStoreBytes;
+        int acc = 0;
         uint32_t acc_phase = 0;
         bool ok = true;
         for (int item = blockIdx.x; item < P.num_items && ok; item += gridDim.x) {
@@ -150,17 +157,17 @@ aff_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__
             const float2 rs = splat(__ldg(P.row_inv + row) * P.scale);
             float2 sum_a = splat(0.f), sum_b = splat(0.f);
             for (int tn = tn0; tn < min(tn0 + kSpan, col_tiles); ++tn) {
-                const int c0 = tn * kAffN + half * 128;
+                const int c0 = tn * kAffN + share * kCols;
                 if (!tc_wait(&acc_full[acc], acc_phase, abort)) { ok = false; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 uint32_t v[2][32];
                 tmem_ld32(taddr0 + (uint32_t)(acc * kAffN), v[0]);
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
+                for (int c = 0; c < kCols / 32; ++c) {
                     tmem_wait_ld(v[c & 1]);
-                    if (c < 3) tmem_ld32(taddr0 + (uint32_t)(acc * kAffN + (c + 1) * 32), v[(c + 1) & 1]);
+                    if (c < kCols / 32 - 1) tmem_ld32(taddr0 + (uint32_t)(acc * kAffN + (c + 1) * 32), v[(c + 1) & 1]);
                     uint32_t (&x)[32] = v[c & 1];
-                    if (c == 3) {                                    // the accumulator is in registers: the next tile may have it
+                    if (c == kCols / 32 - 1) {                       // the accumulator is in registers: the next tile may have it
                         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                         __syncwarp();
                         if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(s32(&acc_empty[acc])) : "memory");
@@ -186,7 +193,7 @@ aff_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__
                     } else {
                         const float4* co = reinterpret_cast<const float4*>(P.col_off + col);
                         if ((c & 1) == 0) {                          // the staging buffer's last store has been read
-                            if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+                            if (lane == 0) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kBufs - 1) : "memory");
                             __syncwarp();
                         }
                         const uint32_t rowaddr = s32(stage_c + buf * kAffStoreBytes) + (uint32_t)lane * 128u;
@@ -216,14 +223,14 @@ aff_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__
                                                  ::"l"(reinterpret_cast<uint64_t>(&tmapC)), "r"(x0), "r"(y0), "r"(s32(stage_c + buf * kAffStoreBytes)) : "memory");
                                 asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                             }
-                            buf ^= 1;
+                            if (++buf == kBufs) buf = 0;
                         }
                     }
                 }
                 if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
             }
             if (MODE == kAffSums && ok)
-                P.part[(long long)((item % P.tiles_n) * 2 + half) * (P.tiles_m * kAffM) + row] = (sum_a.x + sum_a.y) + (sum_b.x + sum_b.y);
+                P.part[(long long)((item % P.tiles_n) * 4 + share) * (P.tiles_m * kAffM) + row] = (sum_a.x + sum_a.y) + (sum_b.x + sum_b.y);
         }
         if (MODE == kAffWrite && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     }
@@ -307,7 +314,7 @@ __global__ void aff_poison_kernel(const int32_t* status, __nv_bfloat16* Mt) {
 // ------------------------------------------------------------------------------------------------
 // host side
 // ------------------------------------------------------------------------------------------------
-// workspace: inv[Npad] | invk[npad] | off[npad] | status | Ek[n, dpad] bf16 | part[2 spans, npad] | Epad[N, dpad] bf16
+// workspace: inv[Npad] | invk[npad] | off[npad] | status | Ek[n, dpad] bf16 | part[4 spans, npad] | Epad[N, dpad] bf16
 struct AffTcLayout { size_t inv, invk, off, status, Ek, part, Epad, total; int Npad, npad, dpad, spans; };
 static AffTcLayout aff_tc_layout(int N, int n, int d) {
     AffTcLayout L;
@@ -321,7 +328,7 @@ static AffTcLayout aff_tc_layout(int N, int n, int d) {
     L.off = o;    o += idx_align((size_t)L.npad * sizeof(float));
     L.status = o; o += idx_align(sizeof(int32_t));
     L.Ek = o;     o += idx_align((size_t)n * L.dpad * sizeof(__nv_bfloat16));
-    L.part = o;   o += idx_align((size_t)2 * L.spans * L.npad * sizeof(float));
+    L.part = o;   o += idx_align((size_t)4 * L.spans * L.npad * sizeof(float));
     L.Epad = o;   o += idx_align((size_t)N * L.dpad * sizeof(__nv_bfloat16));
     L.total = o;
     return L;
@@ -390,13 +397,13 @@ int build_affinity_tc(const __nv_bfloat16* E, int d, long long estride, const in
     const long long items_w = (long long)(L.Npad / kAffM) * (L.npad / kAffN);
     if (items > 0x7fffffffLL || items_w > 0x7fffffffLL) { set_error("rdk_build_affinity: too many tiles"); return RDK_ERR_UNSUPPORTED; }
     P.num_items = (int)items;
-    RDK_CUDA(launch_pdl(aff_tc_kernel<kAffSums>, (unsigned)(items < sms ? items : sms), (unsigned)kAffThreads, (size_t)kAffSmem, s, keptA, tokB, out, P));
-    RDK_CUDA(launch_pdl(aff_offset_kernel, (unsigned)(L.npad / 32), 256u, 0, s, (const float*)part, (const float*)invk, off, 2 * L.spans, L.npad, scale));
+    RDK_CUDA(launch_pdl(aff_tc_kernel<kAffSums>, (unsigned)(items < sms ? items : sms), (unsigned)aff_threads(kAffSums), (size_t)kAffSmem, s, keptA, tokB, out, P));
+    RDK_CUDA(launch_pdl(aff_offset_kernel, (unsigned)(L.npad / 32), 256u, 0, s, (const float*)part, (const float*)invk, off, 4 * L.spans, L.npad, scale));
     // the matrix: rows = tokens, columns = kept ids
     P.tiles_m = L.Npad / kAffM; P.tiles_n = L.npad / kAffN; P.cols = n;
     P.row_inv = inv; P.col_inv = invk; P.col_off = off;
     P.num_items = (int)items_w;
-    RDK_CUDA(launch_pdl(aff_tc_kernel<kAffWrite>, (unsigned)(items_w < sms ? items_w : sms), (unsigned)kAffThreads, (size_t)kAffSmem, s, tokA, keptB, out, P));
+    RDK_CUDA(launch_pdl(aff_tc_kernel<kAffWrite>, (unsigned)(items_w < sms ? items_w : sms), (unsigned)aff_threads(kAffWrite), (size_t)kAffSmem, s, tokA, keptB, out, P));
     RDK_CUDA(launch_pdl(aff_poison_kernel, 1u, 1u, 0, s, (const int32_t*)status, Mt));
     return RDK_OK;
 }

@@ -4,129 +4,172 @@
 // the bf16 layout lives in rdk_exact_tc.cu.
 #include <math.h>
 
-#include "rdk_common.cuh"
+#include "rdk_row.cuh"
 
 namespace rdk {
 
 int launch_exact_tc(const __nv_bfloat16* A, long long lda, const __nv_bfloat16* Mt, long long ldm,
                     float* w_out, float* S_out, int rows, int n, int N, int32_t* status_word, cudaStream_t s);
 
+constexpr int kOperandThreads = 512;
+
 // A[r, i] = q'_{kappa_i}: soft-max over the drafter entries whose id lies in the target vocabulary
 // (Eq. tli-drafter: drop the rest, renormalise), zero for dropped entries and for the padding
-// columns i in [n, lda).
+// columns i in [n, lda); S[r] = 0 for the contraction to add to.
+// Two passes over the row in 16-byte vectors, the second out of L1/L2; the ids are looked at only where the index says
+// that some lie outside the vocabulary.  (Three passes with an element and an id at a time took 99 us for 320 rows of
+// 32064 entries, 10 times the memory time.)
 template <typename TY, typename TA, int KIND>
-__global__ void __launch_bounds__(256)
-exact_operand_kernel(const TY* __restrict__ drafter, long long dstride, const int32_t* __restrict__ ids,
-                     int N, int n, TA* __restrict__ A, long long lda) {
-    __shared__ float red[8];
-    __shared__ float bc[2];
+__global__ void __launch_bounds__(kOperandThreads)
+exact_operand_kernel(const TY* __restrict__ drafter, long long dstride, const int32_t* __restrict__ header, const int32_t* __restrict__ ids,
+                     int N, int n, TA* __restrict__ A, long long lda, float* __restrict__ S) {
+    __shared__ MS red[kOperandThreads / 32];
     const int row = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const TY* y = drafter + (long long)row * dstride;
-    float m = -INFINITY;
-    if (KIND == RDK_LOGITS) {
-        for (int i = tid; i < n; i += 256) {
-            const int id = ids[i];
-            if (id >= 0 && id < N) m = fmaxf(m, to_float<TY>(y[i]));
-        }
-        m = warp_max(m);
-        if (lane == 0) red[warp] = m;
-        __syncthreads();
-        if (tid == 0) { float mm = red[0]; for (int k = 1; k < 8; ++k) mm = fmaxf(mm, red[k]); bc[0] = mm; }
-        __syncthreads();
-        m = bc[0];
-    }
-    float s = 0.f;
-    for (int i = tid; i < n; i += 256) {
-        const int id = ids[i];
-        if (id >= 0 && id < N) {
-            const float v = to_float<TY>(y[i]);
-            s += (KIND == RDK_LOGITS) ? ex2((v - m) * kLog2e) : v;
-        }
-    }
-    s = warp_sum(s);
-    __syncthreads();
-    if (lane == 0) red[warp] = s;
-    __syncthreads();
-    if (tid == 0) { float t = 0.f; for (int k = 0; k < 8; ++k) t += red[k]; bc[1] = 1.f / t; }
-    __syncthreads();
-    const float inv = bc[1];
-    TA* a = A + (long long)row * lda;
-    for (int i = tid; i < lda; i += 256) {
-        float q = 0.f;
-        if (i < n) {
-            const int id = ids[i];
-            if (id >= 0 && id < N) {
-                const float v = to_float<TY>(y[i]);
-                q = ((KIND == RDK_LOGITS) ? ex2((v - m) * kLog2e) : v) * inv;
+    const bool vec = (reinterpret_cast<uintptr_t>(y) & 15u) == 0;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // only now: the contraction may fetch the affinity matrix as soon as it is let go, and that may have been written by
+    // the kernel before this one
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const bool all_valid = __ldg(header + kHdrMagic) == kIdxMagic && __ldg(header + kHdrN) == N && __ldg(header + kHdrn) == n && __ldg(header + kHdrValid) == n;
+    // the row's entries i .. i + 7; what carries no weight reads as -inf (a logit) or 0
+    constexpr float kNone = KIND == RDK_LOGITS ? -INFINITY : 0.f;
+    auto load_y = [&](int i, float (&v)[kVec]) {
+        load8<TY>(y, i, n, vec, kNone, v);
+        if (!all_valid) {
+#pragma unroll
+            for (int k = 0; k < kVec; ++k) {
+                const int id = i + k < n ? __ldg(ids + i + k) : -1;
+                if (id < 0 || id >= N) v[k] = kNone;
             }
         }
-        if (sizeof(TA) == 4) reinterpret_cast<float*>(a)[i] = q;
-        else reinterpret_cast<__nv_bfloat16*>(a)[i] = __float2bfloat16_rn(q);
+    };
+    MS a{KIND == RDK_LOGITS ? -INFINITY : 0.f, 0.f, 0.f};
+#pragma unroll 2
+    for (int i = tid * kVec; i < n; i += kOperandThreads * kVec) {
+        float v[kVec];
+        load_y(i, v);
+        if (KIND == RDK_LOGITS) {
+            float vmax = v[0];
+#pragma unroll
+            for (int k = 1; k < kVec; ++k) vmax = fmaxf(vmax, v[k]);
+            if (vmax > a.m) { a.s *= ex2((a.m - vmax) * kLog2e); a.m = vmax; }
+            const float off = a.m > -INFINITY ? -a.m * kLog2e : 0.f;
+#pragma unroll
+            for (int k = 0; k < kVec; ++k) a.s += ex2(fmaf(v[k], kLog2e, off));
+        } else {
+#pragma unroll
+            for (int k = 0; k < kVec; ++k) a.s += v[k];
+        }
+    }
+    a = ms_warp(a);
+    if (lane == 0) red[warp] = a;
+    __syncthreads();
+    a = ms_warp(lane < kOperandThreads / 32 ? red[lane] : MS{-INFINITY, 0.f, 0.f});
+    const float off = KIND == RDK_LOGITS ? -a.m * kLog2e : 0.f, inv = 1.f / a.s;
+    TA* out = A + (long long)row * lda;
+    for (int i = tid * kVec; i < lda; i += kOperandThreads * kVec) {
+        float v[kVec];
+        load_y(i, v);
+#pragma unroll
+        for (int k = 0; k < kVec; ++k) v[k] = (KIND == RDK_LOGITS ? ex2(fmaf(v[k], kLog2e, off)) : v[k]) * inv;
+        if (sizeof(TA) == 2) {                   // lda is a multiple of 64 and the rows are 16-byte aligned
+            uint32_t w[4];
+#pragma unroll
+            for (int h = 0; h < 4; ++h) asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w[h]) : "f"(v[2 * h + 1]), "f"(v[2 * h]));
+            *reinterpret_cast<uint4*>(out + i) = make_uint4(w[0], w[1], w[2], w[3]);
+        } else {
+#pragma unroll
+            for (int k = 0; k < kVec; ++k) if (i + k < lda) reinterpret_cast<float*>(out)[i + k] = v[k];
+        }
+    }
+    if (tid == 0 && S) S[row] = 0.f;
+}
+
+// w[r, j] = sum_i A[r, i] M[i, j]  with fp32 FMAs (fp32 row layout of M; small problems), S[r] += the sums of w.
+// A CTA takes 8 rows x 32 VC columns; its warps share the contraction (warp w takes i = w, w + 8, ...) and add up in shared
+// memory.  With a thread for a column and all of the contraction, 4 x 1024 x 256 ran on 4 SMs with one load in flight:
+// 27 us.
+constexpr int kFmaRows = 8, kFmaWarps = 8, kFmaChunk = 256;
+template <int VC>
+__global__ void __launch_bounds__(kFmaWarps * 32)
+exact_fma_kernel(const float* __restrict__ A, long long lda, const float* __restrict__ M, long long ldm,
+                 float* __restrict__ w, float* __restrict__ S, int rows, int n, int N) {
+    constexpr int kCols = 32 * VC;
+    __shared__ __align__(16) float a_s[kFmaChunk][kFmaRows];
+    __shared__ float part[kFmaWarps][kFmaRows][kCols];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int j0 = blockIdx.x * kCols, r0 = blockIdx.y * kFmaRows, j = j0 + lane * VC;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    float acc[kFmaRows][VC];
+#pragma unroll
+    for (int r = 0; r < kFmaRows; ++r)
+#pragma unroll
+        for (int c = 0; c < VC; ++c) acc[r][c] = 0.f;
+    for (int i0 = 0; i0 < n; i0 += kFmaChunk) {
+        const int lim = min(kFmaChunk, n - i0);
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < kFmaRows; ++r) a_s[tid][r] = (r0 + r < rows && tid < lim) ? A[(long long)(r0 + r) * lda + i0 + tid] : 0.f;
+        __syncthreads();
+#pragma unroll 8
+        for (int ii = warp; ii < lim; ii += kFmaWarps) {
+            float mv[VC];
+            const float* m = M + (long long)(i0 + ii) * ldm + j;
+            if (VC == 4) {
+                const float4 q = __ldg(reinterpret_cast<const float4*>(m));
+                mv[0] = q.x; mv[VC > 1 ? 1 : 0] = q.y; mv[VC > 2 ? 2 : 0] = q.z; mv[VC > 3 ? 3 : 0] = q.w;
+            } else {
+                mv[0] = j < N ? __ldg(m) : 0.f;
+            }
+            const float4 a0 = *reinterpret_cast<const float4*>(&a_s[ii][0]), a1 = *reinterpret_cast<const float4*>(&a_s[ii][4]);
+            const float av[kFmaRows] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+#pragma unroll
+            for (int r = 0; r < kFmaRows; ++r)
+#pragma unroll
+                for (int c = 0; c < VC; ++c) acc[r][c] = fmaf(av[r], mv[c], acc[r][c]);
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < kFmaRows; ++r)
+#pragma unroll
+        for (int c = 0; c < VC; ++c) part[warp][r][lane * VC + c] = acc[r][c];
+    __syncthreads();
+    for (int o = tid; o < kFmaRows * kCols; o += kFmaWarps * 32) {
+        const int r = o / kCols, c = o % kCols;
+        float v = 0.f;
+#pragma unroll
+        for (int k = 0; k < kFmaWarps; ++k) v += part[k][r][c];
+        const bool in = r0 + r < rows && j0 + c < N;
+        if (in) w[(long long)(r0 + r) * N + j0 + c] = v;
+        if (S) {
+            v = warp_sum(in ? v : 0.f);
+            if (lane == 0 && r0 + r < rows) atomicAdd(S + r0 + r, v);
+        }
     }
 }
 
-constexpr int kSimtRows = 8;
-
-// w[r, j] = sum_i A[r, i] M[i, j]  with fp32 FMAs (fp32 row layout of M; small problems).
-__global__ void __launch_bounds__(256)
-exact_simt_kernel(const float* __restrict__ A, long long lda, const float* __restrict__ M, long long ldm,
-                  float* __restrict__ w, int rows, int n, int N) {
-    __shared__ float a_s[kSimtRows][256];
-    const int j = blockIdx.x * 256 + threadIdx.x;
-    const int r0 = blockIdx.y * kSimtRows;
-    float acc[kSimtRows];
-#pragma unroll
-    for (int r = 0; r < kSimtRows; ++r) acc[r] = 0.f;
-    for (int i0 = 0; i0 < n; i0 += 256) {
-        __syncthreads();
-#pragma unroll
-        for (int r = 0; r < kSimtRows; ++r) {
-            const int i = i0 + threadIdx.x;
-            a_s[r][threadIdx.x] = (r0 + r < rows && i < n) ? A[(long long)(r0 + r) * lda + i] : 0.f;
-        }
-        __syncthreads();
-        if (j < N) {
-            const int lim = min(256, n - i0);
-            for (int ii = 0; ii < lim; ++ii) {
-                const float mv = __ldg(M + (long long)(i0 + ii) * ldm + j);
-#pragma unroll
-                for (int r = 0; r < kSimtRows; ++r) acc[r] = fmaf(a_s[r][ii], mv, acc[r]);
-            }
-        }
-    }
-    if (j < N) {
-#pragma unroll
-        for (int r = 0; r < kSimtRows; ++r)
-            if (r0 + r < rows) w[(long long)(r0 + r) * N + j] = acc[r];
-    }
-}
-
-// S[r] = sum_j w[r, j]
-__global__ void __launch_bounds__(256)
-row_sum_kernel(const float* __restrict__ w, int N, float* __restrict__ S) {
-    __shared__ double red[8];
-    const float* row = w + (long long)blockIdx.x * N;
-    float s = 0.f;
-    double acc = 0.0;
-    int cnt = 0;
-    for (int j = threadIdx.x; j < N; j += 256) {
-        s += row[j];
-        if (++cnt == 64) { acc += (double)s; s = 0.f; cnt = 0; }
-    }
-    acc += (double)s;
-    acc = warp_sum_d(acc);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) { double t = 0.0; for (int k = 0; k < 8; ++k) t += red[k]; S[blockIdx.x] = (float)t; }
+template <typename K, typename... A>
+static cudaError_t launch_pdl(K kern, dim3 grid, unsigned block, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block, 1, 1);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
 template <typename TY, typename TA>
-static void launch_operand(const void* drafter, long long dstride, const int32_t* ids, int N, int n, int kind,
-                           void* A, long long lda, int rows, cudaStream_t s) {
-    if (kind == RDK_LOGITS)
-        exact_operand_kernel<TY, TA, RDK_LOGITS><<<rows, 256, 0, s>>>(static_cast<const TY*>(drafter), dstride, ids, N, n, static_cast<TA*>(A), lda);
-    else
-        exact_operand_kernel<TY, TA, RDK_PROBS><<<rows, 256, 0, s>>>(static_cast<const TY*>(drafter), dstride, ids, N, n, static_cast<TA*>(A), lda);
+static cudaError_t launch_operand(const void* drafter, long long dstride, const KeptIndexView& v, int N, int n, int kind,
+                                  void* A, long long lda, float* S, int rows, cudaStream_t s) {
+    auto k = kind == RDK_LOGITS ? exact_operand_kernel<TY, TA, RDK_LOGITS> : exact_operand_kernel<TY, TA, RDK_PROBS>;
+    return launch_pdl(k, dim3((unsigned)rows), (unsigned)kOperandThreads, s, static_cast<const TY*>(drafter), dstride, v.header, v.ids, N, n,
+                      static_cast<TA*>(A), lda, S);
 }
 
 static long long operand_ld(int n, int layout) {
@@ -186,27 +229,20 @@ extern "C" int rdk_redistribute_exact(const rdk_problem* problem, const void* dr
     const long long dstride = problem->drafter_row_stride ? problem->drafter_row_stride : n;
     const long long lda = operand_ld(n, M->layout);
     const bool bf = M->layout == RDK_AFF_BF16_COLS;
-    if (problem->drafter_dtype == RDK_F32) {
-        if (bf) launch_operand<float, __nv_bfloat16>(drafter, dstride, v.ids, N, n, problem->drafter_kind, ws, lda, rows, s);
-        else launch_operand<float, float>(drafter, dstride, v.ids, N, n, problem->drafter_kind, ws, lda, rows, s);
-    } else {
-        if (bf) launch_operand<__nv_bfloat16, __nv_bfloat16>(drafter, dstride, v.ids, N, n, problem->drafter_kind, ws, lda, rows, s);
-        else launch_operand<__nv_bfloat16, float>(drafter, dstride, v.ids, N, n, problem->drafter_kind, ws, lda, rows, s);
-    }
-    RDK_CUDA(cudaGetLastError());
-    if (bf) {
-        // the tensor-core epilogue also accumulates S (one atomic partial sum per row and tile)
-        return launch_exact_tc(static_cast<const __nv_bfloat16*>(ws), lda, static_cast<const __nv_bfloat16*>(M->data), M->ld,
-                               w_out, S_out, rows, n, N, status_word, s);
-    } else {
-        dim3 grid((N + 255) / 256, (rows + kSimtRows - 1) / kSimtRows);
-        exact_simt_kernel<<<grid, 256, 0, s>>>(static_cast<const float*>(ws), lda, static_cast<const float*>(M->data), M->ld, w_out, rows, n, N);
-        RDK_CUDA(cudaGetLastError());
-    }
-    if (S_out) {
-        row_sum_kernel<<<rows, 256, 0, s>>>(w_out, N, S_out);
-        RDK_CUDA(cudaGetLastError());
-    }
+    using B = __nv_bfloat16;
+    const bool f = problem->drafter_dtype == RDK_F32;
+    const int kind = problem->drafter_kind;
+    if (bf) RDK_CUDA((f ? launch_operand<float, B> : launch_operand<B, B>)(drafter, dstride, v, N, n, kind, ws, lda, S_out, rows, s));
+    else RDK_CUDA((f ? launch_operand<float, float> : launch_operand<B, float>)(drafter, dstride, v, N, n, kind, ws, lda, S_out, rows, s));
+    // either contraction also accumulates S (one atomic partial sum per row and warp or CTA)
+    if (bf)
+        return launch_exact_tc(static_cast<const B*>(ws), lda, static_cast<const B*>(M->data), M->ld, w_out, S_out, rows, n, N, status_word, s);
+    // four columns a thread where that still fills the chip, M's rows are whole 16-byte units and a CTA's columns exist
+    const float *A = static_cast<const float*>(ws), *Mf = static_cast<const float*>(M->data);
+    const unsigned ry = (unsigned)((rows + kFmaRows - 1) / kFmaRows);
+    const bool wide = N % 128 == 0 && M->ld % 4 == 0 && !(reinterpret_cast<uintptr_t>(Mf) & 15u) && (long long)(N / 128) * ry >= 296;
+    if (wide) RDK_CUDA(launch_pdl(exact_fma_kernel<4>, dim3((unsigned)(N / 128), ry), kFmaWarps * 32u, s, A, lda, Mf, (long long)M->ld, w_out, S_out, rows, n, N));
+    else RDK_CUDA(launch_pdl(exact_fma_kernel<1>, dim3((unsigned)((N + 31) / 32), ry), kFmaWarps * 32u, s, A, lda, Mf, (long long)M->ld, w_out, S_out, rows, n, N));
     return RDK_OK;
 }
 

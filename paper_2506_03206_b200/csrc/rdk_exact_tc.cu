@@ -1,14 +1,21 @@
 // Exact redistribution on the tensor cores (Algorithm 1 step 2):  w = q' M,  i.e.
-//   w[r, j] = sum_i A[r, i] Mt[j, i]
+//   w[r, j] = sum_i Mt[j, i] A[r, i]
 // with A = q' (bf16, [rows, K = n], contraction index contiguous) and Mt = the transposed affinity
 // matrix (bf16, [N, K]); products accumulate in fp32.
 //
-// One persistent CTA per SM.  A work item is a 256 x 256 tile of w: two 128 x 256 accumulators in
-// tensor memory (all 512 columns), fed from a 3-stage ring of 64-wide K blocks in shared memory.
-//   warp 0   : TMA producer   (cp.async.bulk.tensor, 128-byte swizzle, out-of-range rows/cols read 0)
-//   warp 1   : MMA issuer     (tcgen05.mma kind::f16, one elected lane) and owner of the TMEM allocation
-//   warps 2-5: epilogue       (tcgen05.ld 32 lanes x 32 columns -> fp32 stores to w)
-// Items are ordered so that the row tiles of one 256-column panel of Mt run at the same time: the
+// The vocabulary takes the M side of the instruction, the rows the N side, which comes in steps of 16: 20 rows cost the
+// tensor cores 32, not 256, and 320 rows cost 320.  A persistent pair of CTAs (cta_group::2, one CTA per SM) computes a
+// work item of 256 tokens x up to 512 rows: each CTA holds its own 128 tokens of Mt and half of the rows of A per 64-wide
+// K block, and the 128 x (T R) fp32 accumulators of its tokens in tensor memory (T = 1 or 2 instructions of R rows).
+// Both operands of a pair are fetched once, so a K block of 512 rows needs 48 KB per CTA for 128 x 512 x 64 products;
+// a CTA by itself with a 256 x 256 tile needs 64 KB, and what an SM can keep in flight bounded it (1024 rows x 32k:
+// 374 us; 320 rows x 128k in padded tiles of 256 rows 3140 us).
+//   warp 0   : TMA producer of its CTA   (128-byte swizzle, out-of-range rows and columns read 0; completion is counted
+//              on the leader's barrier)
+//   warp 1   : in the leader CTA the MMA issuer; in both the owner of the TMEM allocation
+//   warps 2-9: epilogue: a lane is a token, a column a row of w, so a warp stores 32 consecutive tokens per row;
+//              row sums by a butterfly over the lanes and one atomic per row and warp
+// Items are ordered so that the row tiles of one 256-token panel of Mt run at the same time: the
 // panel is fetched from HBM once and shared through L2.
 // Every wait is bounded; on expiry the CTA flags RDK_ERR_TIMEOUT in the status word and winds down.
 #include <atomic>
@@ -17,194 +24,225 @@
 
 namespace rdk {
 
-constexpr int kBM = 128;                 // rows of one MMA
-constexpr int kTileM = 256;              // rows of one work item (two MMAs)
-constexpr int kBN = 256;
+constexpr int kVoc = 128;                // tokens of one CTA
 constexpr int kBK = 64;                  // K block: 64 bf16 = 128 bytes = one swizzle row
-constexpr int kStages = 3;
-constexpr int kABytes = kTileM * kBK * 2;        // 32 KB
-constexpr int kBBytes = kBN * kBK * 2;           // 32 KB
-constexpr int kStageBytes = kABytes + kBBytes;   // 64 KB
-constexpr int kTcThreads = 192;
-constexpr int kTmemCols = 512;
+constexpr int kVocBytes = kVoc * kBK * 2;        // 16 KB
+constexpr int kTcMaxStages = 12;
+constexpr int kTcSmem = 227 * 1024 - 2048;       // for the ring, alignment included
+constexpr int kTcEpiWarps = 8;
+constexpr int kTcThreads = 64 + 32 * kTcEpiWarps;
 
 struct TcParams {
-    float* w; float* S; int rows, N, K;
-    int tiles_m, tiles_n, num_kb;
-    int full_items, num_items;       // items [0, full_items) are 256-row tiles, the rest 128-row halves
+    float* w; float* S; int rows, N;
+    int R, T;                        // rows of one instruction, instructions per item
+    int tiles_r, num_kb, stages;
+    int full_items, num_items;       // items [0, full_items) are whole, the rest halves (one instruction of R rows)
     int32_t* status_word;
 };
 
-// Work item -> first row, column tile and number of 128-row MMAs.  The last partial round of
-// 256-row tiles is cut into 128-row halves so that it costs half a round instead of a whole one.
-__device__ __forceinline__ void decode_item(const TcParams& P, int item, int& row0, int& tn, int& mt) {
-    int tile, half = -1;
-    if (item < P.full_items) tile = item;
-    else { tile = P.full_items + ((item - P.full_items) >> 1); half = (item - P.full_items) & 1; }
-    const int tm = tile % P.tiles_m;
-    tn = tile / P.tiles_m;
-    row0 = tm * kTileM + (half > 0 ? kBM : 0);
-    const int left = P.rows - row0;
-    mt = left <= 0 ? 0 : ((half < 0 && left > kBM) ? 2 : 1);
+// Work item -> token tile, first row, instructions.  The last partial round of items is cut into halves so that it
+// costs half a round instead of a whole one.
+__device__ __forceinline__ void decode_item(const TcParams& P, int item, int& tv, int& row0, int& t) {
+    int tile = item, half = 0;
+    t = P.T;
+    if (item >= P.full_items) { tile = P.full_items + ((item - P.full_items) >> 1); half = (item - P.full_items) & 1; t = 1; }
+    tv = tile / P.tiles_r;
+    row0 = (tile % P.tiles_r) * P.T * P.R + half * P.R;
+    if (row0 >= P.rows) t = 0;                           // a half beyond the last row
+    else if (t == 2 && row0 + P.R >= P.rows) t = 1;
 }
 
-// instruction descriptor: D = fp32, A = B = bf16, both K-major, M = 128, N = 256
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kBN >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
-
-__global__ void __launch_bounds__(kTcThreads, 1)
-exact_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__ CUtensorMap tmapB, const TcParams P) {
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1)
+exact_tc_kernel(const __grid_constant__ CUtensorMap tmapV, const __grid_constant__ CUtensorMap tmapR, const TcParams P) {
     extern __shared__ __align__(1024) unsigned char tc_smem[];
-    unsigned char* tiles = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(tc_smem) + 1023) & ~uintptr_t(1023));
-    __shared__ __align__(8) unsigned long long full_bar[kStages], empty_bar[kStages], tmem_full, tmem_empty;
+    const uint32_t ring = (s32(tc_smem) + 1023u) & ~1023u;               // the same offset in both CTAs
+    __shared__ __align__(8) unsigned long long full_bar[kTcMaxStages], empty_bar[kTcMaxStages], acc_full, acc_empty;
     __shared__ uint32_t tmem_base_s;
     __shared__ int abort_s;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     volatile int* abort = &abort_s;
+    uint32_t rank;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    const bool leader = rank == 0;
 
     if (threadIdx.x == 0) {
         abort_s = 0;
-        for (int s = 0; s < kStages; ++s) {
+        for (int s = 0; s < P.stages; ++s) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(s32(&full_bar[s])));
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(s32(&empty_bar[s])));
         }
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(s32(&tmem_full)));
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 4;" ::"r"(s32(&tmem_empty)));
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(s32(&acc_full)));
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(s32(&acc_empty)), "r"(2 * kTcEpiWarps));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(s32(&tmem_base_s)), "r"(kTmemCols) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(s32(&tmem_base_s)) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = tmem_base_s;
-    const int num_items = P.num_items;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+    const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
+    const uint32_t rbytes = (uint32_t)(P.R / 2) * kBK * 2;               // this CTA's half of one instruction's rows
+    const uint32_t stage_bytes = kVocBytes + (uint32_t)P.T * rbytes;
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
-        {
-            int stage = 0; uint32_t phase = 0;
-            bool ok = true;
-            for (int item = blockIdx.x; item < num_items && ok; item += gridDim.x) {
-                int row0, tn, mt;
-                decode_item(P, item, row0, tn, mt);
-                if (mt == 0) continue;                                        // a half tile beyond the last row
-                for (int kb = 0; kb < P.num_kb; ++kb) {
-                    if (!tc_wait(&empty_bar[stage], phase ^ 1u, abort)) { ok = false; break; }
-                    unsigned char* sa = tiles + stage * kStageBytes;
-                    if (lane == 0) {
-                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(s32(&full_bar[stage])), "r"((uint32_t)kStageBytes) : "memory");
-                    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-                                 ::"r"(s32(sa)), "l"(reinterpret_cast<uint64_t>(&tmapA)), "r"(kb * kBK), "r"(row0), "r"(s32(&full_bar[stage])) : "memory");
-                    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-                                 ::"r"(s32(sa + kABytes)), "l"(reinterpret_cast<uint64_t>(&tmapB)), "r"(kb * kBK), "r"(tn * kBN), "r"(s32(&full_bar[stage])) : "memory");
-                    }
-                    __syncwarp();
-                    if (++stage == kStages) { stage = 0; phase ^= 1u; }
-                }
+        // Mt is not written by the kernel before this one (the operand kernel lets this one start only after everything
+        // before it is complete), so its first blocks are requested before the operand is there.
+        int stage = 0; uint32_t phase = 0;
+        bool ok = true, waited = false;
+        auto full_addr = [&](int s) -> uint32_t {        // the leader's barrier
+            uint32_t a;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(a) : "r"(s32(&full_bar[s])));
+            return a;
+        };
+        auto load_voc = [&](int s, int kb, int tv) {
+            asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+                         ::"r"(ring + (uint32_t)s * stage_bytes), "l"(reinterpret_cast<uint64_t>(&tmapV)), "r"(kb * kBK),
+                           "r"((2 * tv + (int)rank) * kVoc), "r"(full_addr(s)) : "memory");
+        };
+        auto load_rows = [&](int s, int kb, int row0, int t) {
+            for (int k = 0; k < t; ++k)
+                asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+                             ::"r"(ring + (uint32_t)s * stage_bytes + kVocBytes + (uint32_t)k * rbytes), "l"(reinterpret_cast<uint64_t>(&tmapR)), "r"(kb * kBK),
+                               "r"(row0 + k * P.R + (int)rank * (P.R / 2)), "r"(full_addr(s)) : "memory");
+        };
+        auto expect = [&](int s, int t) {                // both CTAs' bytes, announced by the leader
+            if (leader)
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(s32(&full_bar[s])), "r"(2u * (kVocBytes + (uint32_t)t * rbytes)) : "memory");
+        };
+        for (int item = pair; item < P.num_items && ok; item += pairs) {
+            int tv, row0, t;
+            decode_item(P, item, tv, row0, t);
+            if (t == 0) continue;
+            int kb = 0;
+            if (!waited) {                               // the ring is free: the first item's first blocks
+                const int first = min(P.stages, P.num_kb);
+                if (lane == 0) for (int s = 0; s < first; ++s) { expect(s, t); load_voc(s, s, tv); }
+                __syncwarp();
+                asm volatile("griddepcontrol.wait;" ::: "memory");
+                if (lane == 0) for (int s = 0; s < first; ++s) load_rows(s, s, row0, t);
+                __syncwarp();
+                waited = true;
+                kb = first;
+                stage = first;
+                if (stage == P.stages) { stage = 0; phase ^= 1u; }
+            }
+            for (; kb < P.num_kb; ++kb) {
+                if (!tc_wait(&empty_bar[stage], phase ^ 1u, abort)) { ok = false; break; }
+                if (lane == 0) { expect(stage, t); load_voc(stage, kb, tv); load_rows(stage, kb, row0, t); }
+                __syncwarp();
+                if (++stage == P.stages) { stage = 0; phase ^= 1u; }
             }
         }
     } else if (warp == 1) {
-        // ------------------------------------------------------------------ MMA issuer
-        {
+        // ------------------------------------------------------------------ MMA issuer (leader only)
+        if (leader) {
+            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(P.R >> 3) << 17) | (16u << 24);   // fp32 += bf16 bf16, M = 256, N = R
             int stage = 0; uint32_t phase = 0, acc_phase = 0;
             bool ok = true;
-            for (int item = blockIdx.x; item < num_items && ok; item += gridDim.x) {
-                int row0, tn, mt;
-                decode_item(P, item, row0, tn, mt);                           // mt = 1: a lone 128-row remainder or half
-                if (mt == 0) continue;
-                if (!tc_wait(&tmem_empty, acc_phase ^ 1u, abort)) break;      // the epilogue has drained the accumulators
+            for (int item = pair; item < P.num_items && ok; item += pairs) {
+                int tv, row0, t;
+                decode_item(P, item, tv, row0, t);
+                if (t == 0) continue;
+                if (!tc_wait(&acc_empty, acc_phase ^ 1u, abort)) break;       // both epilogues have drained the accumulators
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 for (int kb = 0; kb < P.num_kb; ++kb) {
                     if (!tc_wait(&full_bar[stage], phase, abort)) { ok = false; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint32_t a_addr = s32(tiles + stage * kStageBytes), b_addr = a_addr + kABytes;
+                    const uint32_t va = ring + (uint32_t)stage * stage_bytes, ra = va + kVocBytes;
                     if (lane == 0) {
 #pragma unroll
-                    for (int k = 0; k < kBK / 16; ++k) {
-                        const uint64_t bdesc = smem_desc(b_addr + k * 32);
-                        for (int a = 0; a < mt; ++a) {
-                            const uint64_t adesc = smem_desc(a_addr + a * (kBM * kBK * 2) + k * 32);
-                            const uint32_t accum = (kb > 0 || k > 0) ? 1u : 0u;
-                            asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
-                                         ::"r"(tmem_base + (uint32_t)(a * kBN)), "l"(adesc), "l"(bdesc), "r"(kIdesc), "r"(accum) : "memory");
+                        for (int k = 0; k < kBK / 16; ++k) {
+                            const uint64_t vdesc = smem_desc(va + k * 32);
+                            for (int a = 0; a < t; ++a) {
+                                const uint64_t rdesc = smem_desc(ra + (uint32_t)a * rbytes + k * 32);
+                                asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}"
+                                             ::"r"(tmem_base + (uint32_t)(a * P.R)), "l"(vdesc), "l"(rdesc), "r"(idesc), "r"((kb > 0 || k > 0) ? 1u : 0u) : "memory");
+                            }
                         }
-                    }
-                    // frees the stage once the MMAs above have read it
-                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(s32(&empty_bar[stage])) : "memory");
+                        // frees the stage in both CTAs once the MMAs above have read it
+                        asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+                                     ::"r"(s32(&empty_bar[stage])), "h"((uint16_t)3) : "memory");
                     }
                     __syncwarp();
-                    if (++stage == kStages) { stage = 0; phase ^= 1u; }
+                    if (++stage == P.stages) { stage = 0; phase ^= 1u; }
                 }
                 if (!ok) break;
                 if (lane == 0)
-                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(s32(&tmem_full)) : "memory");
+                    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+                                 ::"r"(s32(&acc_full)), "h"((uint16_t)3) : "memory");
                 __syncwarp();
                 acc_phase ^= 1u;
             }
         }
     } else {
         // ------------------------------------------------------------------ epilogue
-        const int quarter = warp & 3;                    // TMEM lanes 32 * quarter .. + 32 belong to this warp
-        const bool vec_ok = (reinterpret_cast<uintptr_t>(P.w) & 15u) == 0 && (P.N & 3) == 0;
+        const int quarter = warp & 3, share = (warp - 2) >> 2;       // TMEM lanes 32 quarter .. + 32; every second block of 32 columns
+        uint32_t empty_addr;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(empty_addr) : "r"(s32(&acc_empty)));
+        asm volatile("griddepcontrol.wait;" ::: "memory");           // S is zeroed by the kernel before this one
         uint32_t acc_phase = 0;
-        for (int item = blockIdx.x; item < num_items; item += gridDim.x) {
-            int row0, tn, mt;
-            decode_item(P, item, row0, tn, mt);
-            if (mt == 0) continue;
-            if (!tc_wait(&tmem_full, acc_phase, abort)) break;
+        for (int item = pair; item < P.num_items; item += pairs) {
+            int tv, row0, t;
+            decode_item(P, item, tv, row0, t);
+            if (t == 0) continue;
+            if (!tc_wait(&acc_full, acc_phase, abort)) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            for (int a = 0; a < mt; ++a) {
-                const int row = row0 + a * kBM + quarter * 32 + lane;
-                float* wrow = P.w + (long long)row * P.N;
-                float rsum = 0.f;
-#pragma unroll 1
-                for (int c = 0; c < kBN / 32; ++c) {
-                    uint32_t v[32];
-                    const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(a * kBN + c * 32);
-                    asm volatile(
-                        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-                        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-                        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-                        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
-                          "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
-                          "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-                        : "r"(taddr) : "memory");
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                    const int col0 = tn * kBN + c * 32;
+            const int tok = (2 * tv + (int)rank) * kVoc + quarter * 32 + lane;
+            const int cols = t * P.R;
+            for (int c = share * 32; c < cols; c += 64) {
+                uint32_t v[32];
+                tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c, v);
+                tmem_wait_ld(v);
+                const int r = row0 + c;
+                float* wp = P.w + (long long)r * P.N + tok;
+                const int left = min(min(P.rows - r, cols - c), 32);
+                if (tok < P.N) {
+                    if (left == 32) {
 #pragma unroll
-                    for (int q = 0; q < 32; ++q) rsum += (col0 + q < P.N) ? __uint_as_float(v[q]) : 0.f;
-                    if (row < P.rows) {
-                        if (vec_ok && col0 + 32 <= P.N) {
+                        for (int q = 0; q < 32; ++q) wp[(long long)q * P.N] = __uint_as_float(v[q]);
+                    } else {
 #pragma unroll
-                            for (int q = 0; q < 8; ++q)
-                                reinterpret_cast<float4*>(wrow + col0)[q] =
-                                    make_float4(__uint_as_float(v[4 * q]), __uint_as_float(v[4 * q + 1]),
-                                                __uint_as_float(v[4 * q + 2]), __uint_as_float(v[4 * q + 3]));
-                        } else {
-#pragma unroll
-                            for (int q = 0; q < 32; ++q)
-                                if (col0 + q < P.N) wrow[col0 + q] = __uint_as_float(v[q]);
-                        }
+                        for (int q = 0; q < 32; ++q) if (q < left) wp[(long long)q * P.N] = __uint_as_float(v[q]);
                     }
                 }
-                if (P.S && row < P.rows) atomicAdd(P.S + row, rsum);           // S = sum_j w_j, one partial per tile
+                if (P.S) {
+                    // sums over the lanes (tokens beyond the vocabulary are zero): lane q ends up with column q's
+#pragma unroll
+                    for (int s = 16; s > 0; s >>= 1) {
+                        const bool up = lane & s;
+#pragma unroll
+                        for (int q = 0; q < s; ++q) {
+                            const float keep = __uint_as_float(up ? v[q + s] : v[q]), send = __uint_as_float(up ? v[q] : v[q + s]);
+                            v[q] = __float_as_uint(keep + __shfl_xor_sync(0xffffffffu, send, s));
+                        }
+                    }
+                    if (lane < left) atomicAdd(P.S + r + lane, __uint_as_float(v[0]));
+                }
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
-            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(s32(&tmem_empty)) : "memory");
+            if (lane == 0) asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(empty_addr) : "memory");
             acc_phase ^= 1u;
         }
     }
 
+    // after a wait that gave up, copies may still be on their way into shared memory: let them land
+    if (abort_s && warp == 0) for (int k = 0; k < 10000; ++k) __nanosleep(100);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    // neither CTA leaves, nor gives its tensor memory back, while the other may still signal its barriers or read its operands
+    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
     if (warp == 1) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(tmem_base) : "memory");
     }
     if (threadIdx.x == 0 && abort_s && P.status_word) atomicCAS(P.status_word, 0, (int)RDK_ERR_TIMEOUT);
 }
@@ -241,38 +279,62 @@ int make_map(CUtensorMap* map, const void* base, uint64_t inner, uint64_t outer,
     return RDK_OK;
 }
 
+// S_out has to be zeroed by the kernel launched just before, which lets this one start early only once everything before
+// it is complete.
 int launch_exact_tc(const __nv_bfloat16* A, long long lda, const __nv_bfloat16* Mt, long long ldm, float* w_out,
                     float* S_out, int rows, int n, int N, int32_t* status_word, cudaStream_t s) {
     if ((reinterpret_cast<uintptr_t>(A) & 15u) || (lda % 8) || (ldm % 8)) {
         set_error("rdk_redistribute_exact: tensor-core operands need 16-byte aligned rows");
         return RDK_ERR_INVALID_ARG;
     }
-    CUtensorMap mapA, mapB;
-    int st = make_map(&mapA, A, (uint64_t)n, (uint64_t)rows, (uint64_t)lda, kBK, kTileM);
-    if (st != RDK_OK) return st;
-    st = make_map(&mapB, Mt, (uint64_t)n, (uint64_t)N, (uint64_t)ldm, kBK, kBN);
-    if (st != RDK_OK) return st;
+    int dev = 0;
+    RDK_CUDA(cudaGetDevice(&dev));
+    static thread_local int c_dev = -1, sms = 0;
+    if (dev != c_dev) {
+        RDK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        RDK_CUDA(cudaFuncSetAttribute(exact_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem));
+        c_dev = dev;
+    }
     TcParams P;
-    P.w = w_out; P.S = S_out; P.rows = rows; P.N = N; P.K = n;
-    P.tiles_m = (rows + kTileM - 1) / kTileM;
-    P.tiles_n = (N + kBN - 1) / kBN;
+    P.w = w_out; P.S = S_out; P.rows = rows; P.N = N;
     P.num_kb = (n + kBK - 1) / kBK;
     P.status_word = status_word;
-    int dev = 0, sms = 0;
-    RDK_CUDA(cudaGetDevice(&dev));
-    RDK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const long long tiles = (long long)P.tiles_m * P.tiles_n;
+    const long long tiles_v = ((long long)N + 2 * kVoc - 1) / (2 * kVoc);
+    const int pairs_most = sms / 2;
+    // as few row tiles as the 512 accumulator columns allow, more where that leaves pairs without work (down to 64 rows,
+    // below which an item is bound by its part of Mt)
+    long long tiles_r = (rows + 511) / 512;
+    while (tiles_v * tiles_r < pairs_most && rows / tiles_r > 64) ++tiles_r;
+    const int per = (int)((rows + tiles_r - 1) / tiles_r);
+    P.T = per > 256 ? 2 : 1;
+    P.R = P.T == 2 ? ((per + 1) / 2 + 15) / 16 * 16 : (per + 31) / 32 * 32;
+    P.tiles_r = (rows + P.T * P.R - 1) / (P.T * P.R);
+    const int stage_bytes = kVocBytes + P.T * P.R * kBK;
+    P.stages = (kTcSmem - 1024) / stage_bytes;
+    if (P.stages > kTcMaxStages) P.stages = kTcMaxStages;
+    CUtensorMap mapV, mapR;
+    int st = make_map(&mapV, Mt, (uint64_t)n, (uint64_t)N, (uint64_t)ldm, kBK, kVoc);
+    if (st != RDK_OK) return st;
+    st = make_map(&mapR, A, (uint64_t)n, (uint64_t)rows, (uint64_t)lda, kBK, (uint32_t)P.R / 2);
+    if (st != RDK_OK) return st;
+    const long long tiles = tiles_v * P.tiles_r;
     if (tiles > 0x3fffffffLL) { set_error("rdk_redistribute_exact: too many output tiles"); return RDK_ERR_UNSUPPORTED; }
-    const int grid = (int)(tiles < sms ? tiles : sms);
-    const int rest = (int)(tiles % grid);
-    const bool split = rest > 0 && 2 * rest <= grid && tiles > grid;      // cut the last partial round into halves
+    const int pairs = (int)(tiles < pairs_most ? tiles : pairs_most);
+    const int rest = (int)(tiles % pairs);
+    const bool split = P.T == 2 && rest > 0 && 2 * rest <= pairs;         // cut the last partial round into halves
     P.full_items = split ? (int)(tiles - rest) : (int)tiles;
     P.num_items = split ? (int)(tiles + rest) : (int)tiles;
-    if (S_out) RDK_CUDA(cudaMemsetAsync(S_out, 0, (size_t)rows * sizeof(float), s));
-    const size_t smem = (size_t)kStages * kStageBytes + 1024;
-    RDK_CUDA(cudaFuncSetAttribute(exact_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    exact_tc_kernel<<<grid, kTcThreads, smem, s>>>(mapA, mapB, P);
-    RDK_CUDA(cudaGetLastError());
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2u * (unsigned)pairs, 1, 1);
+    cfg.blockDim = dim3(kTcThreads, 1, 1);
+    cfg.dynamicSmemBytes = (size_t)P.stages * stage_bytes + 1024;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    RDK_CUDA(cudaLaunchKernelEx(&cfg, exact_tc_kernel, mapV, mapR, P));
     return RDK_OK;
 }
 

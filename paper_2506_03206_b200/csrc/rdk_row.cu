@@ -470,9 +470,12 @@ static int run_rows(const rdk_problem* pb, int mode, const void* target, const v
     if (e == cudaErrorNotSupported && !(pb->flags & RDK_FLAG_ROW_KERNEL)) {
         RowParams Q = P;
         uint32_t tag = 0;
-        if (Q.accepted_len && Q.accepted && ws && ws_bytes >= stream_workspace_bytes(P.rows, pb->batch, trials)) {
-            Q.arrivals = stream_workspace_arrivals(ws, P.rows);     // accepted_len is counted inside the kernel
-            tag = next_tag();
+        if (Q.accepted_len && Q.accepted && ws) {                   // accepted_len is counted inside the kernel
+            if (mode == RDK_MODE_LINEAR && ws_bytes >= stream_workspace_bytes(P.rows, pb->batch, trials))
+                Q.arrivals = stream_workspace_arrivals(ws, P.rows);
+            else if (mode == RDK_MODE_PRECOMPUTED_W && !(reinterpret_cast<uintptr_t>(ws) & 7u) && ws_bytes / 8 >= (size_t)pb->batch * trials)
+                Q.arrivals = static_cast<unsigned long long*>(ws);
+            if (Q.arrivals) tag = next_tag();
         }
         e = launch_cluster_rows(Q, mode, pb->target_dtype, pb->drafter_dtype, pb->drafter_kind, tag, stream_spin_limit(), s);
         if (e == cudaSuccess && Q.arrivals) return RDK_OK;

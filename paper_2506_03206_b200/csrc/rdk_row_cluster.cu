@@ -714,7 +714,7 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
         const uint32_t all = __ballot_sync(0xffffffffu, on);
         float p[kVec], w[kVec], x[kVec];
         int k_item = 0, turn = 0, held = -1;                     // held: the chunk (by its number) that p, w, x belong to
-        for (uint32_t todo = all; todo; todo &= todo - 1u) {     // the chunks' sums, chunks dealt out to the warps
+        for (uint32_t todo = nch > 1 ? all : 0u; todo; todo &= todo - 1u) {     // the chunks' sums, chunks dealt out to the warps
             const int t = __ffs(todo) - 1, sgm = __shfl_sync(0xffffffffu, seg, t), what = t < kCluRound ? 0 : (from_p ? 2 : 1);
             for (int ch = 0; ch < nch; ++ch, ++k_item) {
                 if (turn == warp) {
@@ -725,14 +725,15 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
                 if (++turn == nw) turn = 0;
             }
         }
-        __syncthreads();
+        if (nch > 1) __syncthreads();
         k_item = 0;
         for (uint32_t todo = all; todo; todo &= todo - 1u, k_item += nch) {
             const int t = __ffs(todo) - 1, sgm = __shfl_sync(0xffffffffu, seg, t), what = t < kCluRound ? 0 : (from_p ? 2 : 1);
             const float remt = __shfl_sync(0xffffffffu, rem, t);
             float cum = 0.f, before = 0.f;
             int chosen = -1, last_pos = -1;
-            for (int ch = 0; ch < nch; ++ch) {
+            if (nch == 1) { chosen = 0; cum = remt; }            // a segment of one chunk: no sums to look at
+            for (int ch = 0; ch < nch && nch > 1; ++ch) {
                 const float s = ds.dsum[t][ch];
                 if (s > 0.f) {
                     if (chosen < 0 && cum + s > remt) { chosen = ch; before = cum; }
@@ -804,7 +805,7 @@ struct CluShape { int C, nw, per; size_t smem; };
 
 // CTAs per row, warps per CTA and vectors per warp; false when a row does not fit a cluster's shared memory.  `lead`: most
 // positions before a row's first token.
-static bool plan_cluster(int N, int rows, size_t es, int variant, bool prior, int lead, CluShape& s) {
+static bool plan_cluster(int N, int rows, int trials, size_t es, int variant, bool prior, int lead, CluShape& s) {
     const size_t bytes = es * (prior ? 2 : 1) + (variant == kVarDense || variant == kVarGiven ? 4 : 0);    // per position
     const long long positions = (long long)N + lead;
     int C = 1;
@@ -822,6 +823,8 @@ static bool plan_cluster(int N, int rows, size_t es, int variant, bool prior, in
     const int per_warp = chunks <= 8 ? 1 : (chunks + 7) / 8;
     const int nw = (chunks + per_warp - 1) / per_warp;
     s.C = C; s.nw = nw < 4 ? 4 : nw;
+    // segments of one chunk and several draws a row: a warp for each draw, also where there is nothing to sweep for it
+    if (per_warp == 1 && (long long)rows * C < 4 * 148 && 2 * trials > s.nw) s.nw = 2 * trials < kCluMaxWarps ? 2 * trials : kCluMaxWarps;
     s.per = per_warp * 32;
     s.smem = (size_t)s.nw * s.per * kVec * bytes;
     if (s.smem < sizeof(DrawSmem)) s.smem = sizeof(DrawSmem);
@@ -888,7 +891,7 @@ cudaError_t launch_cluster_rows(RowParams P, int mode, int tz, int ty, int kind,
                         : (P.qtilde || P.N < kStreamMinN ? kVarDense : (P.prior ? kVarPrior : kVarSparse));
     CluShape sh;
     const bool aligned = !(reinterpret_cast<uintptr_t>(P.target) & 15u) && !((P.target_stride * (long long)es) & 15);
-    if (!plan_cluster(P.N, P.rows, es, variant, P.prior != nullptr, aligned ? 0 : (int)(16 / es) - 1, sh)) return cudaErrorNotSupported;
+    if (!plan_cluster(P.N, P.rows, P.trials, es, variant, P.prior != nullptr, aligned ? 0 : (int)(16 / es) - 1, sh)) return cudaErrorNotSupported;
     if ((long long)P.rows * sh.C > 0x7fffffffLL) return cudaErrorNotSupported;
     CluGeo g;
     g.per = sh.per;
