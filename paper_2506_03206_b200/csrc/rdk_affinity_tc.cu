@@ -99,7 +99,7 @@ aff_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__
             for (int tn = tn0; tn < min(tn0 + kSpan, col_tiles) && ok; ++tn)
                 for (int kb = 0; kb < P.num_kb; ++kb) {
                     if (!tc_wait(&empty_bar[stage], phase ^ 1u, abort)) { ok = false; break; }
-                    if (lane == 0) {
+                    if (elect_one()) {
                         const uint32_t sa = s32(tiles + stage * kAffStage), bar = s32(&full_bar[stage]);
                         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"((uint32_t)kAffStage) : "memory");
                         asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
@@ -112,6 +112,7 @@ aff_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__
                 }
         }
     } else if (warp == 1) {
+        const uint64_t adesc0 = smem_desc(s32(tiles));
         int stage = 0, acc = 0;
         uint32_t phase = 0, acc_phase = 0;
         bool ok = true;
@@ -123,14 +124,9 @@ aff_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__
                 for (int kb = 0; kb < P.num_kb; ++kb) {
                     if (!tc_wait(&full_bar[stage], phase, abort)) { ok = false; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    if (lane == 0) {
-                        const uint32_t a_addr = s32(tiles + stage * kAffStage), b_addr = a_addr + kAffABytes;
-#pragma unroll
-                        for (int k = 0; k < kAffK / 16; ++k) {
-                            const uint64_t adesc = smem_desc(a_addr + k * 32), bdesc = smem_desc(b_addr + k * 32);
-                            asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
-                                         ::"r"(tmem_base + (uint32_t)(acc * kAffN)), "l"(adesc), "l"(bdesc), "r"(kAffIdesc), "r"((kb > 0 || k > 0) ? 1u : 0u) : "memory");
-                        }
+                    if (elect_one()) {
+                        const uint64_t ad = adesc0 + (uint64_t)(stage * (kAffStage >> 4));
+                        mma_kblock<1>(tmem_base + (uint32_t)(acc * kAffN), ad, ad + (kAffABytes >> 4), kAffIdesc, kb > 0);
                         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(s32(&empty_bar[stage])) : "memory");
                     }
                     __syncwarp();

@@ -97,11 +97,9 @@ exact_tc_kernel(const __grid_constant__ CUtensorMap tmapV, const __grid_constant
         // before it is complete), so its first blocks are requested before the operand is there.
         int stage = 0; uint32_t phase = 0;
         bool ok = true, waited = false;
-        auto full_addr = [&](int s) -> uint32_t {        // the leader's barrier
-            uint32_t a;
-            asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(a) : "r"(s32(&full_bar[s])));
-            return a;
-        };
+        uint32_t full0;                                  // the leader's barriers
+        asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(full0) : "r"(s32(&full_bar[0])));
+        auto full_addr = [&](int s) -> uint32_t { return full0 + 8u * (uint32_t)s; };
         auto load_voc = [&](int s, int kb, int tv) {
             asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
                          ::"r"(ring + (uint32_t)s * stage_bytes), "l"(reinterpret_cast<uint64_t>(&tmapV)), "r"(kb * kBK),
@@ -136,7 +134,7 @@ exact_tc_kernel(const __grid_constant__ CUtensorMap tmapV, const __grid_constant
             }
             for (; kb < P.num_kb; ++kb) {
                 if (!tc_wait(&empty_bar[stage], phase ^ 1u, abort)) { ok = false; break; }
-                if (lane == 0) { expect(stage, t); load_voc(stage, kb, tv); load_rows(stage, kb, row0, t); }
+                if (elect_one()) { expect(stage, t); load_voc(stage, kb, tv); load_rows(stage, kb, row0, t); }
                 __syncwarp();
                 if (++stage == P.stages) { stage = 0; phase ^= 1u; }
             }
@@ -145,6 +143,10 @@ exact_tc_kernel(const __grid_constant__ CUtensorMap tmapV, const __grid_constant
         // ------------------------------------------------------------------ MMA issuer (leader only)
         if (leader) {
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(P.R >> 3) << 17) | (16u << 24);   // fp32 += bf16 bf16, M = 256, N = R
+            // (one thread issues everything: the descriptors are prepared so that an instruction costs it a few adds.  Built
+            // anew for every instruction they took 195 to 250 cycles each, whatever the tile, against 128 for 256 rows.)
+            const uint64_t vdesc0 = smem_desc(ring);
+            const uint32_t dstage = stage_bytes >> 4, empty0 = s32(&empty_bar[0]);
             int stage = 0; uint32_t phase = 0, acc_phase = 0;
             bool ok = true;
             for (int item = pair; item < P.num_items && ok; item += pairs) {
@@ -156,20 +158,13 @@ exact_tc_kernel(const __grid_constant__ CUtensorMap tmapV, const __grid_constant
                 for (int kb = 0; kb < P.num_kb; ++kb) {
                     if (!tc_wait(&full_bar[stage], phase, abort)) { ok = false; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint32_t va = ring + (uint32_t)stage * stage_bytes, ra = va + kVocBytes;
-                    if (lane == 0) {
-#pragma unroll
-                        for (int k = 0; k < kBK / 16; ++k) {
-                            const uint64_t vdesc = smem_desc(va + k * 32);
-                            for (int a = 0; a < t; ++a) {
-                                const uint64_t rdesc = smem_desc(ra + (uint32_t)a * rbytes + k * 32);
-                                asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}"
-                                             ::"r"(tmem_base + (uint32_t)(a * P.R)), "l"(vdesc), "l"(rdesc), "r"(idesc), "r"((kb > 0 || k > 0) ? 1u : 0u) : "memory");
-                            }
-                        }
+                    if (elect_one()) {
+                        const uint64_t vd = vdesc0 + (uint64_t)((uint32_t)stage * dstage), rd = vd + (kVocBytes >> 4);
+                        mma_kblock<2>(tmem_base, vd, rd, idesc, kb > 0);
+                        if (t == 2) mma_kblock<2>(tmem_base + (uint32_t)P.R, vd, rd + (rbytes >> 4), idesc, kb > 0);
                         // frees the stage in both CTAs once the MMAs above have read it
                         asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-                                     ::"r"(s32(&empty_bar[stage])), "h"((uint16_t)3) : "memory");
+                                     ::"r"(empty0 + 8u * (uint32_t)stage), "h"((uint16_t)3) : "memory");
                     }
                     __syncwarp();
                     if (++stage == P.stages) { stage = 0; phase ^= 1u; }

@@ -29,6 +29,13 @@ __device__ __forceinline__ bool tc_wait(unsigned long long* bar, uint32_t parity
     return ok;
 }
 
+// true in one lane of a converged warp, in a form the compiler knows to be uniform
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(p));
+    return p != 0;
+}
+
 // shared-memory matrix descriptor: K-major operand, rows of 128 bytes, 128-byte swizzle, groups of
 // 8 rows 1024 bytes apart
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
@@ -39,6 +46,21 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
     d |= (uint64_t)1 << 46;                          // descriptor version of this architecture
     d |= (uint64_t)2 << 61;                          // 128-byte swizzle
     return d;
+}
+
+// D += A B for one 64-wide K block of K-major operands: four instructions of 16, 32 bytes apart in either operand.  One
+// thread issues everything, so the descriptors come prepared and an instruction costs it a few adds: built anew for every
+// instruction they took 195 to 250 cycles each, whatever the tile, against 128 for the largest.
+#define RDK_MMA_KBLOCK(GROUP)                                                                                        \
+    asm volatile("{\n .reg .pred p, q;\n .reg .b64 a, b;\n setp.ne.b32 p, %4, 0;\n setp.eq.b32 q, 0, 0;\n"           \
+                 " tcgen05.mma.cta_group::" GROUP ".kind::f16 [%0], %1, %2, %3, p;\n"                                \
+                 " add.u64 a, %1, 2;\n add.u64 b, %2, 2;\n tcgen05.mma.cta_group::" GROUP ".kind::f16 [%0], a, b, %3, q;\n" \
+                 " add.u64 a, %1, 4;\n add.u64 b, %2, 4;\n tcgen05.mma.cta_group::" GROUP ".kind::f16 [%0], a, b, %3, q;\n" \
+                 " add.u64 a, %1, 6;\n add.u64 b, %2, 6;\n tcgen05.mma.cta_group::" GROUP ".kind::f16 [%0], a, b, %3, q;\n}" \
+                 ::"r"(d), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate ? 1u : 0u) : "memory")
+template <int CTA_GROUP>
+__device__ __forceinline__ void mma_kblock(uint32_t d, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, bool accumulate) {
+    if (CTA_GROUP == 2) RDK_MMA_KBLOCK("2"); else RDK_MMA_KBLOCK("1");
 }
 
 // 32 consecutive columns of this warp's 32 TMEM lanes: v[c] is column c of the lane's row
