@@ -54,9 +54,9 @@ exact_operand_kernel(const TY* __restrict__ drafter, long long dstride, const in
 #pragma unroll
             for (int k = 1; k < kVec; ++k) vmax = fmaxf(vmax, v[k]);
             if (vmax > a.m) { a.s *= ex2((a.m - vmax) * kLog2e); a.m = vmax; }
-            const float off = a.m > -INFINITY ? -a.m * kLog2e : 0.f;
+            const float base = a.m > -INFINITY ? a.m : 0.f;
 #pragma unroll
-            for (int k = 0; k < kVec; ++k) a.s += ex2(fmaf(v[k], kLog2e, off));
+            for (int k = 0; k < kVec; ++k) a.s += ex2((v[k] - base) * kLog2e);
         } else {
 #pragma unroll
             for (int k = 0; k < kVec; ++k) a.s += v[k];
@@ -66,13 +66,13 @@ exact_operand_kernel(const TY* __restrict__ drafter, long long dstride, const in
     if (lane == 0) red[warp] = a;
     __syncthreads();
     a = ms_warp(lane < kOperandThreads / 32 ? red[lane] : MS{-INFINITY, 0.f, 0.f});
-    const float off = KIND == RDK_LOGITS ? -a.m * kLog2e : 0.f, inv = 1.f / a.s;
+    const float inv = 1.f / a.s;
     TA* out = A + (long long)row * lda;
     for (int i = tid * kVec; i < lda; i += kOperandThreads * kVec) {
         float v[kVec];
         load_y(i, v);
 #pragma unroll
-        for (int k = 0; k < kVec; ++k) v[k] = (KIND == RDK_LOGITS ? ex2(fmaf(v[k], kLog2e, off)) : v[k]) * inv;
+        for (int k = 0; k < kVec; ++k) v[k] = (KIND == RDK_LOGITS ? ex2((v[k] - a.m) * kLog2e) : v[k]) * inv;
         if (sizeof(TA) == 2) {                   // lda is a multiple of 64 and the rows are 16-byte aligned
             uint32_t w[4];
 #pragma unroll

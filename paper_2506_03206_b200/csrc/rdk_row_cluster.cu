@@ -513,31 +513,40 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
         const float Kw = fy * Zq - fy * xs * th + theta * xs * K;
         sums = make_float4(oov + Kw, oov + ak, fmaxf(0.f, segP - (oov + ak)), segP);
     } else if (VAR == kVarPrior) {
-        // all tokens as if not kept, w = theta x (1 - x); then the kept ones' difference (what they count too much is
-        // theta x, smaller than 1 / N of a probability: nothing cancels)
-        float2 sw2 = splat(0.f), sa2 = splat(0.f);
-        auto pair = [&](float2 z, float2 pr) {
-            const float2 p = fmul2(ex2_2(ffma2(z, l2e2, zoff2)), fz2), x = fmul2(ex2_2(ffma2(pr, l2e2, poff2)), xs2);
-            const float2 w = fmul2(fmul2(th2, x), ffma2(x, neg2, one2));
-            sw2 = fadd2(sw2, w); sa2 = fadd2(sa2, make_float2(fminf(p.x, w.x), fminf(p.y, w.y)));
-        };
-#pragma unroll 2
+        // All tokens as if not kept, w = theta x (what x^2 takes away is below 1 / N^2 in all); that is the smaller of w and p
+        // nearly everywhere, so the sum of min(p, w) is theta times that of x, less w - p where p is the smaller: where
+        // z - prior falls below a constant of the row.  The difference of the logits (in their own type, with a margin
+        // for its rounding) tells; only vectors with such a token evaluate their exponentials again.  (Evaluating all:
+        // 150 us for 320 rows of 128k.)  Then the kept tokens' own w, in place of theta x.
+        float c = (__log2f(theta * xs) - __log2f(fz) + poff - zoff) * (1.f / kLog2e);
+        c = c == c ? c + fabsf(c) * 0x1p-7f + 0.01f : INFINITY;
+        float viol = 0.f;
+        auto over = [&](float z, float pr) { viol += fmaxf(0.f, theta * xs * ex2(fmaf(pr, kLog2e, poff)) - fz * ex2(fmaf(z, kLog2e, zoff))); };
+#pragma unroll 4
         for (int k = 0; k < nit16; ++k) {
             const uint4 qz = lds128(zb + (uint32_t)(k * 32 + lane) * 16u), qp = lds128(pb + (uint32_t)(k * 32 + lane) * 16u);
+            const uint32_t vz[4] = {qz.x, qz.y, qz.z, qz.w}, vp[4] = {qp.x, qp.y, qp.z, qp.w};
             if (sizeof(TZ) == 2) {
-                pair(make_float2(bf16_lo(qz.x), bf16_hi(qz.x)), make_float2(bf16_lo(qp.x), bf16_hi(qp.x)));
-                pair(make_float2(bf16_lo(qz.y), bf16_hi(qz.y)), make_float2(bf16_lo(qp.y), bf16_hi(qp.y)));
-                pair(make_float2(bf16_lo(qz.z), bf16_hi(qz.z)), make_float2(bf16_lo(qp.z), bf16_hi(qp.z)));
-                pair(make_float2(bf16_lo(qz.w), bf16_hi(qz.w)), make_float2(bf16_lo(qp.w), bf16_hi(qp.w)));
+                __nv_bfloat162 d[4];
+#pragma unroll
+                for (int h = 0; h < 4; ++h) d[h] = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&vz[h]), *reinterpret_cast<const __nv_bfloat162*>(&vp[h]));
+                const __nv_bfloat162 m = __hmin2(__hmin2(d[0], d[1]), __hmin2(d[2], d[3]));
+                if (!(fminf(__low2float(m), __high2float(m)) < c)) continue;
+#pragma unroll
+                for (int h = 0; h < 4; ++h) { over(bf16_lo(vz[h]), bf16_lo(vp[h])); over(bf16_hi(vz[h]), bf16_hi(vp[h])); }
             } else {
-                pair(make_float2(__uint_as_float(qz.x), __uint_as_float(qz.y)), make_float2(__uint_as_float(qp.x), __uint_as_float(qp.y)));
-                pair(make_float2(__uint_as_float(qz.z), __uint_as_float(qz.w)), make_float2(__uint_as_float(qp.z), __uint_as_float(qp.w)));
+                float m = INFINITY;
+#pragma unroll
+                for (int h = 0; h < 4; ++h) m = fminf(m, __uint_as_float(vz[h]) - __uint_as_float(vp[h]));
+                if (!(m < c)) continue;
+#pragma unroll
+                for (int h = 0; h < 4; ++h) over(__uint_as_float(vz[h]), __uint_as_float(vp[h]));
             }
         }
-        float sw = sw2.x + sw2.y, sa = sa2.x + sa2.y, dw = 0.f, da = 0.f;
+        float dw = 0.f, da = 0.f;
         auto again = [&](int pos, float ep, float ey) {
             const float p = ex2(fmaf(lds_z<TZ>(zb + (uint32_t)max(pos, 0) * es), kLog2e, zoff)) * fz, x = ep * xs;
-            const float w0 = theta * x * (1.f - x), w = redistribute1(x, ey * fy, theta);
+            const float w0 = theta * x, w = redistribute1(x, ey * fy, theta);
             if (pos >= 0) { dw += w - w0; da += fminf(p, w) - fminf(p, w0); }
         };
 #pragma unroll
@@ -550,9 +559,8 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
             for (int k = 0; k < 4; ++k)
                 again(pos[k], ex2(fmaf(lds_z<TZ>(pb + (uint32_t)max(pos[k], 0) * es), kLog2e, poff)), KIND == RDK_LOGITS ? ex2(fmaf(y[k], kLog2e, yoff)) : y[k]);
         }
-        sw += dw; sa += da;
-        const float segP = E * fz;
-        sw = warp_sum(sw); sa = warp_sum(sa);
+        const float segP = E * fz, all = theta * xs * Ep;
+        const float sw = all + warp_sum(dw), sa = all + warp_sum(da - viol);
         sums = make_float4(sw, sa, fmaxf(0.f, segP - sa), segP);
     } else {
         float2 sw2 = splat(0.f), sa2 = splat(0.f), sr2 = splat(0.f);
