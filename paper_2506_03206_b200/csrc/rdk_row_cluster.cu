@@ -56,13 +56,14 @@ struct CluGeo {
     unsigned spin_limit;
 };
 
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void st_cluster4(uint32_t local, uint32_t cta, float a, float b, float c, float d) {
-    uint32_t r;
+// Four floats into CTA `cta`'s copy of the shared variable at `local`, counted as 16 bytes on its barrier `bar`: a message and
+// its signal in one, where a barrier over the cluster costs every CTA a round trip and a flush of its stores.
+__device__ __forceinline__ void send_cluster4(uint32_t local, uint32_t bar, uint32_t cta, float a, float b, float c, float d) {
+    uint32_t r, m;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local), "r"(cta));
-    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(r), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(m) : "r"(bar), "r"(cta));
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+                 ::"r"(r), "r"(__float_as_uint(a)), "r"(__float_as_uint(b)), "r"(__float_as_uint(c)), "r"(__float_as_uint(d)), "r"(m) : "memory");
 }
 
 // One segment's share of the row, on the scales m (target), my (drafter), mp (prior)
@@ -171,7 +172,7 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     __shared__ __align__(16) float4 segs[kCluMaxSeg];            // per segment: sums of w, min(p, q~), max(0, p - q~), p
     __shared__ __align__(16) float4 xrec[kCluMaxCtas][2];        // one record per CTA of the cluster
     __shared__ __align__(16) float wrec[kCluMaxWarps][8];
-    __shared__ __align__(8) unsigned long long wbar[kCluMaxWarps];
+    __shared__ __align__(8) unsigned long long wbar[kCluMaxWarps], xbar, sbar;     // a warp's copies; records of all CTAs; sums of all segments (CTA 0)
     __shared__ __align__(16) float4 tot_s[2];
     __shared__ float alpha_s, part_s[kCluMaxWarps];
 
@@ -186,10 +187,20 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     const uint32_t bar = smem_u32(&wbar[warp]);
     if (lane == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar));
+        if (warp == 0) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&xbar)));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&sbar)));
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     __syncwarp();
+    if (tid == 0) {
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&xbar)), "r"(C * 32u) : "memory");
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&sbar)), "r"(rank == 0 ? C * (uint32_t)nw * 16u : 0u) : "memory");
+    }
+    // another CTA's shared memory may be touched only once that CTA runs: arrive here, wait before the first message
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 
     // ---- this warp's segment: positions [sg len, (sg + 1) len) of the row, position = token + phase ----------------
     const TZ* zrow = static_cast<const TZ*>(P.target) + (long long)row * P.target_stride;
@@ -202,26 +213,15 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     const uint32_t zb0 = smem_u32(csm), pb0 = zb0 + g.zoff_p, qb0 = zb0 + g.zoff_q;
     const uint32_t zb = zb0 + (uint32_t)(warp * len) * es, pb = pb0 + (uint32_t)(warp * len) * es, qb = qb0 + (uint32_t)(warp * len) * 4u;
 
-    // header of the index and the ranks of the segment's ends, requested together
-    bool identity = true;
-    int r0 = 0, cnt = 0;                                         // kept tokens of the segment: ranks [r0, r0 + cnt)
+    // header of the index and the ranks of the segment's ends: requested together, looked at when the copies are under way
+    int4 h0 = make_int4(0, 0, 0, 0), h1 = h0;
+    uint32_t end_word = 0;
+    int end_rank = 0;
+    const int end_tok = lane == 0 ? t0 : t1;
     if (kLinear) {
-        const int4 h0 = __ldg(reinterpret_cast<const int4*>(P.header)), h1 = __ldg(reinterpret_cast<const int4*>(P.header) + 1);
-        const int tok = lane == 0 ? t0 : t1;
-        uint32_t word = 0;
-        int r = 0;
-        if (tok < P.N && lane < 2) { word = __ldg(P.mask + (tok >> 5)); r = __ldg(P.rank + (tok >> 5)); }
-        if (h0.x != kIdxMagic || h0.y != P.N || h0.z != P.n) {      // not an index of this problem: the same decision everywhere
-            if (tid == 0 && rank == 0 && P.status_word) atomicCAS(P.status_word, 0, (int)RDK_ERR_INVALID_ARG);
-            return;
-        }
-        identity = h1.y != 0;
-        r = tok < P.N ? r + __popc(word & ((1u << (tok & 31)) - 1u)) : h0.w;
-        r0 = __shfl_sync(0xffffffffu, r, 0);
-        cnt = __shfl_sync(0xffffffffu, r, 1) - r0;
+        h0 = __ldg(reinterpret_cast<const int4*>(P.header)); h1 = __ldg(reinterpret_cast<const int4*>(P.header) + 1);
+        if (end_tok < P.N && lane < 2) { end_word = __ldg(P.mask + (end_tok >> 5)); end_rank = __ldg(P.rank + (end_tok >> 5)); }
     }
-    // another CTA's shared memory may be touched only once that CTA runs: arrive here, wait before the first exchange
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");       // inputs may be the previous kernel's outputs
 
@@ -246,6 +246,19 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
         }
         if (kDense && kLinear)
             for (int i = 0; i < len / 128; ++i) sts128(qb + (uint32_t)(i * 32 + lane) * 16u, 0.f, 0.f, 0.f, 0.f);
+    }
+    bool identity = true;
+    int r0 = 0, cnt = 0;                                         // kept tokens of the segment: ranks [r0, r0 + cnt)
+    if (kLinear) {
+        if (h0.x != kIdxMagic || h0.y != P.N || h0.z != P.n) {      // not an index of this problem: the same decision everywhere
+            if (tid == 0 && rank == 0 && P.status_word) atomicCAS(P.status_word, 0, (int)RDK_ERR_INVALID_ARG);
+            clu_wait(bar, kCluSpinDefault);                      // the copies must land before the CTA leaves
+            return;
+        }
+        identity = h1.y != 0;
+        const int r = end_tok < P.N ? end_rank + __popc(end_word & ((1u << (end_tok & 31)) - 1u)) : h0.w;
+        r0 = __shfl_sync(0xffffffffu, r, 0);
+        cnt = __shfl_sync(0xffffffffu, r, 1) - r0;
     }
     // uniforms of the first round of draws: lane t < 16 has those of the draft draw of trial t, lane 16 + t of its residual draw
     const int trial = lane & (kCluRound - 1), kind = lane / kCluRound;
@@ -400,7 +413,6 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
         reinterpret_cast<float4*>(wrec[warp])[1] = make_float4(my_w, Ep, mp_w, W);
     }
     __syncthreads();
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");      // all CTAs of the cluster run
 
     // ---- first exchange: the row's soft-max sums and theta ------------------------------------------------------------
     if (warp == 0) {
@@ -410,15 +422,16 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
             r = SegRec{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
         }
         r = fold_records<kPrior>(r, lane);
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");      // all CTAs of the cluster run
         if (lane < (int)C) {
-            st_cluster4(smem_u32(&xrec[rank][0]), (uint32_t)lane, r.E, r.Zq, r.th, r.m);
-            st_cluster4(smem_u32(&xrec[rank][1]), (uint32_t)lane, r.my, r.Ep, r.mp, r.W);
+            send_cluster4(smem_u32(&xrec[rank][0]), smem_u32(&xbar), (uint32_t)lane, r.E, r.Zq, r.th, r.m);
+            send_cluster4(smem_u32(&xrec[rank][1]), smem_u32(&xbar), (uint32_t)lane, r.my, r.Ep, r.mp, r.W);
         }
-    }
-    cluster_sync();
-    if (warp == 0) {                                     // fold the cluster's records, once per CTA
-        SegRec r{0.f, 0.f, 0.f, -INFINITY, -INFINITY, 0.f, -INFINITY, 0.f};
-        if (lane < (int)C) {
+        // (the messages are on their way as soon as all CTAs have come this far: no short limit, which would let a CTA leave
+        // before a message to it has arrived)
+        if (!clu_wait(smem_u32(&xbar), kCluSpinDefault) && lane == 0 && P.status_word) atomicCAS(P.status_word, 0, (int)RDK_ERR_TIMEOUT);
+        r = SegRec{0.f, 0.f, 0.f, -INFINITY, -INFINITY, 0.f, -INFINITY, 0.f};
+        if (lane < (int)C) {                             // fold the cluster's records, once per CTA
             const float4 a = xrec[lane][0], b = xrec[lane][1];
             r = SegRec{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
         }
@@ -606,10 +619,9 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     }
 
     // ---- second exchange: CTA 0 gets the sums of all segments; the others are done -----------------------------------------
-    if (lane == 0) st_cluster4(smem_u32(&segs[sg]), 0u, sums.x, sums.y, sums.z, sums.w);
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    if (lane == 0) send_cluster4(smem_u32(&segs[sg]), smem_u32(&sbar), 0u, sums.x, sums.y, sums.z, sums.w);
     if (rank != 0) return;
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (!clu_wait(smem_u32(&sbar), kCluSpinDefault) && lane == 0 && P.status_word) atomicCAS(P.status_word, 0, (int)RDK_ERR_TIMEOUT);
     DrawSmem& ds = *reinterpret_cast<DrawSmem*>(csm);
     double (&cdf)[3][kCluMaxSeg] = ds.cdf;
     for (int job = warp; job < 4; job += nw) {
