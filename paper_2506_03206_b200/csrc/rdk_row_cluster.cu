@@ -163,6 +163,40 @@ __device__ __forceinline__ void redistribute8(const float (&x)[kVec], const floa
 }
 __device__ __forceinline__ float redistribute1(float x, float qp, float theta) { return fmaf(x * (theta - qp), 1.f - x, qp); }
 
+// accepted_len of a sequence (Algorithm 4 step 7): the number of leading accepted positions, counted by the position that
+// arrives last.  The word of a (sequence, trial) holds (tag of the call, accept bits, arrivals), so it needs no
+// initialisation, and one atomic operation carries a position's answer along with its arrival: nothing has to be fenced
+// or read back.  The last one clears the word, for a replayed graph, whose calls carry the same tag.  Sequences longer
+// than the bits count arrivals only and read the flags again.
+constexpr int kCluBits = 24;
+__device__ __forceinline__ void count_accepted(const RowParams& P, uint32_t tag, int row, int t, bool acc) {
+    const int b = row / P.positions, pos = row - b * P.positions;
+    unsigned long long* word = P.arrivals + (long long)b * P.trials + t;
+    int32_t* out = P.accepted_len + (long long)b * P.trials + t;
+    const bool bits = P.positions <= kCluBits;
+    const unsigned long long mine = 1ull | (bits && acc ? 256ull << pos : 0ull), first = (unsigned long long)tag << 32 | mine;
+    if (!bits) __threadfence();
+    unsigned long long old = atomicCAS(word, 0ull, first), now = first;
+    while (old != 0ull) {
+        if ((uint32_t)(old >> 32) == tag) { now = atomicAdd(word, mine) + mine; break; }
+        const unsigned long long seen = atomicCAS(word, old, first);          // left over from something else
+        if (seen == old) break;
+        old = seen;
+    }
+    const int arrived = bits ? (int)(now & 255ull) : (int)(uint32_t)now;
+    if (arrived != P.positions) return;
+    *word = 0ull;
+    int k = 0;
+    if (bits) {
+        k = __ffs(~(int)((uint32_t)now >> 8)) - 1;
+    } else {
+        __threadfence();
+        const volatile uint8_t* af = P.accepted;
+        while (k < P.positions && af[((long long)b * P.positions + k) * P.trials + t]) ++k;
+    }
+    *out = k;
+}
+
 template <typename TZ, typename TY, int KIND, int VAR, bool kPrior>
 __global__ void __launch_bounds__(512, 2)
 rdk_cluster_kernel(const RowParams P, const CluGeo g) {
@@ -663,10 +697,21 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     }
 
     // ---- draws ------------------------------------------------------------------------------------------------------------
+    // Every step here is a round trip to L2 or a chain of barriers that only this row waits for, so the draws of a round
+    // (a draft and a residual draw per trial) go side by side: their segments' 256-position chunks are dealt out to the
+    // warps, two at a time so that both chunks' loads travel together.  (One chunk at a time, binary searches by every
+    // thread, an integer division per draw and a fence with three dependent loads for accepted_len took 18 to 40 thousand
+    // cycles a row, twice what the row itself takes.)
     const bool from_p = !(R_d > 0.0);                    // p and q~ coincide: the replacement comes from p itself
-    const double* cdf_r = from_p ? cdf[2] : cdf[1];
-    const int nch = g.per / 32;
-    // x of this lane's 8 positions in chunk ch of segment sgm, read from global memory again: what = 0: w, 1: max(0, p - q~), 2: p
+    const int nch = g.per / 32, per_lane = (nseg + 31) >> 5;
+    // the first segment whose prefix sum exceeds thr; the last one if rounding leaves none
+    auto find_segment = [&](const double* c, double thr) -> int {
+        const uint32_t lanes = __ballot_sync(0xffffffffu, c[min((lane + 1) * per_lane, nseg) - 1] > thr);
+        if (!lanes) return nseg - 1;
+        const int first = (__ffs(lanes) - 1) * per_lane;
+        const uint32_t in = __ballot_sync(0xffffffffu, lane < per_lane && c[min(first + lane, nseg - 1)] > thr);
+        return min(first + __ffs(in) - 1, nseg - 1);
+    };
     auto load_row8 = [&](const auto* src, int jb, float fill, float (&v)[kVec]) {
         using T = typename std::remove_cv<typename std::remove_pointer<decltype(src)>::type>::type;
         if (jb >= 0) {
@@ -676,106 +721,151 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
             for (int k = 0; k < kVec; ++k) v[k] = jb + k >= 0 && jb + k < P.N ? to_float<T>(src[jb + k]) : fill;
         }
     };
-    auto chunk_x = [&](int sgm, int ch, int what, float (&p)[kVec], float (&w)[kVec], float (&x)[kVec]) -> float {
-        const int jb = sgm * len - phase + (ch * 32 + lane) * kVec;
-        float z[kVec];
-        load_row8(zrow, jb, -INFINITY, z);
-        if (VAR == kVarGiven) {
-            load_row8(P.w + (long long)row * P.w_stride, jb, 0.f, w);
+    const float* wrow = VAR == kVarGiven ? P.w + (long long)row * P.w_stride : nullptr;
+    // x[h] of this lane's 8 positions in chunk ch[h] of segment sgm[h], for H chunks at once, read from global memory again;
+    // what[h] = 0: w, 1: max(0, p - q~), 2: p.  sum[h]: over the warp.
+    auto chunks = [&](auto HC, const int* sgm, const int* ch, const int* what, float (*x)[kVec], float* sum) {
+        constexpr int H = decltype(HC)::value;
+        float z[H][kVec], a[H][kVec];
+        uint32_t mb[H];
+        int i[H][kVec], jb[H];
 #pragma unroll
-            for (int k = 0; k < kVec; ++k) p[k] = ex2(fmaf(z[k], kLog2e, offg)) * inv_zp;
-        } else {
-            // the kept tokens among the 8, looked up in the index
-            const int wi = jb >> 5, sh = jb & 31;
-            const bool in = jb < P.N;
-            const uint32_t lo = wi >= 0 && in ? __ldg(P.mask + wi) : 0u;
-            const uint32_t hi = in && (wi + 1) * 32 < P.N ? __ldg(P.mask + wi + 1) : 0u;
-            const int rw = wi >= 0 && in ? __ldg(P.rank + wi) : 0;
-            float pr[kVec];
-            if (kPrior) load_row8(prow, jb, -INFINITY, pr);
-            const uint32_t mb = __funnelshift_r(lo, hi, sh) & 0xffu;
-            const int rb = wi >= 0 ? rw + __popc(lo & ((1u << sh) - 1u)) : 0;
-            // independent loads: a token that is not kept reads what the first kept one does (or entry 0)
-            int i[kVec];
+        for (int h = 0; h < H; ++h) {
+            jb[h] = sgm[h] * len - phase + (ch[h] * 32 + lane) * kVec;
+            load_row8(zrow, jb[h], -INFINITY, z[h]);
+            if (VAR == kVarGiven) load_row8(wrow, jb[h], 0.f, a[h]);
+            if (kPrior) load_row8(prow, jb[h], -INFINITY, a[h]);
+        }
+        if (kLinear) {       // the kept tokens among the 8, looked up in the index
+            uint32_t lo[H], hi[H];
+            int rw[H];
 #pragma unroll
-            for (int k = 0; k < kVec; ++k) i[k] = (mb >> k) & 1u ? rb + __popc(mb & ((1u << k) - 1u)) : (mb ? rb : 0);
+            for (int h = 0; h < H; ++h) {
+                const int wi = jb[h] >> 5;
+                const bool in = wi >= 0 && jb[h] < P.N;
+                lo[h] = in ? __ldg(P.mask + wi) : 0u;
+                hi[h] = jb[h] < P.N && (wi + 1) * 32 < P.N ? __ldg(P.mask + wi + 1) : 0u;
+                rw[h] = in ? __ldg(P.rank + wi) : 0;
+            }
+#pragma unroll
+            for (int h = 0; h < H; ++h) {
+                const int sh = jb[h] & 31;
+                mb[h] = __funnelshift_r(lo[h], hi[h], sh) & 0xffu;
+                const int rb = rw[h] + __popc(lo[h] & ((1u << sh) - 1u));
+                // independent loads: a token that is not kept reads what the first kept one does (or entry 0)
+#pragma unroll
+                for (int k = 0; k < kVec; ++k) i[h][k] = (mb[h] >> k) & 1u ? rb + __popc(mb[h] & ((1u << k) - 1u)) : (mb[h] ? rb : 0);
+            }
             if (!identity) {
 #pragma unroll
-                for (int k = 0; k < kVec; ++k) i[k] = __ldg(P.slot + i[k]);
-            }
-            float y[kVec];
+                for (int h = 0; h < H; ++h)
 #pragma unroll
-            for (int k = 0; k < kVec; ++k) y[k] = to_float<TY>(yrow[i[k]]);
+                    for (int k = 0; k < kVec; ++k) i[h][k] = __ldg(P.slot + i[h][k]);
+            }
+#pragma unroll
+            for (int h = 0; h < H; ++h)
+#pragma unroll
+                for (int k = 0; k < kVec; ++k) i[h][k] = __float_as_int(to_float<TY>(yrow[i[h][k]]));
+        }
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+            float w[kVec], q[kVec];
 #pragma unroll
             for (int k = 0; k < kVec; ++k) {
-                p[k] = ex2(fmaf(z[k], kLog2e, offg)) * inv_zp;
-                pr[k] = kPrior ? ex2(fmaf(pr[k], kLog2e, poffg)) * inv_zpi * inv_n : p[k] * inv_n;
-                y[k] = (mb >> k) & 1u ? (KIND == RDK_LOGITS ? ex2(fmaf(y[k], kLog2e, yoffg)) : y[k]) * inv_zq : 0.f;
+                z[h][k] = ex2(fmaf(z[h][k], kLog2e, offg)) * inv_zp;
+                if (VAR == kVarGiven) w[k] = a[h][k];
+                if (kLinear) {
+                    const float y = __int_as_float(i[h][k]);
+                    a[h][k] = kPrior ? ex2(fmaf(a[h][k], kLog2e, poffg)) * inv_zpi * inv_n : z[h][k] * inv_n;
+                    q[k] = (mb[h] >> k) & 1u ? (KIND == RDK_LOGITS ? ex2(fmaf(y, kLog2e, yoffg)) : y) * inv_zq : 0.f;
+                }
             }
-            redistribute8(pr, y, theta, small, w);
-        }
-        float s = 0.f;
+            if (kLinear) redistribute8(a[h], q, theta, small, w);
+            float t = 0.f;
 #pragma unroll
-        for (int k = 0; k < kVec; ++k) {
-            x[k] = what == 0 ? w[k] : (what == 1 ? fmaxf(0.f, p[k] - w[k] * inv_s) : p[k]);
-            s += x[k];
+            for (int k = 0; k < kVec; ++k) {
+                x[h][k] = what[h] == 0 ? w[k] : (what[h] == 1 ? fmaxf(0.f, z[h][k] - w[k] * inv_s) : z[h][k]);
+                t += x[h][k];
+            }
+            sum[h] = warp_sum(t);
         }
-        return s;
     };
     for (int base = 0; base < P.trials; base += kCluRound) {
-        const int nt = min(kCluRound, P.trials - base);
-        const bool on = trial < nt;
-        if (base && on) { u_draw = __ldg(u_row + (base + trial) * 4 + 2 * kind); u_test = __ldg(u_row + (base + trial) * 4 + 1); }
-        const double* c = kind == 0 ? cdf[0] : cdf_r;
-        const double thr = (double)u_draw * c[nseg - 1];
-        // the draw's segment is the first whose prefix sum exceeds the threshold (the last one if rounding leaves none)
-        const int seg = min(first_above(c, nseg, thr), nseg - 1);
-        const float rem = (float)(thr - (seg ? c[seg - 1] : 0.0));
-        const uint32_t all = __ballot_sync(0xffffffffu, on);
-        float p[kVec], w[kVec], x[kVec];
-        int k_item = 0, turn = 0, held = -1;                     // held: the chunk (by its number) that p, w, x belong to
-        for (uint32_t todo = nch > 1 ? all : 0u; todo; todo &= todo - 1u) {     // the chunks' sums, chunks dealt out to the warps
-            const int t = __ffs(todo) - 1, sgm = __shfl_sync(0xffffffffu, seg, t), what = t < kCluRound ? 0 : (from_p ? 2 : 1);
-            for (int ch = 0; ch < nch; ++ch, ++k_item) {
-                if (turn == warp) {
-                    held = k_item;
-                    const float s = warp_sum(chunk_x(sgm, ch, what, p, w, x));
-                    if (lane == 0) ds.dsum[t][ch] = s;
-                }
-                if (++turn == nw) turn = 0;
-            }
-        }
-        if (nch > 1) __syncthreads();
-        k_item = 0;
-        for (uint32_t todo = all; todo; todo &= todo - 1u, k_item += nch) {
-            const int t = __ffs(todo) - 1, sgm = __shfl_sync(0xffffffffu, seg, t), what = t < kCluRound ? 0 : (from_p ? 2 : 1);
-            const float remt = __shfl_sync(0xffffffffu, rem, t);
-            float cum = 0.f, before = 0.f;
-            int chosen = -1, last_pos = -1;
-            if (nch == 1) { chosen = 0; cum = remt; }            // a segment of one chunk: no sums to look at
-            for (int ch = 0; ch < nch && nch > 1; ++ch) {
-                const float s = ds.dsum[t][ch];
-                if (s > 0.f) {
-                    if (chosen < 0 && cum + s > remt) { chosen = ch; before = cum; }
-                    last_pos = ch;
-                    cum += s;
-                }
-            }
-            const float r_in = chosen < 0 ? INFINITY : remt - before;    // rounding left no token: the last positive one
-            if (chosen < 0) chosen = max(last_pos, 0);
-            if ((k_item + chosen) % nw != warp) continue;                // the warp that summed the chunk picks the token,
-            if (held != k_item + chosen) {                               // from its registers unless it went on to another chunk
-                (void)chunk_x(sgm, chosen, what, p, w, x);
-                held = k_item + chosen;
-            }
+        const int nt = min(kCluRound, P.trials - base), nd = 2 * nt, items = nd * nch;
+        if (base && trial < nt) { u_draw = __ldg(u_row + (base + trial) * 4 + 2 * kind); u_test = __ldg(u_row + (base + trial) * 4 + 1); }
+        // draw d < nt: the draft draw of trial base + d; nt + d: its residual draw (needed only if the draft is rejected)
+        auto locate = [&](int d, int& sgm, int& what, float& rem) {
+            const bool res = d >= nt;
+            const double* c = res ? (from_p ? cdf[2] : cdf[1]) : cdf[0];
+            const double thr = (double)__shfl_sync(0xffffffffu, u_draw, res ? kCluRound + d - nt : d) * c[nseg - 1];
+            sgm = find_segment(c, thr);
+            rem = (float)(thr - (sgm ? c[sgm - 1] : 0.0));
+            what = res ? (from_p ? 2 : 1) : 0;
+        };
+        // the token of draw d where the running sum of x, from the start of chunk ch, passes r_in
+        auto pick = [&](int d, int sgm, int ch, const float (&x)[kVec], float r_in) {
             const int sel = max(pick_in_segment(x, r_in, lane), 0);
-            float pd = 0.f, wd = 0.f;
+            float wd = 0.f;
 #pragma unroll
-            for (int k = 0; k < kVec; ++k) if (k == (sel & (kVec - 1))) { pd = p[k]; wd = w[k]; }
-            pd = __shfl_sync(0xffffffffu, pd, sel / kVec);
+            for (int k = 0; k < kVec; ++k) if (k == (sel & (kVec - 1))) wd = x[k];
             wd = __shfl_sync(0xffffffffu, wd, sel / kVec);
-            const int tok = sgm * len - phase + chosen * 256 + sel;
-            if (lane == 0) ds.res[t] = make_float4(__int_as_float(min(max(tok, 0), P.N - 1)), pd, wd, 0.f);
+            const int tok = min(max(sgm * len - phase + ch * 256 + sel, 0), P.N - 1);
+            if (lane == 0) ds.res[d] = make_float4(__int_as_float(tok), ex2(fmaf(to_float<TZ>(zrow[tok]), kLog2e, offg)) * inv_zp, wd, 0.f);
+        };
+        // the chunk of draw d in which rem is passed, and what is left of rem there; rounding may leave none: the last positive one
+        auto choose = [&](int d, float rem, int& ch, float& r_in) {
+            const float v = lane < nch ? ds.dsum[d][lane] : 0.f;
+            float incl = v;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const float t = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += t;
+            }
+            const uint32_t pos = __ballot_sync(0xffffffffu, v > 0.f), hit = __ballot_sync(0xffffffffu, v > 0.f && incl > rem);
+            ch = hit ? __ffs(hit) - 1 : (pos ? 31 - __clz(pos) : 0);
+            const float before = __shfl_sync(0xffffffffu, incl - v, ch);
+            r_in = hit ? rem - before : INFINITY;
+        };
+        if (nch == 1) {                                  // no sums to look at: a warp settles its draws by itself
+            for (int d = warp; d < nd; d += nw) {
+                int sgm[1], what[1];
+                const int ch[1] = {0};
+                float rem, x[1][kVec], sum[1];
+                locate(d, sgm[0], what[0], rem);
+                chunks(std::integral_constant<int, 1>(), sgm, ch, what, x, sum);
+                pick(d, sgm[0], 0, x[0], rem);
+            }
+        } else {
+            int d[2] = {0, 0}, ch[2] = {0, 0}, sgm[2] = {0, 0}, what[2] = {0, 0};
+            float rem[2] = {0.f, 0.f}, x[2][kVec], sum[2];
+            for (int it = warp; it < items; it += 2 * nw) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int item = min(it + h * nw, items - 1);
+                    d[h] = item / nch; ch[h] = item - d[h] * nch;
+                    locate(d[h], sgm[h], what[h], rem[h]);
+                }
+                chunks(std::integral_constant<int, 2>(), sgm, ch, what, x, sum);
+                if (lane == 0) { ds.dsum[d[0]][ch[0]] = sum[0]; ds.dsum[d[1]][ch[1]] = sum[1]; }
+            }
+            __syncthreads();
+            int c;
+            float r_in;
+            if (items <= 2 * nw) {                       // every chunk is still in the registers of the warp that summed it
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    if (warp + h * nw >= items) break;
+                    choose(d[h], rem[h], c, r_in);
+                    if (c == ch[h]) pick(d[h], sgm[h], c, x[h], r_in);
+                }
+            } else {
+                for (int e = warp; e < nd; e += nw) {
+                    locate(e, sgm[0], what[0], rem[0]);
+                    choose(e, rem[0], ch[0], r_in);
+                    chunks(std::integral_constant<int, 1>(), sgm, ch, what, x, sum);
+                    pick(e, sgm[0], ch[0], x[0], r_in);
+                }
+            }
         }
         __syncthreads();
         if (tid < nt) {
@@ -786,30 +876,8 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
             if (P.draft_token) P.draft_token[o] = dtok;
             if (P.accepted) P.accepted[o] = acc ? 1 : 0;
             if (P.accept_prob) P.accept_prob[o] = (pd >= qd) ? 1.f : pd / qd;
-            if (P.out_token) P.out_token[o] = acc ? dtok : __float_as_int(ds.res[kCluRound + tid].x);
-            if (P.arrivals && P.accepted_len) {
-                // the last position of a sequence to arrive counts the accepted prefix (Algorithm 4 step 7).  The word
-                // holds (tag of the call, arrivals), so it needs no initialisation; the last one clears it for a replay.
-                const int b = row / P.positions;
-                unsigned long long* word = P.arrivals + (long long)b * P.trials + base + tid;
-                __threadfence();
-                unsigned long long old = *reinterpret_cast<volatile unsigned long long*>(word), want;
-                unsigned n_arrived;
-                for (;;) {
-                    n_arrived = ((uint32_t)(old >> 32) == g.tag ? (unsigned)old : 0u) + 1u;
-                    want = n_arrived == (unsigned)P.positions ? 0ull : ((unsigned long long)g.tag << 32) | n_arrived;
-                    const unsigned long long seen = atomicCAS(word, old, want);
-                    if (seen == old) break;              // at most `positions` CTAs contend for a word
-                    old = seen;
-                }
-                if (n_arrived == (unsigned)P.positions) {
-                    __threadfence();
-                    int k = 0;
-                    const volatile uint8_t* af = P.accepted;
-                    while (k < P.positions && af[((long long)b * P.positions + k) * P.trials + base + tid]) ++k;
-                    P.accepted_len[(long long)b * P.trials + base + tid] = k;
-                }
-            }
+            if (P.out_token) P.out_token[o] = acc ? dtok : __float_as_int(ds.res[nt + tid].x);
+            if (P.arrivals && P.accepted_len) count_accepted(P, g.tag, row, base + tid, acc);
         }
         if (base + kCluRound < P.trials) __syncthreads();        // the round's draws have been read
     }
