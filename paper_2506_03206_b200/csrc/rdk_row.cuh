@@ -85,6 +85,17 @@ __device__ __forceinline__ int first_above(const double* cdf, int count, double 
     return lo;
 }
 
+// The same by a whole warp in two steps (at most 1024 entries), and the last entry where there is none: every lane gets
+// the answer, after two reads instead of one for each halving.
+__device__ __forceinline__ int warp_first_above(const double* cdf, int count, double thr, int lane) {
+    const int per = (count + 31) >> 5;
+    const uint32_t lanes = __ballot_sync(0xffffffffu, cdf[min((lane + 1) * per, count) - 1] > thr);
+    if (!lanes) return count - 1;
+    const int first = (__ffs(lanes) - 1) * per;
+    const uint32_t in = __ballot_sync(0xffffffffu, lane < per && cdf[min(first + lane, count - 1)] > thr);
+    return min(first + __ffs(in) - 1, count - 1);
+}
+
 // Within one 256-token segment held as x[kVec] per lane: the first token whose inclusive prefix
 // sum exceeds rem and whose weight is positive; if rounding leaves none, the last positive token.
 // Returns lane * kVec + k (same value in all lanes), or -1 when the segment has no positive weight.

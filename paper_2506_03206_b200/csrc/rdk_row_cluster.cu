@@ -198,7 +198,9 @@ __device__ __forceinline__ void count_accepted(const RowParams& P, uint32_t tag,
 }
 
 template <typename TZ, typename TY, int KIND, int VAR, bool kPrior>
-__global__ void __launch_bounds__(512, 2)
+// 80 registers where two arrays and the draws' two chunks need them (320 rows of 128k with a prior: 117 -> 111 us, although a
+// CTA of 512 threads then has the SM to itself), 64 elsewhere (given weights of 1024 x 32k: 66 us, with 80 registers 70)
+__global__ void __maxnreg__(VAR == kVarPrior ? 80 : 64)
 rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     constexpr bool kLinear = VAR != kVarGiven, kDense = VAR == kVarDense || VAR == kVarGiven;
     constexpr uint32_t es = (uint32_t)sizeof(TZ);
@@ -703,15 +705,7 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     // thread, an integer division per draw and a fence with three dependent loads for accepted_len took 18 to 40 thousand
     // cycles a row, twice what the row itself takes.)
     const bool from_p = !(R_d > 0.0);                    // p and q~ coincide: the replacement comes from p itself
-    const int nch = g.per / 32, per_lane = (nseg + 31) >> 5;
-    // the first segment whose prefix sum exceeds thr; the last one if rounding leaves none
-    auto find_segment = [&](const double* c, double thr) -> int {
-        const uint32_t lanes = __ballot_sync(0xffffffffu, c[min((lane + 1) * per_lane, nseg) - 1] > thr);
-        if (!lanes) return nseg - 1;
-        const int first = (__ffs(lanes) - 1) * per_lane;
-        const uint32_t in = __ballot_sync(0xffffffffu, lane < per_lane && c[min(first + lane, nseg - 1)] > thr);
-        return min(first + __ffs(in) - 1, nseg - 1);
-    };
+    const int nch = g.per / 32;
     auto load_row8 = [&](const auto* src, int jb, float fill, float (&v)[kVec]) {
         using T = typename std::remove_cv<typename std::remove_pointer<decltype(src)>::type>::type;
         if (jb >= 0) {
@@ -798,7 +792,7 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
             const bool res = d >= nt;
             const double* c = res ? (from_p ? cdf[2] : cdf[1]) : cdf[0];
             const double thr = (double)__shfl_sync(0xffffffffu, u_draw, res ? kCluRound + d - nt : d) * c[nseg - 1];
-            sgm = find_segment(c, thr);
+            sgm = warp_first_above(c, nseg, thr, lane);
             rem = (float)(thr - (sgm ? c[sgm - 1] : 0.0));
             what = res ? (from_p ? 2 : 1) : 0;
         };

@@ -773,7 +773,7 @@ rdk_draw_kernel(const RowParams P, const int nseg, const int Lw) {
     const double* cdf = g == 0 ? cdfW : (from_p ? cdfP : cdfR);
     const int what = g == 0 ? kPickW : (from_p ? kPickP : kPickR);
     const double thr = g == 0 ? (double)u0 * S_d : (double)u2 * (from_p ? Pt_d : R_d);
-    const int seg = min(first_above(cdf, nseg, thr), nseg - 1);
+    const int seg = warp_first_above(cdf, nseg, thr, lane);
     const float rem = (float)(thr - (seg ? cdf[seg - 1] : 0.0));
     const int seg_lo = (int)min((long long)seg * Lw, (long long)P.N);
     const int seg_end = (int)min((long long)P.N, (long long)seg_lo + Lw);
@@ -832,15 +832,22 @@ rdk_draw_kernel(const RowParams P, const int nseg, const int Lw) {
         if (P.accept_prob) P.accept_prob[o] = a_prob;
         if (P.out_token) P.out_token[o] = acc ? dtok : res_tok[1];
         if (P.accepted_len && P.accepted && P.counters) {
-            // the last position of a sequence to finish counts the accepted prefix (Algorithm 4 step 7)
-            const int b = row / P.positions;
-            __threadfence();
-            const int old = atomicAdd(P.counters + b * P.trials + t, 1);
-            if (old == P.positions - 1) {
-                __threadfence();
+            // the last position of a sequence to finish counts the accepted prefix (Algorithm 4 step 7).  The counter
+            // carries the accept bits of up to 24 positions along, so that nothing has to be fenced and read back.
+            const int b = row / P.positions, pos = row - b * P.positions;
+            const bool bits = P.positions <= 24;
+            if (!bits) __threadfence();
+            const unsigned mine = 1u | (bits && acc ? 256u << pos : 0u);
+            const unsigned now = (unsigned)atomicAdd(P.counters + b * P.trials + t, (int)mine) + mine;
+            if ((int)(bits ? now & 255u : now) == P.positions) {
                 int k = 0;
-                const volatile uint8_t* af = P.accepted;
-                while (k < P.positions && af[((long long)b * P.positions + k) * P.trials + t]) ++k;
+                if (bits) {
+                    k = __ffs(~(int)(now >> 8)) - 1;
+                } else {
+                    __threadfence();
+                    const volatile uint8_t* af = P.accepted;
+                    while (k < P.positions && af[((long long)b * P.positions + k) * P.trials + t]) ++k;
+                }
                 P.accepted_len[b * P.trials + t] = k;
             }
         }
