@@ -3,21 +3,24 @@
 // when all drafts were accepted, a fresh draw t ~ p from the target row that follows the last draft
 // (inverse CDF in ascending token id with uniform lane 3 of the sequence's last position).
 //
-// One thread-block cluster per (sequence, trial).  Most sequences need no fresh draw: their clusters leave at once.
-// For the others the row's 16-byte aligned positions are dealt out to the cluster's warps; a warp takes the soft-max
-// sum of its run on a running scale, and these (scale, sum) records are all that the prefix sums need, so the row is
-// read once.  CTA 0 collects them (distributed shared memory), finds the run of the draw and reads that one again.
-// One CTA per sequence with two passes over the row was bound by what one SM can keep in flight: 65 us as soon as one
-// of 64 sequences of 128k tokens needed its draw.
+// A fixed number of thread-block clusters, each with a share of the (sequence, trial) pairs.  A cluster first settles what
+// needs no row -- a warp per pair counts the accepted positions and copies the tokens -- and then takes the pairs whose
+// drafts were all accepted, usually few, one after the other with all of its warps: the row's 16-byte aligned positions
+// are dealt out to the warps, a warp takes the soft-max sum of its run on a running scale, and these (scale, sum) records
+// are all that the prefix sums need, so the row is read once.  CTA 0 collects them (distributed shared memory), finds the
+// run of the draw and reads that one again.  What bounds it is the latency of that chain.  (One CTA per pair with two
+// passes over the row: 65 us as soon as one of 64 sequences of 128k tokens needed its draw; a cluster per pair: 11 us, and
+// 30 us for 512 sequences of 262k.)
 #include "rdk_device.cuh"
 #include "rdk_row.cuh"
 
 namespace rdk {
 
-constexpr int kEmitThreads = 256;
+constexpr int kEmitThreads = 512;
 constexpr int kEmitWarps = kEmitThreads / 32;
 constexpr int kEmitMaxCtas = 8;
 constexpr int kEmitMaxSeg = kEmitMaxCtas * kEmitWarps;
+constexpr int kEmitBatch = 256;           // pairs whose answers are kept at a time
 
 struct EmitParams {
     int N, batch, positions, trials, pad;
@@ -40,6 +43,35 @@ __device__ __forceinline__ void emit_load8(const TZ* zrow, int v, int phase, int
     }
 }
 
+// accepted drafts of one (sequence, trial) pair and the tokens that need no row, by one warp; returns the leading accepts
+__device__ __forceinline__ int emit_accepted(const EmitParams& P, int pair, int lane, bool write) {
+    const int b = pair / P.trials, t = pair - b * P.trials;
+    const long long first = (long long)b * P.positions * P.trials + t;
+    int32_t* seq = P.seq_tokens + (long long)pair * (P.positions + 1);
+    int j = 0;
+    bool run = true;
+    for (int k0 = 0; k0 <= P.positions; k0 += 32) {      // 32 positions at a time
+        const int k = k0 + lane;
+        const long long at = first + (long long)k * P.trials;
+        const bool in = k < P.positions;
+        const uint8_t acc = in ? P.accepted[at] : 0;
+        const int d = write && in ? P.draft_token[at] : -1, o = write && in ? P.out_token[at] : -1;      // (all three loads travel together)
+        if (run) {
+            const uint32_t no = ~__ballot_sync(0xffffffffu, acc != 0);
+            j += no ? __ffs(no) - 1 : 32;
+            run = no == 0;
+        }
+        if (write && k <= P.positions) {
+            if (k < j) seq[k] = d;
+            else if (k == j && in) seq[k] = o;           // the residual draw made there
+            else if (k > j && P.pad) seq[k] = -1;
+        }
+        if (!run && !(write && P.pad)) break;
+    }
+    if (write && lane == 0) P.seq_len[pair] = j + 1;
+    return j;
+}
+
 template <typename TZ>
 __global__ void __launch_bounds__(kEmitThreads)
 emit_kernel(const EmitParams P) {
@@ -47,137 +79,156 @@ emit_kernel(const EmitParams P) {
     __shared__ double cdf[kEmitMaxSeg];
     __shared__ float chunk_sum[32];
     __shared__ float bc[2];
+    __shared__ __align__(8) unsigned long long rbar;     // CTA 0: the records of the row are in rec[]
+    __shared__ uint8_t all_s[kEmitBatch];                // whether all drafts of the pair were accepted
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint32_t rank, C;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
     asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(C));
-    const int g = (int)(blockIdx.x / C), b = g / P.trials, t = g % P.trials;
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    const int cluster = (int)(blockIdx.x / C), clusters = (int)(gridDim.x / C);
+    const int pairs = P.batch * P.trials, mine = pairs > cluster ? (pairs - cluster + clusters - 1) / clusters : 0;
+    if (tid == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&rbar)));
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    uint32_t parity = 0;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");   // the inputs are usually the previous kernel's outputs
 
-    // leading accepted positions, 32 flags at a time
-    int j = 0;
-    for (int k0 = 0; k0 < P.positions; k0 += 32) {
-        const int k = k0 + lane;
-        const bool acc = k < P.positions && P.accepted[((long long)b * P.positions + k) * P.trials + t];
-        const uint32_t no = ~__ballot_sync(0xffffffffu, acc);
-        j += no ? __ffs(no) - 1 : 32;
-        if (no) break;
-    }
-    int32_t* seq = P.seq_tokens + (long long)g * (P.positions + 1);
-    if (rank == 0) {
-        for (int k = tid; k <= P.positions; k += kEmitThreads) {
-            if (k < j) seq[k] = P.draft_token[((long long)b * P.positions + k) * P.trials + t];
-            else if (k == j && j < P.positions) seq[k] = P.out_token[((long long)b * P.positions + k) * P.trials + t];   // the residual draw made there
-            else if (k > j && P.pad) seq[k] = -1;
+    for (int i0 = 0; i0 < mine; i0 += kEmitBatch) {
+        const int cnt = min(kEmitBatch, mine - i0);
+        // every CTA looks at all of the cluster's pairs, CTA 0 writes
+        for (int i = warp; i < cnt; i += kEmitWarps) {
+            const int j = emit_accepted(P, cluster + (i0 + i) * clusters, lane, rank == 0);
+            if (lane == 0) all_s[i] = j == P.positions;
         }
-        if (tid == 0) P.seq_len[g] = j + 1;
-    }
-    if (j < P.positions) return;                         // (the same in every thread of the cluster)
-
-    // every draft accepted: t ~ softmax(bonus row)
-    const TZ* zrow = static_cast<const TZ*>(P.bonus) + (long long)b * P.bonus_stride;
-    const int phase = (int)((reinterpret_cast<uintptr_t>(zrow) & 15u) / sizeof(TZ));
-    const int sg = (int)rank * kEmitWarps + warp, nseg = (int)C * kEmitWarps;
-    MS zs{-INFINITY, 0.f, 0.f};
+        __syncthreads();
+        for (int i = 0; i < cnt; ++i) {
+            if (!all_s[i]) continue;                     // (the same in every thread of the cluster)
+            // every draft accepted: t ~ softmax(bonus row)
+            const int pair = cluster + (i0 + i) * clusters, b = pair / P.trials, t = pair - b * P.trials;
+            const TZ* zrow = static_cast<const TZ*>(P.bonus) + (long long)b * P.bonus_stride;
+            const int phase = (int)((reinterpret_cast<uintptr_t>(zrow) & 15u) / sizeof(TZ));
+            const int sg = (int)rank * kEmitWarps + warp, nseg = (int)C * kEmitWarps;
+            const float u = __ldg(P.uniforms + (((long long)b * P.positions + P.positions - 1) * P.trials + t) * 4 + 3);
+            // CTA 0 runs, and is done with the previous row's records: it says so here, the others wait for it with their sums
+            if (rank == 0 && tid == 0)
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&rbar)), "r"((uint32_t)nseg * 8u) : "memory");
+            __syncwarp();
+            asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+            MS zs{-INFINITY, 0.f, 0.f};
 #pragma unroll 4
-    for (int k = lane; k < P.per; k += 32) {
-        float z[kVec];
-        emit_load8<TZ>(zrow, sg * P.per + k, phase, P.N, z);
-        float vmax = z[0];
+            for (int k = lane; k < P.per; k += 32) {
+                float z[kVec];
+                emit_load8<TZ>(zrow, sg * P.per + k, phase, P.N, z);
+                float vmax = z[0];
 #pragma unroll
-        for (int q = 1; q < kVec; ++q) vmax = fmaxf(vmax, z[q]);
-        if (vmax > zs.m) { zs.s *= ex2((zs.m - vmax) * kLog2e); zs.m = vmax; }
-        const float off = zs.m > -INFINITY ? -zs.m * kLog2e : 0.f;
+                for (int q = 1; q < kVec; ++q) vmax = fmaxf(vmax, z[q]);
+                if (vmax > zs.m) { zs.s *= ex2((zs.m - vmax) * kLog2e); zs.m = vmax; }
+                const float off = zs.m > -INFINITY ? -zs.m * kLog2e : 0.f;
 #pragma unroll
-        for (int q = 0; q < kVec; ++q) zs.s += ex2(fmaf(z[q], kLog2e, off));
-    }
-    zs = ms_warp(zs);
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");      // CTA 0 runs
-    if (lane == 0) {
-        uint32_t r;
-        asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(smem_u32(&rec[sg])));
-        asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(r), "f"(zs.m), "f"(zs.s) : "memory");
-    }
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    if (rank != 0) return;
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    if (warp == 0) {
-        MS a{-INFINITY, 0.f, 0.f};
-        for (int s = lane; s < nseg; s += 32) a = ms_combine(a, MS{rec[s].x, rec[s].y, 0.f});
-        a = ms_warp(a);
-        const float off = -a.m * kLog2e, inv_z = 1.f / a.s;
-        if (lane == 0) { bc[0] = off; bc[1] = inv_z; }
-        // prefix sums of the runs' probabilities, two runs per lane
-        double v[2], x = 0.0;
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int s = 2 * lane + k;
-            if (s < nseg && rec[s].x > -INFINITY) x += (double)(rec[s].y * ex2((rec[s].x - a.m) * kLog2e) * inv_z);
-            v[k] = x;
-        }
-        double incl = x;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const double y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
-        }
-        double before = __shfl_up_sync(0xffffffffu, incl, 1);
-        if (lane == 0) before = 0.0;
-#pragma unroll
-        for (int k = 0; k < 2; ++k) if (2 * lane + k < nseg) cdf[2 * lane + k] = before + v[k];
-    }
-    __syncthreads();
-    const float off = bc[0], inv_z = bc[1];
-    const double thr = (double)__ldg(P.uniforms + (((long long)b * P.positions + P.positions - 1) * P.trials + t) * 4 + 3) * cdf[nseg - 1];
-    const int s = min(first_above(cdf, nseg, thr), nseg - 1);
-    const float rem = (float)(thr - (s ? cdf[s - 1] : 0.0));
-    const int nch = P.per / 32;                          // 256-position chunks of a run, at most 32 taken at a time
-    auto chunk_p = [&](int ch, float (&p)[kVec]) -> float {
-        float z[kVec], sum = 0.f;
-        emit_load8<TZ>(zrow, s * P.per + ch * 32 + lane, phase, P.N, z);
-#pragma unroll
-        for (int q = 0; q < kVec; ++q) { p[q] = ex2(fmaf(z[q], kLog2e, off)) * inv_z; sum += p[q]; }
-        return warp_sum(sum);
-    };
-    float p[kVec], cum = 0.f, before = 0.f;
-    int chosen = -1, last_pos = -1;
-    for (int c0 = 0; c0 < nch && chosen < 0; c0 += 32) {
-        for (int ch = c0 + warp; ch < min(nch, c0 + 32); ch += kEmitWarps) {
-            const float sum = chunk_p(ch, p);
-            if (lane == 0) chunk_sum[ch - c0] = sum;
-        }
-        __syncthreads();
-        for (int ch = c0; ch < min(nch, c0 + 32); ++ch) {
-            const float sum = chunk_sum[ch - c0];
-            if (sum > 0.f) {
-                if (chosen < 0 && cum + sum > rem) { chosen = ch; before = cum; }
-                last_pos = ch;
-                cum += sum;
+                for (int q = 0; q < kVec; ++q) zs.s += ex2(fmaf(z[q], kLog2e, off));
             }
+            zs = ms_warp(zs);
+            asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+            if (lane == 0) {
+                uint32_t r, m;
+                asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(smem_u32(&rec[sg])));
+                asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(m) : "r"(smem_u32(&rbar)));
+                asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];"
+                             ::"r"(r), "r"(__float_as_uint(zs.m)), "r"(__float_as_uint(zs.s)), "r"(m) : "memory");
+            }
+            if (rank != 0) continue;
+            if (warp == 0)                               // the records are on their way from running CTAs; a limit all the same
+                for (unsigned spins = 0, done = 0; !done && spins < (1u << 22); ++spins)
+                    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+                                 : "=r"(done) : "r"(smem_u32(&rbar)), "r"(parity) : "memory");
+            parity ^= 1u;
+            constexpr int K = kEmitMaxSeg / 32;          // runs per lane
+            if (warp == 0) {
+                float2 r[K];
+                MS a{-INFINITY, 0.f, 0.f};
+                const int per = (nseg + 31) >> 5;
+#pragma unroll
+                for (int k = 0; k < K; ++k) {
+                    r[k] = k < per && lane * per + k < nseg ? rec[lane * per + k] : make_float2(-INFINITY, 0.f);
+                    a = ms_combine(a, MS{r[k].x, r[k].y, 0.f});
+                }
+                a = ms_warp(a);
+                const float inv_z = 1.f / a.s;
+                if (lane == 0) { bc[0] = -a.m * kLog2e; bc[1] = inv_z; }
+                double v[K], x = 0.0;                    // prefix sums of the runs' probabilities
+#pragma unroll
+                for (int k = 0; k < K; ++k) {
+                    if (r[k].x > -INFINITY) x += (double)(r[k].y * ex2((r[k].x - a.m) * kLog2e) * inv_z);
+                    v[k] = x;
+                }
+                double incl = x;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const double y = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += y;
+                }
+                double before = __shfl_up_sync(0xffffffffu, incl, 1);
+                if (lane == 0) before = 0.0;
+#pragma unroll
+                for (int k = 0; k < K; ++k) if (k < per && lane * per + k < nseg) cdf[lane * per + k] = before + v[k];
+            }
+            __syncthreads();
+            const float off = bc[0], inv_z = bc[1];
+            const double thr = (double)u * cdf[nseg - 1];
+            const int s = warp_first_above(cdf, nseg, thr, lane);
+            const float rem = (float)(thr - (s ? cdf[s - 1] : 0.0));
+            const int nch = P.per / 32;                  // 256-position chunks of a run, at most 32 taken at a time
+            float p[kVec], cum = 0.f, before = 0.f;
+            int chosen = -1, last_pos = -1, held = -1;
+            auto chunk_p = [&](int ch) -> float {
+                float z[kVec], sum = 0.f;
+                emit_load8<TZ>(zrow, s * P.per + ch * 32 + lane, phase, P.N, z);
+#pragma unroll
+                for (int q = 0; q < kVec; ++q) { p[q] = ex2(fmaf(z[q], kLog2e, off)) * inv_z; sum += p[q]; }
+                held = ch;
+                return warp_sum(sum);
+            };
+            for (int c0 = 0; c0 < nch && chosen < 0; c0 += 32) {
+                for (int ch = c0 + warp; ch < min(nch, c0 + 32); ch += kEmitWarps) {
+                    const float sum = chunk_p(ch);
+                    if (lane == 0) chunk_sum[ch - c0] = sum;
+                }
+                __syncthreads();
+                for (int ch = c0; ch < min(nch, c0 + 32); ++ch) {
+                    const float sum = chunk_sum[ch - c0];
+                    if (sum > 0.f) {
+                        if (chosen < 0 && cum + sum > rem) { chosen = ch; before = cum; }
+                        last_pos = ch;
+                        cum += sum;
+                    }
+                }
+                __syncthreads();
+            }
+            const float r_in = chosen < 0 ? INFINITY : rem - before;     // rounding left no token: the last positive one
+            if (chosen < 0) chosen = max(last_pos, 0);
+            if (chosen % kEmitWarps != warp) continue;
+            if (held != chosen) (void)chunk_p(chosen);
+            const int sel = max(pick_in_segment(p, r_in, lane), 0);
+            if (lane == 0) P.seq_tokens[(long long)pair * (P.positions + 1) + P.positions] = min(max((s * P.per + chosen * 32) * kVec - phase + sel, 0), P.N - 1);
         }
-        __syncthreads();
+        __syncthreads();                                 // all_s has been read
     }
-    if (warp != 0) return;
-    const float r_in = chosen < 0 ? INFINITY : rem - before;     // rounding left no token: the last positive one
-    if (chosen < 0) chosen = max(last_pos, 0);
-    (void)chunk_p(chosen, p);
-    const int sel = max(pick_in_segment(p, r_in, lane), 0);
-    if (lane == 0) seq[j] = min(max((s * P.per + chosen * 32) * kVec - phase + sel, 0), P.N - 1);
 }
 
 template <typename TZ>
 static cudaError_t launch_emit(EmitParams P, cudaStream_t s) {
-    // CTAs per sequence: up to 8, a run of at least 256 positions for each warp, while the clusters are few; with many
-    // sequences most clusters leave at once and their launch is what costs.
-    const long long seqs = (long long)P.batch * P.trials;
+    // CTAs per cluster: a warp's run is at least two 256-position chunks.  Clusters: what is resident at once (four CTAs of
+    // 512 threads to an SM), in the worst case one for each pair.
+    const long long pairs = (long long)P.batch * P.trials;
     unsigned C = 1;
-    while (C < (unsigned)kEmitMaxCtas && (long long)C * 2048 < P.N && seqs * C < 2048) C *= 2;
+    while (C < (unsigned)kEmitMaxCtas && (long long)C * kEmitWarps * 512 < P.N) C *= 2;
+    const long long most = 4 * 148 / C;
     P.per = (int)(((long long)P.N + 8 + C * kEmitWarps * kVec - 1) / (C * kEmitWarps * kVec));
     P.per = (P.per + 31) / 32 * 32;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)seqs * C, 1, 1);
+    cfg.gridDim = dim3((unsigned)(pairs < most ? pairs : most) * C, 1, 1);
     cfg.blockDim = dim3(kEmitThreads, 1, 1);
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
