@@ -461,13 +461,10 @@ static int run_rows(const rdk_problem* pb, int mode, const void* target, const v
     P.num_tiles = (pb->N + kTile - 1) / kTile;
     const size_t smem = (size_t)P.num_tiles * kRowWarps * 24;
     cudaError_t e = cudaErrorNotSupported;
+    bool counted = false;
     P.positions = pb->positions;
     P.accepted_len = out ? out->accepted_len : nullptr;
-    if (mode == RDK_MODE_LINEAR && trials > 0 && !prior && !(pb->flags & RDK_FLAG_ROW_KERNEL)) {
-        e = launch_stream_linear(P, pb->target_dtype, pb->drafter_dtype, pb->drafter_kind, pb->batch, ws, ws_bytes, s);
-        if (e == cudaSuccess) return RDK_OK;          // the streaming kernel also wrote accepted_len
-    }
-    if (e == cudaErrorNotSupported && !(pb->flags & RDK_FLAG_ROW_KERNEL)) {
+    auto cluster = [&]() -> cudaError_t {
         RowParams Q = P;
         uint32_t tag = 0;
         if (Q.accepted_len && Q.accepted && ws) {                   // accepted_len is counted inside the kernel
@@ -477,9 +474,20 @@ static int run_rows(const rdk_problem* pb, int mode, const void* target, const v
                 Q.arrivals = static_cast<unsigned long long*>(ws);
             if (Q.arrivals) tag = next_tag();
         }
-        e = launch_cluster_rows(Q, mode, pb->target_dtype, pb->drafter_dtype, pb->drafter_kind, tag, stream_spin_limit(), s);
-        if (e == cudaSuccess && Q.arrivals) return RDK_OK;
-        if (e == cudaErrorNotSupported) (void)cudaGetLastError();
+        const cudaError_t r = launch_cluster_rows(Q, mode, pb->target_dtype, pb->drafter_dtype, pb->drafter_kind, tag, stream_spin_limit(), s);
+        if (r == cudaErrorNotSupported) (void)cudaGetLastError();
+        counted = r == cudaSuccess && Q.arrivals;
+        return r;
+    };
+    if (!(pb->flags & RDK_FLAG_ROW_KERNEL)) {
+        const bool streams = mode == RDK_MODE_LINEAR && trials > 0 && !prior;
+        if (!streams || stream_few_rows(P, pb->target_dtype, pb->drafter_dtype, pb->drafter_kind)) e = cluster();
+        if (e == cudaErrorNotSupported && streams) {
+            e = launch_stream_linear(P, pb->target_dtype, pb->drafter_dtype, pb->drafter_kind, pb->batch, ws, ws_bytes, s);
+            counted = e == cudaSuccess;
+        }
+        if (e == cudaErrorNotSupported) e = cluster();
+        if (counted) return RDK_OK;                                 // the kernel also wrote accepted_len
     }
     if (e == cudaErrorNotSupported)
         e = (mode == RDK_MODE_LINEAR)

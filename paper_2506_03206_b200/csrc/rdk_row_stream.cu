@@ -1064,6 +1064,21 @@ const char* stream_ineligible(const RowParams& P, int tz, int ty, int kind, int 
     return nullptr;
 }
 
+// Whether so few rows are better served by one cluster launch each than by setting up the streaming grid and a second
+// kernel for the draws (the streaming kernels pay off when a group of CTAs has several rows to stream).  Sampling call, streaming /
+// cluster kernel, a quarter of the tokens kept, us:  8192 bf16: 11.0 / 8.5 for 4 rows, 14.6 / 11.4 for 160, 16.0 / 18.2 for 320;
+// 32768: 12.0 / 8.8 for 4, 16.2 / 15.5 for 96, 17.8 / 18.9 for 160; 128256: 12.8 / 10.3 for 4, 16.6 / 14.6 for 24, 18.6 / 20.9 for
+// 48; 262144: 13.7 / 11.1 for 4, 27.7 / 27.3 for 64; fp32 128256: 13.5 / 10.2 for 4, 32.0 / 31.6 for 96.  The cluster
+// kernel makes a row's draws in one CTA: not with many trials.
+bool stream_few_rows(const RowParams& P, int tz, int ty, int kind) {
+    if (P.trials > 2) return false;
+    StreamSegs sg;
+    const bool one_group = stream_segments(P.N, tz == RDK_F32 ? 4 : 2, sg) && sg.C == kMaxGroup;      // 9 groups of 16 CTAs
+    int most = !fast_types(tz, ty, kind) ? 96 : (one_group ? 56 : 24);
+    if (P.N <= 32768) { const int small = 3200000 / P.N; most = most > small ? most : (small < 192 ? small : 192); }
+    return P.rows <= most;
+}
+
 void set_stream_spin_limit(unsigned limit) { g_spin_limit.store(limit); }
 unsigned stream_spin_limit() { return g_spin_limit.load(); }
 
