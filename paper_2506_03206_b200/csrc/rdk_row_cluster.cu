@@ -39,7 +39,6 @@ constexpr int kCluMaxWarps = 16;
 constexpr int kCluMaxSeg = kCluMaxCtas * kCluMaxWarps;
 constexpr int kCluRound = 16;                       // trials settled between two collections
 constexpr int kCluMaxChunks = 32;                   // 256-position chunks of a segment
-constexpr int kRegSlots = 8;                        // kept tokens per lane held in registers
 constexpr unsigned kCluSpinDefault = 1u << 22;
 
 // What CTA 0 needs for the draws lies where its part of the row was: nobody reads that any more by then.
@@ -173,6 +172,7 @@ __device__ __forceinline__ void count_accepted(const RowParams& P, uint32_t tag,
     const int b = row / P.positions, pos = row - b * P.positions;
     unsigned long long* word = P.arrivals + (long long)b * P.trials + t;
     int32_t* out = P.accepted_len + (long long)b * P.trials + t;
+    if (P.positions == 1) { *out = acc; return; }
     const bool bits = P.positions <= kCluBits;
     const unsigned long long mine = 1ull | (bits && acc ? 256ull << pos : 0ull), first = (unsigned long long)tag << 32 | mine;
     if (!bits) __threadfence();
@@ -204,6 +204,8 @@ __global__ void __maxnreg__(VAR == kVarPrior ? 80 : 64)
 rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     constexpr bool kLinear = VAR != kVarGiven, kDense = VAR == kVarDense || VAR == kVarGiven;
     constexpr uint32_t es = (uint32_t)sizeof(TZ);
+    // kept tokens per lane held in registers between the visits; more cost the others their registers
+    constexpr int kRegSlots = VAR == kVarSparse ? 12 : 8;
     extern __shared__ __align__(128) unsigned char csm[];
     __shared__ __align__(16) float4 segs[kCluMaxSeg];            // per segment: sums of w, min(p, q~), max(0, p - q~), p
     __shared__ __align__(16) float4 xrec[kCluMaxCtas][2];        // one record per CTA of the cluster
@@ -327,22 +329,28 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
                 if (il + k * 32 >= cnt) { y[k] = KIND == RDK_LOGITS ? -INFINITY : 0.f; pos[k] = -1; }
         }
     };
-    float ky[kRegSlots];
-    int kpos[kRegSlots];
+    float ke[kRegSlots];                                             // drafter values, after the first visit e_y
+    uint32_t kpos[kRegSlots / 2] = {};                                 // positions in the segment, two to a word; 0xffff: none
+    auto pos_of = [&](int k) -> int { return (int)(short)(k & 1 ? kpos[k / 2] >> 16 : kpos[k / 2] & 0xffffu); };     // (a segment has at most 8192)
+    auto load_slots = [&](int h) {                                   // slots h .. h + 3
+        if (h * 32 < cnt) {
+            int pos[4];
+            load_kept(h * 32 + lane, ke + h, pos);
+            kpos[h / 2] = (uint32_t)(pos[0] & 0xffff) | (uint32_t)pos[1] << 16;
+            kpos[h / 2 + 1] = (uint32_t)(pos[2] & 0xffff) | (uint32_t)pos[3] << 16;
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) ke[h + k] = KIND == RDK_LOGITS ? -INFINITY : 0.f;
+            kpos[h / 2] = kpos[h / 2 + 1] = 0xffffffffu;
+        }
+    };
     float my_w = KIND == RDK_LOGITS ? -INFINITY : 0.f;
     if (kLinear) {
 #pragma unroll
-        for (int h = 0; h < kRegSlots; h += 4) {
-            if (h * 32 < cnt) {
-                load_kept(h * 32 + lane, ky + h, kpos + h);
-            } else {
-#pragma unroll
-                for (int k = 0; k < 4; ++k) { ky[h + k] = KIND == RDK_LOGITS ? -INFINITY : 0.f; kpos[h + k] = -1; }
-            }
-        }
+        for (int h = 0; h < kRegSlots; h += 4) load_slots(h);
         if (KIND == RDK_LOGITS) {
 #pragma unroll
-            for (int k = 0; k < kRegSlots; ++k) my_w = fmaxf(my_w, ky[k]);
+            for (int k = 0; k < kRegSlots; ++k) my_w = fmaxf(my_w, ke[k]);
             my_w = warp_max_redux(my_w);
         }
     }
@@ -379,11 +387,15 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     };
     float m_w = -INFINITY, mp_w = -INFINITY, zoff = 0.f, poff = 0.f, yoff = 0.f;
     float E = 0.f, Ep = 0.f, K = 0.f, Zq = 0.f, th = 0.f, W = 0.f;
-    float kz[kRegSlots], ke[kRegSlots];                              // e_z and e_y of the first kept tokens
+    float kz[kRegSlots];                                             // e_z (prior: that of the prior) of the first kept tokens
     const uint32_t db = kPrior ? pb : zb;                            // the distribution that enters theta
     for (int attempt = 0; attempt < 2; ++attempt) {
         m_w = seg_max(zb, attempt == 0 ? 1 : nit16);
         if (kPrior) mp_w = seg_max(pb, attempt == 0 ? 1 : nit16);
+        if (attempt == 1 && kLinear) {                               // the values have become exponentials: once more
+#pragma unroll
+            for (int h = 0; h < kRegSlots; h += 4) load_slots(h);
+        }
         if (attempt == 1 && kLinear && KIND == RDK_LOGITS) {
             for (int il = kRegSlots * 32 + lane; il < cnt; il += 128) {
                 float y[4];
@@ -401,7 +413,7 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
         K = 0.f; Zq = 0.f; th = 0.f;
         if (kLinear) {
             const float doff = kPrior ? poff : zoff;
-            auto visit = [&](int pos, float y, float& ed, float& ey) {
+            auto visit = [&](int pos, const float y, float& ed, float& ey) {
                 ed = ex2(fmaf(lds_z<TZ>(db + (uint32_t)max(pos, 0) * es), kLog2e, doff));
                 if (pos < 0) ed = 0.f;
                 ey = KIND == RDK_LOGITS ? ex2(fmaf(y, kLog2e, yoff)) : y;
@@ -412,7 +424,7 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
             for (int h = 0; h < kRegSlots; h += 4) {
                 if (h * 32 < cnt) {
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) visit(kpos[h + k], ky[h + k], kz[h + k], ke[h + k]);
+                    for (int k = 0; k < 4; ++k) visit(pos_of(h + k), ke[h + k], kz[h + k], ke[h + k]);
                 } else {
 #pragma unroll
                     for (int k = 0; k < 4; ++k) { kz[h + k] = 0.f; ke[h + k] = 0.f; }
@@ -599,7 +611,7 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
             if (pos >= 0) { dw += w - w0; da += fminf(p, w) - fminf(p, w0); }
         };
 #pragma unroll
-        for (int k = 0; k < kRegSlots; ++k) if ((k & ~3) * 32 < cnt) again(kpos[k], kz[k], ke[k]);
+        for (int k = 0; k < kRegSlots; ++k) if ((k & ~3) * 32 < cnt) again(pos_of(k), kz[k], ke[k]);
         for (int il = kRegSlots * 32 + lane; il - lane < cnt; il += 128) {
             float y[4];
             int pos[4];
@@ -835,12 +847,18 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
             for (int it = warp; it < items; it += 2 * nw) {
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    const int item = min(it + h * nw, items - 1);
+                    const int item = it + h * nw;
+                    if (item >= items) break;
                     d[h] = item / nch; ch[h] = item - d[h] * nch;
                     locate(d[h], sgm[h], what[h], rem[h]);
                 }
-                chunks(std::integral_constant<int, 2>(), sgm, ch, what, x, sum);
-                if (lane == 0) { ds.dsum[d[0]][ch[0]] = sum[0]; ds.dsum[d[1]][ch[1]] = sum[1]; }
+                if (it + nw < items) {
+                    chunks(std::integral_constant<int, 2>(), sgm, ch, what, x, sum);
+                    if (lane == 0) ds.dsum[d[1]][ch[1]] = sum[1];
+                } else {
+                    chunks(std::integral_constant<int, 1>(), sgm, ch, what, x, sum);
+                }
+                if (lane == 0) ds.dsum[d[0]][ch[0]] = sum[0];
             }
             __syncthreads();
             int c;
