@@ -285,7 +285,7 @@ aff_rows_kernel(const __nv_bfloat16* __restrict__ E, long long stride, const int
 // off[i] = -scale - log2(sum of the parts of i, in order); -inf where the kept id has no token.  One warp per 32 ids and
 // eight warps share their parts.
 __global__ void __launch_bounds__(256)
-aff_offset_kernel(const float* __restrict__ part, const float* __restrict__ invk, float* __restrict__ off, int parts, int npad, float scale) {
+aff_offset_kernel(const float* __restrict__ part, const float* __restrict__ invk, float* __restrict__ off, int parts, int npad, int N, float scale) {
     __shared__ float s[8][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -297,7 +297,9 @@ aff_offset_kernel(const float* __restrict__ part, const float* __restrict__ invk
     __syncthreads();
     if (warp == 0) {
         for (int w = 1; w < 8; ++w) a += s[w][lane];
-        off[i] = invk[i] > 0.f ? -scale - log2f(a) : -INFINITY;
+        // (a zero embedding is equally near to every token: exp(0 - 1 / tau) may be too small to count)
+        const float ik = invk[i];
+        off[i] = ik > 0.f ? (ik < 1e12f ? -scale - log2f(a) : -log2f((float)N)) : -INFINITY;
     }
 }
 
@@ -333,9 +335,8 @@ static AffTcLayout aff_tc_layout(int N, int n, int d) {
 size_t affinity_tc_workspace_bytes(int N, int n, int d) { return aff_tc_layout(N, n, d).total; }
 
 // whether the tensor-core route serves this call (the other route serves everything)
-bool affinity_tc_eligible(const void* embeddings, int emb_dtype, const void* ws, int layout) {
-    return emb_dtype == RDK_BF16 && layout == RDK_AFF_BF16_COLS && (reinterpret_cast<uintptr_t>(embeddings) & 1u) == 0 &&
-           (reinterpret_cast<uintptr_t>(ws) & 15u) == 0;
+bool affinity_tc_eligible(const void* embeddings, int emb_dtype, int layout) {
+    return emb_dtype == RDK_BF16 && layout == RDK_AFF_BF16_COLS && (reinterpret_cast<uintptr_t>(embeddings) & 1u) == 0;
 }
 
 template <typename K, typename... A>
@@ -394,7 +395,7 @@ int build_affinity_tc(const __nv_bfloat16* E, int d, long long estride, const in
     if (items > 0x7fffffffLL || items_w > 0x7fffffffLL) { set_error("rdk_build_affinity: too many tiles"); return RDK_ERR_UNSUPPORTED; }
     P.num_items = (int)items;
     RDK_CUDA(launch_pdl(aff_tc_kernel<kAffSums>, (unsigned)(items < sms ? items : sms), (unsigned)aff_threads(kAffSums), (size_t)kAffSmem, s, keptA, tokB, out, P));
-    RDK_CUDA(launch_pdl(aff_offset_kernel, (unsigned)(L.npad / 32), 256u, 0, s, (const float*)part, (const float*)invk, off, 4 * L.spans, L.npad, scale));
+    RDK_CUDA(launch_pdl(aff_offset_kernel, (unsigned)(L.npad / 32), 256u, 0, s, (const float*)part, (const float*)invk, off, 4 * L.spans, L.npad, N, scale));
     // the matrix: rows = tokens, columns = kept ids
     P.tiles_m = L.Npad / kAffM; P.tiles_n = L.npad / kAffN; P.cols = n;
     P.row_inv = inv; P.col_inv = invk; P.col_off = off;
