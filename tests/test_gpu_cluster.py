@@ -1,0 +1,207 @@
+"""GPU parity of the cluster row kernel, the emitted sequences, the paired tensor-core contraction and the affinity builds
+at the sizes where their tiles and segments end, against the CPU checker (or a float64 product of the same operands)."""
+import numpy as np
+import pytest
+import torch
+
+import parity_util as PU
+import workloads as W
+from oracle import rdk_oracle as O
+from test_gpu_linear import KIND, _run_linear
+
+pytestmark = pytest.mark.gpu
+
+
+def _rdk():
+    import paper_2506_03206_b200 as rdk
+    return rdk
+
+
+def _reference(inp, kept_ids=None, prior=None):
+    cfg, kappa = inp["cfg"], (inp["kept_ids"] if kept_ids is None else kept_ids).numpy()
+    return {r: O.rdk_row(W.to_f64(inp["target"][r]), W.to_f64(inp["drafter"][r]), kappa, np.zeros((1, 4)), "linear",
+                         drafter_kind=cfg.drafter_kind, prior=None if prior is None else W.to_f64(prior)) for r in range(cfg.rows)}
+
+
+# N around the change of variant (4096), segments of one and several 256-token chunks, odd sizes (every row at another
+# alignment), one to sixteen CTAs a row, more than one round of trials (16), more kept tokens than fit a warp's registers
+@pytest.mark.parametrize("N,n,rows,trials,dtype,kind", [
+    (4095, 1000, 3, 17, "f32", "logits"), (4096, 1024, 3, 1, "bf16", "logits"), (4097, 4000, 3, 2, "bf16", "probs"),
+    (8193, 8193, 2, 33, "f32", "logits"), (20001, 2500, 40, 1, "bf16", "logits"), (50257, 25000, 2, 8, "bf16", "logits"),
+    (65537, 300, 2, 3, "f32", "probs"), (131075, 40000, 1, 16, "bf16", "logits")])
+def test_cluster_kernel_shapes(N, n, rows, trials, dtype, kind):
+    cfg = W.tiny_config(N=N, n=n, rows=rows, dtype=dtype, trials=trials, rho=0.6, seed=N, drafter_kind=kind, zipf_bias=True)
+    _run_linear(cfg, W.make_inputs(cfg), check_qtilde=N < 60000).assert_ok()
+
+
+def test_cluster_kernel_unsorted_ids_and_sequences_longer_than_the_accept_bits():
+    cfg = W.tiny_config(N=5003, n=700, rows=60, dtype="bf16", trials=3, rho=0.9, seed=5)
+    cfg = cfg.with_rows(2, 30)                       # 30 positions: arrivals are counted, the flags read again
+    inp = W.make_inputs(cfg)
+    ids = inp["kept_ids"][torch.randperm(cfg.n, generator=torch.Generator().manual_seed(2))].clone()
+    ids[3], ids[cfg.n - 1] = -1, cfg.N + 4           # two drafter tokens outside the vocabulary
+    _run_linear(cfg, inp, kept_override=ids).assert_ok()
+
+
+def test_cluster_kernel_scale_that_does_not_fit_the_segment():
+    """The first tokens of a segment give the scale of its exponentials; here they are far below the others or -inf, so that
+    the sums overflow the limit and the visit is repeated with the maximum."""
+    cfg = W.tiny_config(N=16411, n=3000, rows=4, dtype="f32", trials=4, rho=0.5, seed=12)
+    inp = W.make_inputs(cfg)
+    inp["target"][0, 256:] += 150.0
+    inp["target"][1, :4000] = -float("inf")
+    inp["target"][2, 700:9000] -= 400.0
+    inp["drafter"][3, 2000:] += 120.0
+    _run_linear(cfg, inp).assert_ok()
+
+
+@pytest.mark.parametrize("shift", [0.0, 30.0, -30.0])
+def test_cluster_kernel_prior_above_and_below_the_target(shift):
+    """theta pi / N is the smaller of the two nearly everywhere, or for half of the tokens, or hardly anywhere: the second visit
+    decides it from the difference of the logits."""
+    rdk = _rdk()
+    cfg = W.tiny_config(N=9001, n=1500, rows=3, dtype="bf16", trials=5, rho=0.7, seed=31)
+    inp = W.make_inputs(cfg)
+    g = torch.Generator().manual_seed(3)
+    prior = torch.randn(cfg.N, generator=g)
+    prior[: cfg.N // 2] += shift
+    prior[11] = -float("inf")
+    inp["target"][:, 13] = -float("inf")
+    prior = prior.to(torch.bfloat16)
+    idx = rdk.rdk_prepare_ids(inp["kept_ids"].cuda(), cfg.N)
+    out = rdk.rdk_sample_and_verify_prior(idx, inp["target"].cuda(), prior.cuda(), inp["drafter"].cuda(), inp["uniforms"].cuda(),
+                                          cfg.batch, cfg.positions)
+    qt, _, _ = rdk.rdk_redistribute_linear_prior(idx, inp["target"].cuda(), prior.cuda(), inp["drafter"].cuda(), cfg.batch, cfg.positions)
+    torch.cuda.synchronize()
+    PU.compare_sampling(inp, out, range(cfg.rows), "linear", prior=prior).assert_ok()
+    PU.compare_accepted_len(out, cfg.batch, cfg.positions, cfg.trials)
+    PU.compare_qtilde(qt, _reference(inp, prior=prior), True)
+
+
+@pytest.mark.parametrize("N,batch,positions,trials,counters", [(4096, 3, 2, 20, True), (33000, 2, 3, 1, False), (70001, 1, 1, 4, True)])
+def test_cluster_kernel_given_weights(N, batch, positions, trials, counters):
+    rdk = _rdk()
+    B = rdk.binding
+    cfg = W.tiny_config(N=N, n=50, rows=batch * positions, dtype="bf16", trials=trials, seed=N).with_rows(batch, positions)
+    inp = W.make_inputs(cfg)
+    # a total of about 1, as the exact redistribution gives: S is an fp32 number, so its bound of 1e-5 holds for such totals
+    # (a rounding error is 2^-24 of the total, 2e-4 for one of several thousand)
+    w = torch.rand(cfg.rows, N, generator=torch.Generator().manual_seed(N)) ** 8
+    w = w / w.sum(1, keepdim=True)
+    idx = rdk.rdk_prepare_ids(inp["kept_ids"].cuda(), N)
+    # with room for the counters accepted_len is counted in the same launch, without it in one more
+    ws = torch.full((8 * batch * trials if counters else 4,), 0xA5, dtype=torch.uint8, device="cuda")
+    for _ in range(2):
+        out = rdk.rdk_sample_and_verify(idx, B.RDK_MODE_PRECOMPUTED_W, inp["target"].cuda(), None, w.cuda(), inp["uniforms"].cuda(),
+                                        batch, positions, ws=ws)
+        torch.cuda.synchronize()
+        PU.compare_sampling(inp, out, range(cfg.rows), "given", w_given=w.double().numpy()).assert_ok()
+        PU.compare_accepted_len(out, batch, positions, trials)
+
+
+@pytest.mark.parametrize("N,batch,positions,trials", [(300, 700, 3, 2), (40001, 90, 40, 1), (140000, 3, 1, 1)])
+def test_emitted_sequences_of_many_pairs(N, batch, positions, trials):
+    """More pairs than clusters, more positions than a warp's lanes, one to eight CTAs a row; the accept patterns mix all
+    accepted, none and everything between."""
+    rdk = _rdk()
+    g = torch.Generator().manual_seed(N)
+    bonus = (torch.randn(batch, N, generator=g) * 2).to(torch.bfloat16)
+    u = torch.from_numpy(W.uniforms(N, batch * positions, trials))
+    cut = torch.randint(0, positions + 2, (batch, trials), generator=g)           # leading accepts; beyond it at random
+    acc = torch.rand(batch, positions, trials, generator=g) < 0.5
+    k = torch.arange(positions).view(1, positions, 1)
+    acc = (k < cut.unsqueeze(1)) | (acc & (k > cut.unsqueeze(1)))
+    draft = torch.randint(0, N, (batch, positions, trials), generator=g, dtype=torch.int32)
+    resid = torch.randint(0, N, (batch, positions, trials), generator=g, dtype=torch.int32)
+    seq, ln = rdk.rdk_emit_sequences(N, batch, positions, bonus.cuda(), u.cuda(), draft.cuda(), acc.to(torch.uint8).cuda(), resid.cuda())
+    torch.cuda.synchronize()
+    seq, ln, un, near = seq.cpu().numpy(), ln.cpu().numpy(), u.numpy().reshape(batch, positions, trials, 4), 0
+    for b in range(batch):
+        cdf = None
+        for t in range(trials):
+            a = acc[b, :, t].numpy()
+            j = positions if a.all() else int(np.argmin(a))
+            assert ln[b, t] == j + 1 and np.array_equal(seq[b, t, :j], draft[b, :j, t].numpy()) and np.all(seq[b, t, j + 1:] == -1)
+            if j < positions:
+                assert seq[b, t, j] == resid[b, j, t]
+            else:
+                cdf = np.cumsum(O.softmax(W.to_f64(bonus[b]))) if cdf is None else cdf
+                thr, tok = float(un[b, positions - 1, t, 3]) * cdf[-1], int(seq[b, t, j])
+                near += tok != int(np.searchsorted(cdf, thr, side="right"))
+                assert PU.interval_distance(cdf, tok, thr) <= PU.BOUNDARY_TOL
+    assert near <= max(1, 0.01 * batch * trials)
+
+
+# rows: one instruction of the smallest width, the steps of 16, both instructions, several row tiles, halves of the last
+# round; tokens: less than, exactly and just over a CTA's 128 and a pair's 256; contraction: around one block of 64
+@pytest.mark.parametrize("N,n,rows", [(127, 63, 1), (128, 64, 16), (129, 65, 33), (255, 8, 256), (257, 129, 257), (5000, 200, 300),
+                                      (300, 1000, 513), (19200, 72, 1024), (38000, 640, 320), (4096, 192, 1100)])
+def test_paired_contraction_at_tile_edges(N, n, rows):
+    rdk = _rdk()
+    B = rdk.binding
+    g = torch.Generator(device="cuda").manual_seed(N + rows)
+    ids = torch.sort(torch.randperm(N, generator=g, device="cuda")[: min(n, N)]).values.to(torch.int32)
+    ids = torch.cat([ids, torch.full((n - ids.numel(),), -1, dtype=torch.int32, device="cuda")])        # n > N: tokens outside the vocabulary
+    idx = rdk.rdk_prepare_ids(ids, N)
+    # probabilities that are multiples of 2^-12 and add up to 1: exact in bf16, so that q' is too
+    q = torch.zeros(rows, n, device="cuda")
+    live = min(n, N, 16)
+    q[:, torch.randperm(min(n, N), generator=g, device="cuda")[:live]] = 1.0 / (1 << (live.bit_length() - 1))
+    q = q / q.sum(1, keepdim=True) if live & (live - 1) else q
+    M = {"data": torch.rand(N, (n + 7) // 8 * 8, generator=g, device="cuda").to(torch.bfloat16), "layout": B.RDK_AFF_BF16_COLS, "ld": (n + 7) // 8 * 8}
+    w = torch.full((rows, N), float("nan"), device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    _, S, _ = rdk.rdk_redistribute_exact(idx, q, M, rows, 1, B.RDK_PROBS, w_out=w, status_word=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    ref = q.to(torch.bfloat16).double() @ M["data"][:, :n].double().T
+    # fp32 accumulation of n products: n rounding errors of 2^-24 of the result at most
+    assert ((w.double() - ref).abs() <= (n + 2) * 2.0 ** -24 * ref.abs() + 1e-12).all()
+    assert ((S.double() - ref.sum(1)).abs() <= (N + n) * 2.0 ** -24 * ref.sum(1) + 1e-12).all()
+
+
+@pytest.mark.parametrize("N,n,rows", [(31, 5, 1), (33, 257, 9), (1024, 300, 80), (4736, 1000, 70)])
+def test_fp32_contraction_at_tile_edges(N, n, rows):
+    """One and four columns a thread (the last shape), ragged rows, columns and contraction."""
+    rdk = _rdk()
+    B = rdk.binding
+    g = torch.Generator(device="cuda").manual_seed(N)
+    ids = torch.sort(torch.randperm(N, generator=g, device="cuda")[: min(n, N)]).values.to(torch.int32)
+    ids = torch.cat([ids, torch.full((n - ids.numel(),), -1, dtype=torch.int32, device="cuda")])
+    idx = rdk.rdk_prepare_ids(ids, N)
+    y = torch.randn(rows, n, generator=g, device="cuda")
+    M = {"data": torch.rand(n, N, generator=g, device="cuda"), "layout": B.RDK_AFF_F32_ROWS, "ld": N}
+    w, S, _ = rdk.rdk_redistribute_exact(idx, y, M, rows, 1)
+    torch.cuda.synchronize()
+    q = torch.softmax(torch.where(ids >= 0, y.double(), torch.tensor(-float("inf"), device="cuda", dtype=torch.float64)), -1)
+    ref = q @ M["data"].double()
+    # q' carries a few rounding errors of its own (exponential, sum, quotient): 1e-6; the products add n of 2^-24
+    assert ((w.double() - ref).abs() <= (1e-6 + n * 2.0 ** -24) * ref).all()
+    assert ((S.double() - ref.sum(1)).abs() <= (1e-6 + (N + n) * 2.0 ** -24) * ref.sum(1)).all()
+
+
+@pytest.mark.parametrize("N,n,d,dtype,tau", [(257, 129, 20, "bf16", 0.1), (1030, 260, 100, "bf16", 0.05), (515, 64, 65, "bf16", 0.1),
+                                             (9000, 2400, 64, "f32", 0.1), (1001, 17, 33, "f32", 0.02)])
+def test_affinity_builds_at_tile_edges(N, n, d, dtype, tau):
+    """Ragged tiles on both routes, embedding dimensions whose rows are not whole 16-byte units, a zero embedding (equally near to
+    every token), ids outside the vocabulary, four columns and one a thread."""
+    rdk = _rdk()
+    B = rdk.binding
+    g = torch.Generator(device="cuda").manual_seed(N)
+    E = torch.randn(N, d, generator=g, device="cuda").to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+    ids = torch.sort(torch.randperm(N, generator=g, device="cuda")[:n]).values.to(torch.int32)
+    E[ids[1].long()] = 0
+    ids[2], ids[n - 1] = -1, N
+    M = rdk.rdk_build_affinity(E, ids, tau, B.RDK_AFF_BF16_COLS if dtype == "bf16" else B.RDK_AFF_F32_ROWS)
+    torch.cuda.synchronize()
+    ok = (ids >= 0) & (ids < N)
+    En = torch.nn.functional.normalize(E.double(), dim=1, eps=1e-12)
+    ref = torch.softmax(En[ids.clamp(0, N - 1).long()] @ En.T / tau, -1) * ok.unsqueeze(1)
+    got = M["data"][:, :n].T.double() if dtype == "bf16" else M["data"].double()
+    # the exponent (cos - 1) / tau log2 e carries rounding errors of 2^-24 of its size, d of them in the dot product, in units of
+    # 1 / tau; storing in bf16 adds half a unit in the last place, 2^-9
+    tol = 4 * (d ** 0.5 + 8) * 2.0 ** -24 / tau + (2.0 ** -8 if dtype == "bf16" else 0.0)
+    assert ((got - ref).abs() <= tol * ref).all()
+    assert torch.all(got[~ok] == 0)
+    if dtype == "bf16":
+        assert torch.all(M["data"][:, n:] == 0)
