@@ -327,7 +327,7 @@ def bench_workload(ctx: Ctx, name: str, steps: int, warmup: int, prior: bool, he
             B.rdk_sample_and_verify(index, B.RDK_MODE_PRECOMPUTED_W, sets[0]["target"], None, w_buf, sets[0]["uniforms"],
                                     cfg.batch, cfg.positions, kind, out=out_list[0], ws=ws)
         kernel_fn = contraction
-        launches_per_step = 2 + 2          # operand, contraction; row kernel, accepted length
+        launches_per_step = 2 + 1          # operand, contraction; cluster row kernel (counts the accepted length as well)
         kernels = "exact_operand_kernel + exact_tc_kernel (row sums in its epilogue)"
     elif prior:
         # Eq. rdk-taylor with one shared prior row (a static stand-in for the unknown target distribution)
@@ -338,8 +338,8 @@ def bench_workload(ctx: Ctx, name: str, steps: int, warmup: int, prior: bool, he
             B.rdk_sample_and_verify_prior(index, s["target"], shared_prior, s["drafter"], s["uniforms"],
                                           cfg.batch, cfg.positions, kind, out=out_list[i % nsets])
         kernel_fn = lambda i: step(i, outs_nolen)
-        launches_per_step = 2              # row kernel, accepted length
-        kernels = "rdk_row_kernel (shared prior)"
+        launches_per_step = 2              # cluster row kernel, accepted length
+        kernels = "rdk_cluster_kernel (shared prior)"
     else:
         route, why = B.rdk_sample_route(index, B.RDK_MODE_LINEAR, sets[0]["target"], sets[0]["drafter"], cfg.batch,
                                         cfg.positions, trials, ws, kind)

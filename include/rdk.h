@@ -78,7 +78,7 @@ typedef enum rdk_mode { RDK_MODE_LINEAR = 0, RDK_MODE_PRECOMPUTED_W = 1 } rdk_mo
  * instead of being left untouched.                                                                */
 #define RDK_FLAG_PAD_SEQUENCES 4
 
-/* Which kernel a call of the linear mode takes (see rdk_sample_route).                           */
+/* Whether a call of the linear mode can take the streaming kernels (see rdk_sample_route).       */
 typedef enum rdk_route { RDK_ROUTE_ROW_KERNEL = 0, RDK_ROUTE_STREAM_KERNEL = 1 } rdk_route;
 
 /* Physical layouts of the affinity matrix M (n rows i in I, N columns j in T).
@@ -161,10 +161,10 @@ int rdk_prepare_ids(const int32_t* kept_ids, int32_t n, int32_t N, void* kept_in
  *   M_out        device, layout / ld as in rdk_affinity (data member is ignored; M_out is used)
  *   ws           device workspace of rdk_build_affinity_workspace_bytes(N, n, d) bytes
  * Arithmetic: fp32 dot products and soft-max; the result is rounded to bf16 (nearest even) only
- * when it is stored in the bf16 layout.  bf16 embeddings (d >= 64, 16-byte aligned rows) going to the
- * bf16 layout take the tensor cores for the dot products (bf16 products are exact, accumulation in
- * fp32), in chunks of 2048 kept rows through an fp32 scratch [N, 2048] inside the workspace; every
- * other combination uses fp32 FMAs.  Both routes compute the same quantity.  If a bounded wait
+ * when it is stored in the bf16 layout.  bf16 embeddings going to the bf16 layout take the tensor cores
+ * for the dot products (bf16 products are exact, accumulation in fp32), computed once for the sums and
+ * once for the values; every other combination uses fp32 FMAs, likewise.  Both routes compute the same
+ * quantity.  If a bounded wait
  * inside the tensor-core kernel expires (the call has no status word), element [0, 0] of M_out is
  * set to NaN.
  * ------------------------------------------------------------------------------------------- */
@@ -255,8 +255,11 @@ int rdk_redistribute_linear(const rdk_problem* problem, const void* target, cons
  * the draft token, tests it and draws the replacement from those records, reading again only the
  * few 1024-token chunks the draws fall into.  There the quotient 1 / (N + p_j) is expanded in
  * x = p_j / N <= 2^-12 and terms of relative size x^2 (below 2^-24) are dropped.  Every other
- * problem takes the one-CTA-per-row kernel (three sweeps over the row, exact division), which is
- * several times slower; rdk_sample_route tells which one a call would take and why.  Both
+ * problem, and one of few rows, takes the cluster kernel: a thread-block cluster of up to 16 CTAs holds the
+ * row in its shared memory and goes from the logits to the draws in one launch (any alignment, any order of the ids,
+ * any N whose row fits; exact division below N = 4096).  The one-CTA-per-row kernel (three sweeps over the row,
+ * exact division), several times slower, serves what remains and RDK_FLAG_ROW_KERNEL;
+ * rdk_sample_route tells whether the streaming kernels can serve and why not.  Both
  * streaming kernels are launched with programmatic stream serialisation: each may set itself up
  * while the previous kernel of the stream drains, but reads none of its inputs and touches nothing
  * of the workspace before that kernel is complete, so inputs written by the kernel queued just
@@ -271,13 +274,14 @@ int rdk_sample_and_verify(const rdk_problem* problem, int32_t mode, const void* 
                           void* ws, size_t ws_bytes, void* stream);
 
 /* ---------------------------------------------------------------------------------------------
- * rdk_sample_route -- host-only query (no CUDA call, nothing launched): which kernel
- * rdk_sample_and_verify would run Algorithm 4 steps 4-8 with for these arguments.  It sees what
+ * rdk_sample_route -- host-only query (no CUDA call, nothing launched): whether rdk_sample_and_verify
+ * can run Algorithm 4 steps 4-8 for these arguments with the streaming kernels (few rows are given to
+ * the cluster kernel all the same, where that is faster).  It sees what
  * rdk_stream_geometry cannot: the flags, alignment and strides of the rows, the workspace, and
  * whether the kept ids of problem->kept_index were ascending and valid when the index was built.
  *   why   host const char**, may be NULL: receives a static string naming the first reason the
  *         streaming kernel cannot serve ("" when it can)
- * Returns RDK_ROUTE_STREAM_KERNEL or RDK_ROUTE_ROW_KERNEL, or -(rdk_status) for a bad problem.
+ * Returns RDK_ROUTE_STREAM_KERNEL or RDK_ROUTE_ROW_KERNEL (a row held by one cluster or one CTA), or -(rdk_status) for a bad problem.
  * ------------------------------------------------------------------------------------------- */
 int rdk_sample_route(const rdk_problem* problem, int32_t mode, const void* target,
                      const void* drafter, int32_t trials, const void* ws, size_t ws_bytes,
@@ -303,7 +307,8 @@ void rdk_test_set_spin_limit(uint32_t limit);
  *   prior             device [rows, N] logits of the same dtype as the target, or one shared row
  *   prior_row_stride  elements between prior rows; 0 means one row shared by all rows
  * Everything else as in rdk_sample_and_verify (mode RDK_MODE_LINEAR) and rdk_redistribute_linear.
- * These calls take the one-CTA-per-row kernel and need no workspace.
+ * These calls take the cluster kernel (the one-CTA-per-row kernel where a row does not fit a cluster) and need no
+ * workspace.
  * ------------------------------------------------------------------------------------------- */
 int rdk_sample_and_verify_prior(const rdk_problem* problem, const void* target, const void* prior,
                                 int64_t prior_row_stride, const void* drafter, const float* uniforms,
@@ -315,7 +320,7 @@ int rdk_redistribute_linear_prior(const rdk_problem* problem, const void* target
 /* ---------------------------------------------------------------------------------------------
  * rdk_stream_geometry -- host-only query (no CUDA call): how the streaming kernels of the linear
  * mode would lay a problem of N target tokens and n kept ids out, or supported = 0 when such a
- * problem takes the one-CTA-per-row kernel (N < 4096, or shapes beyond shared memory; unsorted
+ * problem takes another kernel (N < 4096, or shapes beyond shared memory; unsorted
  * or invalid kept ids and unaligned rows also do, but are not known here).  A row is shared by
  * ctas_per_row CTAs of warps_per_cta streaming warps, each owning segment_tokens consecutive
  * tokens (Eq. "rdk-taylor" is evaluated per segment; ctas_per_row * warps_per_cta segments cover
