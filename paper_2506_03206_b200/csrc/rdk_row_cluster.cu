@@ -920,7 +920,10 @@ static bool plan_cluster(int N, int rows, int trials, size_t es, int variant, bo
     // about eight warps of equally many 256-position chunks each: more warps mean more per-warp overhead, fewer do not
     // hide each other's latencies (50257 tokens x 160 rows: 8 warps 29 us, 12 35, 16 46)
     const int chunks = (int)((positions + C * 256 - 1) / (C * 256));
-    const int per_warp = chunks <= 8 ? 1 : (chunks + 7) / 8;
+    // (sixteen, and shorter segments, where the CTAs are few and several draws a row keep the warps busy: 32 rows of 32k with four
+    // trials 16.6 -> 14.1 us, one trial no gain)
+    const int warps = trials >= 3 && (long long)rows * C < 4 * 148 ? kCluMaxWarps : 8;
+    const int per_warp = (chunks + warps - 1) / warps;
     const int nw = (chunks + per_warp - 1) / per_warp;
     s.C = C; s.nw = nw < 4 ? 4 : nw;
     // segments of one chunk and several draws a row: a warp for each draw, also where there is nothing to sweep for it
