@@ -920,9 +920,10 @@ static bool plan_cluster(int N, int rows, int trials, size_t es, int variant, bo
     // about eight warps of equally many 256-position chunks each: more warps mean more per-warp overhead, fewer do not
     // hide each other's latencies (50257 tokens x 160 rows: 8 warps 29 us, 12 35, 16 46)
     const int chunks = (int)((positions + C * 256 - 1) / (C * 256));
-    // (sixteen, and shorter segments, where the CTAs are few and several draws a row keep the warps busy: 32 rows of 32k with four
-    // trials 16.6 -> 14.1 us, one trial no gain)
-    const int warps = trials >= 3 && (long long)rows * C < 4 * 148 ? kCluMaxWarps : 8;
+    // (sixteen, and shorter segments, where several draws a row keep the warps busy -- 32 rows of 32k with four trials 16.6 ->
+    // 14.1 us, 1500 rows of 8k with eight 107 -> 84 -- and where the CTAs are fewer than two an SM and not many share a row:
+    // 100 rows of 3000 10.4 -> 9.0 us, 4 rows of 8k 7.7 -> 7.2, but 5 rows of 128k on 16 CTAs each 8.9 -> 9.3)
+    const int warps = trials >= 3 || ((long long)rows * C < 2 * 148 && C < kCluMaxCtas) ? kCluMaxWarps : 8;
     const int per_warp = (chunks + warps - 1) / warps;
     const int nw = (chunks + per_warp - 1) / per_warp;
     s.C = C; s.nw = nw < 4 ? 4 : nw;
