@@ -9,10 +9,15 @@
 // (2 x 42 us for 32768 x 8192 x 128) than a round trip of fp32 through HBM.  One kernel runs twice over tiles of
 // 128 x 256 dot products, accumulated in tensor memory (two accumulators, so that one is filled while the other is
 // read back):
-//   kAffSums  : rows = kept ids, columns = tokens.  A thread owns a kept id and adds up its exponentials over the
-//               tokens of a work item; a small kernel adds the items' parts in a fixed order.
-//   kAffWrite : rows = tokens, columns = kept ids.  exp(...) / Z_i as one exponential of (cos - 1) / tau - log Z_i,
-//               rounded to bf16, staged in swizzled shared memory and stored by TMA (128-byte rows).
+//   kAffSums  : rows = kept ids, columns = tokens.  A thread owns a kept id and adds up its exponentials over blocks of
+//               64 tokens; a small kernel adds the blocks in order.
+//   kAffWrite : rows = tokens, columns = kept ids.  The same exponential times 1 / Z_i, rounded to bf16, staged in
+//               swizzled shared memory and stored by TMA (128-byte rows).
+// Both evaluate 2^((G x - 1) scale), x the product of the inverse norms, in the same order of operations, so an entry
+// and its share of Z_i carry the same rounding error: where one token has all the weight the entry is 1 however small
+// tau is.  (As one exponential of a scaled G less log2 Z the two differ by the rounding of a number of size scale, 1e-6
+// of the entry at tau = 0.1, 5e-3 at 1e-5; some ten of 32064 diagonal entries, the heaviest of a row, then land on
+// another bf16 number, which moves draws.)
 // Both are bound by the special-function unit (one exponential per element and pass: 2 x 60 us at 16 per clock and SM)
 // and by the write of the matrix (537 MB: 82 us).  The chain that this replaces, with an fp32 scratch between the GEMM
 // and three streaming passes, took 1490 us for that size.
@@ -34,7 +39,12 @@ constexpr int kAffStoreBuffers = 16;
 constexpr int kAffStoreBytes = 32 * 128;                 // a warp's 32 rows x 64 bf16
 constexpr int kAffSmem = kAffStages * kAffStage + kAffStoreBuffers * kAffStoreBytes + 1024;
 constexpr int kAffSpan = 4;                              // column tiles per work item of kAffSums
+constexpr int kAffBlock = 64;                            // tokens summed one after the other: an epilogue warp's columns in kAffSums
+static_assert(4 * kAffN / kAffSumWarps == kAffBlock, "a warp of kAffSums leaves one sum per tile");
 constexpr uint32_t kAffIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kAffN >> 3) << 17) | ((uint32_t)(kAffM >> 4) << 24);
+
+constexpr float kAffZeroInv = 1e12f;                     // inverse norm of a zero embedding
+constexpr float kAffTinySum = 0x1p-100f;                 // exponentials this small are rounded, or flushed to zero
 
 enum { kAffSums = 0, kAffWrite = 1 };
 
@@ -44,9 +54,9 @@ struct AffParams {
     int cols;                          // columns in all
     const float* row_inv;              // 1 / |e| of the rows, zero-padded to whole tiles
     const float* col_inv;              // 1 / |e| of the columns, zero-padded to whole tiles
-    const float* col_off;              // kAffWrite: exponent offset -1 / tau - log2 Z of every column (-inf: weight 0)
+    const float* col_z;                // kAffWrite: 1 / Z of every column (0: no weight)
     float scale;                       // log2(e) / tau
-    float* part;                       // kAffSums: [kAffSumWarps / 4 * tiles_n][row tiles * 128]
+    float* part;                       // kAffSums: [blocks of kAffBlock tokens][row tiles * 128]
     int32_t* status;
 };
 
@@ -150,12 +160,16 @@ aff_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__
         for (int item = blockIdx.x; item < P.num_items && ok; item += gridDim.x) {
             const int tm = item / P.tiles_n, tn0 = (item % P.tiles_n) * kSpan;
             const int row = tm * kAffM + quarter * 32 + lane;
-            const float2 rs = splat(__ldg(P.row_inv + row) * P.scale);
-            float2 sum_a = splat(0.f), sum_b = splat(0.f);
+            const float2 ri = splat(__ldg(P.row_inv + row)), sc = splat(P.scale), neg = splat(-1.f);
+            // 2^((G x - 1) scale) of two columns
+            auto weight2 = [&](uint32_t g0, uint32_t g1, float c0, float c1) -> float2 {
+                return ex2_2(fmul2(ffma2(make_float2(__uint_as_float(g0), __uint_as_float(g1)), fmul2(make_float2(c0, c1), ri), neg), sc));
+            };
             for (int tn = tn0; tn < min(tn0 + kSpan, col_tiles); ++tn) {
                 const int c0 = tn * kAffN + share * kCols;
                 if (!tc_wait(&acc_full[acc], acc_phase, abort)) { ok = false; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                float sum = 0.f;
                 uint32_t v[2][32];
                 tmem_ld32(taddr0 + (uint32_t)(acc * kAffN), v[0]);
 #pragma unroll
@@ -171,12 +185,10 @@ aff_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__
                     const int col = c0 + c * 32;
                     const float4* ci = reinterpret_cast<const float4*>(P.col_inv + col);
                     if (MODE == kAffSums) {
-                        const float2 off = splat(-P.scale);
 #pragma unroll
                         for (int q = 0; q < 8; ++q) {
                             const float4 k4 = __ldg(ci + q);
-                            float2 e0 = ex2_2(ffma2(make_float2(__uint_as_float(x[4 * q]), __uint_as_float(x[4 * q + 1])), fmul2(make_float2(k4.x, k4.y), rs), off));
-                            float2 e1 = ex2_2(ffma2(make_float2(__uint_as_float(x[4 * q + 2]), __uint_as_float(x[4 * q + 3])), fmul2(make_float2(k4.z, k4.w), rs), off));
+                            float2 e0 = weight2(x[4 * q], x[4 * q + 1], k4.x, k4.y), e1 = weight2(x[4 * q + 2], x[4 * q + 3], k4.z, k4.w);
                             if (col + 32 > P.cols) {                 // tokens beyond the vocabulary have no weight
                                 const int left = P.cols - col - 4 * q;
                                 if (left < 1) e0.x = 0.f;
@@ -184,10 +196,10 @@ aff_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__
                                 if (left < 3) e1.x = 0.f;
                                 if (left < 4) e1.y = 0.f;
                             }
-                            sum_a = fadd2(sum_a, e0); sum_b = fadd2(sum_b, e1);
+                            sum += e0.x; sum += e0.y; sum += e1.x; sum += e1.y;
                         }
                     } else {
-                        const float4* co = reinterpret_cast<const float4*>(P.col_off + col);
+                        const float4* cz = reinterpret_cast<const float4*>(P.col_z + col);
                         if ((c & 1) == 0) {                          // the staging buffer's last store has been read
                             if (lane == 0) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kBufs - 1) : "memory");
                             __syncwarp();
@@ -198,10 +210,10 @@ aff_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__
                             uint32_t w[4];
 #pragma unroll
                             for (int h = 0; h < 2; ++h) {
-                                const float4 k4 = __ldg(ci + q + h), o4 = __ldg(co + q + h);
+                                const float4 k4 = __ldg(ci + q + h), z4 = __ldg(cz + q + h);
                                 const int i = 4 * (q + h);
-                                const float2 e0 = ex2_2(ffma2(make_float2(__uint_as_float(x[i]), __uint_as_float(x[i + 1])), fmul2(make_float2(k4.x, k4.y), rs), make_float2(o4.x, o4.y)));
-                                const float2 e1 = ex2_2(ffma2(make_float2(__uint_as_float(x[i + 2]), __uint_as_float(x[i + 3])), fmul2(make_float2(k4.z, k4.w), rs), make_float2(o4.z, o4.w)));
+                                const float2 e0 = fmul2(weight2(x[i], x[i + 1], k4.x, k4.y), make_float2(z4.x, z4.y));
+                                const float2 e1 = fmul2(weight2(x[i + 2], x[i + 3], k4.z, k4.w), make_float2(z4.z, z4.w));
                                 asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w[2 * h]) : "f"(e0.y), "f"(e0.x));
                                 asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w[2 * h + 1]) : "f"(e1.y), "f"(e1.x));
                             }
@@ -223,10 +235,9 @@ aff_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__
                         }
                     }
                 }
+                if (MODE == kAffSums) P.part[(long long)(c0 / kAffBlock) * (P.tiles_m * kAffM) + row] = sum;
                 if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
             }
-            if (MODE == kAffSums && ok)
-                P.part[(long long)((item % P.tiles_n) * 4 + share) * (P.tiles_m * kAffM) + row] = (sum_a.x + sum_a.y) + (sum_b.x + sum_b.y);
         }
         if (MODE == kAffWrite && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     }
@@ -262,71 +273,77 @@ aff_rows_kernel(const __nv_bfloat16* __restrict__ E, long long stride, const int
     __nv_bfloat16* copy = kept ? (i < n ? Ek + (long long)i * dpad : nullptr) : (Epad && i < N ? Epad + (long long)i * dpad : nullptr);
     float ss = 0.f;
     const __nv_bfloat16* row = E + (long long)max(t, 0) * stride;
-    if (vec) {                            // 16-byte aligned rows of a multiple of 8 elements
-        for (int k = lane * 8; k < d; k += 256) {
-            const uint4 q = t >= 0 ? __ldg(reinterpret_cast<const uint4*>(row + k)) : make_uint4(0u, 0u, 0u, 0u);
-            const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-            for (int h = 0; h < 4; ++h) { const float a = bf16_lo(w[h]), b = bf16_hi(w[h]); ss = fmaf(a, a, fmaf(b, b, ss)); }
-            if (copy) *reinterpret_cast<uint4*>(copy + k) = q;
-        }
-    } else {
-        for (int k = lane; k < dpad; k += 32) {
-            const __nv_bfloat16 q = t >= 0 && k < d ? row[k] : __float2bfloat16_rn(0.f);
-            const float a = __bfloat162float(q);
-            ss = fmaf(a, a, ss);
-            if (copy) copy[k] = q;
-        }
+    for (int k = lane; k < d; k += 32) { const float v = t >= 0 ? __bfloat162float(row[k]) : 0.f; ss = fmaf(v, v, ss); }
+    if (copy && vec) {                    // 16-byte aligned rows of a multiple of 8 elements
+        for (int k = lane * 8; k < d; k += 256) *reinterpret_cast<uint4*>(copy + k) = t >= 0 ? __ldg(reinterpret_cast<const uint4*>(row + k)) : make_uint4(0u, 0u, 0u, 0u);
+    } else if (copy) {
+        for (int k = lane; k < dpad; k += 32) copy[k] = t >= 0 && k < d ? row[k] : __float2bfloat16_rn(0.f);
     }
     ss = warp_sum(ss);
     if (lane == 0) (kept ? invk : inv)[i] = t >= 0 ? 1.f / fmaxf(sqrtf(ss), 1e-12f) : 0.f;
 }
 
-// off[i] = -scale - log2(sum of the parts of i, in order); -inf where the kept id has no token.  One warp per 32 ids and
-// eight warps share their parts.
+// z[i] = 1 / Z_i, the blocks' sums added in order; 0 where the kept id has no token, and where a zero embedding (equally
+// near to every token) leaves sums too small to count.  32 ids to a CTA: its warps fetch the sums of 64 blocks at a time into
+// shared memory, one of them adds them up while the next are on their way.
 __global__ void __launch_bounds__(256)
-aff_offset_kernel(const float* __restrict__ part, const float* __restrict__ invk, float* __restrict__ off, int parts, int npad, int N, float scale) {
-    __shared__ float s[8][32];
+aff_norm_kernel(const float* __restrict__ part, const float* __restrict__ invk, float* __restrict__ z, int blocks, int npad) {
+    __shared__ float tile[2][64][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    float a = 0.f;
-#pragma unroll 4
-    for (int p = warp; p < parts; p += 8) a += part[(long long)p * npad + i];
-    s[warp][lane] = a;
-    __syncthreads();
+    float v[8], s = 0.f;
+    auto fetch = [&](int b0) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = b0 + warp * 8 + k < blocks ? part[(long long)(b0 + warp * 8 + k) * npad + i] : 0.f;
+    };
+    fetch(0);
+    for (int b0 = 0, buf = 0; b0 < blocks; b0 += 64, buf ^= 1) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) tile[buf][warp * 8 + k][lane] = v[k];
+        fetch(b0 + 64);
+        __syncthreads();                  // (the tile before this one has been added up)
+        if (warp == 0) {
+#pragma unroll 16
+            for (int k = 0; k < 64; ++k) s += tile[buf][k][lane];
+        }
+    }
     if (warp == 0) {
-        for (int w = 1; w < 8; ++w) a += s[w][lane];
-        // (a zero embedding is equally near to every token: exp(0 - 1 / tau) may be too small to count)
         const float ik = invk[i];
-        off[i] = ik > 0.f ? (ik < 1e12f ? -scale - log2f(a) : -log2f((float)N)) : -INFINITY;
+        z[i] = ik > 0.f && !(ik >= kAffZeroInv && s < kAffTinySum) ? 1.f / s : 0.f;
     }
 }
 
-// a wait inside the tensor-core kernel ran out: the matrix is incomplete, make that impossible to miss
-__global__ void aff_poison_kernel(const int32_t* status, __nv_bfloat16* Mt) {
+// Last: the columns of zero embeddings whose sums were too small to count, 1 / N each (a warp to a kept id; rare).  And if a
+// wait inside the tensor-core kernel ran out, the matrix is incomplete: make that impossible to miss.
+__global__ void __launch_bounds__(256)
+aff_finish_kernel(const int32_t* status, const float* __restrict__ invk, const float* __restrict__ z, __nv_bfloat16* Mt, long long ld, int n, int N) {
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (*status != 0) Mt[0] = __float2bfloat16_rn(NAN);
+    if (i < n && invk[i] >= kAffZeroInv && z[i] == 0.f)
+        for (int j = lane; j < N; j += 32) Mt[(long long)j * ld + i] = __float2bfloat16_rn(1.f / (float)N);
+    __syncwarp();
+    if (i == 0 && lane == 0 && *status != 0) Mt[0] = __float2bfloat16_rn(NAN);
 }
 
 // ------------------------------------------------------------------------------------------------
 // host side
 // ------------------------------------------------------------------------------------------------
-// workspace: inv[Npad] | invk[npad] | off[npad] | status | Ek[n, dpad] bf16 | part[4 spans, npad] | Epad[N, dpad] bf16
-struct AffTcLayout { size_t inv, invk, off, status, Ek, part, Epad, total; int Npad, npad, dpad, spans; };
+// workspace: inv[Npad] | invk[npad] | z[npad] | status | Ek[n, dpad] bf16 | part[blocks, npad] | Epad[N, dpad] bf16
+struct AffTcLayout { size_t inv, invk, z, status, Ek, part, Epad, total; int Npad, npad, dpad, blocks; };
 static AffTcLayout aff_tc_layout(int N, int n, int d) {
     AffTcLayout L;
     L.Npad = (N + kAffN - 1) / kAffN * kAffN;
     L.npad = (n + kAffN - 1) / kAffN * kAffN;
     L.dpad = (d + 7) & ~7;
-    L.spans = (L.Npad / kAffN + kAffSpan - 1) / kAffSpan;
+    L.blocks = L.Npad / kAffBlock;
     size_t o = 0;
     L.inv = o;    o += idx_align((size_t)L.Npad * sizeof(float));
     L.invk = o;   o += idx_align((size_t)L.npad * sizeof(float));
-    L.off = o;    o += idx_align((size_t)L.npad * sizeof(float));
+    L.z = o;      o += idx_align((size_t)L.npad * sizeof(float));
     L.status = o; o += idx_align(sizeof(int32_t));
     L.Ek = o;     o += idx_align((size_t)n * L.dpad * sizeof(__nv_bfloat16));
-    L.part = o;   o += idx_align((size_t)4 * L.spans * L.npad * sizeof(float));
+    L.part = o;   o += idx_align((size_t)L.blocks * L.npad * sizeof(float));
     L.Epad = o;   o += idx_align((size_t)N * L.dpad * sizeof(__nv_bfloat16));
     L.total = o;
     return L;
@@ -360,7 +377,7 @@ int build_affinity_tc(const __nv_bfloat16* E, int d, long long estride, const in
     unsigned char* base = static_cast<unsigned char*>(ws);
     float* inv = reinterpret_cast<float*>(base + L.inv);
     float* invk = reinterpret_cast<float*>(base + L.invk);
-    float* off = reinterpret_cast<float*>(base + L.off);
+    float* z = reinterpret_cast<float*>(base + L.z);
     int32_t* status = reinterpret_cast<int32_t*>(base + L.status);
     __nv_bfloat16* Ek = reinterpret_cast<__nv_bfloat16*>(base + L.Ek);
     float* part = reinterpret_cast<float*>(base + L.part);
@@ -388,20 +405,20 @@ int build_affinity_tc(const __nv_bfloat16* E, int d, long long estride, const in
     AffParams P;
     P.N = N; P.n = n; P.num_kb = (d + kAffK - 1) / kAffK; P.scale = scale; P.status = status; P.part = part;
     // sums: rows = kept ids, columns = tokens
-    P.tiles_m = L.npad / kAffM; P.tiles_n = L.spans; P.cols = N;
-    P.row_inv = invk; P.col_inv = inv; P.col_off = nullptr;
+    P.tiles_m = L.npad / kAffM; P.tiles_n = (L.Npad / kAffN + kAffSpan - 1) / kAffSpan; P.cols = N;
+    P.row_inv = invk; P.col_inv = inv; P.col_z = nullptr;
     const long long items = (long long)P.tiles_m * P.tiles_n;
     const long long items_w = (long long)(L.Npad / kAffM) * (L.npad / kAffN);
     if (items > 0x7fffffffLL || items_w > 0x7fffffffLL) { set_error("rdk_build_affinity: too many tiles"); return RDK_ERR_UNSUPPORTED; }
     P.num_items = (int)items;
     RDK_CUDA(launch_pdl(aff_tc_kernel<kAffSums>, (unsigned)(items < sms ? items : sms), (unsigned)aff_threads(kAffSums), (size_t)kAffSmem, s, keptA, tokB, out, P));
-    RDK_CUDA(launch_pdl(aff_offset_kernel, (unsigned)(L.npad / 32), 256u, 0, s, (const float*)part, (const float*)invk, off, 4 * L.spans, L.npad, N, scale));
+    RDK_CUDA(launch_pdl(aff_norm_kernel, (unsigned)(L.npad / 32), 256u, 0, s, (const float*)part, (const float*)invk, z, L.blocks, L.npad));
     // the matrix: rows = tokens, columns = kept ids
     P.tiles_m = L.Npad / kAffM; P.tiles_n = L.npad / kAffN; P.cols = n;
-    P.row_inv = inv; P.col_inv = invk; P.col_off = off;
+    P.row_inv = inv; P.col_inv = invk; P.col_z = z;
     P.num_items = (int)items_w;
     RDK_CUDA(launch_pdl(aff_tc_kernel<kAffWrite>, (unsigned)(items_w < sms ? items_w : sms), (unsigned)aff_threads(kAffWrite), (size_t)kAffSmem, s, tokA, keptB, out, P));
-    RDK_CUDA(launch_pdl(aff_poison_kernel, 1u, 1u, 0, s, (const int32_t*)status, Mt));
+    RDK_CUDA(launch_pdl(aff_finish_kernel, (unsigned)((n + wpb - 1) / wpb), 256u, 0, s, (const int32_t*)status, (const float*)invk, (const float*)z, Mt, ld, n, N));
     return RDK_OK;
 }
 

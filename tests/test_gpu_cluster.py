@@ -205,3 +205,22 @@ def test_affinity_builds_at_tile_edges(N, n, d, dtype, tau):
     assert torch.all(got[~ok] == 0)
     if dtype == "bf16":
         assert torch.all(M["data"][:, n:] == 0)
+
+
+@pytest.mark.parametrize("N,n,d", [(3000, 700, 64), (1111, 300, 200)])
+def test_affinity_of_a_small_temperature_is_the_identity(N, n, d):
+    """At tau = 1e-5 every other token is thousands of units of the exponent away, so a kept id's own entry is its whole sum and
+    has to be 1 to the last bit, whatever rounding errors the cosine carries (units of 1e-2 of the exponent here): entry and sum
+    are the same number.  Some 1e-2 off shows as another bf16 number, of which there is one every 2^-8 below 1.  A zero embedding
+    is equally near to every token."""
+    rdk = _rdk()
+    B = rdk.binding
+    g = torch.Generator(device="cuda").manual_seed(d)
+    E = torch.randn(N, d, generator=g, device="cuda").to(torch.bfloat16)
+    ids = torch.randperm(N, generator=g, device="cuda")[:n].to(torch.int32)
+    E[ids[7].long()] = 0
+    M = rdk.rdk_build_affinity(E, ids, 1e-5, B.RDK_AFF_BF16_COLS)["data"][:, :n].double()
+    ref = torch.zeros_like(M)
+    ref[ids.long(), torch.arange(n, device="cuda")] = 1.0
+    ref[:, 7] = torch.tensor(1.0 / N).to(torch.bfloat16).double()
+    assert torch.equal(M, ref)
