@@ -12,18 +12,21 @@ int launch_exact_tc(const __nv_bfloat16* A, long long lda, const __nv_bfloat16* 
                     float* w_out, float* S_out, int rows, int n, int N, int32_t* status_word, cudaStream_t s);
 
 constexpr int kOperandThreads = 512;
+constexpr int kOperandSums = 256;        // partial sums of a row: entries i, i + 256, ... one after the other
 
 // A[r, i] = q'_{kappa_i}: soft-max over the drafter entries whose id lies in the target vocabulary
 // (Eq. tli-drafter: drop the rest, renormalise), zero for dropped entries and for the padding
 // columns i in [n, lda); S[r] = 0 for the contraction to add to.
-// Two passes over the row in 16-byte vectors, the second out of L1/L2; the ids are looked at only where the index says
-// that some lie outside the vocabulary.  (Three passes with an element and an id at a time took 99 us for 320 rows of
-// 32064 entries, 10 times the memory time.)
+// The maximum and the result in passes of 16-byte vectors, all but the first out of L1/L2; the ids are looked at only where
+// the index says that some lie outside the vocabulary.  The sum is taken over 256 interleaved runs: its order decides on
+// which side of a bf16 boundary an entry falls (added up vector by vector, 30 to 500 of 10 million entries of q' change),
+// so it does not follow the width of the loads.  (Three passes with an element and an id at a time took 99 us for 320 rows
+// of 32064 entries, 10 times the memory time.)
 template <typename TY, typename TA, int KIND>
 __global__ void __launch_bounds__(kOperandThreads)
 exact_operand_kernel(const TY* __restrict__ drafter, long long dstride, const int32_t* __restrict__ header, const int32_t* __restrict__ ids,
                      int N, int n, TA* __restrict__ A, long long lda, float* __restrict__ S) {
-    __shared__ MS red[kOperandThreads / 32];
+    __shared__ float red[kOperandThreads / 32];
     const int row = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const TY* y = drafter + (long long)row * dstride;
     const bool vec = (reinterpret_cast<uintptr_t>(y) & 15u) == 0;
@@ -44,35 +47,42 @@ exact_operand_kernel(const TY* __restrict__ drafter, long long dstride, const in
             }
         }
     };
-    MS a{KIND == RDK_LOGITS ? -INFINITY : 0.f, 0.f, 0.f};
+    float m = -INFINITY;
+    if (KIND == RDK_LOGITS) {
 #pragma unroll 2
-    for (int i = tid * kVec; i < n; i += kOperandThreads * kVec) {
-        float v[kVec];
-        load_y(i, v);
-        if (KIND == RDK_LOGITS) {
-            float vmax = v[0];
+        for (int i = tid * kVec; i < n; i += kOperandThreads * kVec) {
+            float v[kVec];
+            load_y(i, v);
 #pragma unroll
-            for (int k = 1; k < kVec; ++k) vmax = fmaxf(vmax, v[k]);
-            if (vmax > a.m) { a.s *= ex2((a.m - vmax) * kLog2e); a.m = vmax; }
-            const float base = a.m > -INFINITY ? a.m : 0.f;
-#pragma unroll
-            for (int k = 0; k < kVec; ++k) a.s += ex2((v[k] - base) * kLog2e);
-        } else {
-#pragma unroll
-            for (int k = 0; k < kVec; ++k) a.s += v[k];
+            for (int k = 0; k < kVec; ++k) m = fmaxf(m, v[k]);
         }
+        m = warp_max(m);
+        if (lane == 0) red[warp] = m;
+        __syncthreads();
+        m = warp_max(red[lane & (kOperandThreads / 32 - 1)]);
+        __syncthreads();
     }
-    a = ms_warp(a);
-    if (lane == 0) red[warp] = a;
+    float s = 0.f;
+    if (tid < kOperandSums) {
+#pragma unroll 16
+        for (int i = tid; i < n; i += kOperandSums) {
+            const int id = all_valid ? 0 : __ldg(ids + i);
+            const float v = to_float<TY>(y[i]);
+            if (id >= 0 && id < N) s += KIND == RDK_LOGITS ? ex2((v - m) * kLog2e) : v;
+        }
+        s = warp_sum(s);
+        if (lane == 0) red[warp] = s;
+    }
     __syncthreads();
-    a = ms_warp(lane < kOperandThreads / 32 ? red[lane] : MS{-INFINITY, 0.f, 0.f});
-    const float inv = 1.f / a.s;
+    s = 0.f;
+    for (int k = 0; k < kOperandSums / 32; ++k) s += red[k];
+    const float inv = 1.f / s;
     TA* out = A + (long long)row * lda;
     for (int i = tid * kVec; i < lda; i += kOperandThreads * kVec) {
         float v[kVec];
         load_y(i, v);
 #pragma unroll
-        for (int k = 0; k < kVec; ++k) v[k] = (KIND == RDK_LOGITS ? ex2((v[k] - a.m) * kLog2e) : v[k]) * inv;
+        for (int k = 0; k < kVec; ++k) v[k] = (KIND == RDK_LOGITS ? ex2((v[k] - m) * kLog2e) : v[k]) * inv;
         if (sizeof(TA) == 2) {                   // lda is a multiple of 64 and the rows are 16-byte aligned
             uint32_t w[4];
 #pragma unroll

@@ -272,3 +272,37 @@ def test_config5_full_size_sampled_outputs():
     t = PU.compare_sampling(inp, out, rows, "given", w_given=w_rows.double().numpy())
     print("C5", t.summary())
     t.assert_ok(max_ambiguous_frac=0.2)
+
+
+@pytest.mark.parametrize("n,dropped", [(1, False), (255, False), (257, True), (5000, False), (8197, True)])
+def test_drafter_sum_has_a_fixed_order(n, dropped):
+    """q' of a probability drafter is a quotient of two fp32 numbers, so it can be had to the last bit: the row's sum is taken over
+    256 interleaved runs, the runs of 32 neighbours are added in pairs and these eight one after the other.  With the identity as
+    affinity the contraction returns it unchanged."""
+    rdk = _rdk()
+    B = rdk.binding
+    N, rows = n + 3, 3
+    g = torch.Generator().manual_seed(n)
+    q = torch.rand(rows, n, generator=g) ** 4
+    ids = torch.arange(n, dtype=torch.int32)
+    if dropped:
+        ids[5], ids[n - 2] = -1, N
+    valid = ((ids >= 0) & (ids < N)).numpy()
+    M = torch.zeros(n, N)
+    M[torch.arange(n)[valid], ids[valid].long()] = 1.0
+    idx = rdk.rdk_prepare_ids(ids.cuda(), N)
+    w, _, _ = rdk.rdk_redistribute_exact(idx, q.cuda(), {"data": M.cuda(), "layout": B.RDK_AFF_F32_ROWS, "ld": N}, rows, 1, B.RDK_PROBS)
+    v = np.zeros((rows, (n + 255) // 256 * 256), dtype=np.float32)
+    v[:, :n] = np.where(valid, q.numpy(), np.float32(0))
+    run = np.zeros((rows, 256), dtype=np.float32)
+    for part in v.reshape(rows, -1, 256).transpose(1, 0, 2):
+        run = run + part
+    run = run.reshape(rows, 8, 32)
+    for o in (16, 8, 4, 2, 1):
+        run = run + run[:, :, np.arange(32) ^ o]
+    total = np.zeros(rows, dtype=np.float32)
+    for k in range(8):
+        total = total + run[:, k, 0]
+    want = np.zeros((rows, N), dtype=np.float32)
+    want[:, ids.numpy()[valid]] = (q.numpy() * (np.float32(1) / total)[:, None])[:, valid]
+    assert np.array_equal(w.cpu().numpy(), want)
