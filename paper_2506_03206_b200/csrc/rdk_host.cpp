@@ -95,18 +95,31 @@ void arity(Py_ssize_t got, Py_ssize_t want) {
     if (got != want) raise(PyExc_TypeError, "wrong number of arguments");
 }
 
-// the library's calls run without the interpreter lock: a launch may have to wait for room in the stream's queue
+// The library's calls run without the interpreter lock: a launch may have to wait for room in the stream's queue.  Only the
+// C call itself belongs in here: whatever may throw (a pointer of a tensor without storage, a stride, the current stream) is
+// worked out before, and the lock comes back on every way out.
+class Unlocked {
+public:
+    Unlocked() : state_(PyEval_SaveThread()) {}
+    ~Unlocked() { PyEval_RestoreThread(state_); }
+    Unlocked(const Unlocked&) = delete;
+    Unlocked& operator=(const Unlocked&) = delete;
+private:
+    PyThreadState* state_;
+};
 template <typename F> int unlocked(F f) {
-    PyThreadState* s = PyEval_SaveThread();
-    const int st = f();
-    PyEval_RestoreThread(s);
-    return st;
+    Unlocked lock;
+    return f();
 }
+template <typename T> T* pointer(const at::Tensor& t) { return static_cast<T*>(t.data_ptr()); }
 
 template <typename F> PyObject* guarded(F f) {
     try {
         return f();
     } catch (const Raised&) {
+        return nullptr;
+    } catch (const c10::IndexError& e) {
+        PyErr_SetString(PyExc_IndexError, e.what_without_backtrace());
         return nullptr;
     } catch (const std::exception& e) {
         PyErr_SetString(PyExc_RuntimeError, e.what());
@@ -127,12 +140,12 @@ PyObject* sample(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const rdk_outputs o = outputs(a[12]);
         const at::Tensor& ws = tensor(a[13], "ws");
         const int mode = (int)integer(a[3]);
-        return PyLong_FromLong(unlocked([&] {
-            return rdk_sample_and_verify(&pb, mode, target.data_ptr(), drafter ? drafter->data_ptr() : nullptr,
-                                         w ? static_cast<const float*>(w->data_ptr()) : nullptr, w ? w->stride(0) : 0,
-                                         static_cast<const float*>(u.data_ptr()), (int32_t)trials, &o, ws.data_ptr(),
-                                         (size_t)ws.numel(), stream());
-        }));
+        const void *z = pointer<void>(target), *y = drafter ? pointer<void>(*drafter) : nullptr;
+        const float *wp = w ? pointer<float>(*w) : nullptr, *up = pointer<float>(u);
+        const int64_t w_stride = w ? w->stride(0) : 0;
+        void *wsp = pointer<void>(ws), *s = stream();
+        const size_t ws_bytes = (size_t)ws.numel();
+        return PyLong_FromLong(unlocked([&] { return rdk_sample_and_verify(&pb, mode, z, y, wp, w_stride, up, (int32_t)trials, &o, wsp, ws_bytes, s); }));
     });
 }
 
@@ -158,10 +171,10 @@ PyObject* sample_prior(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const long long trials = per_row(u, (long long)pb.batch * pb.positions, false);
         const rdk_outputs o = outputs(a[10]);
         const long long stride = prior_stride(prior, a[4], target, pb.N);
-        return PyLong_FromLong(unlocked([&] {
-            return rdk_sample_and_verify_prior(&pb, target.data_ptr(), prior.data_ptr(), stride, drafter.data_ptr(),
-                                               static_cast<const float*>(u.data_ptr()), (int32_t)trials, &o, stream());
-        }));
+        const void *z = pointer<void>(target), *pr = pointer<void>(prior), *y = pointer<void>(drafter);
+        const float* up = pointer<float>(u);
+        void* s = stream();
+        return PyLong_FromLong(unlocked([&] { return rdk_sample_and_verify_prior(&pb, z, pr, stride, y, up, (int32_t)trials, &o, s); }));
     });
 }
 
@@ -177,10 +190,11 @@ PyObject* linear(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const at::Tensor qt = at::empty({rows, pb.N}, opt), theta = at::empty({rows}, opt), S = at::empty({rows}, opt);
         const at::Tensor* prior = a[4] == Py_None ? nullptr : &tensor(a[4], "prior");
         const long long stride = prior ? prior_stride(*prior, a[4], target, pb.N) : 0;
-        float *q = static_cast<float*>(qt.data_ptr()), *t = static_cast<float*>(theta.data_ptr()), *z = static_cast<float*>(S.data_ptr());
+        float *q = pointer<float>(qt), *th = pointer<float>(theta), *sum = pointer<float>(S);
+        const void *z = pointer<void>(target), *pr = prior ? pointer<void>(*prior) : nullptr, *y = pointer<void>(drafter);
+        void* s = stream();
         const int st = unlocked([&] {
-            return prior ? rdk_redistribute_linear_prior(&pb, target.data_ptr(), prior->data_ptr(), stride, drafter.data_ptr(), q, t, z, stream())
-                         : rdk_redistribute_linear(&pb, target.data_ptr(), drafter.data_ptr(), q, t, z, stream());
+            return prior ? rdk_redistribute_linear_prior(&pb, z, pr, stride, y, q, th, sum, s) : rdk_redistribute_linear(&pb, z, y, q, th, sum, s);
         });
         return Py_BuildValue("(iNNN)", st, THPVariable_Wrap(qt), THPVariable_Wrap(theta), THPVariable_Wrap(S));
     });
@@ -198,10 +212,11 @@ PyObject* exact(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const at::Tensor& ws = tensor(a[11], "ws");
         void* status = a[12] == Py_None ? nullptr : tensor(a[12], "status_word").data_ptr();
         const at::Tensor S = at::empty({(int64_t)pb.batch * pb.positions}, drafter.options().dtype(at::kFloat));
-        const int st = unlocked([&] {
-            return rdk_redistribute_exact(&pb, drafter.data_ptr(), &M, static_cast<float*>(w.data_ptr()), static_cast<float*>(S.data_ptr()),
-                                          ws.data_ptr(), (size_t)ws.numel(), static_cast<int32_t*>(status), stream());
-        });
+        const void* y = pointer<void>(drafter);
+        float *wp = pointer<float>(w), *sum = pointer<float>(S);
+        void *wsp = pointer<void>(ws), *s = stream();
+        const size_t ws_bytes = (size_t)ws.numel();
+        const int st = unlocked([&] { return rdk_redistribute_exact(&pb, y, &M, wp, sum, wsp, ws_bytes, static_cast<int32_t*>(status), s); });
         return Py_BuildValue("(iN)", st, THPVariable_Wrap(S));
     });
 }
@@ -220,12 +235,14 @@ PyObject* emit(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const auto opt = bonus.options().dtype(at::kInt);
         const at::Tensor seq = at::empty({pb.batch, trials, (int64_t)pb.positions + 1}, opt), len = at::empty({pb.batch, trials}, opt);
         const at::Tensor &draft = tensor(a[5], "draft_token"), &acc = tensor(a[6], "accepted"), &out = tensor(a[7], "out_token");
-        const int st = unlocked([&] {
-            return rdk_emit_sequences(&pb, bonus.data_ptr(), bonus.stride(0), static_cast<const float*>(u.data_ptr()), (int32_t)trials,
-                                      static_cast<const int32_t*>(draft.data_ptr()), static_cast<const uint8_t*>(acc.data_ptr()),
-                                      static_cast<const int32_t*>(out.data_ptr()), static_cast<int32_t*>(seq.data_ptr()),
-                                      static_cast<int32_t*>(len.data_ptr()), stream());
-        });
+        const void* z = pointer<void>(bonus);
+        const int64_t z_stride = bonus.stride(0);
+        const float* up = pointer<float>(u);
+        const int32_t *d = pointer<int32_t>(draft), *o = pointer<int32_t>(out);
+        const uint8_t* ap = pointer<uint8_t>(acc);
+        int32_t *sp = pointer<int32_t>(seq), *lp = pointer<int32_t>(len);
+        void* s = stream();
+        const int st = unlocked([&] { return rdk_emit_sequences(&pb, z, z_stride, up, (int32_t)trials, d, ap, o, sp, lp, s); });
         return Py_BuildValue("(iNN)", st, THPVariable_Wrap(seq), THPVariable_Wrap(len));
     });
 }

@@ -154,3 +154,39 @@ def test_stream_geometry_covers_the_vocabulary_and_fits_shared_memory(B):
     assert big["live_rows"] * (big["cached_slots_per_warp"] // 64) * 4 <= 128 and big["stages"] >= 3
     assert rdk.rdk_stream_geometry(1000, 10)["supported"] == 0              # small vocabularies take the row kernel
     assert rdk.rdk_stream_geometry(1 << 21, 1000)["supported"] == 0         # too large for shared memory
+
+
+def test_what_the_marshalling_cannot_take_raises():
+    """A 0-d tensor of weights (it has no row stride) and a machine without a CUDA stream: each is found out while the arguments are
+    taken apart, where it raises; several times over and from two threads, so that an interpreter lock that was not given back
+    would show.  In a process of its own, which a crash ends."""
+    code = """
+import threading, torch
+import paper_2506_03206_b200.binding as B
+h, buf = B.host(), torch.zeros(64, dtype=torch.uint8)
+z, y, u = torch.zeros(2, 8), torch.zeros(2, 4), torch.zeros(2, 1, 4)
+seen = []
+def call(f, kind):
+    try:
+        f()
+    except kind as e:
+        seen.append(type(e).__name__)
+def work():
+    for _ in range(3):
+        call(lambda: h.sample(buf, 8, 4, 1, z, None, torch.tensor(1.0), u, 2, 1, 0, 0, {}, buf), IndexError)
+        if not torch.cuda.is_available():
+            call(lambda: h.linear(buf, 8, 4, z, None, y, 2, 1, 0), RuntimeError)
+            call(lambda: h.sample(buf, 8, 4, 0, z, y, None, u, 2, 1, 0, 0, {}, buf), RuntimeError)
+            call(lambda: h.sample_prior(buf, 8, 4, z, z, y, u, 2, 1, 0, {}), RuntimeError)
+            call(lambda: h.exact(buf, 8, 4, y, z, 0, 8, 2, 1, 0, z, buf, None), RuntimeError)
+            call(lambda: h.emit(8, 2, 1, z, u, buf, buf, buf), RuntimeError)
+t = threading.Thread(target=work)
+t.start(); work(); t.join()
+assert len(seen) == (6 if torch.cuda.is_available() else 36), seen
+print("fine")
+"""
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    res = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
+    assert res.returncode == 0 and "fine" in res.stdout, (res.returncode, res.stderr[-2000:])
