@@ -16,7 +16,7 @@ constexpr int kOperandSums = 256;        // partial sums of a row: entries i, i 
 
 // A[r, i] = q'_{kappa_i}: soft-max over the drafter entries whose id lies in the target vocabulary
 // (Eq. tli-drafter: drop the rest, renormalise), zero for dropped entries and for the padding
-// columns i in [n, lda); S[r] = 0 for the contraction to add to.
+// columns i in [n, lda); S[r] = 0 for the contraction to add to (or to count in).
 // The maximum and the result in passes of 16-byte vectors, all but the first out of L1/L2; the ids are looked at only where
 // the index says that some lie outside the vocabulary.  The sum is taken over 256 interleaved runs: its order decides on
 // which side of a bf16 boundary an entry falls (added up vector by vector, 30 to 500 of 10 million entries of q' change),
@@ -96,11 +96,53 @@ exact_operand_kernel(const TY* __restrict__ drafter, long long dstride, const in
     if (tid == 0 && S) S[row] = 0.f;
 }
 
-// w[r, j] = sum_i A[r, i] M[i, j]  with fp32 FMAs (fp32 row layout of M; small problems), S[r] += the sums of w.
+// S[r] = sum_j w[r, j], by one warp: fp32 runs of 16 per lane, carried in fp64, the lanes added in a fixed order.  w is read
+// from L2, where other CTAs have just written it.
+__device__ __forceinline__ void warp_row_sum(const float* __restrict__ row, int N, float* S, int lane) {
+    double acc = 0.0;
+#pragma unroll 2
+    for (int j0 = lane; j0 < N; j0 += 32 * 16) {
+        float v[16], s = 0.f;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) v[k] = j0 + k * 32 < N ? __ldcg(row + j0 + k * 32) : 0.f;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) s += v[k];
+        acc += (double)s;
+    }
+    acc = warp_sum_d(acc);
+    if (lane == 0) *S = (float)acc;
+}
+// The same for long rows, a CTA each.
+constexpr int kSumThreads = 256;
+__global__ void __launch_bounds__(kSumThreads)
+row_sum_kernel(const float* __restrict__ w, int N, float* __restrict__ S) {
+    __shared__ double red[kSumThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31;
+    const float* row = w + (long long)blockIdx.x * N;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    double acc = 0.0;
+    for (int j0 = tid; j0 < N; j0 += kSumThreads * 16) {
+        float v[16], s = 0.f;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) v[k] = j0 + k * kSumThreads < N ? row[j0 + k * kSumThreads] : 0.f;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) s += v[k];
+        acc += (double)s;
+    }
+    acc = warp_sum_d(acc);
+    if (lane == 0) red[tid >> 5] = acc;
+    __syncthreads();
+    if (tid == 0) { double t = 0.0; for (int k = 0; k < kSumThreads / 32; ++k) t += red[k]; S[blockIdx.x] = (float)t; }
+}
+
+// w[r, j] = sum_i A[r, i] M[i, j]  with fp32 FMAs (fp32 row layout of M; small problems).  Where S is given, the CTA of a
+// row block that arrives last adds up its rows of w; until then the block's first S counts the arrivals (the operand kernel
+// has zeroed it).  Sums added as they come, by fp32 atomics, are not the same twice and three times as far off.
 // A CTA takes 8 rows x 32 VC columns; its warps share the contraction (warp w takes i = w, w + 8, ...) and add up in shared
 // memory.  With a thread for a column and all of the contraction, 4 x 1024 x 256 ran on 4 SMs with one load in flight:
 // 27 us.
-constexpr int kFmaRows = 8, kFmaWarps = 8, kFmaChunk = 256;
+constexpr int kFmaRows = 8, kFmaWarps = 8, kFmaChunk = 256, kFmaSumMax = 4096;
 template <int VC>
 __global__ void __launch_bounds__(kFmaWarps * 32)
 exact_fma_kernel(const float* __restrict__ A, long long lda, const float* __restrict__ M, long long ldm,
@@ -153,11 +195,19 @@ exact_fma_kernel(const float* __restrict__ A, long long lda, const float* __rest
         for (int k = 0; k < kFmaWarps; ++k) v += part[k][r][c];
         const bool in = r0 + r < rows && j0 + c < N;
         if (in) w[(long long)(r0 + r) * N + j0 + c] = v;
-        if (S) {
-            v = warp_sum(in ? v : 0.f);
-            if (lane == 0 && r0 + r < rows) atomicAdd(S + r0 + r, v);
-        }
     }
+    if (!S) return;
+    __shared__ bool last;
+    __syncthreads();
+    if (tid == 0) {                              // releases the whole CTA's w, and acquires that of those before it
+        unsigned before;
+        asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(before) : "l"(S + r0) : "memory");
+        last = before == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    static_assert(kFmaRows == kFmaWarps, "a warp to a row");
+    if (r0 + warp < rows) warp_row_sum(w + (long long)(r0 + warp) * N, N, S + r0 + warp, lane);
 }
 
 template <typename K, typename... A>
@@ -244,15 +294,18 @@ extern "C" int rdk_redistribute_exact(const rdk_problem* problem, const void* dr
     const int kind = problem->drafter_kind;
     if (bf) RDK_CUDA((f ? launch_operand<float, B> : launch_operand<B, B>)(drafter, dstride, v, N, n, kind, ws, lda, S_out, rows, s));
     else RDK_CUDA((f ? launch_operand<float, float> : launch_operand<B, float>)(drafter, dstride, v, N, n, kind, ws, lda, S_out, rows, s));
-    // either contraction also accumulates S (one atomic partial sum per row and warp or CTA)
-    if (bf)
+    if (bf)                                      // also accumulates S (one atomic partial sum per row and warp)
         return launch_exact_tc(static_cast<const B*>(ws), lda, static_cast<const B*>(M->data), M->ld, w_out, S_out, rows, n, N, status_word, s);
     // four columns a thread where that still fills the chip, M's rows are whole 16-byte units and a CTA's columns exist
     const float *A = static_cast<const float*>(ws), *Mf = static_cast<const float*>(M->data);
     const unsigned ry = (unsigned)((rows + kFmaRows - 1) / kFmaRows);
     const bool wide = N % 128 == 0 && M->ld % 4 == 0 && !(reinterpret_cast<uintptr_t>(Mf) & 15u) && (long long)(N / 128) * ry >= 296;
-    if (wide) RDK_CUDA(launch_pdl(exact_fma_kernel<4>, dim3((unsigned)(N / 128), ry), kFmaWarps * 32u, s, A, lda, Mf, (long long)M->ld, w_out, S_out, rows, n, N));
-    else RDK_CUDA(launch_pdl(exact_fma_kernel<1>, dim3((unsigned)((N + 31) / 32), ry), kFmaWarps * 32u, s, A, lda, Mf, (long long)M->ld, w_out, S_out, rows, n, N));
+    // S by a kernel of its own where one CTA's turn at eight long rows would take longer than that launch
+    const bool sum_after = S_out && N > kFmaSumMax;
+    float* S_in = sum_after ? nullptr : S_out;
+    if (wide) RDK_CUDA(launch_pdl(exact_fma_kernel<4>, dim3((unsigned)(N / 128), ry), kFmaWarps * 32u, s, A, lda, Mf, (long long)M->ld, w_out, S_in, rows, n, N));
+    else RDK_CUDA(launch_pdl(exact_fma_kernel<1>, dim3((unsigned)((N + 31) / 32), ry), kFmaWarps * 32u, s, A, lda, Mf, (long long)M->ld, w_out, S_in, rows, n, N));
+    if (sum_after) RDK_CUDA(launch_pdl(row_sum_kernel, dim3((unsigned)rows), (unsigned)kSumThreads, s, (const float*)w_out, N, S_out));
     return RDK_OK;
 }
 

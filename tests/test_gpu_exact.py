@@ -306,3 +306,24 @@ def test_drafter_sum_has_a_fixed_order(n, dropped):
     want = np.zeros((rows, N), dtype=np.float32)
     want[:, ids.numpy()[valid]] = (q.numpy() * (np.float32(1) / total)[:, None])[:, valid]
     assert np.array_equal(w.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("N,rows", [(31, 1), (1024, 4), (4096, 21), (4097, 9), (20000, 5)])
+def test_fp32_row_sums_are_repeatable(N, rows):
+    """S of the fp32 layout: runs of 16 fp32 additions carried in fp64, in a fixed order, so the same bits every time, and within 15
+    roundings of 2^-24 of the terms (16 with the result's own) of the sum of w."""
+    rdk = _rdk()
+    B = rdk.binding
+    n = 64
+    g = torch.Generator(device="cuda").manual_seed(N)
+    ids = torch.cat([torch.arange(min(n, N)), torch.full((max(0, n - N),), -1)]).to(torch.int32).cuda()
+    idx = rdk.rdk_prepare_ids(ids, N)
+    M = {"data": torch.rand(n, N, generator=g, device="cuda") ** 6, "layout": B.RDK_AFF_F32_ROWS, "ld": N}
+    y = torch.randn(rows, n, generator=g, device="cuda")
+    first = None
+    for _ in range(20):
+        w, S, _ = rdk.rdk_redistribute_exact(idx, y, M, rows, 1)
+        first = S.clone() if first is None else first
+        assert torch.equal(S, first)
+    ref = w.double().sum(1)
+    assert ((S.double() - ref).abs() <= 16 * 2.0 ** -24 * ref).all()
