@@ -27,7 +27,7 @@ __global__ void __launch_bounds__(kOperandThreads)
 exact_operand_kernel(const TY* __restrict__ drafter, long long dstride, const int32_t* __restrict__ header, const int32_t* __restrict__ ids,
                      int N, int n, TA* __restrict__ A, long long lda, float* __restrict__ S) {
     __shared__ float red[kOperandThreads / 32];
-    const int row = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int row = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, threads = blockDim.x;
     const TY* y = drafter + (long long)row * dstride;
     const bool vec = (reinterpret_cast<uintptr_t>(y) & 15u) == 0;
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -50,7 +50,7 @@ exact_operand_kernel(const TY* __restrict__ drafter, long long dstride, const in
     float m = -INFINITY;
     if (KIND == RDK_LOGITS) {
 #pragma unroll 2
-        for (int i = tid * kVec; i < n; i += kOperandThreads * kVec) {
+        for (int i = tid * kVec; i < n; i += threads * kVec) {
             float v[kVec];
             load_y(i, v);
 #pragma unroll
@@ -59,7 +59,7 @@ exact_operand_kernel(const TY* __restrict__ drafter, long long dstride, const in
         m = warp_max(m);
         if (lane == 0) red[warp] = m;
         __syncthreads();
-        m = warp_max(red[lane & (kOperandThreads / 32 - 1)]);
+        m = warp_max(red[lane & (threads / 32 - 1)]);
         __syncthreads();
     }
     float s = 0.f;
@@ -78,7 +78,7 @@ exact_operand_kernel(const TY* __restrict__ drafter, long long dstride, const in
     for (int k = 0; k < kOperandSums / 32; ++k) s += red[k];
     const float inv = 1.f / s;
     TA* out = A + (long long)row * lda;
-    for (int i = tid * kVec; i < lda; i += kOperandThreads * kVec) {
+    for (int i = tid * kVec; i < lda; i += threads * kVec) {
         float v[kVec];
         load_y(i, v);
 #pragma unroll
@@ -227,8 +227,9 @@ static cudaError_t launch_pdl(K kern, dim3 grid, unsigned block, cudaStream_t s,
 template <typename TY, typename TA>
 static cudaError_t launch_operand(const void* drafter, long long dstride, const KeptIndexView& v, int N, int n, int kind,
                                   void* A, long long lda, float* S, int rows, cudaStream_t s) {
+    // half the threads where a vector each covers the row
     auto k = kind == RDK_LOGITS ? exact_operand_kernel<TY, TA, RDK_LOGITS> : exact_operand_kernel<TY, TA, RDK_PROBS>;
-    return launch_pdl(k, dim3((unsigned)rows), (unsigned)kOperandThreads, s, static_cast<const TY*>(drafter), dstride, v.header, v.ids, N, n,
+    return launch_pdl(k, dim3((unsigned)rows), (unsigned)(n <= kOperandSums * kVec ? kOperandSums : kOperandThreads), s, static_cast<const TY*>(drafter), dstride, v.header, v.ids, N, n,
                       static_cast<TA*>(A), lda, S);
 }
 

@@ -274,7 +274,7 @@ def test_config5_full_size_sampled_outputs():
     t.assert_ok(max_ambiguous_frac=0.2)
 
 
-@pytest.mark.parametrize("n,dropped", [(1, False), (255, False), (257, True), (5000, False), (8197, True)])
+@pytest.mark.parametrize("n,dropped", [(1, False), (255, False), (257, True), (2048, False), (2049, True), (5000, False), (8197, True)])
 def test_drafter_sum_has_a_fixed_order(n, dropped):
     """q' of a probability drafter is a quotient of two fp32 numbers, so it can be had to the last bit: the row's sum is taken over
     256 interleaved runs, the runs of 32 neighbours are added in pairs and these eight one after the other.  With the identity as
