@@ -14,7 +14,10 @@
 //              on the leader's barrier)
 //   warp 1   : in the leader CTA the MMA issuer; in both the owner of the TMEM allocation
 //   warps 2-9: epilogue: a lane is a token, a column a row of w, so a warp stores 32 consecutive tokens per row;
-//              row sums by a butterfly over the lanes and one atomic per row and warp
+//              row sums by a butterfly over the lanes, kept in registers while the CTA's items are of the same rows
+//              (in shared memory where they are not); the four warps of a column are added up at the end: one atomic
+//              per row and CTA.  (One per row, warp and item put 4008 fp32 additions behind each other for 128256
+//              tokens: S off by 8e-7, now 1.6e-7.)
 // Items are ordered so that the row tiles of one 256-token panel of Mt run at the same time: the
 // panel is fetched from HBM once and shared through L2.
 // Every wait is bounded; on expiry the CTA flags RDK_ERR_TIMEOUT in the status word and winds down.
@@ -28,6 +31,8 @@ constexpr int kVoc = 128;                // tokens of one CTA
 constexpr int kBK = 64;                  // K block: 64 bf16 = 128 bytes = one swizzle row
 constexpr int kVocBytes = kVoc * kBK * 2;        // 16 KB
 constexpr int kTcMaxStages = 12;
+constexpr int kTcSumRows = 8192;         // most rows with a sum in shared memory
+constexpr int kTcMaxRows = 512;          // rows of an item: the columns of the accumulators
 constexpr int kTcSmem = 227 * 1024 - 2048;       // for the ring, alignment included
 constexpr int kTcEpiWarps = 8;
 constexpr int kTcThreads = 64 + 32 * kTcEpiWarps;
@@ -36,6 +41,7 @@ struct TcParams {
     float* w; float* S; int rows, N;
     int R, T;                        // rows of one instruction, instructions per item
     int tiles_r, num_kb, stages;
+    int sum_rows;                    // rows with a sum in shared memory behind the ring: all, or 0
     int full_items, num_items;       // items [0, full_items) are whole, the rest halves (one instruction of R rows)
     int32_t* status_word;
 };
@@ -56,9 +62,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1)
 exact_tc_kernel(const __grid_constant__ CUtensorMap tmapV, const __grid_constant__ CUtensorMap tmapR, const TcParams P) {
     extern __shared__ __align__(1024) unsigned char tc_smem[];
     const uint32_t ring = (s32(tc_smem) + 1023u) & ~1023u;               // the same offset in both CTAs
+    float* row_sums = reinterpret_cast<float*>(tc_smem + (ring - s32(tc_smem)) + (size_t)P.stages * (size_t)(kVocBytes + P.T * P.R * kBK));
+    for (int r = threadIdx.x; r < P.sum_rows; r += kTcThreads) row_sums[r] = 0.f;
+    float (*tc_sums)[kTcMaxRows] = reinterpret_cast<float (*)[kTcMaxRows]>(tc_smem);      // [4 quarters], at the end of the kernel
     __shared__ __align__(8) unsigned long long full_bar[kTcMaxStages], empty_bar[kTcMaxStages], acc_full, acc_empty;
     __shared__ uint32_t tmem_base_s;
-    __shared__ int abort_s;
+    __shared__ int abort_s, sum_row0_s;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     volatile int* abort = &abort_s;
@@ -68,6 +77,7 @@ exact_tc_kernel(const __grid_constant__ CUtensorMap tmapV, const __grid_constant
 
     if (threadIdx.x == 0) {
         abort_s = 0;
+        sum_row0_s = -1;
         for (int s = 0; s < P.stages; ++s) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(s32(&full_bar[s])));
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(s32(&empty_bar[s])));
@@ -184,10 +194,26 @@ exact_tc_kernel(const __grid_constant__ CUtensorMap tmapV, const __grid_constant
         asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(empty_addr) : "r"(s32(&acc_empty)));
         asm volatile("griddepcontrol.wait;" ::: "memory");           // S is zeroed by the kernel before this one
         uint32_t acc_phase = 0;
+        constexpr int kBlocks = kTcMaxRows / 64;                     // this warp's blocks of 32 columns
+        float sums[kBlocks];                                         // lane q: row sum_row0 + 32 share + 64 k + q
+        int sum_row0 = -1;
+        auto keep_sums = [&](auto&& put) {
+#pragma unroll
+            for (int k = 0; k < kBlocks; ++k) { put(k, sums[k]); sums[k] = 0.f; }
+        };
+        keep_sums([](int, float) {});
+        auto hand_over = [&](int k, float v) {
+            const int r = sum_row0 + share * 32 + k * 64 + lane;
+            if (v != 0.f && r < P.rows) atomicAdd((P.sum_rows ? row_sums : P.S) + r, v);
+        };
         for (int item = pair; item < P.num_items; item += pairs) {
             int tv, row0, t;
             decode_item(P, item, tv, row0, t);
             if (t == 0) continue;
+            if (P.S && row0 != sum_row0) {                           // other rows: what there is goes to them (while the tensor cores work)
+                if (sum_row0 >= 0) keep_sums(hand_over);
+                sum_row0 = row0;
+            }
             if (!tc_wait(&acc_full, acc_phase, abort)) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const int tok = (2 * tv + (int)rank) * kVoc + quarter * 32 + lane;
@@ -219,7 +245,9 @@ exact_tc_kernel(const __grid_constant__ CUtensorMap tmapV, const __grid_constant
                             v[q] = __float_as_uint(keep + __shfl_xor_sync(0xffffffffu, send, s));
                         }
                     }
-                    if (lane < left) atomicAdd(P.S + r + lane, __uint_as_float(v[0]));
+                    const float mine = lane < left ? __uint_as_float(v[0]) : 0.f;
+#pragma unroll
+                    for (int k = 0; k < kBlocks; ++k) sums[k] += k == c / 64 ? mine : 0.f;
                 }
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -227,12 +255,26 @@ exact_tc_kernel(const __grid_constant__ CUtensorMap tmapV, const __grid_constant
             if (lane == 0) asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(empty_addr) : "memory");
             acc_phase ^= 1u;
         }
+        // every item of the CTA is through the tensor cores: the ring holds nothing that is still needed
+        if (P.S && sum_row0 >= 0 && P.sum_rows) {
+            keep_sums(hand_over);
+        } else if (P.S && sum_row0 >= 0 && !*abort) {
+            keep_sums([&](int k, float v) { tc_sums[quarter][share * 32 + k * 64 + lane] = v; });
+            if (lane == 0) sum_row0_s = sum_row0;                    // (the same in all eight warps)
+        }
     }
 
     // after a wait that gave up, copies may still be on their way into shared memory: let them land
     if (abort_s && warp == 0) for (int k = 0; k < 10000; ++k) __nanosleep(100);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    if (sum_row0_s >= 0 && !abort_s)
+        for (int c = threadIdx.x; c < kTcMaxRows; c += kTcThreads) {
+            const float v = (tc_sums[0][c] + tc_sums[1][c]) + (tc_sums[2][c] + tc_sums[3][c]);
+            if (v != 0.f && sum_row0_s + c < P.rows) atomicAdd(P.S + sum_row0_s + c, v);
+        }
+    for (int r = threadIdx.x; r < P.sum_rows; r += kTcThreads)
+        if (row_sums[r] != 0.f) atomicAdd(P.S + r, row_sums[r]);
     // neither CTA leaves, nor gives its tensor memory back, while the other may still signal its barriers or read its operands
     asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
     if (warp == 1) {
@@ -298,31 +340,33 @@ int launch_exact_tc(const __nv_bfloat16* A, long long lda, const __nv_bfloat16* 
     const int pairs_most = sms / 2;
     // as few row tiles as the 512 accumulator columns allow, more where that leaves pairs without work (down to 64 rows,
     // below which an item is bound by its part of Mt)
-    long long tiles_r = (rows + 511) / 512;
+    long long tiles_r = (rows + kTcMaxRows - 1) / kTcMaxRows;
     while (tiles_v * tiles_r < pairs_most && rows / tiles_r > 64) ++tiles_r;
     const int per = (int)((rows + tiles_r - 1) / tiles_r);
     P.T = per > 256 ? 2 : 1;
     P.R = P.T == 2 ? ((per + 1) / 2 + 15) / 16 * 16 : (per + 31) / 32 * 32;
     P.tiles_r = (rows + P.T * P.R - 1) / (P.T * P.R);
     const int stage_bytes = kVocBytes + P.T * P.R * kBK;
-    P.stages = (kTcSmem - 1024) / stage_bytes;
+    const long long tiles = tiles_v * P.tiles_r;
+    if (tiles > 0x3fffffffLL) { set_error("rdk_redistribute_exact: too many output tiles"); return RDK_ERR_UNSUPPORTED; }
+    const int pairs = (int)(tiles < pairs_most ? tiles : pairs_most);
+    const int rest = (int)(tiles % pairs);
+    const bool split = P.T == 2 && rest > 0 && 2 * rest <= pairs;         // cut the last partial round into halves
+    // a pair's items have rows of their own each where the row tiles do not divide the pairs, or in halves
+    P.sum_rows = S_out && tiles > pairs && (pairs % P.tiles_r || split) && rows <= kTcSumRows ? rows : 0;
+    P.stages = (kTcSmem - 1024 - 4 * P.sum_rows) / stage_bytes;
     if (P.stages > kTcMaxStages) P.stages = kTcMaxStages;
     CUtensorMap mapV, mapR;
     int st = make_map(&mapV, Mt, (uint64_t)n, (uint64_t)N, (uint64_t)ldm, kBK, kVoc);
     if (st != RDK_OK) return st;
     st = make_map(&mapR, A, (uint64_t)n, (uint64_t)rows, (uint64_t)lda, kBK, (uint32_t)P.R / 2);
     if (st != RDK_OK) return st;
-    const long long tiles = tiles_v * P.tiles_r;
-    if (tiles > 0x3fffffffLL) { set_error("rdk_redistribute_exact: too many output tiles"); return RDK_ERR_UNSUPPORTED; }
-    const int pairs = (int)(tiles < pairs_most ? tiles : pairs_most);
-    const int rest = (int)(tiles % pairs);
-    const bool split = P.T == 2 && rest > 0 && 2 * rest <= pairs;         // cut the last partial round into halves
     P.full_items = split ? (int)(tiles - rest) : (int)tiles;
     P.num_items = split ? (int)(tiles + rest) : (int)tiles;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2u * (unsigned)pairs, 1, 1);
     cfg.blockDim = dim3(kTcThreads, 1, 1);
-    cfg.dynamicSmemBytes = (size_t)P.stages * stage_bytes + 1024;
+    cfg.dynamicSmemBytes = (size_t)P.stages * stage_bytes + 1024 + 4 * (size_t)P.sum_rows;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -327,3 +327,20 @@ def test_fp32_row_sums_are_repeatable(N, rows):
         assert torch.equal(S, first)
     ref = w.double().sum(1)
     assert ((S.double() - ref).abs() <= 16 * 2.0 ** -24 * ref).all()
+
+
+@pytest.mark.parametrize("N,rows", [(128000, 320), (100003, 40), (70000, 700), (8192, 300), (33000, 1500)])
+def test_bf16_row_sums_take_one_addition_per_cta(N, rows):
+    """S of the bf16 layout: a CTA keeps the sums of its rows and adds them to S once, in whatever order.  k fp32 additions of equal
+    terms, each off by up to 2^-24 of a running sum that grows to the total, leave a root mean square error of 2^-24 sqrt(k / 3)
+    at most; k is one for each SM, and 16 for what a CTA adds up by itself."""
+    rdk = _rdk()
+    B = rdk.binding
+    n = 64
+    g = torch.Generator(device="cuda").manual_seed(N)
+    idx = rdk.rdk_prepare_ids(torch.arange(n, dtype=torch.int32, device="cuda"), N)
+    M = {"data": torch.rand(N, n, generator=g, device="cuda").to(torch.bfloat16), "layout": B.RDK_AFF_BF16_COLS, "ld": n}
+    w, S, _ = rdk.rdk_redistribute_exact(idx, torch.randn(rows, n, generator=g, device="cuda"), M, rows, 1)
+    ref = torch.cat([x.double().sum(1) for x in w.split(64)])
+    k = torch.cuda.get_device_properties(0).multi_processor_count + 16
+    assert float(((S.double() / ref - 1) ** 2).mean().sqrt()) <= 2.0 ** -24 * (k / 3) ** 0.5
