@@ -65,7 +65,12 @@ __device__ __forceinline__ void send_cluster4(uint32_t local, uint32_t bar, uint
                  ::"r"(r), "r"(__float_as_uint(a)), "r"(__float_as_uint(b)), "r"(__float_as_uint(c)), "r"(__float_as_uint(d)), "r"(m) : "memory");
 }
 
-// One segment's share of the row, on the scales m (target), my (drafter), mp (prior)
+// Scales of exponentials are whole powers of two: 2^(z log2 e - k) then has the rounding error of its own exponent only, and
+// going from one scale to another is exact.  (On the scale e^m itself m log2 e is rounded for each segment apart, an error of the
+// size of m that all tokens of the segment share.)
+__device__ __forceinline__ float scale_of(float m) { return m > -INFINITY ? rintf(m * kLog2e) : -INFINITY; }
+
+// One segment's share of the row, on the scales 2^m (target), 2^my (drafter), 2^mp (prior)
 struct SegRec { float E, Zq, th, m, my, Ep, mp, W; };
 
 // Folds the records of the warp's lanes into one (lanes without a record hold m = my = mp = -inf and zeros); the
@@ -74,13 +79,13 @@ template <bool PRIOR>
 __device__ __forceinline__ SegRec fold_records(const SegRec& r, int lane) {
     SegRec o;
     o.m = warp_max_redux(r.m); o.my = warp_max_redux(r.my);
-    const float f = r.m > -INFINITY ? ex2((r.m - o.m) * kLog2e) : 0.f;
-    const float g = r.my > -INFINITY ? ex2((r.my - o.my) * kLog2e) : 0.f;
+    const float f = r.m > -INFINITY ? ex2(r.m - o.m) : 0.f;
+    const float g = r.my > -INFINITY ? ex2(r.my - o.my) : 0.f;
     float fp = f;
     o.mp = 0.f; o.Ep = 0.f;
     if (PRIOR) {
         o.mp = warp_max_redux(r.mp);
-        fp = r.mp > -INFINITY ? ex2((r.mp - o.mp) * kLog2e) : 0.f;
+        fp = r.mp > -INFINITY ? ex2(r.mp - o.mp) : 0.f;
     }
     const float t = warp_sum4(r.E * f, r.Zq * g, r.th * (fp * g), PRIOR ? r.Ep * fp : r.W, lane);
     o.E = __shfl_sync(0xffffffffu, t, 0); o.Zq = __shfl_sync(0xffffffffu, t, 8); o.th = __shfl_sync(0xffffffffu, t, 16);
@@ -368,9 +373,10 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     __syncwarp();
 
     // ---- first visit ------------------------------------------------------------------------------------------------
-    // Scale of a segment's exponentials: not their maximum (finding it is a pass of its own) but that of the first vectors;
-    // any scale gives the same result as long as no sum grows beyond 1e18, in which case (or with nothing but -inf among
-    // the first) the visit is repeated with the maximum.
+    // Scale of a segment's exponentials: its maximum, so that the heaviest tokens have the smallest exponents and with them the
+    // smallest errors.  (On the maximum of the first vectors, which saves a pass over shared memory, q~ is 1.2 to 1.9 times
+    // as far off.)  The drafter's is the maximum of the tokens in registers; any scale will do as long as the sum does not grow
+    // beyond 1e18, in which case (or with nothing but -inf among them) the visit is repeated with the maximum of all.
     const int nit16 = g.per * kVec * (int)es / 512;              // 16-byte vectors per lane
     auto seg_max = [&](uint32_t base, int nit) -> float {
         MaxAcc<TZ> a;
@@ -385,19 +391,18 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
         for (int k = 0; k < nit16; ++k) exp_sum_vec<TZ>(lds128(base + (uint32_t)(k * 32 + lane) * 16u), l2, of, Ea, Eb);
         return (Ea.x + Ea.y) + (Eb.x + Eb.y);
     };
-    float m_w = -INFINITY, mp_w = -INFINITY, zoff = 0.f, poff = 0.f, yoff = 0.f;
-    float E = 0.f, Ep = 0.f, K = 0.f, Zq = 0.f, th = 0.f, W = 0.f;
+    const float m_w = scale_of(seg_max(zb, nit16)), mp_w = kPrior ? scale_of(seg_max(pb, nit16)) : -INFINITY;
+    const float zoff = m_w > -INFINITY ? -m_w : 0.f, poff = mp_w > -INFINITY ? -mp_w : 0.f;
+    float yoff = 0.f, my_s = KIND == RDK_LOGITS ? -INFINITY : 0.f;   // the drafter's scale (probabilities: 1)
+    float E = seg_sum(zb, zoff), Ep = kPrior ? seg_sum(pb, poff) : 0.f;
+    float K = 0.f, Zq = 0.f, th = 0.f, W = 0.f;
     float kz[kRegSlots];                                             // e_z (prior: that of the prior) of the first kept tokens
     const uint32_t db = kPrior ? pb : zb;                            // the distribution that enters theta
-    for (int attempt = 0; attempt < 2; ++attempt) {
-        m_w = seg_max(zb, attempt == 0 ? 1 : nit16);
-        if (kPrior) mp_w = seg_max(pb, attempt == 0 ? 1 : nit16);
-        if (attempt == 1 && kLinear) {                               // the values have become exponentials: once more
+    for (int attempt = 0; kLinear && attempt < 2; ++attempt) {
+        if (attempt == 1) {                                          // the values have become exponentials: once more
 #pragma unroll
             for (int h = 0; h < kRegSlots; h += 4) load_slots(h);
-        }
-        if (attempt == 1 && kLinear && KIND == RDK_LOGITS) {
-            for (int il = kRegSlots * 32 + lane; il < cnt; il += 128) {
+            for (int il = kRegSlots * 32 + lane; il - lane < cnt; il += 128) {
                 float y[4];
                 int pos[4];
                 load_kept(il, y, pos);
@@ -405,13 +410,9 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
             }
             my_w = warp_max_redux(my_w);
         }
-        zoff = m_w > -INFINITY ? -m_w * kLog2e : 0.f;
-        poff = mp_w > -INFINITY ? -mp_w * kLog2e : 0.f;
-        yoff = my_w > -INFINITY ? -my_w * kLog2e : 0.f;
-        E = seg_sum(zb, zoff);
-        if (kPrior) Ep = seg_sum(pb, poff);
+        if (KIND == RDK_LOGITS) { my_s = scale_of(my_w); yoff = my_s > -INFINITY ? -my_s : 0.f; }
         K = 0.f; Zq = 0.f; th = 0.f;
-        if (kLinear) {
+        {
             const float doff = kPrior ? poff : zoff;
             auto visit = [&](int pos, const float y, float& ed, float& ey) {
                 ed = ex2(fmaf(lds_z<TZ>(db + (uint32_t)max(pos, 0) * es), kLog2e, doff));
@@ -438,8 +439,7 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
                 for (int k = 0; k < 4; ++k) visit(pos[k], y[k], ed, ey);
             }
         }
-        const bool poor = !(fmaxf(E, fmaxf(Ep, KIND == RDK_LOGITS ? Zq : 0.f)) < 1e18f) || !(m_w > -INFINITY) || (kPrior && !(mp_w > -INFINITY)) ||
-                          (kLinear && KIND == RDK_LOGITS && cnt > kRegSlots * 32 && !(my_w > -INFINITY));
+        const bool poor = KIND == RDK_LOGITS && cnt > kRegSlots * 32 && (!(Zq < 1e18f) || !(my_s > -INFINITY));
         if (!__any_sync(0xffffffffu, poor)) break;
     }
     if (VAR == kVarGiven) {
@@ -458,7 +458,7 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     }
     if (lane == 0) {
         reinterpret_cast<float4*>(wrec[warp])[0] = make_float4(E, Zq, th, m_w);
-        reinterpret_cast<float4*>(wrec[warp])[1] = make_float4(my_w, Ep, mp_w, W);
+        reinterpret_cast<float4*>(wrec[warp])[1] = make_float4(my_s, Ep, mp_w, W);
     }
     __syncthreads();
 
@@ -492,18 +492,18 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     const float inv_zp = tot_b.x, inv_zq = tot_b.y, inv_zpi = tot_b.z;
     const float theta = kLinear ? tot_b.w * inv_zpi * inv_zq : 0.f;
     const float inv_n = 1.f / (float)P.N;
-    const float offg = -tot_m * kLog2e, poffg = kPrior ? -tot_mp * kLog2e : 0.f;
-    const float yoffg = KIND == RDK_LOGITS ? -tot_my * kLog2e : 0.f;
+    const float offg = -tot_m, poffg = kPrior ? -tot_mp : 0.f;
+    const float yoffg = KIND == RDK_LOGITS ? -tot_my : 0.f;
     // factor that turns the e_y of a segment with scale my into q'
     auto y_factor = [&](float my) -> float {
-        return !kLinear ? 1.f : (KIND == RDK_LOGITS ? (my > -INFINITY ? ex2((my - tot_my) * kLog2e) : 0.f) : 1.f) * inv_zq;
+        return !kLinear ? 1.f : (KIND == RDK_LOGITS ? (my > -INFINITY ? ex2(my - tot_my) : 0.f) : 1.f) * inv_zq;
     };
-    const float fy = y_factor(my_w);
+    const float fy = y_factor(my_s);
     float inv_s = 1.f;
 
     // p and w of two neighbouring positions, from their logits (pr: prior's) and e_y (or w)
-    const float fz = (m_w > -INFINITY ? ex2((m_w - tot_m) * kLog2e) : 0.f) * inv_zp;      // e on the segment's scale -> p
-    const float xs = kPrior ? (mp_w > -INFINITY ? ex2((mp_w - tot_mp) * kLog2e) : 0.f) * inv_zpi * inv_n : fz * inv_n;    // -> x
+    const float fz = (m_w > -INFINITY ? ex2(m_w - tot_m) : 0.f) * inv_zp;      // e on the segment's scale -> p
+    const float xs = kPrior ? (mp_w > -INFINITY ? ex2(mp_w - tot_mp) : 0.f) * inv_zpi * inv_n : fz * inv_n;    // -> x
     const float2 l2e2 = splat(kLog2e), zoff2 = splat(zoff), poff2 = splat(poff), fz2 = splat(fz), xs2 = splat(xs), fy2 = splat(fy), th2 = splat(theta), neg2 = splat(-1.f), one2 = splat(1.f);
     auto dense_pair = [&](float2 z, float2 pr, float2 q, float2& p, float2& w) {
         const float2 e = ex2_2(ffma2(z, l2e2, zoff2));

@@ -224,3 +224,34 @@ def test_affinity_of_a_small_temperature_is_the_identity(N, n, d):
     ref[ids.long(), torch.arange(n, device="cuda")] = 1.0
     ref[:, 7] = torch.tensor(1.0 / N).to(torch.bfloat16).double()
     assert torch.equal(M, ref)
+
+
+@pytest.mark.parametrize("N,n,dtype,order", [(50257, 12565, "bf16", "ascending"), (32000, 8000, "f32", "ranked"), (9001, 3000, "f32", "ascending")])
+def test_cluster_kernel_errors_against_64_bits(N, n, dtype, order):
+    """alpha and the residual's mass of 320 long-tailed rows, relative error in the 2-norm: an exponential is off by 2^-24 of itself
+    in the mean; its sum, the reciprocal, the product and the sum of the products by a rounding each (2^-24 / sqrt 3): sqrt(7 / 3) in
+    units of 2^-24 in all where one token has the weight, and less where several share it.  Scales that are rounded for each segment apart, and exponents far
+    above zero, show here."""
+    rdk = _rdk()
+    B = rdk.binding
+    rows, dt, g = 32, {"bf16": torch.bfloat16, "f32": torch.float32}[dtype], torch.Generator(device="cuda").manual_seed(N)
+    square = {"alpha": 0.0, "residual_mass": 0.0}
+    for _ in range(10):
+        ranking = torch.randperm(N, generator=g, device="cuda")
+        ids = ranking[:n] if order == "ranked" else torch.sort(ranking[:n]).values
+        bias = torch.empty(N, device="cuda")
+        bias[ranking] = -1.1 * torch.log(torch.arange(1, N + 1, device="cuda", dtype=torch.float32))
+        z0 = torch.randn(rows, N, generator=g, device="cuda")
+        z = (3 * z0 + bias).to(dt)
+        y = (bias[ids] + 3 * (0.8 * z0[:, ids] + 0.6 * torch.randn(rows, n, generator=g, device="cuda"))).to(dt)
+        out = rdk.rdk_sample_and_verify(rdk.rdk_prepare_ids(ids.to(torch.int32), N), B.RDK_MODE_LINEAR, z, y, None,
+                                        torch.rand(rows, 4, 4, generator=g, device="cuda"), rows, 1)
+        B.check_status_word(out)
+        p, q = torch.softmax(z.double(), 1), torch.zeros(rows, N, dtype=torch.float64, device="cuda")
+        q[:, ids] = torch.softmax(y.double(), 1)
+        theta = (p * q).sum(1, keepdim=True)
+        w = (N * q + theta * p) / (N + p)
+        m = torch.minimum(p, w / w.sum(1, keepdim=True))
+        for k, ref in (("alpha", m.sum(1)), ("residual_mass", (p - m).sum(1))):
+            square[k] += float(((out[k].double() - ref) ** 2).sum() / (ref ** 2).sum()) / 10
+    assert max(square.values()) ** 0.5 <= (7 / 3) ** 0.5 * 2.0 ** -24, {k: v ** 0.5 * 2 ** 24 for k, v in square.items()}
