@@ -75,8 +75,9 @@ struct SegRec { float E, Zq, th, m, my, Ep, mp, W; };
 
 // Folds the records of the warp's lanes into one (lanes without a record hold m = my = mp = -inf and zeros); the
 // scale of th is that of the target (or the prior) times that of the drafter.
+// exact_q: the drafter's sum in fp64 (see the warp totals).
 template <bool PRIOR>
-__device__ __forceinline__ SegRec fold_records(const SegRec& r, int lane) {
+__device__ __forceinline__ SegRec fold_records(const SegRec& r, int lane, bool exact_q) {
     SegRec o;
     o.m = warp_max_redux(r.m); o.my = warp_max_redux(r.my);
     const float f = r.m > -INFINITY ? ex2(r.m - o.m) : 0.f;
@@ -89,6 +90,7 @@ __device__ __forceinline__ SegRec fold_records(const SegRec& r, int lane) {
     }
     const float t = warp_sum4(r.E * f, r.Zq * g, r.th * (fp * g), PRIOR ? r.Ep * fp : r.W, lane);
     o.E = __shfl_sync(0xffffffffu, t, 0); o.Zq = __shfl_sync(0xffffffffu, t, 8); o.th = __shfl_sync(0xffffffffu, t, 16);
+    if (exact_q) o.Zq = (float)warp_sum_d((double)(r.Zq * g));
     const float last = __shfl_sync(0xffffffffu, t, 24);
     if (PRIOR) { o.Ep = last; o.W = 0.f; } else o.W = last;
     return o;
@@ -398,17 +400,25 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     float K = 0.f, Zq = 0.f, th = 0.f, W = 0.f;
     float kz[kRegSlots];                                             // e_z (prior: that of the prior) of the first kept tokens
     const uint32_t db = kPrior ? pb : zb;                            // the distribution that enters theta
+    // q~ is written out as it stands, not divided by its sum: the roundings of the 15 additions that fold the drafter's sum over
+    // warp, CTA and cluster, each of the size of the whole, would be in all of a row's q~, and so would those of
+    // exponents above zero (9e-8 to 1.1e-7 off 64 bits instead of 6e-8 to 7e-8)
+    const bool exact_q = VAR == kVarDense && P.qtilde;
+    auto max_of_rest = [&]() {                                       // the drafter's maximum, of the tokens beyond the registers too
+        for (int il = kRegSlots * 32 + lane; il - lane < cnt; il += 128) {
+            float y[4];
+            int pos[4];
+            load_kept(il, y, pos);
+            my_w = fmaxf(fmaxf(my_w, fmaxf(y[0], y[1])), fmaxf(y[2], y[3]));
+        }
+        my_w = warp_max_redux(my_w);
+    };
+    if (KIND == RDK_LOGITS && exact_q && cnt > kRegSlots * 32) max_of_rest();
     for (int attempt = 0; kLinear && attempt < 2; ++attempt) {
         if (attempt == 1) {                                          // the values have become exponentials: once more
 #pragma unroll
             for (int h = 0; h < kRegSlots; h += 4) load_slots(h);
-            for (int il = kRegSlots * 32 + lane; il - lane < cnt; il += 128) {
-                float y[4];
-                int pos[4];
-                load_kept(il, y, pos);
-                my_w = fmaxf(fmaxf(my_w, fmaxf(y[0], y[1])), fmaxf(y[2], y[3]));
-            }
-            my_w = warp_max_redux(my_w);
+            max_of_rest();
         }
         if (KIND == RDK_LOGITS) { my_s = scale_of(my_w); yoff = my_s > -INFINITY ? -my_s : 0.f; }
         K = 0.f; Zq = 0.f; th = 0.f;
@@ -450,6 +460,10 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
         }
     }
     {   // warp totals
+        if (exact_q) {
+            const float all = (float)warp_sum_d((double)Zq);
+            Zq = lane == 0 ? all : 0.f;
+        }
         const float t = warp_sum4(E, K, Zq, th, lane);
         E = __shfl_sync(0xffffffffu, t, 0); K = __shfl_sync(0xffffffffu, t, 8);
         Zq = __shfl_sync(0xffffffffu, t, 16); th = __shfl_sync(0xffffffffu, t, 24);
@@ -469,7 +483,7 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
             const float4 a = reinterpret_cast<const float4*>(wrec[lane])[0], b = reinterpret_cast<const float4*>(wrec[lane])[1];
             r = SegRec{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
         }
-        r = fold_records<kPrior>(r, lane);
+        r = fold_records<kPrior>(r, lane, exact_q);
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");      // all CTAs of the cluster run
         if (lane < (int)C) {
             send_cluster4(smem_u32(&xrec[rank][0]), smem_u32(&xbar), (uint32_t)lane, r.E, r.Zq, r.th, r.m);
@@ -483,7 +497,7 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
             const float4 a = xrec[lane][0], b = xrec[lane][1];
             r = SegRec{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
         }
-        r = fold_records<kPrior>(r, lane);
+        r = fold_records<kPrior>(r, lane, exact_q);
         if (lane == 0) { tot_s[0] = make_float4(r.m, r.my, r.mp, r.W); tot_s[1] = make_float4(1.f / r.E, kLinear ? 1.f / r.Zq : 1.f, kPrior ? 1.f / r.Ep : 1.f / r.E, r.th); }
     }
     __syncthreads();

@@ -255,3 +255,25 @@ def test_cluster_kernel_errors_against_64_bits(N, n, dtype, order):
         for k, ref in (("alpha", m.sum(1)), ("residual_mass", (p - m).sum(1))):
             square[k] += float(((out[k].double() - ref) ** 2).sum() / (ref ** 2).sum()) / 10
     assert max(square.values()) ** 0.5 <= (7 / 3) ** 0.5 * 2.0 ** -24, {k: v ** 0.5 * 2 ** 24 for k, v in square.items()}
+
+
+@pytest.mark.parametrize("N,n", [(128256, 12826), (262143, 90000)])
+def test_written_out_q_errors_against_64_bits(N, n):
+    """q~ of 64 long-tailed rows, relative error in the 2-norm: the exponential's 2^-24 and a rounding (2^-24 / sqrt 3) each for the
+    reciprocal of the sum, the product and the redistribution; the sum's own, which all of a row would share, are not among them."""
+    rdk = _rdk()
+    rows, g, square = 8, torch.Generator(device="cuda").manual_seed(N), 0.0
+    for _ in range(8):
+        ranking = torch.randperm(N, generator=g, device="cuda")
+        ids = torch.sort(ranking[:n]).values
+        bias = torch.empty(N, device="cuda")
+        bias[ranking] = -1.1 * torch.log(torch.arange(1, N + 1, device="cuda", dtype=torch.float32))
+        z = (3 * torch.randn(rows, N, generator=g, device="cuda") + bias).to(torch.bfloat16)
+        y = (bias[ids] + 3 * torch.randn(rows, n, generator=g, device="cuda")).to(torch.bfloat16)
+        got, _, _ = rdk.rdk_redistribute_linear(rdk.rdk_prepare_ids(ids.to(torch.int32), N), z, y, rows, 1)
+        p, q = torch.softmax(z.double(), 1), torch.zeros(rows, N, dtype=torch.float64, device="cuda")
+        q[:, ids] = torch.softmax(y.double(), 1)
+        w = (N * q + (p * q).sum(1, keepdim=True) * p) / (N + p)
+        w = w / w.sum(1, keepdim=True)
+        square += float(((got.double() - w) ** 2).sum() / (w ** 2).sum()) / 8
+    assert square ** 0.5 <= 2.0 ** 0.5 * 2.0 ** -24, square ** 0.5 * 2 ** 24
