@@ -180,6 +180,7 @@ extern "C" int rdk_build_affinity(const void* embeddings, int32_t emb_dtype, int
         return RDK_ERR_WORKSPACE_TOO_SMALL;
     }
     const size_t smem = (size_t)d * kAffRows * sizeof(float);
+    if (smem > 200 * 1024) { set_error("rdk_build_affinity: embedding dimension %d too large", d); return RDK_ERR_UNSUPPORTED; }
     const int st = check_arch();
     if (st != RDK_OK) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -187,7 +188,6 @@ extern "C" int rdk_build_affinity(const void* embeddings, int32_t emb_dtype, int
     if (affinity_tc_eligible(embeddings, emb_dtype, M_desc->layout))
         return build_affinity_tc(static_cast<const __nv_bfloat16*>(embeddings), d, estride, kept_ids, n, N, tau,
                                  static_cast<__nv_bfloat16*>(M_out), M_desc->ld, ws, s);
-    if (smem > 200 * 1024) { set_error("rdk_build_affinity: embedding dimension %d too large", d); return RDK_ERR_UNSUPPORTED; }
     float* Et = static_cast<float*>(ws);
     const int Npad = aff_npad(N);
     float* part = reinterpret_cast<float*>(static_cast<unsigned char*>(ws) + idx_align((size_t)Npad * d * sizeof(float)));

@@ -190,3 +190,15 @@ print("fine")
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     res = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
     assert res.returncode == 0 and "fine" in res.stdout, (res.returncode, res.stderr[-2000:])
+
+
+@pytest.mark.skipif("__import__('torch').cuda.is_available()", reason="host logic, with addresses that no device may see")
+def test_embedding_dimensions_beyond_the_limit_are_refused_by_every_route(B):
+    """3200 is the largest dimension (16 rows in shared memory); the limit is the call's, whichever kernel would serve it."""
+    L, dummy = B.lib(), C.c_void_p(1 << 20)
+    for layout in (B.RDK_AFF_F32_ROWS, B.RDK_AFF_BF16_COLS):
+        for dtype in (B.RDK_F32, B.RDK_BF16):
+            for d in (3201, 4096):
+                a = B.rdk_affinity(1 << 20, layout, 0, 64)
+                st = L.rdk_build_affinity(dummy, dtype, d, 0, dummy, 8, 64, 0.1, C.byref(a), dummy, dummy, 1 << 40, None)
+                assert st == B.RDK_ERR_UNSUPPORTED, (layout, dtype, d, st)
