@@ -16,10 +16,9 @@
 
 namespace rdk {
 
-constexpr int kEmitThreads = 512;
-constexpr int kEmitWarps = kEmitThreads / 32;
+constexpr int kEmitMaxWarps = 16;
 constexpr int kEmitMaxCtas = 8;
-constexpr int kEmitMaxSeg = kEmitMaxCtas * kEmitWarps;
+constexpr int kEmitMaxSeg = kEmitMaxCtas * kEmitMaxWarps;
 constexpr int kEmitBatch = 256;           // pairs whose answers are kept at a time
 
 struct EmitParams {
@@ -73,7 +72,7 @@ __device__ __forceinline__ int emit_accepted(const EmitParams& P, int pair, int 
 }
 
 template <typename TZ>
-__global__ void __launch_bounds__(kEmitThreads)
+__global__ void __launch_bounds__(kEmitMaxWarps * 32)
 emit_kernel(const EmitParams P) {
     __shared__ float2 rec[kEmitMaxSeg];                  // CTA 0: (scale, sum) of every warp of the cluster
     __shared__ double cdf[kEmitMaxSeg];
@@ -81,7 +80,7 @@ emit_kernel(const EmitParams P) {
     __shared__ float bc[2];
     __shared__ __align__(8) unsigned long long rbar;     // CTA 0: the records of the row are in rec[]
     __shared__ uint8_t all_s[kEmitBatch];                // whether all drafts of the pair were accepted
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     uint32_t rank, C;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
     asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(C));
@@ -98,7 +97,7 @@ emit_kernel(const EmitParams P) {
     for (int i0 = 0; i0 < mine; i0 += kEmitBatch) {
         const int cnt = min(kEmitBatch, mine - i0);
         // every CTA looks at all of the cluster's pairs, CTA 0 writes
-        for (int i = warp; i < cnt; i += kEmitWarps) {
+        for (int i = warp; i < cnt; i += nw) {
             const int j = emit_accepted(P, cluster + (i0 + i) * clusters, lane, rank == 0);
             if (lane == 0) all_s[i] = j == P.positions;
         }
@@ -109,7 +108,7 @@ emit_kernel(const EmitParams P) {
             const int pair = cluster + (i0 + i) * clusters, b = pair / P.trials, t = pair - b * P.trials;
             const TZ* zrow = static_cast<const TZ*>(P.bonus) + (long long)b * P.bonus_stride;
             const int phase = (int)((reinterpret_cast<uintptr_t>(zrow) & 15u) / sizeof(TZ));
-            const int sg = (int)rank * kEmitWarps + warp, nseg = (int)C * kEmitWarps;
+            const int sg = (int)rank * nw + warp, nseg = (int)C * nw;
             const float u = __ldg(P.uniforms + (((long long)b * P.positions + P.positions - 1) * P.trials + t) * 4 + 3);
             // CTA 0 runs, and is done with the previous row's records: it says so here, the others wait for it with their sums
             if (rank == 0 && tid == 0)
@@ -191,7 +190,7 @@ emit_kernel(const EmitParams P) {
                 return warp_sum(sum);
             };
             for (int c0 = 0; c0 < nch && chosen < 0; c0 += 32) {
-                for (int ch = c0 + warp; ch < min(nch, c0 + 32); ch += kEmitWarps) {
+                for (int ch = c0 + warp; ch < min(nch, c0 + 32); ch += nw) {
                     const float sum = chunk_p(ch);
                     if (lane == 0) chunk_sum[ch - c0] = sum;
                 }
@@ -208,7 +207,7 @@ emit_kernel(const EmitParams P) {
             }
             const float r_in = chosen < 0 ? INFINITY : rem - before;     // rounding left no token: the last positive one
             if (chosen < 0) chosen = max(last_pos, 0);
-            if (chosen % kEmitWarps != warp) continue;
+            if (chosen % nw != warp) continue;
             if (held != chosen) (void)chunk_p(chosen);
             const int sel = max(pick_in_segment(p, r_in, lane), 0);
             if (lane == 0) P.seq_tokens[(long long)pair * (P.positions + 1) + P.positions] = min(max((s * P.per + chosen * 32) * kVec - phase + sel, 0), P.N - 1);
@@ -219,17 +218,27 @@ emit_kernel(const EmitParams P) {
 
 template <typename TZ>
 static cudaError_t launch_emit(EmitParams P, cudaStream_t s) {
-    // CTAs per cluster: a warp's run is at least two 256-position chunks.  Clusters: what is resident at once (four CTAs of
-    // 512 threads to an SM), in the worst case one for each pair.
+    // Warps: few for few tokens, so that more rows are under way (2048 rows of 1000 tokens, all drawn from: 12 us, with
+    // sixteen 32), and eight where rows are many (512 of 8000: 7.2 us, with sixteen 8.1; 64 or 160: 5.9 either way).
+    // CTAs per cluster: a warp's run is at least two 256-position chunks, and all pairs can have such a cluster at once:
+    // beyond that a larger one only serialises what would run side by side (2048 rows of 32000 tokens, all drawn from: 65 us, on
+    // clusters of four 187).  Up to four pairs to a cluster for rows that one CTA takes longer over than their chain: 512 rows
+    // of 262143, a tenth drawn from, 27 us, with single CTAs 37.  Clusters: what is resident at once.
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
     const long long pairs = (long long)P.batch * P.trials;
+    const unsigned nw = P.N <= 1000 ? 4 : (P.N <= 4000 || (P.N <= 65536 && pairs > 2 * sms) ? 8 : kEmitMaxWarps);
+    const long long resident = (long long)sms * 64 / nw;        // CTAs, at 64 warps an SM
     unsigned C = 1;
-    while (C < (unsigned)kEmitMaxCtas && (long long)C * kEmitWarps * 512 < P.N) C *= 2;
-    const long long most = 4 * 148 / C;
-    P.per = (int)(((long long)P.N + 8 + C * kEmitWarps * kVec - 1) / (C * kEmitWarps * kVec));
+    while (C < (unsigned)kEmitMaxCtas && (long long)C * nw * 512 < P.N && pairs * 2 * C <= (P.N > 65536 ? 4 : 1) * resident) C *= 2;
+    const long long most = resident / C;
+    P.per = (int)(((long long)P.N + 8 + C * nw * kVec - 1) / (C * nw * kVec));
     P.per = (P.per + 31) / 32 * 32;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(pairs < most ? pairs : most) * C, 1, 1);
-    cfg.blockDim = dim3(kEmitThreads, 1, 1);
+    cfg.blockDim = dim3(nw * 32, 1, 1);
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;

@@ -99,7 +99,8 @@ def test_cluster_kernel_given_weights(N, batch, positions, trials, counters):
         PU.compare_accepted_len(out, batch, positions, trials)
 
 
-@pytest.mark.parametrize("N,batch,positions,trials", [(300, 700, 3, 2), (40001, 90, 40, 1), (140000, 3, 1, 1)])
+@pytest.mark.parametrize("N,batch,positions,trials", [(300, 700, 3, 2), (40001, 90, 40, 1), (140000, 3, 1, 1), (1001, 20, 2, 2), (4001, 400, 2, 1),
+                                                      (65537, 400, 1, 1), (70001, 70, 2, 1)])
 def test_emitted_sequences_of_many_pairs(N, batch, positions, trials):
     """More pairs than clusters, more positions than a warp's lanes, one to eight CTAs a row; the accept patterns mix all
     accepted, none and everything between."""
