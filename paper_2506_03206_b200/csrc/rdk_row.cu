@@ -430,6 +430,22 @@ static int validate_problem(const rdk_problem* pb, const char* who, bool need_in
     return RDK_OK;
 }
 
+// Whether the one-CTA-per-row kernel is the better one because draws outweigh the sweep: the cluster kernel makes a row's
+// draws in one of its CTAs, sums the chunks of a segment for each and makes the residual draw of every trial, needed or not;
+// there a row's warps share the trials, from sums of 256 tokens.  Row / cluster kernel, us: linear, 160 rows x 64 trials of
+// 32768 tokens 104 / 149, of 50257 154 / 257, of 128257 371 / 471, 40 x 64 of 128257 295 / 169, 160 x 32 356 / 282; with a prior,
+// 600 x 16 of 32768 208 / 243, 160 x 16 of 128256 274 / 169; given weights, 160 x 32 of 50257 70 / 73, of 128257 145 / 154, x 16
+// 64 / 49 and 139 / 96.  Rows on 16-byte boundaries are quicker in the row kernel: given, 100 x 16 of 32768 18 / 21, of 128256
+// 50 / 60, of 262144 149 / 89, 40 x 64 of 262144 102 / 136, 40 x 32 of 32768 21 / 17.
+static bool many_draws(const RowParams& P, int mode, size_t es) {
+    if (P.N < kStreamMinN || P.trials < 16) return false;
+    const long long draws = (long long)P.rows * P.trials;
+    if (mode == RDK_MODE_LINEAR) return draws >= (P.prior ? 9600 : 10240);
+    const bool aligned = !(((uintptr_t)P.target | (uintptr_t)P.w) & 15u) && !((P.target_stride * (long long)es | P.w_stride * 4) & 15);
+    if (!aligned) return draws >= 5120;
+    return P.trials >= 64 ? draws >= 2560 : draws >= (P.N <= 131072 ? 1600 : 5120);
+}
+
 static int run_rows(const rdk_problem* pb, int mode, const void* target, const void* drafter,
                     const float* w, long long w_stride, const float* uniforms, int trials,
                     const rdk_outputs* out, float* qtilde, float* theta_out, float* S_out,
@@ -481,12 +497,13 @@ static int run_rows(const rdk_problem* pb, int mode, const void* target, const v
     };
     if (!(pb->flags & RDK_FLAG_ROW_KERNEL)) {
         const bool streams = mode == RDK_MODE_LINEAR && trials > 0 && !prior;
-        if (!streams || stream_few_rows(P, pb->target_dtype, pb->drafter_dtype, pb->drafter_kind)) e = cluster();
+        const bool many = many_draws(P, mode, pb->target_dtype == RDK_F32 ? 4 : 2);
+        if (!many && (!streams || stream_few_rows(P, pb->target_dtype, pb->drafter_dtype, pb->drafter_kind))) e = cluster();
         if (e == cudaErrorNotSupported && streams) {
             e = launch_stream_linear(P, pb->target_dtype, pb->drafter_dtype, pb->drafter_kind, pb->batch, ws, ws_bytes, s);
             counted = e == cudaSuccess;
         }
-        if (e == cudaErrorNotSupported) e = cluster();
+        if (e == cudaErrorNotSupported && !many) e = cluster();
         if (counted) return RDK_OK;                                 // the kernel also wrote accepted_len
     }
     if (e == cudaErrorNotSupported)

@@ -278,3 +278,26 @@ def test_written_out_q_errors_against_64_bits(N, n):
         w = w / w.sum(1, keepdim=True)
         square += float(((got.double() - w) ** 2).sum() / (w ** 2).sum()) / 8
     assert square ** 0.5 <= 2.0 ** 0.5 * 2.0 ** -24, square ** 0.5 * 2 ** 24
+
+
+@pytest.mark.parametrize("mode,N,rows,trials", [("given", 4096, 100, 16), ("given", 33001, 20, 256), ("given", 262144, 40, 64), ("linear", 5000, 160, 64),
+                                                ("linear", 70001, 5, 2048), ("prior", 9000, 150, 64)])
+def test_many_draws_take_the_row_kernel(mode, N, rows, trials):
+    """Where draws outweigh the sweep the one-CTA-per-row kernel serves, so every output has that kernel's bits."""
+    rdk = _rdk()
+    B = rdk.binding
+    g = torch.Generator(device="cuda").manual_seed(N)
+    ids = torch.randperm(N, generator=g, device="cuda")[: N // 4].to(torch.int32)      # (not ascending: the streaming kernels cannot serve)
+    idx = rdk.rdk_prepare_ids(ids, N)
+    z = torch.randn(rows, N, generator=g, device="cuda").to(torch.bfloat16)
+    y = torch.randn(rows, N // 4, generator=g, device="cuda").to(torch.bfloat16) if mode != "given" else None
+    w = torch.softmax(torch.randn(rows, N, generator=g, device="cuda"), -1) if mode == "given" else None
+    u = torch.rand(rows, trials, 4, generator=g, device="cuda")
+    m = B.RDK_MODE_LINEAR if mode != "given" else B.RDK_MODE_PRECOMPUTED_W
+    if mode == "prior":      # (the call with a prior has no flags: the row kernel's numbers are those of a prior that is the target)
+        a = rdk.rdk_sample_and_verify_prior(idx, z, z, y, u, rows, 1)
+        b = rdk.rdk_sample_and_verify(idx, m, z, y, None, u, rows, 1, flags=B.RDK_FLAG_ROW_KERNEL)
+    else:
+        a, b = (rdk.rdk_sample_and_verify(idx, m, z, y, w, u, rows, 1, flags=f) for f in (0, B.RDK_FLAG_ROW_KERNEL))
+    for k in ("draft_token", "out_token", "accepted", "accept_prob", "alpha", "S", "residual_mass", "accepted_len"):
+        assert torch.equal(a[k], b[k]), k
