@@ -78,7 +78,8 @@ typedef enum rdk_mode { RDK_MODE_LINEAR = 0, RDK_MODE_PRECOMPUTED_W = 1 } rdk_mo
  * instead of being left untouched.                                                                */
 #define RDK_FLAG_PAD_SEQUENCES 4
 
-/* Whether a call of the linear mode can take the streaming kernels (see rdk_sample_route).       */
+/* What serves a call (see rdk_sample_route): a row kernel -- a row to a thread-block cluster, or to a
+ * CTA -- or the streaming kernels.                                                              */
 typedef enum rdk_route { RDK_ROUTE_ROW_KERNEL = 0, RDK_ROUTE_STREAM_KERNEL = 1 } rdk_route;
 
 /* Physical layouts of the affinity matrix M (n rows i in I, N columns j in T).
@@ -240,7 +241,7 @@ int rdk_redistribute_linear(const rdk_problem* problem, const void* target, cons
  *              aligned (may be NULL when that size is 0; the precomputed mode counts accepted_len in the
  *              kernel that draws if given 8 bytes per (sequence, trial), else in one more launch).  The streaming kernels keep there one
  *              record of 4160 bytes per row (row scalars and per-segment sums of w, min(p, q~),
- *              max(0, p - q~), p), one 4-byte counter per (sequence, trial), and 64 bytes per
+ *              max(0, p - q~), p), one 8-byte counter per (sequence, trial), and 64 bytes per
  *              (row, CTA sharing the row) through which those CTAs exchange their partial
  *              soft-max sums.  Its contents need no initialisation.  One workspace serves one call
  *              at a time: calls that share it must be ordered on one stream (they may be queued
@@ -275,13 +276,15 @@ int rdk_sample_and_verify(const rdk_problem* problem, int32_t mode, const void* 
 
 /* ---------------------------------------------------------------------------------------------
  * rdk_sample_route -- host-only query (no CUDA call, nothing launched): whether rdk_sample_and_verify
- * can run Algorithm 4 steps 4-8 for these arguments with the streaming kernels (few rows are given to
- * the cluster kernel all the same, where that is faster).  It sees what
- * rdk_stream_geometry cannot: the flags, alignment and strides of the rows, the workspace, and
- * whether the kept ids of problem->kept_index were ascending and valid when the index was built.
+ * runs Algorithm 4 steps 4-8 for these arguments with the streaming kernels.  It sees what
+ * rdk_stream_geometry cannot: the flags, alignment and strides of the rows, the workspace, the number
+ * of rows (few are given to the cluster kernel, where that is faster), and whether the kept ids of
+ * problem->kept_index were ascending and valid when the index was built.
  *   why   host const char**, may be NULL: receives a static string naming the first reason the
- *         streaming kernel cannot serve ("" when it can)
- * Returns RDK_ROUTE_STREAM_KERNEL or RDK_ROUTE_ROW_KERNEL (a row held by one cluster or one CTA), or -(rdk_status) for a bad problem.
+ *         streaming kernels do not serve ("" when they do)
+ * Returns RDK_ROUTE_STREAM_KERNEL or RDK_ROUTE_ROW_KERNEL (the cluster kernel; the one-CTA-per-row
+ * kernel with RDK_FLAG_ROW_KERNEL, where a row does not fit a cluster, and for very many draws), or
+ * -(rdk_status) for a bad problem.
  * ------------------------------------------------------------------------------------------- */
 int rdk_sample_route(const rdk_problem* problem, int32_t mode, const void* target,
                      const void* drafter, int32_t trials, const void* ws, size_t ws_bytes,

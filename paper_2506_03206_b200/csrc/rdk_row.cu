@@ -589,6 +589,7 @@ extern "C" int rdk_sample_route(const rdk_problem* problem, int32_t mode, const 
     P.header = static_cast<const int32_t*>(problem->kept_index);
     const char* no = stream_ineligible(P, problem->target_dtype, problem->drafter_dtype, problem->drafter_kind,
                                        problem->batch, ws, ws_bytes);
+    if (!no && stream_few_rows(P, problem->target_dtype, problem->drafter_dtype, problem->drafter_kind)) no = "few rows: one cluster each is faster";
     if (no) { if (why) *why = no; return RDK_ROUTE_ROW_KERNEL; }
     return RDK_ROUTE_STREAM_KERNEL;
 }

@@ -383,7 +383,7 @@ def test_strided_rows_through_the_streaming_kernels():
     not a multiple of 8, so the drafter rows start at varying 16-byte phases)."""
     rdk = _rdk()
     B = rdk.binding
-    cfg = W.tiny_config(N=24576, n=5001, rows=40, dtype="bf16", trials=2, kept_rule="zipf", zipf_bias=True,
+    cfg = W.tiny_config(N=24576, n=5001, rows=40, dtype="bf16", trials=3, kept_rule="zipf", zipf_bias=True,
                         rho=0.7, seed=57)
     inp = W.make_inputs(cfg)
     tw = torch.zeros(cfg.rows, cfg.N + 24, dtype=torch.bfloat16)
@@ -391,9 +391,11 @@ def test_strided_rows_through_the_streaming_kernels():
     dw = torch.zeros(cfg.rows, cfg.n + 5, dtype=torch.bfloat16)
     dw[:, : cfg.n] = inp["drafter"]
     idx = rdk.rdk_prepare_ids(inp["kept_ids"].cuda(), cfg.N)
-    out = rdk.rdk_sample_and_verify(idx, B.RDK_MODE_LINEAR, tw.cuda()[:, : cfg.N], dw.cuda()[:, : cfg.n], None,
-                                    inp["uniforms"].cuda(), cfg.batch, cfg.positions)
+    z, y = tw.cuda()[:, : cfg.N], dw.cuda()[:, : cfg.n]
+    out = rdk.rdk_sample_and_verify(idx, B.RDK_MODE_LINEAR, z, y, None, inp["uniforms"].cuda(), cfg.batch, cfg.positions)
     torch.cuda.synchronize()
+    route, why = rdk.rdk_sample_route(idx, B.RDK_MODE_LINEAR, z, y, cfg.batch, cfg.positions, cfg.trials, out["_ws"])
+    assert route == B.RDK_ROUTE_STREAM_KERNEL, why
     B.check_status_word(out)
     PU.compare_sampling(inp, out, range(cfg.rows), "linear").assert_ok()
 
@@ -587,3 +589,17 @@ def test_linear_with_a_separate_prior(dtype, N, n, kind):
                                         inp["uniforms"].cuda(), cfg.batch, cfg.positions, KIND[kind])
     torch.cuda.synchronize()
     PU.compare_sampling(inp, a, range(cfg.rows), "linear").assert_ok()
+
+
+@pytest.mark.parametrize("N,n,rows,trials,streams", [(32768, 8192, 97, 1, False), (32768, 8192, 98, 1, True), (32768, 8192, 4, 3, True),
+                                                     (262144, 49152, 40, 1, False), (262144, 65536, 40, 1, True), (262144, 65536, 24, 1, False),
+                                                     (262144, 131072, 24, 1, True), (262144, 131072, 4, 1, False)])
+def test_route_of_few_rows(N, n, rows, trials, streams):
+    """The query names the kernel that runs: with few rows the cluster kernel, fewer of them where many tokens are kept."""
+    rdk = _rdk()
+    B = rdk.binding
+    idx = rdk.rdk_prepare_ids(torch.arange(n, dtype=torch.int32, device="cuda") * (N // n), N)
+    z, y = (torch.zeros(rows, k, dtype=torch.bfloat16, device="cuda") for k in (N, n))
+    ws = B.sample_workspace(B.make_problem(idx, z, y, rows, 1), B.RDK_MODE_LINEAR, trials, "cuda")
+    route, why = rdk.rdk_sample_route(idx, B.RDK_MODE_LINEAR, z, y, rows, 1, trials, ws)
+    assert (route == B.RDK_ROUTE_STREAM_KERNEL) == streams and ("few rows" in why) == (not streams), (route, why)
