@@ -1069,13 +1069,18 @@ const char* stream_ineligible(const RowParams& P, int tz, int ty, int kind, int 
 // cluster kernel, a quarter of the tokens kept, us:  8192 bf16: 11.0 / 8.5 for 4 rows, 14.6 / 11.4 for 160, 16.0 / 18.2 for 320;
 // 32768: 12.0 / 8.8 for 4, 16.2 / 15.5 for 96, 17.8 / 18.9 for 160; 128256: 12.8 / 10.3 for 4, 16.6 / 14.6 for 24, 18.6 / 20.9 for
 // 48; 262144: 13.7 / 11.1 for 4, 27.7 / 27.3 for 64; fp32 128256: 13.5 / 10.2 for 4, 32.0 / 31.6 for 96.  The cluster
-// kernel makes a row's draws in one CTA: not with many trials.
+// kernel makes a row's draws in one CTA: not with many trials.  It visits kept tokens beyond a warp's 384 register slots in
+// memory, twice: with more of them (a warp of the largest cluster has n / 128) fewer rows, and few beyond twice as many.  262144
+// tokens: 65536 kept, 24 rows 21.7 / 19.5, 56 rows 28.2 / 30.7; 131072 kept, 1 row 17.2 / 15.4, 8 17.7 / 18.2, 24 25.2 / 26.9.
 bool stream_few_rows(const RowParams& P, int tz, int ty, int kind) {
     if (P.trials > 2) return false;
     StreamSegs sg;
     const bool one_group = stream_segments(P.N, tz == RDK_F32 ? 4 : 2, sg) && sg.C == kMaxGroup;      // 9 groups of 16 CTAs
     int most = !fast_types(tz, ty, kind) ? 96 : (one_group ? 56 : 24);
     if (P.N <= 32768) { const int small = 3200000 / P.N; most = most > small ? most : (small < 192 ? small : 192); }
+    const int kept = P.n / 128;
+    if (kept > 384 && most > 24) most = 24;
+    if (kept > 768) most = 4;
     return P.rows <= most;
 }
 
