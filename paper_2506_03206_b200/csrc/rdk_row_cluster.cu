@@ -12,8 +12,8 @@
 // CTAs then exchange one record each through distributed shared memory (theta, 1/Z_p, 1/Z_q), the warps finish
 // their segment sums of w, min(p, q~), max(0, p - q~) and p and leave them in CTA 0.  The other CTAs are done then and
 // make room for the next rows; CTA 0 draws: prefix sums over the segments, the draw's segment read again (from L2), its
-// 256-position chunks shared by the warps.  (Draws made in place by the CTA that holds the segment kept whole clusters
-// waiting for two chains of dependent loads: 212 instead of 156 us for 320 rows of 128k with a prior.)
+// 256-position chunks shared by the warps.  (Draws made in place by the CTA that holds the segment would keep whole clusters
+// waiting for two chains of dependent loads.)
 //
 // Four variants:
 //   kVarSparse  N >= 4096, Eq. rdk-taylor with p itself.  A token that is not kept has q~ = theta x < p, x = p / N, so such
@@ -258,6 +258,9 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     const uint32_t zb0 = smem_u32(csm), pb0 = zb0 + g.zoff_p, qb0 = zb0 + g.zoff_q;
     const uint32_t zb = zb0 + (uint32_t)(warp * len) * es, pb = pb0 + (uint32_t)(warp * len) * es, qb = qb0 + (uint32_t)(warp * len) * 4u;
 
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");       // inputs may be the previous kernel's outputs, the index (a copy of one) too
+
     // header of the index and the ranks of the segment's ends: requested together, looked at when the copies are under way
     int4 h0 = make_int4(0, 0, 0, 0), h1 = h0;
     uint32_t end_word = 0;
@@ -267,8 +270,6 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
         h0 = __ldg(reinterpret_cast<const int4*>(P.header)); h1 = __ldg(reinterpret_cast<const int4*>(P.header) + 1);
         if (end_tok < P.N && lane < 2) { end_word = __ldg(P.mask + (end_tok >> 5)); end_rank = __ldg(P.rank + (end_tok >> 5)); }
     }
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");       // inputs may be the previous kernel's outputs
 
     {   // start the copies; positions without a token weigh nothing
         int zh, zl, ph = 0, pl = 0, qh = 0, ql = 0;
@@ -924,8 +925,7 @@ static bool plan_cluster(int N, int rows, int trials, size_t es, int variant, bo
     const long long positions = (long long)N + lead;
     int C = 1;
     if (N >= kStreamMinN) {
-        // three CTAs to an SM (their phases of copying, exponentials and waiting overlap; with one to an SM a prior of
-        // 128k tokens takes 515 us for 320 rows, with three 147) ...
+        // three CTAs to an SM, whose phases of copying, exponentials and waiting overlap (320 rows of 128k with a prior: 112 us) ...
         while (C < kCluMaxCtas && (long long)bytes * (positions / C) > 64 * 1024) C *= 2;
         // ... and, with few rows, enough CTAs to fill the chip four times over, while each has 4096 positions or more (with
         // less the exchange between the CTAs costs more than the sweep)

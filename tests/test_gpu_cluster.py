@@ -301,3 +301,26 @@ def test_many_draws_take_the_row_kernel(mode, N, rows, trials):
         a, b = (rdk.rdk_sample_and_verify(idx, m, z, y, w, u, rows, 1, flags=f) for f in (0, B.RDK_FLAG_ROW_KERNEL))
     for k in ("draft_token", "out_token", "accepted", "accept_prob", "alpha", "S", "residual_mass", "accepted_len"):
         assert torch.equal(a[k], b[k]), k
+
+
+def test_index_written_by_the_kernel_queued_just_before_the_call():
+    """An index is an input like any other: a copy of one, made on the stream just before the call into a buffer that held another
+    list's, is the one that the call uses.  The strided copy is a kernel that a long one holds up."""
+    rdk = _rdk()
+    B = rdk.binding
+    N, n, rows = 20011, 3001, 4
+    g = torch.Generator(device="cuda").manual_seed(4)
+    lists = [torch.randperm(N, generator=g, device="cuda")[:n].to(torch.int32) for _ in range(2)]
+    idx = [rdk.rdk_prepare_ids(x, N) for x in lists]
+    z = torch.randn(rows, N, generator=g, device="cuda").to(torch.bfloat16)
+    y, u = torch.randn(rows, n, generator=g, device="cuda").to(torch.bfloat16), torch.rand(rows, 1, 4, generator=g, device="cuda")
+    want = [rdk.rdk_sample_and_verify(i, B.RDK_MODE_LINEAR, z, y, None, u, rows, 1) for i in idx]
+    wide = [torch.stack([i.buffer, i.buffer], 1) for i in idx]
+    moved, big = B.KeptIndex(torch.empty_like(idx[0].buffer), N, n, n), torch.zeros(1 << 27, device="cuda")
+    moved.buffer.copy_(idx[0].buffer)
+    for k in range(1, 9):
+        big.add_(1.0)
+        moved.buffer.copy_(wide[k & 1][:, 0])
+        out = rdk.rdk_sample_and_verify(moved, B.RDK_MODE_LINEAR, z, y, None, u, rows, 1)
+        for name in ("draft_token", "alpha", "theta", "S"):
+            assert torch.equal(out[name], want[k & 1][name]), (k, name)
