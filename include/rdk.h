@@ -292,9 +292,9 @@ int rdk_sample_route(const rdk_problem* problem, int32_t mode, const void* targe
 
 /* ---------------------------------------------------------------------------------------------
  * rdk_test_set_spin_limit -- for tests of the failure path only (the paper has no counterpart).
- * Every wait inside the streaming kernel (on a shared-memory barrier, on a record another CTA
- * publishes) gives up after a number of failed tries, records RDK_ERR_TIMEOUT in
- * out->status_word and lets the kernel run to its end.  This sets that number for later calls of
+ * Every wait inside the streaming and cluster kernels (on a shared-memory barrier, on a record another
+ * CTA publishes) gives up after a number of failed tries, records RDK_ERR_TIMEOUT in
+ * out->status_word (rdk_emit_sequences: marks the token) and lets the kernel run to its end.  This sets that number for later calls of
  * this process; 0 restores the default (2^17 tries of up to 2 us each).  With a limit of 1 the waits of an ordinary call
  * run out, which is how the tests reach the failure path without hanging or faulting anything.
  * ------------------------------------------------------------------------------------------- */
@@ -354,6 +354,8 @@ int rdk_stream_geometry(int32_t N, int32_t n, int32_t target_dtype, int32_t draf
  *                            distribution after all drafts -- by inverse CDF with uniform lane 3 of
  *                            the sequence's last position,
  *   seq_len[b, t]          = j + 1  (between 1 and positions + 1).
+ * If a bounded wait inside the kernel expires (the call has no status word), the bonus token of that
+ * (sequence, trial) is -1.
  *   bonus_target  device [batch, N] target logits of problem->target_dtype, row stride in elements
  *                 (0 means N)
  *   uniforms, draft_token, accepted, out_token: as given to / produced by rdk_sample_and_verify

@@ -20,6 +20,7 @@ constexpr int kEmitMaxWarps = 16;
 constexpr int kEmitMaxCtas = 8;
 constexpr int kEmitMaxSeg = kEmitMaxCtas * kEmitMaxWarps;
 constexpr int kEmitBatch = 256;           // pairs whose answers are kept at a time
+constexpr unsigned kEmitSpin = 1u << 22;
 
 struct EmitParams {
     int N, batch, positions, trials, pad;
@@ -28,7 +29,23 @@ struct EmitParams {
     const float* uniforms;
     const int32_t* draft_token; const uint8_t* accepted; const int32_t* out_token;
     int32_t* seq_tokens; int32_t* seq_len;
+    unsigned spin_limit;
 };
+
+// Bounded wait of a warp for the phase of `bar`; a try may park the warp, except under the small limits of the failure-path
+// tests, whose tries must be able to run out.
+__device__ __forceinline__ bool emit_wait(uint32_t bar, uint32_t parity, unsigned limit) {
+    uint32_t done = 0;
+    for (unsigned spins = 0; !done && spins < limit; ++spins) {
+        if (limit < 64)
+            asm volatile("{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+                         : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+        else
+            asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+                         : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+    }
+    return __all_sync(0xffffffffu, done != 0);
+}
 
 // the 8 logits at position v * 8 of a row whose token 0 is at position `phase` (so that vectors are 16-byte aligned)
 template <typename TZ>
@@ -79,6 +96,7 @@ emit_kernel(const EmitParams P) {
     __shared__ float chunk_sum[32];
     __shared__ float bc[2];
     __shared__ __align__(8) unsigned long long rbar;     // CTA 0: the records of the row are in rec[]
+    __shared__ bool lost_s;                              // the wait for the records gave up
     __shared__ uint8_t all_s[kEmitBatch];                // whether all drafts of the pair were accepted
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     uint32_t rank, C;
@@ -138,10 +156,11 @@ emit_kernel(const EmitParams P) {
                              ::"r"(r), "r"(__float_as_uint(zs.m)), "r"(__float_as_uint(zs.s)), "r"(m) : "memory");
             }
             if (rank != 0) continue;
-            if (warp == 0)                               // the records are on their way from running CTAs; a limit all the same
-                for (unsigned spins = 0, done = 0; !done && spins < (1u << 22); ++spins)
-                    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-                                 : "=r"(done) : "r"(smem_u32(&rbar)), "r"(parity) : "memory");
+            if (warp == 0) {                             // the records are on their way from running CTAs; a limit all the same
+                const bool in = emit_wait(smem_u32(&rbar), parity, P.spin_limit);
+                if (!in) (void)emit_wait(smem_u32(&rbar), parity, kEmitSpin);      // (they must have landed before the CTA goes on, or leaves)
+                if (lane == 0) lost_s = !in;
+            }
             parity ^= 1u;
             constexpr int K = kEmitMaxSeg / 32;          // runs per lane
             if (warp == 0) {
@@ -174,6 +193,10 @@ emit_kernel(const EmitParams P) {
                 for (int k = 0; k < K; ++k) if (k < per && lane * per + k < nseg) cdf[lane * per + k] = before + v[k];
             }
             __syncthreads();
+            if (lost_s) {                                // no draw from records that may not be the row's
+                if (tid == 0) P.seq_tokens[(long long)pair * (P.positions + 1) + P.positions] = -1;
+                continue;
+            }
             const float off = bc[0], inv_z = bc[1];
             const double thr = (double)u * cdf[nseg - 1];
             const int s = warp_first_above(cdf, nseg, thr, lane);
@@ -278,6 +301,7 @@ extern "C" int rdk_emit_sequences(const rdk_problem* problem, const void* bonus_
     P.bonus = bonus_target; P.bonus_stride = bonus_row_stride ? bonus_row_stride : problem->N;
     P.uniforms = uniforms; P.draft_token = draft_token; P.accepted = accepted; P.out_token = out_token;
     P.seq_tokens = seq_tokens; P.seq_len = seq_len;
+    P.spin_limit = stream_spin_limit() ? stream_spin_limit() : kEmitSpin;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const cudaError_t e = problem->target_dtype == RDK_F32 ? launch_emit<float>(P, s) : launch_emit<__nv_bfloat16>(P, s);
     if (e != cudaSuccess) return cuda_fail(e, "emit kernel launch");

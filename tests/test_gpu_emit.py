@@ -46,3 +46,27 @@ def test_emit_sequences(N, positions, dtype):
                 ambiguous += 1
             assert np.all(seq[b, t, ln[b, t]:] == -1)                      # entries beyond the length are untouched
     assert ambiguous <= 1
+
+
+def test_a_bonus_draw_whose_wait_runs_out_is_marked():
+    """With one try for the wait for the records of the other CTAs, rows that clusters share give -1 in place of the bonus token
+    (or the right one, where the records were there already); nothing else changes, and the next call is right."""
+    rdk = _rdk()
+    N, batch = 140000, 64
+    g = torch.Generator(device="cuda").manual_seed(6)
+    bonus = torch.randn(batch, N, generator=g, device="cuda").to(torch.bfloat16)
+    u = torch.rand(batch * 2, 1, 4, generator=g, device="cuda")
+    acc, tok = torch.ones(batch, 2, 1, dtype=torch.uint8, device="cuda"), torch.arange(batch * 2, dtype=torch.int32, device="cuda")
+    acc[5, 1] = 0
+    good, ln = rdk.rdk_emit_sequences(N, batch, 2, bonus, u, tok, acc, tok)
+    try:
+        rdk.rdk_test_set_spin_limit(1)
+        seq, ln1 = rdk.rdk_emit_sequences(N, batch, 2, bonus, u, tok, acc, tok)
+        torch.cuda.synchronize()
+    finally:
+        rdk.rdk_test_set_spin_limit(0)
+    last = seq[:, 0, 2] == good[:, 0, 2]
+    assert torch.equal(ln, ln1) and torch.equal(seq[:, :, :2], good[:, :, :2]) and torch.all(last | (seq[:, 0, 2] == -1))
+    assert int((~last).sum()) > 0
+    again, _ = rdk.rdk_emit_sequences(N, batch, 2, bonus, u, tok, acc, tok)
+    assert torch.equal(again, good)
