@@ -4,6 +4,7 @@ from __future__ import annotations
 import json
 import math
 import os
+import tempfile
 from typing import Dict, Iterable, Optional
 
 import numpy as np
@@ -79,14 +80,11 @@ class Tally:
         assert amb <= allowed, f"{amb} ambiguous draws, {allowed} allowed: " + self.summary()
 
     def record(self, name: str):
-        """Keep the tally: one JSON line per comparison in parity_tallies.jsonl (next to the other run
-        outputs when that folder exists, else in the working directory), and on stdout."""
+        """Keep the tally: one JSON line per comparison in parity_tallies.jsonl, among the temporary files, and on stdout."""
         line = {"case": name, "rows": self.rows, "draws": self.draws, "ambiguous_draft": self.ambiguous_draft,
                 "ambiguous_accept": self.ambiguous_accept, "ambiguous_residual": self.ambiguous_residual,
                 "failures": len(self.failures), "max_abs": {k: float("%.3g" % v) for k, v in self.max_abs.items()}}
-        root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
-        folder = os.path.join(root, "gpurun_out")
-        path = os.path.join(folder if os.path.isdir(folder) else os.getcwd(), "parity_tallies.jsonl")
+        path = os.path.join(tempfile.gettempdir(), "parity_tallies.jsonl")
         try:
             with open(path, "a") as f:
                 f.write(json.dumps(line) + "\n")

@@ -136,7 +136,11 @@ def test_emitted_sequences_of_many_pairs(N, batch, positions, trials):
 # rows: one instruction of the smallest width, the steps of 16, both instructions, several row tiles, halves of the last
 # round; tokens: less than, exactly and just over a CTA's 128 and a pair's 256; contraction: around one block of 64
 @pytest.mark.parametrize("N,n,rows", [(127, 63, 1), (128, 64, 16), (129, 65, 33), (255, 8, 256), (257, 129, 257), (5000, 200, 300),
-                                      (300, 1000, 513), (19200, 72, 1024), (38000, 640, 320), (4096, 192, 1100)])
+                                      (300, 1000, 513), (19200, 72, 1024), (38000, 640, 320), (4096, 192, 1100),
+                                      # two instructions of R rows each, 74 pairs: R = 144, in one round and with halved items; 176,
+                                      # 208 and 240; two and three row tiles; a last row tile of one instruction
+                                      (18944, 300, 257), (19100, 300, 288), (25000, 200, 340), (25000, 200, 410), (30000, 136, 470),
+                                      (20000, 100, 700), (33000, 70, 1030), (2000, 70, 8200)])
 def test_paired_contraction_at_tile_edges(N, n, rows):
     rdk = _rdk()
     B = rdk.binding
@@ -146,8 +150,8 @@ def test_paired_contraction_at_tile_edges(N, n, rows):
     idx = rdk.rdk_prepare_ids(ids, N)
     # probabilities that are multiples of 2^-12 and add up to 1: exact in bf16, so that q' is too
     q = torch.zeros(rows, n, device="cuda")
-    live = min(n, N, 16)
-    q[:, torch.randperm(min(n, N), generator=g, device="cuda")[:live]] = 1.0 / (1 << (live.bit_length() - 1))
+    live = min(n, N, 16)                             # columns of its own for every row: a row in another's place shows
+    q.scatter_(1, torch.rand(rows, min(n, N), generator=g, device="cuda").argsort(1)[:, :live], 1.0 / (1 << (live.bit_length() - 1)))
     q = q / q.sum(1, keepdim=True) if live & (live - 1) else q
     M = {"data": torch.rand(N, (n + 7) // 8 * 8, generator=g, device="cuda").to(torch.bfloat16), "layout": B.RDK_AFF_BF16_COLS, "ld": (n + 7) // 8 * 8}
     w = torch.full((rows, N), float("nan"), device="cuda")

@@ -190,7 +190,7 @@ def test_exact_probability_drafter_fp32():
 @pytest.mark.parametrize("N,n,rows", [(300, 33, 9), (2050, 130, 17), (1000, 520, 300), (4096, 1024, 384),
                                       (777, 64, 129), (256, 8, 1)])
 def test_exact_tensor_core_shapes(N, n, rows):
-    # several 256 x 256 output tiles, ragged edges in all three dimensions, one- and two-MMA row tiles
+    # several tiles of 256 tokens, ragged edges in all three dimensions, up to five row tiles of one instruction each
     _exact_case(W.tiny_config(N=N, n=n, rows=rows, trials=2, emb_dim=8, seed=N + n + rows, dtype="bf16"), "bf16")
 
 
