@@ -51,7 +51,7 @@ def test_emit_sequences(N, positions, dtype):
 def test_a_bonus_draw_whose_wait_runs_out_is_marked():
     """With one try for the wait for the records of the other CTAs, rows that clusters share give -1 in place of the bonus token
     (or the right one, where the records were there already); nothing else changes, and the next call is right."""
-    rdk = _rdk()
+    import paper_2506_03206_b200 as rdk
     N, batch = 140000, 64
     g = torch.Generator(device="cuda").manual_seed(6)
     bonus = torch.randn(batch, N, generator=g, device="cuda").to(torch.bfloat16)
