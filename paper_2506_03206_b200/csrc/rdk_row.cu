@@ -442,6 +442,7 @@ static bool many_draws(const RowParams& P, int mode, size_t es) {
     const long long draws = (long long)P.rows * P.trials;
     if (mode == RDK_MODE_LINEAR) return draws >= (P.prior ? 9600 : 10240);
     const bool aligned = !(((uintptr_t)P.target | (uintptr_t)P.w) & 15u) && !((P.target_stride * (long long)es | P.w_stride * 4) & 15);
+    if (P.trials >= 256 && P.N > 65536) return true;         // (4 rows x 256 of 262143: 194 / 310)
     if (!aligned) return draws >= 5120;
     return P.trials >= 64 ? draws >= 2560 : draws >= (P.N <= 131072 ? 1600 : 5120);
 }

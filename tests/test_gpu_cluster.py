@@ -284,7 +284,7 @@ def test_written_out_q_errors_against_64_bits(N, n):
     assert square ** 0.5 <= 2.0 ** 0.5 * 2.0 ** -24, square ** 0.5 * 2 ** 24
 
 
-@pytest.mark.parametrize("mode,N,rows,trials", [("given", 4096, 100, 16), ("given", 33001, 20, 256), ("given", 262144, 40, 64), ("linear", 5000, 160, 64),
+@pytest.mark.parametrize("mode,N,rows,trials", [("given", 4096, 100, 16), ("given", 33001, 20, 256), ("given", 262144, 40, 64), ("given", 70001, 2, 256), ("linear", 5000, 160, 64),
                                                 ("linear", 70001, 5, 2048), ("prior", 9000, 150, 64)])
 def test_many_draws_take_the_row_kernel(mode, N, rows, trials):
     """Where draws outweigh the sweep the one-CTA-per-row kernel serves, so every output has that kernel's bits."""
