@@ -259,8 +259,9 @@ int rdk_redistribute_linear(const rdk_problem* problem, const void* target, cons
  * problem, and one of few rows, takes the cluster kernel: a thread-block cluster of up to 16 CTAs holds the
  * row in its shared memory and goes from the logits to the draws in one launch (any alignment, any order of the ids,
  * any N whose row fits; exact division below N = 4096).  The one-CTA-per-row kernel (three sweeps over the row,
- * exact division), several times slower, serves what remains and RDK_FLAG_ROW_KERNEL;
- * rdk_sample_route tells whether the streaming kernels can serve and why not.  Both
+ * exact division), several times slower, serves what remains, calls of very many draws (which outweigh the sweep)
+ * and RDK_FLAG_ROW_KERNEL;
+ * rdk_sample_route tells whether the streaming kernels serve and why not.  Both
  * streaming kernels are launched with programmatic stream serialisation: each may set itself up
  * while the previous kernel of the stream drains, but reads none of its inputs and touches nothing
  * of the workspace before that kernel is complete, so inputs written by the kernel queued just
