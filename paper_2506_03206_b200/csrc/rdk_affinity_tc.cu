@@ -19,8 +19,10 @@
 // of the entry at tau = 0.1, 5e-3 at 1e-5; some ten of 32064 diagonal entries, the heaviest of a row, then land on
 // another bf16 number, which moves draws.)
 // Both are bound by the special-function unit (one exponential per element and pass: 2 x 60 us at 16 per clock and SM)
-// and by the write of the matrix (537 MB: 82 us).  The chain that this replaces, with an fp32 scratch between the GEMM
-// and three streaming passes, took 1490 us for that size.
+// and by the write of the matrix (537 MB: 82 us).  CTAs side by side share an operand tile in either pass, and the epilogue of
+// both has sixteen warps with a block of 64 columns each: 277 us for that size (with four tiles in a row to a CTA for the sums and
+// eight warps with two store buffers each for the write 288).  Sums of one panel of kept ids and the matrix of
+// another in one launch, so that exponentials and stores overlap, were slower: two panels 286, four 311.
 #include <math.h>
 
 #include "rdk_device.cuh"
@@ -32,15 +34,13 @@ constexpr int kAffM = 128, kAffN = 256, kAffK = 64;
 constexpr int kAffABytes = kAffM * kAffK * 2, kAffBBytes = kAffN * kAffK * 2;       // 16 KB, 32 KB
 constexpr int kAffStage = kAffABytes + kAffBBytes;
 constexpr int kAffStages = 3;
-// Epilogue warps: 16 for the sums, whose exponentials need the latency hidden (101 us instead of 118 with 8), 8 with two
-// store buffers each for the write, which waits for memory (170 us instead of 181 with 16).
-constexpr int kAffSumWarps = 16, kAffWriteWarps = 8;
-constexpr int kAffStoreBuffers = 16;
+constexpr int kAffEpiWarps = 16;                         // their exponentials need the latency hidden (sums alone: 101 us, with 8 118)
+constexpr int kAffCols = 4 * kAffN / kAffEpiWarps;       // columns of a tile per epilogue warp
 constexpr int kAffStoreBytes = 32 * 128;                 // a warp's 32 rows x 64 bf16
-constexpr int kAffSmem = kAffStages * kAffStage + kAffStoreBuffers * kAffStoreBytes + 1024;
-constexpr int kAffSpan = 4;                              // column tiles per work item of kAffSums
-constexpr int kAffBlock = 64;                            // tokens summed one after the other: an epilogue warp's columns in kAffSums
-static_assert(4 * kAffN / kAffSumWarps == kAffBlock, "a warp of kAffSums leaves one sum per tile");
+constexpr int kAffSmem = kAffStages * kAffStage + kAffEpiWarps * kAffStoreBytes + 1024;
+constexpr int kAffBlock = 64;                            // tokens summed one after the other
+static_assert(kAffCols == kAffBlock, "an epilogue warp leaves one sum per tile, or fills one store buffer");
+constexpr int kAffThreads = 64 + 32 * kAffEpiWarps;
 constexpr uint32_t kAffIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kAffN >> 3) << 17) | ((uint32_t)(kAffM >> 4) << 24);
 
 constexpr float kAffZeroInv = 1e12f;                     // inverse norm of a zero embedding
@@ -50,23 +50,20 @@ enum { kAffSums = 0, kAffWrite = 1 };
 
 struct AffParams {
     int N, n, num_kb;
-    int tiles_m, tiles_n, num_items;   // row tiles, column tiles (kAffSums: spans of kAffSpan column tiles), work items
-    int cols;                          // columns in all
-    const float* row_inv;              // 1 / |e| of the rows, zero-padded to whole tiles
-    const float* col_inv;              // 1 / |e| of the columns, zero-padded to whole tiles
-    const float* col_z;                // kAffWrite: 1 / Z of every column (0: no weight)
+    int row_tiles, col_tiles;          // sums: kept ids x tokens; write: tokens x kept ids
+    const float* row_inv;              // 1 / |e| of the rows and of the columns, zero-padded to whole tiles
+    const float* col_inv;
+    const float* z;                    // kAffWrite: 1 / Z of every kept id (0: no weight)
     float scale;                       // log2(e) / tau
-    float* part;                       // kAffSums: [blocks of kAffBlock tokens][row tiles * 128]
+    float* part;                       // kAffSums: [blocks of kAffBlock tokens][npad]
+    int npad;
     int32_t* status;
 };
 
-constexpr int aff_threads(int mode) { return 64 + 32 * (mode == kAffSums ? kAffSumWarps : kAffWriteWarps); }
-
 template <int MODE>
-__global__ void __launch_bounds__(aff_threads(MODE), 1)
+__global__ void __launch_bounds__(kAffThreads, 1)
 aff_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__ CUtensorMap tmapB, const __grid_constant__ CUtensorMap tmapC, const AffParams P) {
-    constexpr int kEpi = MODE == kAffSums ? kAffSumWarps : kAffWriteWarps, kCols = 4 * kAffN / kEpi;     // columns per epilogue warp
-    constexpr int kBufs = kAffStoreBuffers / kEpi;
+    constexpr bool kWrite = MODE == kAffWrite;
     extern __shared__ __align__(1024) unsigned char aff_smem[];
     unsigned char* tiles = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(aff_smem) + 1023) & ~uintptr_t(1023));
     __shared__ __align__(8) unsigned long long full_bar[kAffStages], empty_bar[kAffStages], acc_full[2], acc_empty[2];
@@ -82,7 +79,7 @@ aff_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__
         }
         for (int a = 0; a < 2; ++a) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(s32(&acc_full[a])));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(s32(&acc_empty[a])), "r"(kEpi));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(s32(&acc_empty[a])), "r"(kAffEpiWarps));
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -94,152 +91,150 @@ aff_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = tmem_base_s;
-    constexpr int kSpan = MODE == kAffSums ? kAffSpan : 1;
-    const int col_tiles = (P.cols + kAffN - 1) / kAffN;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-    // every role walks the same sequence: items blockIdx.x, + gridDim.x, ...; in an item up to kSpan column tiles
+    // Every role walks the same sequence of tiles: blockIdx.x, + gridDim.x, ...  CTAs side by side take the tiles of one row of
+    // tiles of the matrix when it is written (whole rows of it are under way then) and those of one column of tiles, the
+    // same tokens, for the sums.
+    const int num_tiles = P.row_tiles * P.col_tiles;
+    auto walk = [&](auto&& tile) {
+        for (int j = blockIdx.x; j < num_tiles; j += gridDim.x) {
+            const int row = kWrite ? j / P.col_tiles : j % P.row_tiles, col = kWrite ? j % P.col_tiles : j / P.row_tiles;
+            if (!tile(row * kAffM, col * kAffN)) return;
+        }
+    };
     if (warp == 0) {
         int stage = 0;
         uint32_t phase = 0;
-        bool ok = true;
-        for (int item = blockIdx.x; item < P.num_items && ok; item += gridDim.x) {
-            const int tm = item / P.tiles_n, tn0 = (item % P.tiles_n) * kSpan;
-            for (int tn = tn0; tn < min(tn0 + kSpan, col_tiles) && ok; ++tn)
-                for (int kb = 0; kb < P.num_kb; ++kb) {
-                    if (!tc_wait(&empty_bar[stage], phase ^ 1u, abort)) { ok = false; break; }
-                    if (elect_one()) {
-                        const uint32_t sa = s32(tiles + stage * kAffStage), bar = s32(&full_bar[stage]);
-                        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"((uint32_t)kAffStage) : "memory");
-                        asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-                                     ::"r"(sa), "l"(reinterpret_cast<uint64_t>(&tmapA)), "r"(kb * kAffK), "r"(tm * kAffM), "r"(bar) : "memory");
-                        asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-                                     ::"r"(sa + kAffABytes), "l"(reinterpret_cast<uint64_t>(&tmapB)), "r"(kb * kAffK), "r"(tn * kAffN), "r"(bar) : "memory");
-                    }
-                    __syncwarp();
-                    if (++stage == kAffStages) { stage = 0; phase ^= 1u; }
+        walk([&](int row, int col) -> bool {
+            for (int kb = 0; kb < P.num_kb; ++kb) {
+                if (!tc_wait(&empty_bar[stage], phase ^ 1u, abort)) return false;
+                if (elect_one()) {
+                    const uint32_t sa = s32(tiles + stage * kAffStage), bar = s32(&full_bar[stage]);
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"((uint32_t)kAffStage) : "memory");
+                    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+                                 ::"r"(sa), "l"(reinterpret_cast<uint64_t>(&tmapA)), "r"(kb * kAffK), "r"(row), "r"(bar) : "memory");
+                    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+                                 ::"r"(sa + kAffABytes), "l"(reinterpret_cast<uint64_t>(&tmapB)), "r"(kb * kAffK), "r"(col), "r"(bar) : "memory");
                 }
-        }
+                __syncwarp();
+                if (++stage == kAffStages) { stage = 0; phase ^= 1u; }
+            }
+            return true;
+        });
     } else if (warp == 1) {
         const uint64_t adesc0 = smem_desc(s32(tiles));
         int stage = 0, acc = 0;
         uint32_t phase = 0, acc_phase = 0;
-        bool ok = true;
-        for (int item = blockIdx.x; item < P.num_items && ok; item += gridDim.x) {
-            const int tn0 = (item % P.tiles_n) * kSpan;
-            for (int tn = tn0; tn < min(tn0 + kSpan, col_tiles) && ok; ++tn) {
-                if (!tc_wait(&acc_empty[acc], acc_phase ^ 1u, abort)) { ok = false; break; }
+        walk([&](int, int) -> bool {
+            if (!tc_wait(&acc_empty[acc], acc_phase ^ 1u, abort)) return false;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            for (int kb = 0; kb < P.num_kb; ++kb) {
+                if (!tc_wait(&full_bar[stage], phase, abort)) return false;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                for (int kb = 0; kb < P.num_kb; ++kb) {
-                    if (!tc_wait(&full_bar[stage], phase, abort)) { ok = false; break; }
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    if (elect_one()) {
-                        const uint64_t ad = adesc0 + (uint64_t)(stage * (kAffStage >> 4));
-                        mma_kblock<1>(tmem_base + (uint32_t)(acc * kAffN), ad, ad + (kAffABytes >> 4), kAffIdesc, kb > 0);
-                        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(s32(&empty_bar[stage])) : "memory");
-                    }
-                    __syncwarp();
-                    if (++stage == kAffStages) { stage = 0; phase ^= 1u; }
+                if (elect_one()) {
+                    const uint64_t ad = adesc0 + (uint64_t)(stage * (kAffStage >> 4));
+                    mma_kblock<1>(tmem_base + (uint32_t)(acc * kAffN), ad, ad + (kAffABytes >> 4), kAffIdesc, kb > 0);
+                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(s32(&empty_bar[stage])) : "memory");
                 }
-                if (!ok) break;
-                if (lane == 0)
-                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(s32(&acc_full[acc])) : "memory");
                 __syncwarp();
-                if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+                if (++stage == kAffStages) { stage = 0; phase ^= 1u; }
             }
-        }
+            if (lane == 0)
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(s32(&acc_full[acc])) : "memory");
+            __syncwarp();
+            if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+            return true;
+        });
     } else {
-        int buf = 0;
-        const int quarter = warp & 3, share = (warp - 2) >> 2;       // TMEM lanes 32 quarter .. + 32, columns kCols share .. + kCols
-        const uint32_t taddr0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(share * kCols);
-        unsigned char* stage_c = tiles + kAffStages * kAffStage + (warp - 2) * kBufs * kAffStoreBytes;
+        const int quarter = warp & 3, share = (warp - 2) >> 2;       // TMEM lanes 32 quarter .. + 32, columns kAffCols share .. + kAffCols
+        const uint32_t taddr0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(share * kAffCols);
+        const uint32_t store = s32(tiles + kAffStages * kAffStage + (warp - 2) * kAffStoreBytes);
         int acc = 0;
         uint32_t acc_phase = 0;
-        bool ok = true;
-        for (int item = blockIdx.x; item < P.num_items && ok; item += gridDim.x) {
-            const int tm = item / P.tiles_n, tn0 = (item % P.tiles_n) * kSpan;
-            const int row = tm * kAffM + quarter * 32 + lane;
-            const float2 ri = splat(__ldg(P.row_inv + row)), sc = splat(P.scale), neg = splat(-1.f);
+        const float2 sc = splat(P.scale), neg = splat(-1.f);
+        walk([&](int row0, int col0) -> bool {
+            const int row = row0 + quarter * 32 + lane, c0 = col0 + share * kAffCols;
+            const float2 ri = splat(__ldg(P.row_inv + row));
             // 2^((G x - 1) scale) of two columns
-            auto weight2 = [&](uint32_t g0, uint32_t g1, float c0, float c1) -> float2 {
-                return ex2_2(fmul2(ffma2(make_float2(__uint_as_float(g0), __uint_as_float(g1)), fmul2(make_float2(c0, c1), ri), neg), sc));
+            auto weight2 = [&](uint32_t g0, uint32_t g1, float k0, float k1) -> float2 {
+                return ex2_2(fmul2(ffma2(make_float2(__uint_as_float(g0), __uint_as_float(g1)), fmul2(make_float2(k0, k1), ri), neg), sc));
             };
-            for (int tn = tn0; tn < min(tn0 + kSpan, col_tiles); ++tn) {
-                const int c0 = tn * kAffN + share * kCols;
-                if (!tc_wait(&acc_full[acc], acc_phase, abort)) { ok = false; break; }
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                float sum = 0.f;
-                uint32_t v[2][32];
-                tmem_ld32(taddr0 + (uint32_t)(acc * kAffN), v[0]);
+            if (!tc_wait(&acc_full[acc], acc_phase, abort)) return false;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            float sum = 0.f;
+            uint32_t v[2][32];
+            tmem_ld32(taddr0 + (uint32_t)(acc * kAffN), v[0]);
+            if (kWrite) {                                            // the warp's last store has been read
+                if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                __syncwarp();
+            }
 #pragma unroll
-                for (int c = 0; c < kCols / 32; ++c) {
-                    tmem_wait_ld(v[c & 1]);
-                    if (c < kCols / 32 - 1) tmem_ld32(taddr0 + (uint32_t)(acc * kAffN + (c + 1) * 32), v[(c + 1) & 1]);
-                    uint32_t (&x)[32] = v[c & 1];
-                    if (c == kCols / 32 - 1) {                       // the accumulator is in registers: the next tile may have it
-                        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                        __syncwarp();
-                        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(s32(&acc_empty[acc])) : "memory");
+            for (int c = 0; c < 2; ++c) {
+                tmem_wait_ld(v[c]);
+                uint32_t (&x)[32] = v[c];
+                if (c == 0) {
+                    tmem_ld32(taddr0 + (uint32_t)(acc * kAffN + 32), v[1]);
+                } else {                                             // the accumulator is in registers: the next tile may have it
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(s32(&acc_empty[acc])) : "memory");
+                }
+                const int col = c0 + c * 32;
+                const float4* ci = reinterpret_cast<const float4*>(P.col_inv + col);
+                if (!kWrite) {
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        const float4 k4 = __ldg(ci + q);
+                        float2 e0 = weight2(x[4 * q], x[4 * q + 1], k4.x, k4.y), e1 = weight2(x[4 * q + 2], x[4 * q + 3], k4.z, k4.w);
+                        if (col + 32 > P.N) {                        // tokens beyond the vocabulary have no weight
+                            const int left = P.N - col - 4 * q;
+                            if (left < 1) e0.x = 0.f;
+                            if (left < 2) e0.y = 0.f;
+                            if (left < 3) e1.x = 0.f;
+                            if (left < 4) e1.y = 0.f;
+                        }
+                        sum += e0.x; sum += e0.y; sum += e1.x; sum += e1.y;
                     }
-                    const int col = c0 + c * 32;
-                    const float4* ci = reinterpret_cast<const float4*>(P.col_inv + col);
-                    if (MODE == kAffSums) {
+                } else {
+                    const float4* cz = reinterpret_cast<const float4*>(P.z + col);
+                    const uint32_t rowaddr = store + (uint32_t)lane * 128u;
 #pragma unroll
-                        for (int q = 0; q < 8; ++q) {
-                            const float4 k4 = __ldg(ci + q);
-                            float2 e0 = weight2(x[4 * q], x[4 * q + 1], k4.x, k4.y), e1 = weight2(x[4 * q + 2], x[4 * q + 3], k4.z, k4.w);
-                            if (col + 32 > P.cols) {                 // tokens beyond the vocabulary have no weight
-                                const int left = P.cols - col - 4 * q;
-                                if (left < 1) e0.x = 0.f;
-                                if (left < 2) e0.y = 0.f;
-                                if (left < 3) e1.x = 0.f;
-                                if (left < 4) e1.y = 0.f;
-                            }
-                            sum += e0.x; sum += e0.y; sum += e1.x; sum += e1.y;
-                        }
-                    } else {
-                        const float4* cz = reinterpret_cast<const float4*>(P.col_z + col);
-                        if ((c & 1) == 0) {                          // the staging buffer's last store has been read
-                            if (lane == 0) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kBufs - 1) : "memory");
-                            __syncwarp();
-                        }
-                        const uint32_t rowaddr = s32(stage_c + buf * kAffStoreBytes) + (uint32_t)lane * 128u;
+                    for (int q = 0; q < 8; q += 2) {
+                        uint32_t w[4];
 #pragma unroll
-                        for (int q = 0; q < 8; q += 2) {
-                            uint32_t w[4];
-#pragma unroll
-                            for (int h = 0; h < 2; ++h) {
-                                const float4 k4 = __ldg(ci + q + h), z4 = __ldg(cz + q + h);
-                                const int i = 4 * (q + h);
-                                const float2 e0 = fmul2(weight2(x[i], x[i + 1], k4.x, k4.y), make_float2(z4.x, z4.y));
-                                const float2 e1 = fmul2(weight2(x[i + 2], x[i + 3], k4.z, k4.w), make_float2(z4.z, z4.w));
-                                asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w[2 * h]) : "f"(e0.y), "f"(e0.x));
-                                asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w[2 * h + 1]) : "f"(e1.y), "f"(e1.x));
-                            }
-                            // 16-byte chunk (c & 1) * 4 + q / 2 of the row, at its place in the 128-byte swizzle
-                            const uint32_t chunk = (uint32_t)((c & 1) * 4 + q / 2) ^ (uint32_t)(lane & 7);
-                            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(rowaddr + chunk * 16u), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]) : "memory");
+                        for (int h = 0; h < 2; ++h) {
+                            const float4 k4 = __ldg(ci + q + h), z4 = __ldg(cz + q + h);
+                            const int i = 4 * (q + h);
+                            const float2 e0 = fmul2(weight2(x[i], x[i + 1], k4.x, k4.y), make_float2(z4.x, z4.y));
+                            const float2 e1 = fmul2(weight2(x[i + 2], x[i + 3], k4.z, k4.w), make_float2(z4.z, z4.w));
+                            asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w[2 * h]) : "f"(e0.y), "f"(e0.x));
+                            asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w[2 * h + 1]) : "f"(e1.y), "f"(e1.x));
                         }
-                        if (c & 1) {                                 // 64 columns are complete
-                            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                            __syncwarp();
-                            if (lane == 0) {
-                                const int x0 = c0 + (c >> 1) * 64, y0 = tm * kAffM + quarter * 32;
-                                if (x0 < P.n && y0 < P.N)
-                                    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];"
-                                                 ::"l"(reinterpret_cast<uint64_t>(&tmapC)), "r"(x0), "r"(y0), "r"(s32(stage_c + buf * kAffStoreBytes)) : "memory");
-                                asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-                            }
-                            if (++buf == kBufs) buf = 0;
-                        }
+                        // 16-byte chunk c * 4 + q / 2 of the row, at its place in the 128-byte swizzle
+                        const uint32_t chunk = (uint32_t)(c * 4 + q / 2) ^ (uint32_t)(lane & 7);
+                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(rowaddr + chunk * 16u), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]) : "memory");
                     }
                 }
-                if (MODE == kAffSums) P.part[(long long)(c0 / kAffBlock) * (P.tiles_m * kAffM) + row] = sum;
-                if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
             }
-        }
-        if (MODE == kAffWrite && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+            if (kWrite) {                                            // (read while the next tile is waited for and evaluated)
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) {
+                    const int y0 = row0 + quarter * 32;
+                    if (c0 < P.n && y0 < P.N)
+                        asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];"
+                                     ::"l"(reinterpret_cast<uint64_t>(&tmapC)), "r"(c0), "r"(y0), "r"(store) : "memory");
+                    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                }
+            } else {
+                P.part[(long long)(c0 / kAffBlock) * P.npad + row] = sum;
+            }
+            if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+            return true;
+        });
+        if (kWrite && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     }
     // after a wait that gave up, copies may still be on their way into shared memory: let them land (bounded as well)
     if (abort_s && warp == 0)
@@ -403,21 +398,15 @@ int build_affinity_tc(const __nv_bfloat16* E, int d, long long estride, const in
     RDK_CUDA(cudaFuncSetAttribute(aff_tc_kernel<kAffSums>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAffSmem));
     RDK_CUDA(cudaFuncSetAttribute(aff_tc_kernel<kAffWrite>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAffSmem));
     AffParams P;
-    P.N = N; P.n = n; P.num_kb = (d + kAffK - 1) / kAffK; P.scale = scale; P.status = status; P.part = part;
-    // sums: rows = kept ids, columns = tokens
-    P.tiles_m = L.npad / kAffM; P.tiles_n = (L.Npad / kAffN + kAffSpan - 1) / kAffSpan; P.cols = N;
-    P.row_inv = invk; P.col_inv = inv; P.col_z = nullptr;
-    const long long items = (long long)P.tiles_m * P.tiles_n;
-    const long long items_w = (long long)(L.Npad / kAffM) * (L.npad / kAffN);
-    if (items > 0x7fffffffLL || items_w > 0x7fffffffLL) { set_error("rdk_build_affinity: too many tiles"); return RDK_ERR_UNSUPPORTED; }
-    P.num_items = (int)items;
-    RDK_CUDA(launch_pdl(aff_tc_kernel<kAffSums>, (unsigned)(items < sms ? items : sms), (unsigned)aff_threads(kAffSums), (size_t)kAffSmem, s, keptA, tokB, out, P));
+    P.N = N; P.n = n; P.num_kb = (d + kAffK - 1) / kAffK; P.scale = scale; P.status = status; P.part = part; P.npad = L.npad; P.z = z;
+    const long long tiles = (long long)(L.npad / kAffM) * (L.Npad / kAffN);       // of either pass
+    if (tiles > 0x7fffffffLL) { set_error("rdk_build_affinity: too many tiles"); return RDK_ERR_UNSUPPORTED; }
+    const unsigned grid = (unsigned)(tiles < sms ? tiles : sms);
+    P.row_tiles = L.npad / kAffM; P.col_tiles = L.Npad / kAffN; P.row_inv = invk; P.col_inv = inv;
+    RDK_CUDA(launch_pdl(aff_tc_kernel<kAffSums>, grid, (unsigned)kAffThreads, (size_t)kAffSmem, s, keptA, tokB, out, P));
     RDK_CUDA(launch_pdl(aff_norm_kernel, (unsigned)(L.npad / 32), 256u, 0, s, (const float*)part, (const float*)invk, z, L.blocks, L.npad));
-    // the matrix: rows = tokens, columns = kept ids
-    P.tiles_m = L.Npad / kAffM; P.tiles_n = L.npad / kAffN; P.cols = n;
-    P.row_inv = inv; P.col_inv = invk; P.col_z = z;
-    P.num_items = (int)items_w;
-    RDK_CUDA(launch_pdl(aff_tc_kernel<kAffWrite>, (unsigned)(items_w < sms ? items_w : sms), (unsigned)aff_threads(kAffWrite), (size_t)kAffSmem, s, tokA, keptB, out, P));
+    P.row_tiles = L.Npad / kAffM; P.col_tiles = L.npad / kAffN; P.row_inv = inv; P.col_inv = invk;
+    RDK_CUDA(launch_pdl(aff_tc_kernel<kAffWrite>, grid, (unsigned)kAffThreads, (size_t)kAffSmem, s, tokA, keptB, out, P));
     RDK_CUDA(launch_pdl(aff_finish_kernel, (unsigned)((n + wpb - 1) / wpb), 256u, 0, s, (const int32_t*)status, (const float*)invk, (const float*)z, Mt, ld, n, N));
     return RDK_OK;
 }
