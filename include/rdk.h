@@ -312,11 +312,18 @@ void rdk_test_set_spin_limit(uint32_t limit);
  *   prior_row_stride  elements between prior rows; 0 means one row shared by all rows
  * Everything else as in rdk_sample_and_verify (mode RDK_MODE_LINEAR) and rdk_redistribute_linear.
  * These calls take the cluster kernel (the one-CTA-per-row kernel where a row does not fit a cluster) and need no
- * workspace.
+ * workspace.  Given one (rdk_sample_and_verify_prior_ws; contents, alignment and sharing as in rdk_sample_and_verify), many
+ * rows with one shared prior are served by the streaming kernels: rdk_sample_prior_workspace_bytes (host only, no CUDA
+ * call) says how many bytes that takes, 0 where they would not serve.  A smaller or missing workspace is no error.
  * ------------------------------------------------------------------------------------------- */
 int rdk_sample_and_verify_prior(const rdk_problem* problem, const void* target, const void* prior,
                                 int64_t prior_row_stride, const void* drafter, const float* uniforms,
                                 int32_t trials, const rdk_outputs* out, void* stream);
+size_t rdk_sample_prior_workspace_bytes(const rdk_problem* problem, const void* target, const void* prior,
+                                        int64_t prior_row_stride, const void* drafter, int32_t trials);
+int rdk_sample_and_verify_prior_ws(const rdk_problem* problem, const void* target, const void* prior,
+                                   int64_t prior_row_stride, const void* drafter, const float* uniforms,
+                                   int32_t trials, const rdk_outputs* out, void* ws, size_t ws_bytes, void* stream);
 int rdk_redistribute_linear_prior(const rdk_problem* problem, const void* target, const void* prior,
                                   int64_t prior_row_stride, const void* drafter, float* qtilde_out,
                                   float* theta_out, float* S_out, void* stream);
@@ -328,8 +335,8 @@ int rdk_redistribute_linear_prior(const rdk_problem* problem, const void* target
  * or invalid kept ids and unaligned rows also do, but are not known here).  A row is shared by
  * ctas_per_row CTAs of warps_per_cta streaming warps, each owning segment_tokens consecutive
  * tokens (Eq. "rdk-taylor" is evaluated per segment; ctas_per_row * warps_per_cta segments cover
- * the vocabulary); stages = depth of the shared-memory ring; live_rows - 1 = rows by which the
- * second visit of a row trails its first.  Returns RDK_OK, or RDK_ERR_INVALID_ARG.
+ * the vocabulary); stages = depth of the shared-memory ring; live_rows = rows whose second
+ * visit may be outstanding.  Returns RDK_OK, or RDK_ERR_INVALID_ARG.
  * ------------------------------------------------------------------------------------------- */
 typedef struct rdk_stream_geometry_t {
     int32_t supported;

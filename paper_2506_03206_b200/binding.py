@@ -37,7 +37,8 @@ EXPORTS = [
     "rdk_redistribute_exact", "rdk_redistribute_exact_static", "rdk_redistribute_linear",
     "rdk_sample_workspace_bytes", "rdk_sample_and_verify", "rdk_emit_sequences",
     "rdk_sample_and_verify_host", "rdk_stream_geometry", "rdk_sample_and_verify_prior",
-    "rdk_redistribute_linear_prior", "rdk_sample_route", "rdk_test_set_spin_limit",
+    "rdk_sample_and_verify_prior_ws", "rdk_sample_prior_workspace_bytes", "rdk_redistribute_linear_prior", "rdk_sample_route",
+    "rdk_test_set_spin_limit",
 ]
 
 

@@ -173,8 +173,16 @@ PyObject* sample_prior(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const long long stride = prior_stride(prior, a[4], target, pb.N);
         const void *z = pointer<void>(target), *pr = pointer<void>(prior), *y = pointer<void>(drafter);
         const float* up = pointer<float>(u);
-        void* s = stream();
-        return PyLong_FromLong(unlocked([&] { return rdk_sample_and_verify_prior(&pb, z, pr, stride, y, up, (int32_t)trials, &o, s); }));
+        const c10::cuda::CUDAStream current = c10::cuda::getCurrentCUDAStream();
+        // A workspace of this call's own from torch's allocator, which hands the memory out again in the order of the stream;
+        // none while the stream is captured, where the allocator may have to be kept out of it.
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        const size_t ws_bytes = rdk_sample_prior_workspace_bytes(&pb, z, pr, stride, y, (int32_t)trials);
+        at::Tensor ws;
+        if (ws_bytes && cudaStreamIsCapturing(current.stream(), &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone)
+            ws = at::empty({(int64_t)ws_bytes}, target.options().dtype(at::kByte));
+        void *wsp = ws.defined() ? pointer<void>(ws) : nullptr, *s = current.stream();
+        return PyLong_FromLong(unlocked([&] { return rdk_sample_and_verify_prior_ws(&pb, z, pr, stride, y, up, (int32_t)trials, &o, wsp, wsp ? ws_bytes : 0, s); }));
     });
 }
 

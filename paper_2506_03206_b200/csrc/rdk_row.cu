@@ -447,6 +447,17 @@ static bool many_draws(const RowParams& P, int mode, size_t es) {
     return P.trials >= 64 ? draws >= 2560 : draws >= (P.N <= 131072 ? 1600 : 5120);
 }
 
+// what the host-only queries look at
+static RowParams linear_rows(const rdk_problem* problem, const void* target, const void* drafter, int trials, const void* prior) {
+    RowParams P{};
+    P.N = problem->N; P.n = problem->n; P.rows = problem->batch * problem->positions; P.trials = trials;
+    P.target = target; P.target_stride = problem->target_row_stride ? problem->target_row_stride : problem->N;
+    P.drafter = drafter; P.drafter_stride = problem->drafter_row_stride ? problem->drafter_row_stride : problem->n;
+    P.header = static_cast<const int32_t*>(problem->kept_index);
+    P.prior = prior;
+    return P;
+}
+
 static int run_rows(const rdk_problem* pb, int mode, const void* target, const void* drafter,
                     const float* w, long long w_stride, const float* uniforms, int trials,
                     const rdk_outputs* out, float* qtilde, float* theta_out, float* S_out,
@@ -497,7 +508,7 @@ static int run_rows(const rdk_problem* pb, int mode, const void* target, const v
         return r;
     };
     if (!(pb->flags & RDK_FLAG_ROW_KERNEL)) {
-        const bool streams = mode == RDK_MODE_LINEAR && trials > 0 && !prior;
+        const bool streams = mode == RDK_MODE_LINEAR && trials > 0 && (!prior || ws);     // (a prior's call may come without a workspace)
         const bool many = many_draws(P, mode, pb->target_dtype == RDK_F32 ? 4 : 2);
         if (!many && (!streams || stream_few_rows(P, pb->target_dtype, pb->drafter_dtype, pb->drafter_kind))) e = cluster();
         if (e == cudaErrorNotSupported && streams) {
@@ -555,6 +566,23 @@ extern "C" int rdk_redistribute_linear_prior(const rdk_problem* problem, const v
 extern "C" int rdk_sample_and_verify_prior(const rdk_problem* problem, const void* target, const void* prior,
                                            int64_t prior_row_stride, const void* drafter, const float* uniforms,
                                            int32_t trials, const rdk_outputs* out, void* stream) {
+    return rdk_sample_and_verify_prior_ws(problem, target, prior, prior_row_stride, drafter, uniforms, trials, out, nullptr, 0, stream);
+}
+
+extern "C" size_t rdk_sample_prior_workspace_bytes(const rdk_problem* problem, const void* target, const void* prior,
+                                                   int64_t prior_row_stride, const void* drafter, int32_t trials) {
+    if (!prior || prior_row_stride != 0 || trials < 1 || validate_problem(problem, "rdk_sample_prior_workspace_bytes", true) != RDK_OK) return 0;
+    const RowParams P = linear_rows(problem, target, drafter, trials, prior);
+    const size_t bytes = stream_workspace_bytes(P.rows, problem->batch, trials);
+    const bool streams = !(problem->flags & RDK_FLAG_ROW_KERNEL) && !many_draws(P, RDK_MODE_LINEAR, problem->target_dtype == RDK_F32 ? 4 : 2) &&
+                         !stream_few_rows(P, problem->target_dtype, problem->drafter_dtype, problem->drafter_kind) &&
+                         !stream_ineligible(P, problem->target_dtype, problem->drafter_dtype, problem->drafter_kind, problem->batch, reinterpret_cast<const void*>(uintptr_t(256)), bytes);
+    return streams ? bytes : 0;
+}
+
+extern "C" int rdk_sample_and_verify_prior_ws(const rdk_problem* problem, const void* target, const void* prior,
+                                              int64_t prior_row_stride, const void* drafter, const float* uniforms,
+                                              int32_t trials, const rdk_outputs* out, void* ws, size_t ws_bytes, void* stream) {
     int st = validate_problem(problem, "rdk_sample_and_verify_prior", true);
     if (st != RDK_OK) return st;
     if (!target || !prior || !drafter || !uniforms || !out || trials < 1 ||
@@ -569,7 +597,7 @@ extern "C" int rdk_sample_and_verify_prior(const rdk_problem* problem, const voi
     st = check_arch();
     if (st != RDK_OK) return st;
     return run_rows(problem, RDK_MODE_LINEAR, target, drafter, nullptr, 0, uniforms, trials, out, nullptr,
-                    nullptr, nullptr, nullptr, 0, static_cast<cudaStream_t>(stream), prior, prior_row_stride);
+                    nullptr, nullptr, ws, ws_bytes, static_cast<cudaStream_t>(stream), prior, prior_row_stride);
 }
 
 extern "C" int rdk_sample_route(const rdk_problem* problem, int32_t mode, const void* target, const void* drafter,
@@ -583,11 +611,7 @@ extern "C" int rdk_sample_route(const rdk_problem* problem, int32_t mode, const 
         return -RDK_ERR_INVALID_ARG;
     }
     if (problem->flags & RDK_FLAG_ROW_KERNEL) { if (why) *why = "RDK_FLAG_ROW_KERNEL is set"; return RDK_ROUTE_ROW_KERNEL; }
-    RowParams P{};
-    P.N = problem->N; P.n = problem->n; P.rows = problem->batch * problem->positions; P.trials = trials;
-    P.target = target; P.target_stride = problem->target_row_stride ? problem->target_row_stride : problem->N;
-    P.drafter = drafter; P.drafter_stride = problem->drafter_row_stride ? problem->drafter_row_stride : problem->n;
-    P.header = static_cast<const int32_t*>(problem->kept_index);
+    const RowParams P = linear_rows(problem, target, drafter, trials, nullptr);
     const char* no = stream_ineligible(P, problem->target_dtype, problem->drafter_dtype, problem->drafter_kind,
                                        problem->batch, ws, ws_bytes);
     if (!no && stream_few_rows(P, problem->target_dtype, problem->drafter_dtype, problem->drafter_kind)) no = "few rows: one cluster each is faster";

@@ -36,6 +36,11 @@
 //   through sum p_j per segment, which comes out of the soft-max sweep itself.
 // * S = sum_j w_j = 1 + O(N^-2), because sum q' = 1 and sum q'_j p_j = theta cancel the
 //   first-order terms; it is taken as 1.
+//
+// With one prior row pi for all rows in place of p inside the formula the same kernel keeps the CTA's slice of pi and all that
+// no row changes about it, so that a row costs it one set of exponentials more at the kept tokens' second visit only in
+// arithmetic.  320 rows of 128256 tokens: 54 us, with the draws; the cluster kernel, which reads pi and takes its soft-max
+// anew for every row, 111.
 #include <atomic>
 #include <chrono>
 
@@ -61,9 +66,9 @@ constexpr int kFastNit = 64 / kSW;       // 16-byte vectors per lane in a segmen
 constexpr int kMaxFastSteps = 6;         // kept-token passes of up to this many steps are unrolled, their offsets in registers
 
 // scalars of a row's record
-enum { kRecOffg = 0, kRecInvZp, kRecYoffg, kRecInvZq, kRecTheta };
+enum { kRecOffg = 0, kRecInvZp, kRecYoffg, kRecInvZq, kRecTheta, kRecOffPrior, kRecInvZprior };
 
-struct Scal { float offg, inv_zp, yoffg, inv_zq, theta, inv_n, inv_s; };
+struct Scal { float offg, inv_zp, yoffg, inv_zq, theta, inv_n, inv_s, offpi, inv_zpi; };
 
 struct StreamGeo {
     int C, G;              // CTAs per group, groups
@@ -80,7 +85,7 @@ struct StreamGeo {
     const uint16_t* goff;  // per slot: byte offset of its target logit in the CTA's slice
 };
 
-// w_j for given p_j and q'_j:  (q' + theta x) (1 - x + x^2),  x = p / N
+// w_j for given p_j (the prior's, where there is one) and q'_j:  (q' + theta x) (1 - x + x^2),  x = p / N
 __device__ __forceinline__ float taylor_w(const Scal& c, float p, float qp) {
     const float x = p * c.inv_n;
     return fmaf(c.theta, x, qp) * fmaf(x, x - 1.f, 1.f);
@@ -100,11 +105,32 @@ __device__ __forceinline__ uint4 tmem_ld4(uint32_t taddr) {
     return v;
 }
 
+__device__ __forceinline__ void tmem_st2(uint32_t taddr, float a, float b) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1, %2};" ::"r"(taddr), "r"(__float_as_uint(a)), "r"(__float_as_uint(b)) : "memory");
+}
+__device__ __forceinline__ float2 tmem_ld2(uint32_t taddr) {
+    uint32_t a, b;
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];" : "=r"(a), "=r"(b) : "r"(taddr) : "memory");
+    return make_float2(__uint_as_float(a), __uint_as_float(b));
+}
+__device__ __forceinline__ void tmem_st1(uint32_t taddr, float a) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%0], {%1};" ::"r"(taddr), "r"(__float_as_uint(a)) : "memory");
+}
+__device__ __forceinline__ float tmem_ld1(uint32_t taddr) {
+    uint32_t a;
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(a) : "r"(taddr) : "memory");
+    return __uint_as_float(a);
+}
+// Columns of a warp's share of the tensor memory: with a prior first its e_pi at the kept slots and a column per live row for
+// the smallest z - pi of each lane, then the rows' pairs, 4 columns per step.
+__host__ __device__ constexpr int tmem_epi_cols(int nst, bool prior) { return prior ? (2 * nst + 3) & ~3 : 0; }
+__host__ __device__ constexpr int tmem_rows_at(int nst, bool prior) { return prior ? tmem_epi_cols(nst, true) + kMaxNB : 0; }
+
 // ------------------------------------------------------------------------------------------------
 // helpers of the draw kernel (Algorithm 4 steps 4-8)
 // ------------------------------------------------------------------------------------------------
 struct DrawCtx {
-    const void* zrow; const void* yrow; bool zvec;
+    const void* zrow; const void* yrow; const void* prior; bool zvec;
     const uint32_t* mask; const int32_t* rank;
     int N;
     Scal c;
@@ -113,10 +139,12 @@ struct DrawCtx {
 // p and w of the 8 tokens starting at global token jb (a multiple of 8).  The drafter values of the kept
 // tokens among them are fetched by eight independent loads (tokens that are not kept re-read the first
 // fetched index), so that one round trip serves them all.
-template <typename TZ, typename TY, int KIND>
+template <typename TZ, typename TY, int KIND, bool PRI>
 __device__ __forceinline__ void draw_pw(const DrawCtx& d, int jb, float (&p)[kVec], float (&w)[kVec]) {
     float z[kVec];
     load8<TZ>(static_cast<const TZ*>(d.zrow), jb, d.N, d.zvec, -INFINITY, z);
+    [[maybe_unused]] float pr[kVec];
+    if constexpr (PRI) load8<TZ>(static_cast<const TZ*>(d.prior), jb, d.N, true, -INFINITY, pr);
     const uint32_t word = __ldg(d.mask + (jb >> 5));
     const int rbase = __ldg(d.rank + (jb >> 5));          // issued together with the mask and the logits
     const int sh = jb & 31;
@@ -135,18 +163,19 @@ __device__ __forceinline__ void draw_pw(const DrawCtx& d, int jb, float (&p)[kVe
         p[k] = ex2(fmaf(z[k], kLog2e, d.c.offg)) * d.c.inv_zp;
         const bool kept = (mb >> k) & 1u;
         const float qp = kept ? (KIND == RDK_LOGITS ? ex2(fmaf(y[k], kLog2e, d.c.yoffg)) : y[k]) * d.c.inv_zq : 0.f;
-        w[k] = taylor_w(d.c, p[k], qp);
+        if constexpr (PRI) w[k] = taylor_w(d.c, ex2(fmaf(pr[k], kLog2e, d.c.offpi)) * d.c.inv_zpi, qp);
+        else w[k] = taylor_w(d.c, p[k], qp);
     }
 }
 
 enum { kPickW = 0, kPickR = 1, kPickP = 2 };
 
-template <typename TZ, typename TY, int KIND>
+template <typename TZ, typename TY, int KIND, bool PRI>
 __device__ __forceinline__ void draw_x(const DrawCtx& d, int what, int jb, int seg_end, float (&p)[kVec], float (&w)[kVec], float (&x)[kVec]) {
 #pragma unroll
     for (int k = 0; k < kVec; ++k) { p[k] = 0.f; w[k] = 0.f; x[k] = 0.f; }
     if (jb >= seg_end) return;
-    draw_pw<TZ, TY, KIND>(d, jb, p, w);
+    draw_pw<TZ, TY, KIND, PRI>(d, jb, p, w);
 #pragma unroll
     for (int k = 0; k < kVec; ++k)
         x[k] = what == kPickW ? w[k] : (what == kPickR ? fmaxf(0.f, p[k] - w[k] * d.c.inv_s) : p[k]);
@@ -159,7 +188,11 @@ __device__ __forceinline__ void draw_x(const DrawCtx& d, int what, int jb, int s
 // and the exponential pass; NIT = 0: any segment length, two passes over shared memory.
 // NST > 0: the kept-token passes take exactly NST steps of 64 slots, unrolled, with the slots' offsets in
 // registers; NST = 0: any number of steps, offsets in shared memory.
-template <typename TZ, typename TY, int KIND, int NIT, int NST>
+// PRI: one prior row pi for all rows stands in for p inside Eq. rdk-taylor.  The CTA keeps its slice of it (in shared memory) and
+// what of it no row changes: sum of e_pi over the segments, e_pi at the kept slots (in tensor memory).  Tokens that are not kept
+// have w = theta x, x = pi_j / N, the smaller of w and p nearly everywhere; where p is the smaller, z - pi lies below a
+// constant of the row (see violations).
+template <typename TZ, typename TY, int KIND, int NIT, int NST, bool PRI>
 __global__ void __launch_bounds__(kSThreads, 1)
 rdk_stream_kernel(const RowParams P, const StreamGeo g) {
     extern __shared__ __align__(128) unsigned char dsm[];
@@ -172,6 +205,9 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
     __shared__ __align__(8) unsigned long long bbar[kMaxNB];   // [row mod NB]: akv[] of the row is set
     __shared__ __align__(8) unsigned long long pbar[16];    // [row mod 16]: the publish warp has parked the row in pend[]
     __shared__ __align__(16) float pend[16][kSW][8];    // publish and collect warps only, [row mod 16][warp]: the warp's sums, its factors, theta, a row scalar
+    __shared__ __align__(8) unsigned long long prbar;   // PRI: the slice of the prior has landed
+    __shared__ float xs_s[16];                             // PRI: [row mod 16]: e_pi -> x
+    __shared__ float epi_s[kSW], epm_s[kSW];               // PRI: sum of e_pi over the warp's segment, on the CTA's scale; the segment's maximum
     __shared__ int fail;
     __shared__ uint32_t tmem_base_s;                       // base address of the CTA's tensor memory (unrolled route)
     constexpr bool kTmem = NST > 0;                        // the pair cache lives in tensor memory, not in shared memory
@@ -207,7 +243,8 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
     const uint32_t stage = zslice + 16u + (uint32_t)kSW * (uint32_t)g.ystage;
     const uint32_t off_cache = (uint32_t)g.NS * stage;
     const int nb = g.NB, defer = g.NB - 1;
-    const uint32_t off_goff = off_cache + (kTmem ? 0u : (uint32_t)kSW * (uint32_t)nb * (uint32_t)g.ycap * 8u);
+    const uint32_t pr_a = smem_u32(dsm) + off_cache;        // PRI (which has no cache in shared memory): the slice of the prior and 16 bytes of -inf
+    const uint32_t off_goff = off_cache + (PRI ? zslice + 16u : 0u) + (kTmem ? 0u : (uint32_t)kSW * (uint32_t)nb * (uint32_t)g.ycap * 8u);
     const uint32_t off_bar = off_goff + (NST > 0 ? 0u : (uint32_t)kSW * (uint32_t)g.ycap * 2u);
     const uint32_t dsm_a = smem_u32(dsm);
     const uint32_t full_a = dsm_a + off_bar, empty_a = full_a + 8u * (uint32_t)g.NS;
@@ -221,6 +258,7 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&bbar[k])), "r"(kSW));
         }
         for (int k = 0; k < 16; ++k) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&pbar[k])));
+        if (PRI) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&prbar)));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     // per-warp quantities of the streaming warps (taken from lane 0 so that the compiler knows they are uniform)
@@ -314,8 +352,8 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
         {
             const uint32_t ninf16 = sizeof(TZ) == 2 ? 0xff80ff80u : 0xff800000u;      // -inf
             const uint32_t z0 = zbytes, z1 = zslice + 16u;        // [end of the copied vectors, spare bytes included)
-            for (int k = 0; k < g.NS; ++k) {
-                const uint32_t base = dsm_a + (uint32_t)k * stage;
+            for (int k = 0; k < (PRI ? g.NS + 1 : g.NS); ++k) {
+                const uint32_t base = dsm_a + (uint32_t)k * stage;       // (the prior's slice lies behind the last stage)
 #pragma unroll 8
                 for (uint32_t o = z0 + 16u * lane; o < z1; o += 512u)
                     asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(base + o), "r"(ninf16) : "memory");
@@ -323,6 +361,8 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
         }
         __syncwarp();
         asm volatile("griddepcontrol.wait;" ::: "memory");     // the inputs may be the previous kernel's outputs
+        // (the few elements of the prior's slice that a 16-byte copy cannot cover)
+        if (PRI && lane < lenc - lenc_v) reinterpret_cast<TZ*>(dsm + off_cache)[lenc_v + lane] = static_cast<const TZ*>(P.prior)[j0c + lenc_v + lane];
         for (int k = 0; k < pre_rows; ++k) load_row();
     }
 
@@ -347,6 +387,17 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();                        // barriers initialised, padding and tables in place, tensor memory allocated
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (PRI && warp == kWPublish && lane == 0) {     // the slice of the prior
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        if (zbytes == 0) {
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&prbar)) : "memory");
+        } else {
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&prbar)), "r"(zbytes) : "memory");
+            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                         ::"r"(pr_a), "l"(static_cast<const TZ*>(P.prior) + j0c), "r"(zbytes), "r"(smem_u32(&prbar)) : "memory");
+        }
+    }
 
     if (warp < kSW) {
         // ================================ streaming warps ============================================
@@ -358,7 +409,8 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
         const uint32_t csz = (uint32_t)g.ycap * 8u;
         const uint32_t cb0 = dsm_a + off_cache + (uint32_t)warp * (uint32_t)nb * csz + (uint32_t)lane * 16u;
         // tensor memory: this warp's quarter of the lanes (warp % 4), its 128 columns there, 4 columns per step and live row
-        const uint32_t tb0 = tmem_base_s + ((uint32_t)(warp & 3) << 21) + (uint32_t)(warp >> 2) * (uint32_t)kTmemWarpCols;
+        const uint32_t tb_w = tmem_base_s + ((uint32_t)(warp & 3) << 21) + (uint32_t)(warp >> 2) * (uint32_t)kTmemWarpCols;
+        const uint32_t tb0 = tb_w + (uint32_t)tmem_rows_at(NST, PRI), tb_min = tb_w + (uint32_t)tmem_epi_cols(NST, PRI);
         constexpr int kRowCols = 4 * (NST > 0 ? NST : 1);
         const uint32_t gl = dsm_a + off_goff + (uint32_t)warp * (uint32_t)g.ycap * 2u + (uint32_t)lane * 4u;
         // slot il = 64 st + 2 lane + h of the pair grid holds a kept token of the segment iff il < kcs, and
@@ -369,15 +421,78 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
         const long long ystep = (long long)g.G * P.drafter_stride;
         const float2 l2e = splat(kLog2e);
 
+        // ---- what of the prior no row changes ------------------------------------------------------------
+        float poff = 0.f;                                // its exponentials are on one scale in the CTA, a whole power of two
+        const uint32_t prw_a = pr_a + zw_off;            // this warp's segment of it
+        if (PRI) {
+            mbar_wait(smem_u32(&prbar), 0, &fail, spin_limit);
+            MaxAcc<TZ> mp;
+#pragma unroll
+            for (int k = 0; k < (NIT > 0 ? NIT : 1); ++k) mp.push(lds128(prw_a + (uint32_t)(k * 32 + lane) * 16u));
+            const float m = warp_max_redux(mp.result());
+            if (lane == 0) epm_s[warp] = m;
+            asm volatile("bar.sync 1, %0;" ::"n"(kSW * 32) : "memory");          // the streaming warps
+            const float mc = warp_max_redux(epm_s[lane & (kSW - 1)]);
+            poff = mc > -INFINITY ? -rintf(mc * kLog2e) : 0.f;
+            float2 Ea = splat(0.f), Eb = splat(0.f);
+#pragma unroll
+            for (int k = 0; k < (NIT > 0 ? NIT : 1); ++k) exp_sum_vec<TZ>(lds128(prw_a + (uint32_t)(k * 32 + lane) * 16u), l2e, splat(poff), Ea, Eb);
+            const float e = warp_sum((Ea.x + Ea.y) + (Eb.x + Eb.y));
+            if (lane == 0) epi_s[warp] = e;              // (read by the publish warp, after this warp's first record)
+#pragma unroll
+            for (int st = 0; st < (NST > 0 ? NST : 1); ++st)
+                tmem_st2(tb_w + 2u * (uint32_t)st, ex2(fmaf(lds_z<TZ>(pr_a + (gor[st] & 0xffffu)), kLog2e, poff)), ex2(fmaf(lds_z<TZ>(pr_a + (gor[st] >> 16)), kLog2e, poff)));
+            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        }
+
         // ---- second visit of a row: sum of min(p, q~) over the cached kept tokens ----------------------
-        // sv_sum: this lane's share, once the row's scalars are in place (par = row mod NB)
+        // PRI: sum of max(0, theta x - p) over this lane's tokens of the segment.  theta x > p where z - pi lies below a constant c
+        // of the row; `least` is the lane's smallest difference, taken in bf16 (hence the margin), and a lane with such a
+        // token, one in some thirty, reads its part of the row again.  tx: theta x / e_pi, fz: p / e_z.
+        auto violations = [&](int itb, int par, float tx, float fz, float least) -> float {
+            const float m_w = wrec[par][warp][4];
+            const float zoff = m_w > -INFINITY ? -m_w * kLog2e : 0.f;
+            float c = (__log2f(tx) - __log2f(fz) + poff - zoff) * (1.f / kLog2e);
+            c = c == c ? c + fabsf(c) * 0x1p-7f + 0.01f : INFINITY;
+            float v = 0.f;
+            if (least < c) {
+                const TZ* zrow = static_cast<const TZ*>(P.target) + (grp + (long long)itb * g.G) * P.target_stride;
+#pragma unroll 1
+                for (int k = 0; k < (NIT > 0 ? NIT : 1); ++k) {
+                    const int tok = j0 + (k * 32 + lane) * kVec;
+                    if (tok >= P.N) break;
+                    float z[kVec];
+                    load8<TZ>(zrow, tok, P.N, true, -INFINITY, z);
+                    const uint4 q = lds128(prw_a + (uint32_t)(k * 32 + lane) * 16u);          // (-inf beyond the vocabulary)
+                    const uint32_t qw[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+                    for (int h = 0; h < kVec; ++h) {
+                        const float pi = h & 1 ? bf16_hi(qw[h / 2]) : bf16_lo(qw[h / 2]);
+                        if (z[h] - pi < c) v += fmaxf(0.f, tx * ex2(fmaf(pi, kLog2e, poff)) - fz * ex2(fmaf(z[h], kLog2e, zoff)));
+                    }
+                }
+            }
+            __syncwarp();
+            return v;
+        };
+        // sv_sum: this lane's share, once the row's scalars are in place (itb: row of the group, par = itb mod NB)
         auto sv_sum = [&](int itb, int par) -> float {
             const float theta = scal[par][4];
             const float2 f = fzy[par][warp];                  // p = f.x e_z,  q' = f.y e_y
             // q~ = q' + x (theta - q'),  x = p / N
-            const float2 fz2 = splat(f.x), fy2 = splat(f.y), xs2 = splat(f.x * inv_n), th2 = splat(theta), neg1 = splat(-1.f);
+            const float xs = PRI ? scal[par][5] : f.x * inv_n;                                  // e_z (or e_pi) -> x
+            const float2 fz2 = splat(f.x), fy2 = splat(f.y), xs2 = splat(xs), th2 = splat(theta), neg1 = splat(-1.f);
             float2 ak2 = splat(0.f);
             const uint32_t cb = cb0 + (uint32_t)par * csz;
+            // PRI: what min(p, w) is above min(p, theta x), which stands for it in the segment's sum
+            auto sv_math_prior = [&](uint4 c4, float2 ep) {
+                const float2 ez = make_float2(__uint_as_float(c4.x), __uint_as_float(c4.y));
+                const float2 ey = make_float2(__uint_as_float(c4.z), __uint_as_float(c4.w));
+                const float2 p = fmul2(ez, fz2), qp = fmul2(ey, fy2), x = fmul2(ep, xs2);
+                const float2 w = ffma2(x, ffma2(qp, neg1, th2), qp), w0 = fmul2(x, th2);
+                ak2 = fadd2(ak2, make_float2(fminf(p.x, w.x), fminf(p.y, w.y)));
+                ak2 = ffma2(make_float2(fminf(p.x, w0.x), fminf(p.y, w0.y)), neg1, ak2);
+            };
             auto sv_math = [&](uint4 c4) {
                 const float2 ez = make_float2(__uint_as_float(c4.x), __uint_as_float(c4.y));
                 const float2 ey = make_float2(__uint_as_float(c4.z), __uint_as_float(c4.w));
@@ -391,10 +506,22 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
 #pragma unroll
                 for (int st = 0; st < (NST > 0 ? NST : 1); ++st)
                     if (st < NST - 1 || NST == 1 || last_step) c4[st] = tmem_ld4(tb0 + (uint32_t)(par * kRowCols + st * 4));
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                if constexpr (PRI) {
+                    float2 ep[NST > 0 ? NST : 1];
 #pragma unroll
-                for (int st = 0; st < (NST > 0 ? NST : 1); ++st)
-                    if (st < NST - 1 || NST == 1 || last_step) sv_math(c4[st]);
+                    for (int st = 0; st < (NST > 0 ? NST : 1); ++st) ep[st] = tmem_ld2(tb_w + 2u * (uint32_t)st);
+                    const float least = tmem_ld1(tb_min + (uint32_t)par);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                    for (int st = 0; st < (NST > 0 ? NST : 1); ++st)
+                        if (st < NST - 1 || NST == 1 || last_step) sv_math_prior(c4[st], ep[st]);
+                    ak2.x -= violations(itb, par, theta * xs, f.x, least);
+                } else {
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                    for (int st = 0; st < (NST > 0 ? NST : 1); ++st)
+                        if (st < NST - 1 || NST == 1 || last_step) sv_math(c4[st]);
+                }
             } else {
 #pragma unroll 2
                 for (int st = 0; st < nst; ++st) sv_math(lds128(cb + (uint32_t)st * 512u));
@@ -411,7 +538,12 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
                     const float y = to_float<TY>(yrow[r0 + il]);
                     const float ey = KIND == RDK_LOGITS ? ex2(fmaf(y, kLog2e, yoff)) : y;
                     const float p = ez * f.x, qp = ey * f.y;
-                    ak += fminf(p, fmaf(p * inv_n, theta - qp, qp));
+                    if constexpr (PRI) {
+                        const float x = ex2(fmaf(lds_z<TZ>(prw_a + (uint32_t)(__ldg(P.ids + r0 + il) - j0) * (uint32_t)sizeof(TZ)), kLog2e, poff)) * xs;
+                        ak += fminf(p, fmaf(x, theta - qp, qp)) - fminf(p, theta * x);
+                    } else {
+                        ak += fminf(p, fmaf(p * inv_n, theta - qp, qp));
+                    }
                 }
             }
             return ak;
@@ -472,6 +604,24 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
                         exp_sum_vec<TZ>(lds128(zs_a + (uint32_t)t * (uint32_t)sizeof(TZ)), l2e, of, Ea, Eb);
                 }
             }
+            if (PRI) {                                   // the smallest z - pi of the lane, for the second visit
+                __nv_bfloat162 da = __float2bfloat162_rn(INFINITY), db = da;
+#pragma unroll
+                for (int k = 0; k < (NIT > 0 ? NIT : 1); ++k) {
+                    const uint4 q = lds128(prw_a + (uint32_t)(k * 32 + lane) * 16u);
+                    auto diff = [](uint32_t a, uint32_t b) { return __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b)); };
+                    da = __hmin2(__hmin2(da, diff(zv[k].x, q.x)), diff(zv[k].y, q.y));
+                    db = __hmin2(__hmin2(db, diff(zv[k].z, q.z)), diff(zv[k].w, q.w));
+                }
+                da = __hmin2(da, db);
+                tmem_st1(tb_min + (uint32_t)par, fminf(__low2float(da), __high2float(da)));
+            }
+            float2 ep[NST > 0 ? NST : 1];                // e_pi at the kept slots
+            if (PRI) {
+#pragma unroll
+                for (int st = 0; st < (NST > 0 ? NST : 1); ++st) ep[st] = tmem_ld2(tb_w + 2u * (uint32_t)st);
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            }
             // kept tokens: e_z, e_y, their sums; the pairs go to the cache
             float K1s, Zqs, ths;
             const uint32_t cbA = cb0 + (uint32_t)par * csz;
@@ -488,7 +638,8 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
                 } else {
                     ey = make_float2(v0 ? y.x : 0.f, v1 ? y.y : 0.f);
                 }
-                K1 = fadd2(K1, ez); Zq = fadd2(Zq, ey); th = ffma2(ez, ey, th);
+                if (!PRI) K1 = fadd2(K1, ez);
+                Zq = fadd2(Zq, ey); th = ffma2(PRI ? ep[NST > 0 ? st : 0] : ez, ey, th);
                 if (kTmem) tmem_st4(tb0 + (uint32_t)(par * kRowCols + st * 4), ez.x, ez.y, ey.x, ey.y);
                 else sts128(cbA + (uint32_t)st * 512u, ez.x, ez.y, ey.x, ey.y);
             };
@@ -510,7 +661,8 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
                         const float ez = ex2(fmaf(lds_z<TZ>(zs_a + (uint32_t)(__ldg(P.ids + r0 + il) - j0) * (uint32_t)sizeof(TZ)), kLog2e, zoff));
                         const float y = to_float<TY>(cy[il]);
                         const float ey = KIND == RDK_LOGITS ? ex2(fmaf(y, kLog2e, yoff)) : y;
-                        K1s += ez; Zqs += ey; ths = fmaf(ez, ey, ths);
+                        K1s += ez; Zqs += ey;
+                        ths = fmaf(PRI ? ex2(fmaf(lds_z<TZ>(prw_a + (uint32_t)(__ldg(P.ids + r0 + il) - j0) * (uint32_t)sizeof(TZ)), kLog2e, poff)) : ez, ey, ths);
                     }
                 }
             };
@@ -581,12 +733,14 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
                 const float theta = f4.z, ak = akv[pf][lane];
                 // sums over the segment: p; w of the not-kept tokens (theta x); w of the kept tokens from the moments
                 const float segP = w0.x * f4.x;
-                const float xs = f4.x * inv_n;
-                const float oov = theta * xs * fmaxf(0.f, w0.x - w0.y);
-                const float Kw = f4.y * w0.z - f4.y * xs * w0.w + theta * xs * w0.y;
+                const float xs = PRI ? xs_s[itf & 15] : f4.x * inv_n;
+                // (with a prior all tokens count as not kept here, and ak has what the kept ones are above that)
+                const float oov = theta * xs * (PRI ? epi_s[lane] : fmaxf(0.f, w0.x - w0.y));
+                const float Kw = f4.y * w0.z - f4.y * xs * w0.w + (PRI ? 0.f : theta * xs * w0.y);
                 const float a_s = oov + ak;
                 reinterpret_cast<float4*>(rec + 16)[seg] = make_float4(oov + Kw, a_s, fmaxf(0.f, segP - a_s), segP);
-                if (crank == 0 && lane < 5) rec[lane] = lane == 4 ? theta : f4.w;     // -m log2e, 1/Zp, -my log2e, 1/Zq, theta
+                // -m log2e, 1/Zp, -my log2e, 1/Zq, theta; the prior's scale and 1/Zpi
+                if (crank == 0 && lane < (PRI ? 7 : 5)) rec[lane] = lane == kRecTheta ? theta : f4.w;
             }
         };
         for (int it = 0; it < rows_g + nb; ++it) {
@@ -601,7 +755,16 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
                     *reinterpret_cast<float4*>(&pend[it & 15][lane][0]) = make_float4(E1, K1, Zq, th);
                     *reinterpret_cast<float2*>(&pend[it & 15][lane][4]) = make_float2(m, my);     // the warp's maxima, until the factors replace them
                 }
-                combine_records(E1, Zq, th, m, my, lane);
+                if constexpr (PRI) {
+                    float Ep = lane < kSW ? epi_s[lane] : 0.f;
+                    const float mc = warp_max_redux(epm_s[lane & (kSW - 1)]);
+                    combine_records_prior(E1, Zq, th, m, my, Ep, lane);
+                    // and two words more
+                    const float v = lane == 5 ? Ep : (mc > -INFINITY ? rintf(mc * kLog2e) : -INFINITY);
+                    if (lane == 5 || lane == 6) st_tagged(P.xrec + ((size_t)row * g.C + crank) * kXrecBytes + 8 * lane, v, g.tag);
+                } else {
+                    combine_records(E1, Zq, th, m, my, lane);
+                }
                 {
                     // five (value, tag) words, one per lane
                     const float v = lane == 0 ? E1 : (lane == 1 ? Zq : (lane == 2 ? th : (lane == 3 ? m : my)));
@@ -617,30 +780,41 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
         // Per row: gather the C records of the row from global memory, leave the row scalars and every
         // warp's factors in shared memory for the second visits.
         asm volatile("griddepcontrol.wait;" ::: "memory");     // see the publish warp
+        constexpr int kWords = PRI ? 7 : 5;
         for (int it = 0; it < rows_g; ++it) {
             const int pc = it % nb;
             const long long row = grp + (long long)it * g.G;
-            float E1 = 0.f, Zq = 0.f, th = 0.f, m = -INFINITY, my = -INFINITY;
+            float E1 = 0.f, Zq = 0.f, th = 0.f, m = -INFINITY, my = -INFINITY, Ep = 0.f, mp = -INFINITY;
             if (lane < g.C) {
                 const unsigned char* xr = P.xrec + ((size_t)row * g.C + lane) * kXrecBytes;
-                unsigned long long w[5];
+                unsigned long long w[kWords];
                 unsigned spins = 0;
                 for (;;) {
                     bool ok = true;
 #pragma unroll
-                    for (int k = 0; k < 5; ++k) w[k] = ld_tagged(xr + 8 * k);
+                    for (int k = 0; k < kWords; ++k) w[k] = ld_tagged(xr + 8 * k);
 #pragma unroll
-                    for (int k = 0; k < 5; ++k) ok = ok && (uint32_t)(w[k] >> 32) == g.tag;
+                    for (int k = 0; k < kWords; ++k) ok = ok && (uint32_t)(w[k] >> 32) == g.tag;
                     if (ok) break;
                     if (++spins > spin_limit || ld_volatile_s32(&fail)) { atomicExch(&fail, 1); break; }
                     __nanosleep(20);
                 }
                 E1 = __uint_as_float((uint32_t)w[0]); Zq = __uint_as_float((uint32_t)w[1]); th = __uint_as_float((uint32_t)w[2]);
                 m = __uint_as_float((uint32_t)w[3]); my = __uint_as_float((uint32_t)w[4]);
+                if (PRI) { Ep = __uint_as_float((uint32_t)w[kWords - 2]); mp = __uint_as_float((uint32_t)w[kWords - 1]); }
             }
-            combine_records(E1, Zq, th, m, my, lane);
-            const float inv_zp = 1.f / E1, inv_zq = 1.f / Zq;
-            const float theta = th * inv_zp * inv_zq;
+            float mpm = 0.f;
+            if constexpr (PRI) {                         // (the prior is the same for every row)
+                __syncwarp();
+                mpm = warp_max_redux(mp);
+                const float fp = mp > -INFINITY ? ex2(mp - mpm) : 0.f;
+                Ep *= fp; th *= fp;
+                combine_records_prior(E1, Zq, th, m, my, Ep, lane);
+            } else {
+                combine_records(E1, Zq, th, m, my, lane);
+            }
+            const float inv_zp = 1.f / E1, inv_zq = 1.f / Zq, inv_zpi = PRI ? 1.f / Ep : inv_zp;
+            const float theta = th * inv_zpi * inv_zq;
             mbar_wait(smem_u32(&pbar[it & 15]), (uint32_t)((it >> 4) & 1), &fail, spin_limit);     // this CTA's own record of the row is parked
             if (lane < kSW) {
                 const float2 mw = *reinterpret_cast<const float2*>(&pend[it & 15][lane][4]);
@@ -649,8 +823,17 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
                 f.y = (KIND == RDK_LOGITS ? (mw.y > -INFINITY ? ex2((mw.y - my) * kLog2e) : 0.f) : 1.f) * inv_zq;
                 fzy[pc][lane] = f;
                 // lanes 0..3 also carry the row scalars the draws need: -m log2e, 1/Zp, -my log2e, 1/Zq
-                const float sc = lane == 0 ? -m * kLog2e : (lane == 1 ? inv_zp : (lane == 2 ? (KIND == RDK_LOGITS ? -my * kLog2e : 0.f) : inv_zq));
+                float sc = lane == 0 ? -m * kLog2e : (lane == 1 ? inv_zp : (lane == 2 ? (KIND == RDK_LOGITS ? -my * kLog2e : 0.f) : inv_zq));
+                if (PRI && lane >= kRecOffPrior) sc = lane == kRecOffPrior ? -mpm : inv_zpi;
                 *reinterpret_cast<float4*>(&pend[it & 15][lane][4]) = make_float4(f.x, f.y, theta, sc);
+            }
+            if (PRI) {                                   // e_pi on this CTA's scale -> x
+                const float mc = warp_max_redux(epm_s[lane & (kSW - 1)]);
+                if (lane == 0) {
+                    const float xs = (mc > -INFINITY ? ex2(rintf(mc * kLog2e) - mpm) : 0.f) * inv_zpi * inv_n;
+                    scal[pc][5] = xs;
+                    xs_s[it & 15] = xs;
+                }
             }
             if (lane == 0) scal[pc][4] = theta;
             __syncwarp();
@@ -675,6 +858,14 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
                     if (!done) __nanosleep(100);
                 }
             }
+            if (PRI) {
+                uint32_t done = 0;
+                for (unsigned spins = 0; !done && spins < (1u << 16); ++spins) {
+                    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n selp.u32 %0, 1, 0, p;\n}"
+                                 : "=r"(done) : "r"(smem_u32(&prbar)) : "memory");
+                    if (!done) __nanosleep(100);
+                }
+            }
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -694,7 +885,7 @@ __device__ __forceinline__ bool index_matches(const RowParams& P) {
 // kernel 2: one CTA per (row, trial) turns the row's record into draws
 // ------------------------------------------------------------------------------------------------
 // DT threads per CTA: half of the warps work on the draft draw, half on the residual draw.
-template <typename TZ, typename TY, int KIND, int DT>
+template <typename TZ, typename TY, int KIND, int DT, bool PRI>
 __global__ void __launch_bounds__(DT)
 rdk_draw_kernel(const RowParams P, const int nseg, const int Lw) {
     __shared__ double cdfW[kMaxSeg], cdfR[kMaxSeg], cdfP[kMaxSeg];
@@ -716,6 +907,7 @@ rdk_draw_kernel(const RowParams P, const int nseg, const int Lw) {
     d.c.offg = __ldcg(rec + kRecOffg); d.c.inv_zp = __ldcg(rec + kRecInvZp); d.c.yoffg = __ldcg(rec + kRecYoffg);
     d.c.inv_zq = __ldcg(rec + kRecInvZq); d.c.theta = __ldcg(rec + kRecTheta); d.c.inv_n = 1.f / (float)P.N;
     d.c.inv_s = 1.f;
+    if constexpr (PRI) { d.c.offpi = __ldcg(rec + kRecOffPrior); d.c.inv_zpi = __ldcg(rec + kRecInvZprior); d.prior = P.prior; }
 
     if (warp < 3) {   // fp64 prefix sums over the segments: warp 0 those of w, warp 1 of max(0, p - q~), warp 2 of p
         double* cdf = warp == 0 ? cdfW : (warp == 1 ? cdfR : cdfP);
@@ -780,7 +972,7 @@ rdk_draw_kernel(const RowParams P, const int nseg, const int Lw) {
     const int nch = (Lw + kSeg - 1) / kSeg;
     float p[kVec], w[kVec], x[kVec];          // of the last chunk this warp summed
     for (int ch = wg; ch < nch; ch += kGW) {
-        draw_x<TZ, TY, KIND>(d, what, seg_lo + ch * kSeg + lane * kVec, seg_end, p, w, x);
+        draw_x<TZ, TY, KIND, PRI>(d, what, seg_lo + ch * kSeg + lane * kVec, seg_end, p, w, x);
         float s = 0.f;
 #pragma unroll
         for (int k = 0; k < kVec; ++k) s += x[k];
@@ -805,7 +997,7 @@ rdk_draw_kernel(const RowParams P, const int nseg, const int Lw) {
             if (wg == 0 && lane == 0) { res_tok[g] = seg_lo; res_p[g] = 0.f; res_w[g] = 0.f; }
         } else if (chosen % kGW == wg) {
             // the chunk is still in this warp's registers unless the warp went on to a later one
-            if (chosen + kGW < nch) draw_x<TZ, TY, KIND>(d, what, seg_lo + chosen * kSeg + lane * kVec, seg_end, p, w, x);
+            if (chosen + kGW < nch) draw_x<TZ, TY, KIND, PRI>(d, what, seg_lo + chosen * kSeg + lane * kVec, seg_end, p, w, x);
             int sel = pick_in_segment(x, r_in, lane);
             if (sel < 0) sel = 0;
             float ps = 0.f, ws = 0.f;
@@ -863,17 +1055,17 @@ static int fast_steps(const StreamGeo& g, int nit) {
 }
 
 // offsets_in_smem = false is the unrolled route: offsets in registers and the pair cache in tensor memory
-static size_t stream_smem(const StreamGeo& g, size_t es, bool offsets_in_smem) {
-    const size_t stage = (size_t)kSW * g.Lw * es + 16 + (size_t)kSW * g.ystage;
-    // + cache (8 bytes per slot and live row) and offsets (2 bytes per slot) where they live here, barriers
-    return (size_t)g.NS * stage + (offsets_in_smem ? (size_t)kSW * g.ycap * (8 * g.NB + 2) : 0) + (size_t)g.NS * 16;
+static size_t stream_smem(const StreamGeo& g, size_t es, bool offsets_in_smem, bool prior) {
+    const size_t slice = (size_t)kSW * g.Lw * es + 16, stage = slice + (size_t)kSW * g.ystage;
+    // + the slice of a prior, cache (8 bytes per slot and live row) and offsets (2 bytes per slot) where they live here, barriers
+    return (size_t)g.NS * stage + (prior ? slice : 0) + (offsets_in_smem ? (size_t)kSW * g.ycap * (8 * g.NB + 2) : 0) + (size_t)g.NS * 16;
 }
 
 constexpr size_t kStreamSmemBudget = 212 * 1024;    // dynamic shared memory a CTA may ask for: 227 KB less the static part (14.2 KB)
 
 // Stage count, live rows and cache capacity for a vocabulary of N tokens with n kept ids; false when
 // the shapes do not fit shared memory.
-static bool plan_stream(int N, int n, size_t es, size_t ys, bool fast_types, StreamGeo& g) {
+static bool plan_stream(int N, int n, size_t es, size_t ys, bool fast_types, bool prior, StreamGeo& g) {
     const size_t budget = kStreamSmemBudget;
     StreamSegs sg;
     if (!stream_segments(N, es, sg)) return false;
@@ -888,7 +1080,7 @@ static bool plan_stream(int N, int n, size_t es, size_t ys, bool fast_types, Str
         g.ycap = (int)c;
         g.ystage = (int)((((size_t)c + 16) * ys + 15) & ~size_t(15));
         const bool in_regs = fast_types && fast_steps(g, g.nv) > 0;
-        return stream_smem(g, es, !in_regs) <= budget;
+        return stream_smem(g, es, !in_regs, prior) <= budget;
     };
     // The exchange of a row between the CTAs of its group takes several microseconds (two round trips to L2
     // and the folding on either side), and a row holds its place in the pair cache for that long: the
@@ -898,11 +1090,12 @@ static bool plan_stream(int N, int n, size_t es, size_t ys, bool fast_types, Str
     g.ycap = (int)cap;
     if (fast_types && fast_steps(g, g.nv) > 0) {
         const int nst = fast_steps(g, g.nv);
-        g.NB = kTmemWarpCols / (4 * nst);
+        g.NB = (kTmemWarpCols - tmem_rows_at(nst, prior)) / (4 * nst);
         if (g.NB > kMaxNB) g.NB = kMaxNB;
         for (g.NS = 4; g.NS >= 2; --g.NS)
             if (fits(cap)) return true;
     }
+    if (prior) return false;
     // Otherwise the cache shares shared memory with the stages: prefer live rows over stages, then give up cache.
     static const int pref[][2] = {{4, 3}, {5, 2}, {4, 2}, {3, 3}, {3, 2}};     // {NB, NS}, by measured speed
     for (const auto& pr : pref) {
@@ -916,10 +1109,10 @@ static bool plan_stream(int N, int n, size_t es, size_t ys, bool fast_types, Str
 
 static std::atomic<unsigned> g_spin_limit{0};     // 0: the default
 
-template <typename TZ, typename TY, int KIND, int NIT, int NST>
+template <typename TZ, typename TY, int KIND, int NIT, int NST, bool PRI>
 static cudaError_t launch_stream(const RowParams& P, StreamGeo g, cudaStream_t s) {
-    auto kern = rdk_stream_kernel<TZ, TY, KIND, NIT, NST>;
-    const size_t smem = stream_smem(g, sizeof(TZ), NST == 0);
+    auto kern = rdk_stream_kernel<TZ, TY, KIND, NIT, NST, PRI>;
+    const size_t smem = stream_smem(g, sizeof(TZ), NST == 0, PRI);
     // how many CTAs are resident at once (cached per kernel instance, shared-memory size and device)
     static thread_local int c_dev = -1, c_ctas = 0, sms = 0;
     static thread_local size_t c_smem = 0;
@@ -993,15 +1186,15 @@ static cudaError_t launch_stream(const RowParams& P, StreamGeo g, cudaStream_t s
     dattr[0].val.programmaticStreamSerializationAllowed = 1;
     dcfg.attrs = dattr;
     dcfg.numAttrs = 1;
-    if (small_ctas) return cudaLaunchKernelEx(&dcfg, rdk_draw_kernel<TZ, TY, KIND, 128>, P, g.C * kSW, g.Lw);
-    return cudaLaunchKernelEx(&dcfg, rdk_draw_kernel<TZ, TY, KIND, 256>, P, g.C * kSW, g.Lw);
+    if (small_ctas) return cudaLaunchKernelEx(&dcfg, rdk_draw_kernel<TZ, TY, KIND, 128, PRI>, P, g.C * kSW, g.Lw);
+    return cudaLaunchKernelEx(&dcfg, rdk_draw_kernel<TZ, TY, KIND, 256, PRI>, P, g.C * kSW, g.Lw);
 }
 
 template <typename TZ, typename TY, int KIND>
 static cudaError_t launch_nit(const RowParams& P, const StreamGeo& g, cudaStream_t s) {
     // the common segment length (four 16-byte vectors per lane) gets the register-resident sweep
-    if (g.nv == kFastNit) return launch_stream<TZ, TY, KIND, kFastNit, 0>(P, g, s);
-    return launch_stream<TZ, TY, KIND, 0, 0>(P, g, s);
+    if (g.nv == kFastNit) return launch_stream<TZ, TY, KIND, kFastNit, 0, false>(P, g, s);
+    return launch_stream<TZ, TY, KIND, 0, 0, false>(P, g, s);
 }
 
 template <typename TZ, typename TY>
@@ -1010,15 +1203,16 @@ static cudaError_t launch_kind_s(const RowParams& P, int kind, const StreamGeo& 
 }
 
 // bf16 logits on both sides with the common segment length: the kept-token passes unrolled
+template <bool PRI>
 static cudaError_t launch_fast(const RowParams& P, const StreamGeo& g, int nst, cudaStream_t s) {
     using B = __nv_bfloat16;
     switch (nst) {
-        case 1: return launch_stream<B, B, RDK_LOGITS, kFastNit, 1>(P, g, s);
-        case 2: return launch_stream<B, B, RDK_LOGITS, kFastNit, 2>(P, g, s);
-        case 3: return launch_stream<B, B, RDK_LOGITS, kFastNit, 3>(P, g, s);
-        case 4: return launch_stream<B, B, RDK_LOGITS, kFastNit, 4>(P, g, s);
-        case 5: return launch_stream<B, B, RDK_LOGITS, kFastNit, 5>(P, g, s);
-        case 6: return launch_stream<B, B, RDK_LOGITS, kFastNit, 6>(P, g, s);
+        case 1: return launch_stream<B, B, RDK_LOGITS, kFastNit, 1, PRI>(P, g, s);
+        case 2: return launch_stream<B, B, RDK_LOGITS, kFastNit, 2, PRI>(P, g, s);
+        case 3: return launch_stream<B, B, RDK_LOGITS, kFastNit, 3, PRI>(P, g, s);
+        case 4: return launch_stream<B, B, RDK_LOGITS, kFastNit, 4, PRI>(P, g, s);
+        case 5: return launch_stream<B, B, RDK_LOGITS, kFastNit, 5, PRI>(P, g, s);
+        case 6: return launch_stream<B, B, RDK_LOGITS, kFastNit, 6, PRI>(P, g, s);
         default: return cudaErrorNotSupported;
     }
 }
@@ -1051,7 +1245,7 @@ const char* stream_ineligible(const RowParams& P, int tz, int ty, int kind, int 
     if (P.N < kStreamMinN) return "N < 4096";
     if (P.qtilde) return "q~ is written out";
     if (P.rows <= 0 || P.trials <= 0) return "no draws";
-    if (P.prior) return "separate prior";
+    if (P.prior && (P.prior_stride || (reinterpret_cast<uintptr_t>(P.prior) & 15u))) return "a prior for each row, or not 16-byte aligned";
     // rows of the target start on 16-byte boundaries; drafter values are read in aligned pairs
     if ((reinterpret_cast<uintptr_t>(P.target) & 15u) || ((P.target_stride * (long long)es) & 15)) return "target rows not 16-byte aligned";
     if ((reinterpret_cast<uintptr_t>(P.drafter) & 15u) || (P.drafter_stride & 1)) return "drafter base not 16-byte aligned or odd drafter row stride";
@@ -1060,7 +1254,8 @@ const char* stream_ineligible(const RowParams& P, int tz, int ty, int kind, int 
     // ascending, valid kept ids only, as recorded when the index was built (the kernel re-checks the header)
     if (index_order(P.header, P.N, P.n) != 1) return "kept ids not ascending and valid (or index not prepared at this address)";
     StreamGeo g;
-    if (!plan_stream(P.N, P.n, es, ys, fast_types(tz, ty, kind), g)) return "shapes beyond shared memory";
+    if (!plan_stream(P.N, P.n, es, ys, fast_types(tz, ty, kind), P.prior != nullptr, g)) return "shapes beyond shared memory";
+    if (P.prior && !(fast_types(tz, ty, kind) && fast_steps(g, g.nv) > 0)) return "a prior beside other types or segment lengths than the common ones";
     return nullptr;
 }
 
@@ -1091,7 +1286,7 @@ cudaError_t launch_stream_linear(RowParams P, int tz, int ty, int kind, int batc
     const size_t es = tz == RDK_F32 ? 4 : 2, ys = ty == RDK_F32 ? 4 : 2;
     if (stream_ineligible(P, tz, ty, kind, batch, ws, ws_bytes)) return cudaErrorNotSupported;
     StreamGeo g;
-    if (!plan_stream(P.N, P.n, es, ys, fast_types(tz, ty, kind), g)) return cudaErrorNotSupported;
+    if (!plan_stream(P.N, P.n, es, ys, fast_types(tz, ty, kind), P.prior != nullptr, g)) return cudaErrorNotSupported;
     g.G = 0;
     g.tag = next_tag();
     g.spin_limit = stream_spin_limit() ? stream_spin_limit() : kSpinLimitDefault;
@@ -1103,7 +1298,7 @@ cudaError_t launch_stream_linear(RowParams P, int tz, int ty, int kind, int batc
     P.xrec = reinterpret_cast<unsigned char*>(ws) + ws_off_xrec(P.rows, batch, P.trials);
     if (fast_types(tz, ty, kind)) {
         const int nst = fast_steps(g, g.nv);
-        if (nst > 0) return launch_fast(P, g, nst, s);
+        if (nst > 0) return P.prior ? launch_fast<true>(P, g, nst, s) : launch_fast<false>(P, g, nst, s);
     }
     if (tz == RDK_F32) return ty == RDK_F32 ? launch_kind_s<float, float>(P, kind, g, s) : launch_kind_s<float, __nv_bfloat16>(P, kind, g, s);
     return ty == RDK_F32 ? launch_kind_s<__nv_bfloat16, float>(P, kind, g, s) : launch_kind_s<__nv_bfloat16, __nv_bfloat16>(P, kind, g, s);
@@ -1122,10 +1317,10 @@ extern "C" int rdk_stream_geometry(int32_t N, int32_t n, int32_t target_dtype, i
     const bool ft = fast_types(target_dtype, drafter_dtype, RDK_LOGITS);
     StreamGeo g;
     *out = rdk_stream_geometry_t{};
-    out->supported = plan_stream(N, n, es, ys, ft, g) ? 1 : 0;
+    out->supported = plan_stream(N, n, es, ys, ft, false, g) ? 1 : 0;
     if (!out->supported) return RDK_OK;
     out->ctas_per_row = g.C; out->warps_per_cta = kSW; out->segment_tokens = g.Lw; out->stages = g.NS;
     out->live_rows = g.NB; out->cached_slots_per_warp = g.ycap;
-    out->dynamic_shared_bytes = (int64_t)stream_smem(g, es, !(ft && fast_steps(g, g.nv) > 0));
+    out->dynamic_shared_bytes = (int64_t)stream_smem(g, es, !(ft && fast_steps(g, g.nv) > 0), false);
     return RDK_OK;
 }

@@ -328,3 +328,47 @@ def test_index_written_by_the_kernel_queued_just_before_the_call():
         out = rdk.rdk_sample_and_verify(moved, B.RDK_MODE_LINEAR, z, y, None, u, rows, 1)
         for name in ("draft_token", "alpha", "theta", "S"):
             assert torch.equal(out[name], want[k & 1][name]), (k, name)
+
+
+# One prior row for all rows through the streaming kernels, and the same shapes without it: groups of unequal length and of one
+# row; kept tokens per segment from none to all of them (segments that outgrow the cached slots), one to six steps of 64 slots
+@pytest.mark.parametrize("N,n,rows,kept", [
+    (16384, 900, 450, "random"), (65536, 8000, 190, "random"), (65536, 11000, 149, "highest"), (65536, 13000, 131, "random"),
+    (65536, 20000, 160, "lowest"), (131072, 7000, 90, "highest"), (131064, 34000, 83, "random"), (262144, 4000, 70, "random")])
+@pytest.mark.parametrize("shared_prior", [False, True])
+def test_stream_kernel_shared_prior(N, n, rows, kept, shared_prior):
+    cfg = W.tiny_config(N=N, n=n, rows=rows, dtype="bf16", trials=1, rho=0.7, seed=n, zipf_bias=True)
+    g = torch.Generator().manual_seed(n)
+    ids = {"random": torch.sort(torch.randperm(N, generator=g)[:n]).values, "lowest": torch.arange(n), "highest": torch.arange(N - n, N)}[kept]
+    inp = W.make_inputs(cfg)
+    inp["kept_ids"] = ids.to(inp["kept_ids"].dtype)
+    rdk = _rdk()
+    idx = rdk.rdk_prepare_ids(inp["kept_ids"].to(torch.int32).cuda(), N)
+    z, y, u = inp["target"].cuda(), inp["drafter"].cuda(), inp["uniforms"].cuda()
+    z[rows // 2, : N // 3] = -float("inf")               # whole segments without weight
+    y[rows - 1, n // 2:] += 60.0                         # the first kept value is a poor scale
+    inp["target"], inp["drafter"] = z, y
+    B = rdk.binding
+    prior = None
+    if shared_prior:
+        prior = (torch.randn(N, generator=g) * 2).to(torch.bfloat16)
+        prior[5] = -float("inf")
+        pb = B.make_problem(idx, z, y, cfg.batch, cfg.positions)
+        wanted = B.lib().rdk_sample_prior_workspace_bytes(B.C.byref(pb), z.data_ptr(), prior.cuda().data_ptr(), 0, y.data_ptr(), 1)
+        assert wanted > 0                                # the streaming kernels serve
+        out = rdk.rdk_sample_and_verify_prior(idx, z, prior.cuda(), y, u, cfg.batch, cfg.positions)
+    else:
+        out = rdk.rdk_sample_and_verify(idx, B.RDK_MODE_LINEAR, z, y, None, u, cfg.batch, cfg.positions)
+    torch.cuda.synchronize()
+    B.check_status_word(out)
+    some = sorted({0, 1, rows // 2, rows - 2, rows - 1})
+    PU.compare_sampling(inp, out, some, "linear", prior=prior).assert_ok()
+    # every row against the one-CTA-per-row or the cluster kernel
+    if shared_prior:
+        ref = rdk.rdk_sample_and_verify_prior(idx, z, prior.cuda().expand(rows, N).contiguous(), y, u, cfg.batch, cfg.positions)
+    else:
+        ref = rdk.rdk_sample_and_verify(idx, B.RDK_MODE_LINEAR, z, y, None, u, cfg.batch, cfg.positions, flags=B.RDK_FLAG_ROW_KERNEL)
+    torch.cuda.synchronize()
+    for k in ("alpha", "theta", "S", "residual_mass"):
+        assert float((out[k] - ref[k]).abs().max()) < 1e-5, k
+    assert int((out["draft_token"] != ref["draft_token"]).sum()) <= max(2, rows // 20)
