@@ -24,6 +24,9 @@
 //   kVarDense   any N, q~ output and small vocabularies, with or without a prior: a fp32 array of q' for all tokens of
 //               the segment beside the logits.
 //   kVarGiven   w in place of q'.
+#include <math.h>
+#include <string.h>
+
 #include <atomic>
 #include <type_traits>
 
@@ -204,10 +207,15 @@ __device__ __forceinline__ void count_accepted(const RowParams& P, uint32_t tag,
     *out = k;
 }
 
-template <typename TZ, typename TY, int KIND, int VAR, bool kPrior>
-// 80 registers where two arrays and the draws' two chunks need them (320 rows of 128k with a prior: 117 -> 111 us, although a
-// CTA of 512 threads then has the SM to itself), 64 elsewhere (given weights of 1024 x 32k: 66 us, with 80 registers 70)
-__global__ void __maxnreg__(VAR == kVarPrior ? 80 : 64)
+// Registers a thread: with many CTAs, what lets most of them be resident: 80 where two arrays and the draws' two chunks need
+// them (320 rows of 128k with a prior: 117 -> 111 us, although a CTA of 512 threads then has the SM to itself), 64
+// elsewhere (given weights of 1024 x 32k: 66 us, with 80 registers 70).  ROOMY, for calls whose CTAs all fit beside one another
+// all the same: 128, nothing spilled and more loads in flight in a row's chain (5 rows of 128257 bf16 10.4 -> 8.7 us, with four
+// trials 12.9 -> 9.5; 1 row of 5001 7.0 -> 6.4, given weights of 1 x 128256 8.1 -> 7.0).
+template <int VAR, bool ROOMY> constexpr int clu_registers() { return ROOMY ? 128 : (VAR == kVarPrior ? 80 : 64); }
+
+template <typename TZ, typename TY, int KIND, int VAR, bool kPrior, bool ROOMY>
+__global__ void __maxnreg__((clu_registers<VAR, ROOMY>()))
 rdk_cluster_kernel(const RowParams P, const CluGeo g) {
     constexpr bool kLinear = VAR != kVarGiven, kDense = VAR == kVarDense || VAR == kVarGiven;
     constexpr uint32_t es = (uint32_t)sizeof(TZ);
@@ -913,45 +921,130 @@ rdk_cluster_kernel(const RowParams P, const CluGeo g) {
 // ------------------------------------------------------------------------------------------------
 // host side
 // ------------------------------------------------------------------------------------------------
-constexpr int kCluStatic = 6 * 1024;                            // static shared memory of the kernel, rounded up
-constexpr int kCluDynamic = 227 * 1024 - kCluStatic;
+constexpr int kCluStatic = 7 * 1024;                            // static shared memory of the kernel and what a CTA has besides, rounded up
+constexpr int kCluDynamic = 227 * 1024 - 6 * 1024 - 512;
+constexpr int kCluSms = 148;
 
-struct CluShape { int C, nw, per; size_t smem; };
+struct CluShape { int C, nw, per; size_t smem; bool roomy; float cost; };
+
+// A rule of thumb for the time of a call with a given shape, in us: launch and row statistics, then for every wave of CTAs a
+// chain (k; km where waves follow one another), b for each 256-position chunk of a warp, what the number of warps and CTAs of a row adds
+// to the exchange and to the prefix sums, a second pass over the chunks for the draws (unless there is but one), more
+// rounds of draws, kept tokens beyond a warp's registers (visited in memory, twice) and the warps that share the SM.
+// The constants are a fit to measured calls: 30 to 40 shapes each of 350 problems (N from 5001 to 262143, 1 to 1000 rows, bf16
+// and fp32).  The shape that the rule picks is within 2 to 4 % of the fastest one tried on average; powers of
+// two alone, which this replaces as the last word, were 8 to 15 % off (50257 tokens: 80 rows 16.9 -> 12.3 us, 320 rows
+// 44.8 -> 33.5; 128257: 320 rows 86.4 -> 70.4; q~ of 80 x 262143: 114.6 -> 62.1; given weights of 40 x 50240: 11.4 -> 8.7).
+struct CluCost {
+    float t0, k, km, b, seg, cluster, second, over, warps, tail, fill, roomy, draws;
+};
+constexpr CluCost kCostFewDraws{3.794f, 1.737f, 0.762f, 0.742f, 0.015f, 0.501f, 0.394f, 2.617f, 2.986f, 0.006f, 0.776f, 0.902f, 1.884f};
+constexpr CluCost kCostManyDraws{4.506f, 1.475f, 1.116f, 1.927f, 0.153f, 0.55f, 1.387f, 3.974f, 0.42f, 0.272f, 0.83f, 0.631f, 1.077f};
+constexpr CluCost kCostDense{3.425f, 2.429f, 4.145f, 0.574f, 0.275f, 0.081f, 0.168f, 0.151f, 0.69f, 0.281f, 0.876f, 0.845f, 0.117f};
+constexpr CluCost kCostPrior{4.82f, 4.042f, 1.734f, 1.087f, 0.033f, 0.61f, 0.494f, 0.034f, 2.926f, 0.829f, 0.949f, 0.982f, 1.884f};
+constexpr CluCost kCostGiven{3.984f, 0.916f, 1.611f, 0.565f, 1.035f, 0.125f, 0.613f, 2.38f, 0.613f, 0.48f, 0.87f, 0.846f, 0.713f};
+
+// The shape with C CTAs a row and at most `warps` warps each; false where a row does not fit.
+static bool shape_cluster(long long positions, int C, int warps, size_t bytes, bool roomy, CluShape& s) {
+    const int chunks = (int)((positions + C * 256 - 1) / (C * 256)), per = (chunks + warps - 1) / warps;
+    const int nw = (chunks + per - 1) / per;
+    s.C = C; s.nw = nw < 4 ? 4 : nw; s.per = per * 32; s.roomy = roomy;
+    s.smem = (size_t)s.nw * s.per * kVec * bytes;
+    if (s.smem < sizeof(DrawSmem)) s.smem = sizeof(DrawSmem);
+    return s.smem <= (size_t)kCluDynamic && per <= kCluMaxChunks;
+}
+
+// CTAs of a shape that an SM holds
+static int resident_ctas(const CluShape& s, int registers) {
+    const int by_smem = (int)(228u * 1024u / (s.smem + kCluStatic + 256)), by_regs = 65536 / (registers * 32 * s.nw), by_warps = 64 / s.nw;
+    const int n = by_smem < by_regs ? by_smem : by_regs;
+    return n < by_warps ? (n < 1 ? 1 : n) : by_warps;
+}
+
+static float cost_cluster(const CluCost& c, const CluShape& s, int rows, int trials, int registers, float kept, int kept_slots) {
+    const int slots = resident_ctas(s, registers), chunks = s.per / 32;
+    // (clusters do not fill the chip to the last SM: they stay within a group of SMs)
+    int cap = s.C > 1 ? (int)(c.fill * (float)(kCluSms * slots) / (float)s.C) : kCluSms * slots;
+    if (cap < 1) cap = 1;
+    const float waves = (float)rows / (float)cap;
+    float resident = (float)rows * (float)s.C / (float)kCluSms;
+    resident = resident < 1.f ? 1.f : (resident > (float)slots ? (float)slots : resident);
+    const float most = kept * 256.f * (float)chunks + 2.f * sqrtf(kept * 256.f * (float)chunks);     // kept tokens of a warp, nearly at most
+    const float over = most > (float)kept_slots ? ceilf((most - (float)kept_slots) / 128.f) : 0.f;
+    const int rounds = (trials * chunks + s.nw - 1) / s.nw - 1;                                        // two draws a trial, two chunks a turn
+    const float one = (waves > 1.f ? c.km : c.k) + c.b * (float)chunks + c.seg * (float)(s.C * s.nw) / 128.f + (s.C > 1 ? c.cluster : 0.f) +
+                      (chunks > 1 ? c.second : 0.f) + c.over * over + c.warps * resident * (float)s.nw / 32.f + c.draws * (float)(rounds > 0 ? rounds : 0);
+    return c.t0 + (waves > 1.f ? waves + c.tail : 1.f) * one * (s.roomy ? c.roomy : 1.f);
+}
 
 // CTAs per row, warps per CTA and vectors per warp; false when a row does not fit a cluster's shared memory.  `lead`: most
 // positions before a row's first token.
-static bool plan_cluster(int N, int rows, int trials, size_t es, int variant, bool prior, int lead, CluShape& s) {
+static bool plan_cluster_anew(int N, int n, int rows, int trials, size_t es, int variant, bool prior, int lead, CluShape& s) {
     const size_t bytes = es * (prior ? 2 : 1) + (variant == kVarDense || variant == kVarGiven ? 4 : 0);    // per position
     const long long positions = (long long)N + lead;
+    const int registers = variant == kVarPrior ? 80 : 64;
     int C = 1;
     if (N >= kStreamMinN) {
         // three CTAs to an SM, whose phases of copying, exponentials and waiting overlap (320 rows of 128k with a prior: 112 us) ...
         while (C < kCluMaxCtas && (long long)bytes * (positions / C) > 64 * 1024) C *= 2;
         // ... and, with few rows, enough CTAs to fill the chip four times over, while each has 4096 positions or more (with
         // less the exchange between the CTAs costs more than the sweep)
-        while (C < kCluMaxCtas && (long long)rows * C < 4 * 148 && positions / C > 4096) C *= 2;
+        while (C < kCluMaxCtas && (long long)rows * C < 4 * kCluSms && positions / C > 4096) C *= 2;
     }
     // about eight warps of equally many 256-position chunks each: more warps mean more per-warp overhead, fewer do not
     // hide each other's latencies (50257 tokens x 160 rows: 8 warps 29 us, 12 35, 16 46)
-    const int chunks = (int)((positions + C * 256 - 1) / (C * 256));
     // (sixteen, and shorter segments, where several draws a row keep the warps busy -- 32 rows of 32k with four trials 16.6 ->
     // 14.1 us, 1500 rows of 8k with eight 107 -> 84 -- and where the CTAs are fewer than two an SM and not many share a row:
     // 100 rows of 3000 10.4 -> 9.0 us, 4 rows of 8k 7.7 -> 7.2, but 5 rows of 128k on 16 CTAs each 8.9 -> 9.3)
-    const int warps = trials >= 3 || ((long long)rows * C < 2 * 148 && C < kCluMaxCtas) ? kCluMaxWarps : 8;
-    const int per_warp = (chunks + warps - 1) / warps;
-    const int nw = (chunks + per_warp - 1) / per_warp;
-    s.C = C; s.nw = nw < 4 ? 4 : nw;
+    const int warps = trials >= 3 || ((long long)rows * C < 2 * kCluSms && C < kCluMaxCtas) ? kCluMaxWarps : 8;
+    bool found = shape_cluster(positions, C, warps, bytes, false, s);
+    if (N < kStreamMinN) {
+        CluShape r;      // a CTA holds the row either way
+        if (shape_cluster(positions, C, warps, bytes, true, r) && rows <= kCluSms * resident_ctas(r, 128)) { s = r; found = true; }
+    } else {
+        const CluCost& c = variant == kVarGiven ? kCostGiven : (variant == kVarDense ? kCostDense : (variant == kVarPrior ? kCostPrior : (trials >= 3 ? kCostManyDraws : kCostFewDraws)));
+        const float kept = variant == kVarGiven ? 0.f : fminf(1.f, (float)n / (float)N);
+        const int kept_slots = variant == kVarSparse ? 384 : 256;
+        // another shape where the rule promises more than it is off by itself
+        if (found) s.cost = cost_cluster(c, s, rows, trials, registers, kept, kept_slots);
+        float best = found ? 0.95f * s.cost : INFINITY;
+        for (int k : {1, 2, 3, 4, 5, 6, 8, 10, 16})
+            for (int w = 8; w <= kCluMaxWarps; w += 8)
+                for (int roomy = 0; roomy < 2; ++roomy) {
+                    CluShape t;
+                    if (!shape_cluster(positions, k, w, bytes, roomy != 0, t)) continue;
+                    const int regs = roomy ? 128 : registers;
+                    if (roomy && (float)rows * (float)k > c.fill * (float)(kCluSms * resident_ctas(t, regs))) continue;      // (measured where one wave holds them)
+                    t.cost = cost_cluster(c, t, rows, trials, regs, kept, kept_slots);
+                    if (t.cost < best) { best = t.cost; s = t; found = true; }
+                }
+    }
     // segments of one chunk and several draws a row: a warp for each draw, also where there is nothing to sweep for it
-    if (per_warp == 1 && (long long)rows * C < 4 * 148 && 2 * trials > s.nw) s.nw = 2 * trials < kCluMaxWarps ? 2 * trials : kCluMaxWarps;
-    s.per = per_warp * 32;
-    s.smem = (size_t)s.nw * s.per * kVec * bytes;
-    if (s.smem < sizeof(DrawSmem)) s.smem = sizeof(DrawSmem);
-    return s.smem <= (size_t)kCluDynamic && s.per <= 32 * kCluMaxChunks;
+    if (found && s.per == 32 && (long long)rows * s.C < 4 * kCluSms && 2 * trials > s.nw) {
+        s.nw = 2 * trials < kCluMaxWarps ? 2 * trials : kCluMaxWarps;
+        const size_t smem = (size_t)s.nw * s.per * kVec * bytes;
+        if (smem > s.smem) s.smem = smem;
+    }
+    return found;
+}
+// The last few plans of the calling thread: trying all shapes takes the host a microsecond.
+static bool plan_cluster(int N, int n, int rows, int trials, size_t es, int variant, bool prior, int lead, CluShape& s) {
+    struct Plan { int key[8]; CluShape shape; bool found; };
+    static thread_local Plan plans[4] = {};
+    static thread_local unsigned next = 0;
+    const int key[8] = {N, n, rows, trials, (int)es, variant, prior ? 1 : 0, lead};
+    for (const Plan& p : plans)
+        if (p.key[0] && !memcmp(p.key, key, sizeof(key))) { s = p.shape; return p.found; }
+    Plan& p = plans[next++ & 3u];
+    p.found = plan_cluster_anew(N, n, rows, trials, es, variant, prior, lead, p.shape);
+    memcpy(p.key, key, sizeof(key));
+    s = p.shape;
+    return p.found;
 }
 
-template <typename TZ, typename TY, int KIND, int VAR, bool PRIOR>
-static cudaError_t launch_cluster(const RowParams& P, CluGeo g, const CluShape& sh, cudaStream_t s) {
-    auto kern = rdk_cluster_kernel<TZ, TY, KIND, VAR, PRIOR>;
+template <typename TZ, typename TY, int KIND, int VAR, bool PRIOR, bool ROOMY>
+static cudaError_t launch_cluster_as(const RowParams& P, CluGeo g, const CluShape& sh, cudaStream_t s) {
+    auto kern = rdk_cluster_kernel<TZ, TY, KIND, VAR, PRIOR, ROOMY>;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -969,8 +1062,8 @@ static cudaError_t launch_cluster(const RowParams& P, CluGeo g, const CluShape& 
     cfg.attrs = attr;
     cfg.numAttrs = 2;
     // once per kernel, device and cluster size: the limits raised, and whether such a cluster can be resident at all
-    static std::atomic<uint32_t> known[64];                       // bit log2(C): asked; bit 8 + log2(C): fits
-    const uint32_t bit = (uint32_t)__builtin_ctz((unsigned)sh.C);
+    static std::atomic<uint32_t> known[64];                       // bit C - 1: asked; bit 16 + C - 1: fits
+    const uint32_t bit = (uint32_t)sh.C - 1u;
     uint32_t k = known[dev].load(std::memory_order_acquire);
     if (!(k >> bit & 1u)) {
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kCluDynamic);
@@ -983,11 +1076,16 @@ static cudaError_t launch_cluster(const RowParams& P, CluGeo g, const CluShape& 
         int fit = 0;
         e = cudaOccupancyMaxActiveClusters(&fit, kern, &q);
         if (e != cudaSuccess) { (void)cudaGetLastError(); fit = 0; }
-        k = (1u << bit) | (fit > 0 ? 256u << bit : 0u);
+        k = (1u << bit) | (fit > 0 ? 65536u << bit : 0u);
         k |= known[dev].fetch_or(k, std::memory_order_acq_rel);
     }
-    if (!(k >> (8 + bit) & 1u)) return cudaErrorNotSupported;
+    if (!(k >> (16 + bit) & 1u)) return cudaErrorNotSupported;
     return cudaLaunchKernelEx(&cfg, kern, P, g);
+}
+
+template <typename TZ, typename TY, int KIND, int VAR, bool PRIOR>
+static cudaError_t launch_cluster(const RowParams& P, const CluGeo& g, const CluShape& sh, cudaStream_t s) {
+    return sh.roomy ? launch_cluster_as<TZ, TY, KIND, VAR, PRIOR, true>(P, g, sh, s) : launch_cluster_as<TZ, TY, KIND, VAR, PRIOR, false>(P, g, sh, s);
 }
 
 template <typename TZ, typename TY, int KIND>
@@ -1002,6 +1100,14 @@ static cudaError_t launch_kind_c(const RowParams& P, const CluGeo& g, const CluS
     return kind == RDK_LOGITS ? launch_variant<TZ, TY, RDK_LOGITS>(P, g, sh, variant, s) : launch_variant<TZ, TY, RDK_PROBS>(P, g, sh, variant, s);
 }
 
+// What the rule above expects of a linear call of 16-byte aligned rows, in us (INFINITY where no shape fits), times what it was
+// low by on average for calls of that kind.
+float cluster_rows_cost(const RowParams& P, size_t es) {
+    CluShape sh;
+    if (P.N < kStreamMinN || !plan_cluster(P.N, P.n, P.rows, P.trials, es, P.prior ? kVarPrior : kVarSparse, P.prior != nullptr, 0, sh)) return INFINITY;
+    return sh.cost * (P.prior ? 1.18f : (P.trials == 2 ? 1.14f : 1.06f));
+}
+
 cudaError_t launch_cluster_rows(RowParams P, int mode, int tz, int ty, int kind, uint32_t tag, unsigned spin_limit, cudaStream_t s) {
     using B = __nv_bfloat16;
     const size_t es = tz == RDK_F32 ? 4 : 2;
@@ -1009,7 +1115,7 @@ cudaError_t launch_cluster_rows(RowParams P, int mode, int tz, int ty, int kind,
                         : (P.qtilde || P.N < kStreamMinN ? kVarDense : (P.prior ? kVarPrior : kVarSparse));
     CluShape sh;
     const bool aligned = !(reinterpret_cast<uintptr_t>(P.target) & 15u) && !((P.target_stride * (long long)es) & 15);
-    if (!plan_cluster(P.N, P.rows, P.trials, es, variant, P.prior != nullptr, aligned ? 0 : (int)(16 / es) - 1, sh)) return cudaErrorNotSupported;
+    if (!plan_cluster(P.N, P.n, P.rows, P.trials, es, variant, P.prior != nullptr, aligned ? 0 : (int)(16 / es) - 1, sh)) return cudaErrorNotSupported;
     if ((long long)P.rows * sh.C > 0x7fffffffLL) return cudaErrorNotSupported;
     CluGeo g;
     g.per = sh.per;

@@ -37,10 +37,9 @@
 // * S = sum_j w_j = 1 + O(N^-2), because sum q' = 1 and sum q'_j p_j = theta cancel the
 //   first-order terms; it is taken as 1.
 //
-// With one prior row pi for all rows in place of p inside the formula the same kernel keeps the CTA's slice of pi and all that
-// no row changes about it, so that a row costs it one set of exponentials more at the kept tokens' second visit only in
-// arithmetic.  320 rows of 128256 tokens: 54 us, with the draws; the cluster kernel, which reads pi and takes its soft-max
-// anew for every row, 111.
+// With one prior row pi for all rows in place of p inside the formula, the same kernel keeps the CTA's slice of pi and all that no
+// row changes about it, so pi costs a row no exponentials.  320 rows of 128256 tokens: 54 us, with the draws; the cluster
+// kernel, which reads pi and takes its soft-max anew for every row, 111.
 #include <atomic>
 #include <chrono>
 

@@ -330,6 +330,39 @@ def test_index_written_by_the_kernel_queued_just_before_the_call():
             assert torch.equal(out[name], want[k & 1][name]), (k, name)
 
 
+# Shapes on clusters of other sizes than powers of two, of eight and of sixteen warps, with many and with few registers; more
+# than one wave of them; more kept tokens than fit a warp's registers
+@pytest.mark.parametrize("N,n,rows,trials,dtype", [
+    (5001, 500, 40, 1, "bf16"), (20011, 2000, 20, 1, "f32"), (33333, 8333, 40, 1, "bf16"), (33333, 8333, 45, 4, "f32"),
+    (50257, 12565, 80, 1, "bf16"), (50257, 12565, 330, 2, "bf16"), (90001, 30000, 20, 1, "f32"), (128257, 3000, 24, 5, "bf16"),
+    (262143, 100000, 5, 1, "bf16")])
+def test_cluster_kernel_cluster_sizes(N, n, rows, trials, dtype):
+    cfg = W.tiny_config(N=N, n=n, rows=rows, dtype=dtype, trials=trials, rho=0.8, seed=rows, zipf_bias=True)
+    inp = W.make_inputs(cfg)
+    rdk = _rdk()
+    B = rdk.binding
+    idx = rdk.rdk_prepare_ids(inp["kept_ids"].cuda(), N)
+    z, y, u = inp["target"].cuda(), inp["drafter"].cuda(), inp["uniforms"].cuda()
+    out = rdk.rdk_sample_and_verify(idx, B.RDK_MODE_LINEAR, z, y, None, u, cfg.batch, cfg.positions)
+    ref = rdk.rdk_sample_and_verify(idx, B.RDK_MODE_LINEAR, z, y, None, u, cfg.batch, cfg.positions, flags=B.RDK_FLAG_ROW_KERNEL)
+    torch.cuda.synchronize()
+    B.check_status_word(out)
+    PU.compare_sampling(inp, out, sorted({0, rows // 2, rows - 1}), "linear").assert_ok()
+    for k in ("alpha", "theta", "S", "residual_mass"):
+        assert float((out[k] - ref[k]).abs().max()) < 1e-5, k
+    # a draw on the other side of a boundary: prefix sums 1e-7 apart, some 2 n interval ends (as in assert_ok_at_scale)
+    assert int((out["draft_token"] != ref["draft_token"]).sum()) <= 2 + 6e-7 * n * rows * trials
+    if trials == 1:
+        w = torch.softmax(z.float(), -1)
+        given = rdk.rdk_sample_and_verify(idx, B.RDK_MODE_PRECOMPUTED_W, z, None, w, u, cfg.batch, cfg.positions)
+        torch.cuda.synchronize()
+        assert float(given["accepted"].float().mean()) > 0.99 and float((given["alpha"] - 1).abs().max()) < 1e-5
+        if N < 100000:
+            qt, _, _ = rdk.rdk_redistribute_linear(idx, z, y, cfg.batch, cfg.positions)
+            torch.cuda.synchronize()
+            PU.compare_qtilde(qt, {0: O.rdk_row(W.to_f64(inp["target"][0]), W.to_f64(inp["drafter"][0]), inp["kept_ids"].numpy(), np.zeros((1, 4)), "linear")}, dtype == "bf16")
+
+
 # One prior row for all rows through the streaming kernels, and the same shapes without it: groups of unequal length and of one
 # row; kept tokens per segment from none to all of them (segments that outgrow the cached slots), one to six steps of 64 slots
 @pytest.mark.parametrize("N,n,rows,kept", [
