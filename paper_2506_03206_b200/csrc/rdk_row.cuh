@@ -145,6 +145,7 @@ void set_stream_spin_limit(unsigned limit);
 unsigned stream_spin_limit();
 
 bool stream_few_rows(const RowParams& P, int tz, int ty, int kind);
+float cluster_rows_cost(const RowParams& P, size_t es);
 // Launches the cluster kernel (rdk_row_cluster.cu) in either mode; cudaErrorNotSupported (nothing launched) when a row does
 // not fit the shared memory of a cluster.
 cudaError_t launch_cluster_rows(RowParams P, int mode, int tz, int ty, int kind, uint32_t tag, unsigned spin_limit, cudaStream_t s);

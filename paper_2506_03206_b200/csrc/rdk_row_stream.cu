@@ -1258,24 +1258,40 @@ const char* stream_ineligible(const RowParams& P, int tz, int ty, int kind, int 
     return nullptr;
 }
 
-// Whether so few rows are better served by one cluster launch each than by setting up the streaming grid and a second
-// kernel for the draws (the streaming kernels pay off when a group of CTAs has several rows to stream).  Sampling call, streaming /
-// cluster kernel, a quarter of the tokens kept, us:  8192 bf16: 11.0 / 8.5 for 4 rows, 14.6 / 11.4 for 160, 16.0 / 18.2 for 320;
-// 32768: 12.0 / 8.8 for 4, 16.2 / 15.5 for 96, 17.8 / 18.9 for 160; 128256: 12.8 / 10.3 for 4, 16.6 / 14.6 for 24, 18.6 / 20.9 for
-// 48; 262144: 13.7 / 11.1 for 4, 27.7 / 27.3 for 64; fp32 128256: 13.5 / 10.2 for 4, 32.0 / 31.6 for 96.  The cluster
-// kernel makes a row's draws in one CTA: not with many trials.  It visits kept tokens beyond a warp's 384 register slots in
-// memory, twice: with more of them (a warp of the largest cluster has n / 128) fewer rows, and few beyond twice as many.  262144
-// tokens: 65536 kept, 24 rows 21.7 / 19.5, 56 rows 28.2 / 30.7; 131072 kept, 1 row 17.2 / 15.4, 8 17.7 / 18.2, 24 25.2 / 26.9.
+// Whether the rows are better served by one cluster launch each than by setting up the streaming grid and a second kernel
+// for the draws (the streaming kernels pay off when a group of CTAs has several rows to stream): where the cluster kernel's
+// rule of thumb expects less time than this one.  12.3 us for one row a group, 1.8 more for the second kernel once it has a CTA
+// for nearly every SM, 1.9 for every further row of a group of four 16-byte vectors a lane (1.3 times that without the
+// unrolled pass), 3 where the draws take a second wave of CTAs, 4.7 for a prior's slice.  Measured, streaming / cluster, a quarter of
+// the tokens kept, us:  4608 bf16: 11.3 / 6.2 for 4 rows, 14.8 / 9.6 for 256, four draws a row 13.2 / 6.7 for 64; 8192: 15.1 / 10.5 for
+// 256, 16.4 / 16.5 for 320; 65536: 16.8 / 12.0 for 64, 20.0 / 21.3 for 128; 128256: 13.4 / 8.7 for 4, 17.3 / 15.5 for 32,
+// 20.3 / 21.8 for 64; with a prior 128256: 16.6 / 13.4 for 4, 21.6 / 24.7 for 32.  Over 540 such calls the faster kernel is
+// missed by 1.8 % on average; limits on the number of rows alone missed it by 6 %.
+// Rows of 16385 to 49152 tokens, and those that take a group of sixteen CTAs, keep such limits without a prior, as the route query
+// has told them: one or two draws, and up to 3200000 / N rows (24 or 96 above 32768; 56 for a group of sixteen).  The cluster
+// kernel visits kept tokens beyond a warp's 384 register slots in memory, twice: with more of them (a warp of the largest
+// cluster has n / 128) fewer rows, and few beyond twice as many.
 bool stream_few_rows(const RowParams& P, int tz, int ty, int kind) {
-    if (P.trials > 2) return false;
+    const size_t es = tz == RDK_F32 ? 4 : 2;
+    const bool fast = fast_types(tz, ty, kind);
     StreamSegs sg;
-    const bool one_group = stream_segments(P.N, tz == RDK_F32 ? 4 : 2, sg) && sg.C == kMaxGroup;      // 9 groups of 16 CTAs
-    int most = !fast_types(tz, ty, kind) ? 96 : (one_group ? 56 : 24);
-    if (P.N <= 32768) { const int small = 3200000 / P.N; most = most > small ? most : (small < 192 ? small : 192); }
-    const int kept = P.n / 128;
-    if (kept > 384 && most > 24) most = 24;
-    if (kept > 768) most = 4;
-    return P.rows <= most;
+    if (P.trials < 1 || !stream_segments(P.N, es, sg)) return false;
+    const bool sixteen = sg.C == kMaxGroup;                  // 9 groups of 16 CTAs
+    if (!P.prior && ((P.N > 16384 && P.N <= 49152) || sixteen)) {
+        if (P.trials > 2) return false;
+        int most = !fast ? 96 : (sixteen ? 56 : 24);
+        if (P.N <= 32768) most = most > 3200000 / P.N ? most : 3200000 / P.N;
+        const int kept = P.n / 128;
+        if (kept > 384 && most > 24) most = 24;
+        if (kept > 768) most = 4;
+        return P.rows <= most;
+    }
+    const int groups = 148 / sg.C, per_group = (P.rows + groups - 1) / groups;
+    const long long draws = (long long)P.rows * P.trials;
+    const float row = 1.87f * (float)sg.nv / 4.f * (fast && sg.nv == kFastNit ? 1.f : (es == 4 ? 0.85f : 1.3f));
+    const float t = 12.3f + (per_group > 1 ? 1.8f + row * (float)(per_group - 1) : (draws >= 120 ? 1.8f : 0.f)) + (draws > 740 && draws <= 8 * 148 ? 3.f : 0.f) +
+                    (P.prior ? 4.7f : 0.f) + (sg.C > 8 ? 0.9f : 0.f);
+    return cluster_rows_cost(P, es) < 0.97f * t;
 }
 
 void set_stream_spin_limit(unsigned limit) { g_spin_limit.store(limit); }
