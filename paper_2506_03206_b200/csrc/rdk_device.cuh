@@ -189,12 +189,12 @@ __device__ __forceinline__ void combine_records(float& E1, float& Zq, float& th,
     m = mm; my = mmy;
 }
 
-// The same where th is on the scale of Zq alone (E1 of a prior, all of whose records are on one scale, is not this E1); x is
-// summed up as it is.
+// The same on scales 2^m and 2^my, with th on that of Zq alone (e_pi, which it has in place of e_z, is on one scale in all
+// records); x is summed up as it is.
 __device__ __forceinline__ void combine_records_prior(float& E1, float& Zq, float& th, float& m, float& my, float& x, int lane) {
     const float mm = warp_max_redux(m), mmy = warp_max_redux(my);
-    const float f = m > -INFINITY ? ex2((m - mm) * kLog2e) : 0.f;
-    const float g = my > -INFINITY ? ex2((my - mmy) * kLog2e) : 0.f;
+    const float f = m > -INFINITY ? ex2(m - mm) : 0.f;
+    const float g = my > -INFINITY ? ex2(my - mmy) : 0.f;
     const float tot = warp_sum4(E1 * f, Zq * g, th * g, x, lane);
     E1 = __shfl_sync(0xffffffffu, tot, 0); Zq = __shfl_sync(0xffffffffu, tot, 8); th = __shfl_sync(0xffffffffu, tot, 16); x = __shfl_sync(0xffffffffu, tot, 24);
     m = mm; my = mmy;

@@ -419,6 +419,10 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
         const bool skip0 = w_dummy && lane == 0;
         const long long ystep = (long long)g.G * P.drafter_stride;
         const float2 l2e = splat(kLog2e);
+        // A scale of exponentials as it goes into the records, and what it adds to an exponent.  With a prior a whole power of two,
+        // as in the cluster kernel, which served these calls before: going from one scale to another is exact then.
+        auto scale = [](float m) -> float { return PRI ? (m > -INFINITY ? rintf(m * kLog2e) : -INFINITY) : m; };
+        auto offset = [](float s) -> float { return PRI ? (s > -INFINITY ? -s : 0.f) : (s > -INFINITY ? -s * kLog2e : 0.f); };
 
         // ---- what of the prior no row changes ------------------------------------------------------------
         float poff = 0.f;                                // its exponentials are on one scale in the CTA, a whole power of two
@@ -449,8 +453,7 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
         // of the row; `least` is the lane's smallest difference, taken in bf16 (hence the margin), and a lane with such a
         // token, one in some thirty, reads its part of the row again.  tx: theta x / e_pi, fz: p / e_z.
         auto violations = [&](int itb, int par, float tx, float fz, float least) -> float {
-            const float m_w = wrec[par][warp][4];
-            const float zoff = m_w > -INFINITY ? -m_w * kLog2e : 0.f;
+            const float zoff = offset(wrec[par][warp][4]);
             float c = (__log2f(tx) - __log2f(fz) + poff - zoff) * (1.f / kLog2e);
             c = c == c ? c + fabsf(c) * 0x1p-7f + 0.01f : INFINITY;
             float v = 0.f;
@@ -531,7 +534,7 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
                 const TZ* zrow = static_cast<const TZ*>(P.target) + row * P.target_stride;
                 const TY* yrow = static_cast<const TY*>(P.drafter) + row * P.drafter_stride;
                 const float m_w = wrec[par][warp][4], my_w = wrec[par][warp][5];
-                const float zoff = m_w > -INFINITY ? -m_w * kLog2e : 0.f, yoff = my_w > -INFINITY ? -my_w * kLog2e : 0.f;
+                const float zoff = offset(m_w), yoff = offset(my_w);
                 for (int il = kcs + lane; il < kcp; il += 32) {
                     const float ez = ex2(fmaf(to_float<TZ>(zrow[__ldg(P.ids + r0 + il)]), kLog2e, zoff));
                     const float y = to_float<TY>(yrow[r0 + il]);
@@ -586,9 +589,19 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
             float my_w = KIND == RDK_LOGITS ? -INFINITY : 0.f;
             if (KIND == RDK_LOGITS && kcp > w_dummy)
                 my_w = kcs > w_dummy ? lds_z<TY>(ysb_a + (uint32_t)w_dummy * (uint32_t)sizeof(TY)) : to_float<TY>(cy[w_dummy]);
-            const float m_w = warp_max_redux(mz.result());
-            const float zoff = m_w > -INFINITY ? -m_w * kLog2e : 0.f;
-            float yoff = my_w > -INFINITY ? -my_w * kLog2e : 0.f;
+            const float m_w = scale(warp_max_redux(mz.result()));
+            const float zoff = offset(m_w);
+            if constexpr (PRI) {     // theta is a sum of products here that no other sum has the rounding of: the maximum after all
+                my_w = -INFINITY;
+#pragma unroll
+                for (int st = 0; st < (NST > 0 ? NST : 1); ++st) {
+                    const float2 y = lds_ypair<TY>(ys_a + (uint32_t)st * 64u * (uint32_t)sizeof(TY));
+                    const bool v0 = (lim > st * 64) && !(st == 0 && skip0), v1 = lim > st * 64 + 1;
+                    my_w = fmaxf(my_w, fmaxf(v0 ? y.x : -INFINITY, v1 ? y.y : -INFINITY));
+                }
+                my_w = scale(warp_max_redux(my_w));
+            }
+            float yoff = offset(my_w);
 
             // soft-max sweep: sum of e over the segment
             float2 Ea = splat(0.f), Eb = splat(0.f);
@@ -677,8 +690,8 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
                         ym = fmaxf(ym, fmaxf(v0 ? y.x : -INFINITY, v1 ? y.y : -INFINITY));
                     }
                     if (ovf) for (int il = kcs + lane; il < kcp; il += 32) ym = fmaxf(ym, to_float<TY>(cy[il]));
-                    my_w = warp_max_redux(ym);
-                    yoff = my_w > -INFINITY ? -my_w * kLog2e : 0.f;
+                    my_w = scale(warp_max_redux(ym));
+                    yoff = offset(my_w);
                     kept_pass();
                 }
             }
@@ -818,11 +831,12 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
             if (lane < kSW) {
                 const float2 mw = *reinterpret_cast<const float2*>(&pend[it & 15][lane][4]);
                 float2 f;
-                f.x = (mw.x > -INFINITY ? ex2((mw.x - m) * kLog2e) : 0.f) * inv_zp;
-                f.y = (KIND == RDK_LOGITS ? (mw.y > -INFINITY ? ex2((mw.y - my) * kLog2e) : 0.f) : 1.f) * inv_zq;
+                constexpr float kUnit = PRI ? 1.f : kLog2e;      // of the scales
+                f.x = (mw.x > -INFINITY ? ex2((mw.x - m) * kUnit) : 0.f) * inv_zp;
+                f.y = (KIND == RDK_LOGITS ? (mw.y > -INFINITY ? ex2((mw.y - my) * kUnit) : 0.f) : 1.f) * inv_zq;
                 fzy[pc][lane] = f;
                 // lanes 0..3 also carry the row scalars the draws need: -m log2e, 1/Zp, -my log2e, 1/Zq
-                float sc = lane == 0 ? -m * kLog2e : (lane == 1 ? inv_zp : (lane == 2 ? (KIND == RDK_LOGITS ? -my * kLog2e : 0.f) : inv_zq));
+                float sc = lane == 0 ? -m * kUnit : (lane == 1 ? inv_zp : (lane == 2 ? (KIND == RDK_LOGITS ? -my * kUnit : 0.f) : inv_zq));
                 if (PRI && lane >= kRecOffPrior) sc = lane == kRecOffPrior ? -mpm : inv_zpi;
                 *reinterpret_cast<float4*>(&pend[it & 15][lane][4]) = make_float4(f.x, f.y, theta, sc);
             }
@@ -1267,24 +1281,25 @@ const char* stream_ineligible(const RowParams& P, int tz, int ty, int kind, int 
 // 256, 16.4 / 16.5 for 320; 65536: 16.8 / 12.0 for 64, 20.0 / 21.3 for 128; 128256: 13.4 / 8.7 for 4, 17.3 / 15.5 for 32,
 // 20.3 / 21.8 for 64; with a prior 128256: 16.6 / 13.4 for 4, 21.6 / 24.7 for 32.  Over 540 such calls the faster kernel is
 // missed by 1.8 % on average; limits on the number of rows alone missed it by 6 %.
-// Rows of 16385 to 49152 tokens, and those that take a group of sixteen CTAs, keep such limits without a prior, as the route query
-// has told them: one or two draws, and up to 3200000 / N rows (24 or 96 above 32768; 56 for a group of sixteen).  The cluster
-// kernel visits kept tokens beyond a warp's 384 register slots in memory, twice: with more of them (a warp of the largest
-// cluster has n / 128) fewer rows, and few beyond twice as many.
+// Calls that such limits gave to the cluster kernel stay there (its sums are the more exact by half): one or two draws and up
+// to 3200000 / N rows, 192 at most (24, or 96 in other types, above 32768 tokens; 56 for groups of sixteen CTAs).  It visits kept
+// tokens beyond a warp's 384 register slots in memory, twice: with more of them (a warp of the largest cluster has n / 128) fewer
+// rows, and few beyond twice as many.  Rows of 16385 to 49152 tokens, and those that take a group of sixteen CTAs, keep the limits
+// both ways, as the route query has told them.
 bool stream_few_rows(const RowParams& P, int tz, int ty, int kind) {
     const size_t es = tz == RDK_F32 ? 4 : 2;
     const bool fast = fast_types(tz, ty, kind);
     StreamSegs sg;
     if (P.trials < 1 || !stream_segments(P.N, es, sg)) return false;
     const bool sixteen = sg.C == kMaxGroup;                  // 9 groups of 16 CTAs
-    if (!P.prior && ((P.N > 16384 && P.N <= 49152) || sixteen)) {
-        if (P.trials > 2) return false;
+    if (!P.prior) {
         int most = !fast ? 96 : (sixteen ? 56 : 24);
-        if (P.N <= 32768) most = most > 3200000 / P.N ? most : 3200000 / P.N;
+        if (P.N <= 32768) { const int small = 3200000 / P.N; most = most > small ? most : (small < 192 ? small : 192); }
         const int kept = P.n / 128;
         if (kept > 384 && most > 24) most = 24;
         if (kept > 768) most = 4;
-        return P.rows <= most;
+        if (P.trials <= 2 && P.rows <= most) return true;
+        if ((P.N > 16384 && P.N <= 49152) || sixteen) return false;
     }
     const int groups = 148 / sg.C, per_group = (P.rows + groups - 1) / groups;
     const long long draws = (long long)P.rows * P.trials;
