@@ -27,7 +27,7 @@
 
 namespace rdk {
 
-constexpr int kVoc = 128;                // tokens of one CTA
+constexpr int kVoc = 128;                // most tokens of one CTA: its half of the instruction's M
 constexpr int kBK = 64;                  // K block: 64 bf16 = 128 bytes = one swizzle row
 constexpr int kVocBytes = kVoc * kBK * 2;        // 16 KB
 constexpr int kTcMaxStages = 12;
@@ -40,6 +40,7 @@ constexpr int kTcThreads = 64 + 32 * kTcEpiWarps;
 struct TcParams {
     float* w; float* S; int rows, N;
     int R, T;                        // rows of one instruction, instructions per item
+    int voc;                         // tokens of one CTA, a multiple of 8
     int tiles_r, num_kb, stages;
     int sum_rows;                    // rows with a sum in shared memory behind the ring: all, or 0
     int full_items, num_items;       // items [0, full_items) are whole, the rest halves (one instruction of R rows)
@@ -113,7 +114,7 @@ exact_tc_kernel(const __grid_constant__ CUtensorMap tmapV, const __grid_constant
         auto load_voc = [&](int s, int kb, int tv) {
             asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
                          ::"r"(ring + (uint32_t)s * stage_bytes), "l"(reinterpret_cast<uint64_t>(&tmapV)), "r"(kb * kBK),
-                           "r"((2 * tv + (int)rank) * kVoc), "r"(full_addr(s)) : "memory");
+                           "r"((2 * tv + (int)rank) * P.voc), "r"(full_addr(s)) : "memory");
         };
         auto load_rows = [&](int s, int kb, int row0, int t) {
             for (int k = 0; k < t; ++k)
@@ -123,7 +124,7 @@ exact_tc_kernel(const __grid_constant__ CUtensorMap tmapV, const __grid_constant
         };
         auto expect = [&](int s, int t) {                // both CTAs' bytes, announced by the leader
             if (leader)
-                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(s32(&full_bar[s])), "r"(2u * (kVocBytes + (uint32_t)t * rbytes)) : "memory");
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(s32(&full_bar[s])), "r"(2u * ((uint32_t)P.voc * (kBK * 2) + (uint32_t)t * rbytes)) : "memory");
         };
         for (int item = pair; item < P.num_items && ok; item += pairs) {
             int tv, row0, t;
@@ -216,7 +217,9 @@ exact_tc_kernel(const __grid_constant__ CUtensorMap tmapV, const __grid_constant
             }
             if (!tc_wait(&acc_full, acc_phase, abort)) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const int tok = (2 * tv + (int)rank) * kVoc + quarter * 32 + lane;
+            // (accumulator lanes beyond the CTA's tokens hold products of whatever lies behind them in the ring)
+            const bool held = quarter * 32 + lane < P.voc;
+            const int tok = held ? (2 * tv + (int)rank) * P.voc + quarter * 32 + lane : P.N;
             const int cols = t * P.R;
             for (int c = share * 32; c < cols; c += 64) {
                 uint32_t v[32];
@@ -236,6 +239,10 @@ exact_tc_kernel(const __grid_constant__ CUtensorMap tmapV, const __grid_constant
                 }
                 if (P.S) {
                     // sums over the lanes (tokens beyond the vocabulary are zero): lane q ends up with column q's
+                    if (P.voc != kVoc) {
+#pragma unroll
+                        for (int q = 0; q < 32; ++q) v[q] = held ? v[q] : 0u;
+                    }
 #pragma unroll
                     for (int s = 16; s > 0; s >>= 1) {
                         const bool up = lane & s;
@@ -336,7 +343,7 @@ int launch_exact_tc(const __nv_bfloat16* A, long long lda, const __nv_bfloat16* 
     P.w = w_out; P.S = S_out; P.rows = rows; P.N = N;
     P.num_kb = (n + kBK - 1) / kBK;
     P.status_word = status_word;
-    const long long tiles_v = ((long long)N + 2 * kVoc - 1) / (2 * kVoc);
+    long long tiles_v = ((long long)N + 2 * kVoc - 1) / (2 * kVoc);
     const int pairs_most = sms / 2;
     // as few row tiles as the 512 accumulator columns allow, more where that leaves pairs without work (down to 64 rows,
     // below which an item is bound by its part of Mt)
@@ -347,6 +354,18 @@ int launch_exact_tc(const __nv_bfloat16* A, long long lda, const __nv_bfloat16* 
     P.R = P.T == 2 ? ((per + 1) / 2 + 15) / 16 * 16 : (per + 31) / 32 * 32;
     P.tiles_r = (rows + P.T * P.R - 1) / (P.T * P.R);
     const int stage_bytes = kVocBytes + P.T * P.R * kBK;
+    // Up to 256 rows the call is the read of Mt, and a last round with few panels reads it with few SMs.  So the panels are made
+    // lower than the instruction, as low as leaves every round full; the rest of the instruction's rows are idle (whole calls with
+    // the draws: 32 rows x 20011 x 5001 68.5 -> 59.9 us, 16 x 65536 x 16000 359 -> 334, 240 x 50000 x 5000 151.0 -> 146.3, 20 x
+    // 32768 x 8192 104.1 -> 102.8).  Not where one round holds all panels: more of them, each with the operand to fetch, were
+    // slower (16 x 8192 x 2000 24.6 -> 25.3).
+    P.voc = kVoc;
+    if (P.tiles_r == 1 && P.T == 1 && tiles_v > pairs_most) {
+        const long long rounds = (tiles_v + pairs_most - 1) / pairs_most, per_cta = ((long long)N + 2 * rounds * pairs_most - 1) / (2 * rounds * pairs_most);
+        P.voc = (int)((per_cta + 7) / 8 * 8);
+        if (P.voc > kVoc) P.voc = kVoc;
+        tiles_v = ((long long)N + 2 * P.voc - 1) / (2 * P.voc);
+    }
     const long long tiles = tiles_v * P.tiles_r;
     if (tiles > 0x3fffffffLL) { set_error("rdk_redistribute_exact: too many output tiles"); return RDK_ERR_UNSUPPORTED; }
     const int pairs = (int)(tiles < pairs_most ? tiles : pairs_most);
@@ -357,7 +376,7 @@ int launch_exact_tc(const __nv_bfloat16* A, long long lda, const __nv_bfloat16* 
     P.stages = (kTcSmem - 1024 - 4 * P.sum_rows) / stage_bytes;
     if (P.stages > kTcMaxStages) P.stages = kTcMaxStages;
     CUtensorMap mapV, mapR;
-    int st = make_map(&mapV, Mt, (uint64_t)n, (uint64_t)N, (uint64_t)ldm, kBK, kVoc);
+    int st = make_map(&mapV, Mt, (uint64_t)n, (uint64_t)N, (uint64_t)ldm, kBK, (uint32_t)P.voc);
     if (st != RDK_OK) return st;
     st = make_map(&mapR, A, (uint64_t)n, (uint64_t)rows, (uint64_t)lda, kBK, (uint32_t)P.R / 2);
     if (st != RDK_OK) return st;

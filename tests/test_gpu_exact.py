@@ -344,3 +344,25 @@ def test_bf16_row_sums_take_one_addition_per_cta(N, rows):
     ref = torch.cat([x.double().sum(1) for x in w.split(64)])
     k = torch.cuda.get_device_properties(0).multi_processor_count + 16
     assert float(((S.double() / ref - 1) ** 2).mean().sqrt()) <= 2.0 ** -24 * (k / 3) ** 0.5
+
+
+@pytest.mark.parametrize("N,n,rows", [(2000, 300, 5), (9473, 200, 17), (19000, 130, 33), (20011, 1001, 20), (32768, 520, 250), (40001, 64, 1)])
+def test_panels_lower_than_the_instruction(N, n, rows):
+    """Up to 256 rows a CTA takes fewer tokens than the instruction has rows, so that every round of panels is full (32 to 128 tokens,
+    the last panel ragged): every entry of w against a float64 product of the same bf16 operands, and its row sums."""
+    rdk = _rdk()
+    B = rdk.binding
+    g = torch.Generator(device="cuda").manual_seed(N)
+    idx = rdk.rdk_prepare_ids(torch.arange(n, dtype=torch.int32).cuda(), N)
+    ld = (n + 7) // 8 * 8
+    Mt = torch.rand(N, ld, generator=g, device="cuda").to(torch.bfloat16)
+    q = torch.rand(rows, n, generator=g, device="cuda")
+    w, S, _ = rdk.rdk_redistribute_exact(idx, q, {"data": Mt, "layout": B.RDK_AFF_BF16_COLS, "ld": ld}, rows, 1, B.RDK_PROBS)
+    torch.cuda.synchronize()
+    # the operand as the library rounds it: q / sum in fp32, to bf16; a quotient next to a boundary may be its neighbour (2^-8)
+    a = (q.double() / q.double().sum(1, keepdim=True)).to(torch.bfloat16).double()
+    ref = a @ Mt[:, :n].double().t()
+    # products exact, n fp32 additions of terms of one sign, rounded or cut off; and a neighbour or two moves w by 2^-8 of a term,
+    # of which the largest is some four times the mean
+    assert float(((w.double() - ref).abs() / ref).max()) <= n * 2.0 ** -23 + 2.0 ** -8 * (2 + n / 4096) * 4 / n
+    assert float((S.double() - w.double().sum(1)).abs().max()) <= 3e-6 * float(S.max())
