@@ -34,13 +34,15 @@ constexpr int kAffM = 128, kAffN = 256, kAffK = 64;
 constexpr int kAffABytes = kAffM * kAffK * 2, kAffBBytes = kAffN * kAffK * 2;       // 16 KB, 32 KB
 constexpr int kAffStage = kAffABytes + kAffBBytes;
 constexpr int kAffStages = 3;
-constexpr int kAffEpiWarps = 16;                         // their exponentials need the latency hidden (sums alone: 101 us, with 8 118)
-constexpr int kAffCols = 4 * kAffN / kAffEpiWarps;       // columns of a tile per epilogue warp
+// Epilogue warps: sixteen, whose exponentials need the latency hidden (sums alone: 101 us, with eight 118); eight for the write where
+// a CTA has one tile (see build_affinity_tc).
+constexpr int kAffEpiWarps = 16, kAffFewWarps = 8;
+constexpr int kAffStoreBuffers = 16;
 constexpr int kAffStoreBytes = 32 * 128;                 // a warp's 32 rows x 64 bf16
-constexpr int kAffSmem = kAffStages * kAffStage + kAffEpiWarps * kAffStoreBytes + 1024;
+constexpr int kAffSmem = kAffStages * kAffStage + kAffStoreBuffers * kAffStoreBytes + 1024;
 constexpr int kAffBlock = 64;                            // tokens summed one after the other
-static_assert(kAffCols == kAffBlock, "an epilogue warp leaves one sum per tile, or fills one store buffer");
-constexpr int kAffThreads = 64 + 32 * kAffEpiWarps;
+static_assert(4 * kAffN / kAffEpiWarps == kAffBlock, "an epilogue warp leaves one sum per tile");
+constexpr int aff_threads(int epi) { return 64 + 32 * epi; }
 constexpr uint32_t kAffIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kAffN >> 3) << 17) | ((uint32_t)(kAffM >> 4) << 24);
 
 constexpr float kAffZeroInv = 1e12f;                     // inverse norm of a zero embedding
@@ -60,10 +62,11 @@ struct AffParams {
     int32_t* status;
 };
 
-template <int MODE>
-__global__ void __launch_bounds__(kAffThreads, 1)
+template <int MODE, int EPI>
+__global__ void __launch_bounds__(aff_threads(EPI), 1)
 aff_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__ CUtensorMap tmapB, const __grid_constant__ CUtensorMap tmapC, const AffParams P) {
     constexpr bool kWrite = MODE == kAffWrite;
+    constexpr int kCols = 4 * kAffN / EPI, kBufs = kAffStoreBuffers / EPI;       // columns and store buffers of an epilogue warp
     extern __shared__ __align__(1024) unsigned char aff_smem[];
     unsigned char* tiles = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(aff_smem) + 1023) & ~uintptr_t(1023));
     __shared__ __align__(8) unsigned long long full_bar[kAffStages], empty_bar[kAffStages], acc_full[2], acc_empty[2];
@@ -79,7 +82,7 @@ aff_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__
         }
         for (int a = 0; a < 2; ++a) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(s32(&acc_full[a])));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(s32(&acc_empty[a])), "r"(kAffEpiWarps));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(s32(&acc_empty[a])), "r"(EPI));
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -148,14 +151,14 @@ aff_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__
             return true;
         });
     } else {
-        const int quarter = warp & 3, share = (warp - 2) >> 2;       // TMEM lanes 32 quarter .. + 32, columns kAffCols share .. + kAffCols
-        const uint32_t taddr0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(share * kAffCols);
-        const uint32_t store = s32(tiles + kAffStages * kAffStage + (warp - 2) * kAffStoreBytes);
-        int acc = 0;
+        const int quarter = warp & 3, share = (warp - 2) >> 2;       // TMEM lanes 32 quarter .. + 32, columns kCols share .. + kCols
+        const uint32_t taddr0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(share * kCols);
+        const uint32_t store0 = s32(tiles + kAffStages * kAffStage + (warp - 2) * kBufs * kAffStoreBytes);
+        int acc = 0, buf = 0;
         uint32_t acc_phase = 0;
         const float2 sc = splat(P.scale), neg = splat(-1.f);
         walk([&](int row0, int col0) -> bool {
-            const int row = row0 + quarter * 32 + lane, c0 = col0 + share * kAffCols;
+            const int row = row0 + quarter * 32 + lane, c0 = col0 + share * kCols;
             const float2 ri = splat(__ldg(P.row_inv + row));
             // 2^((G x - 1) scale) of two columns
             auto weight2 = [&](uint32_t g0, uint32_t g1, float k0, float k1) -> float2 {
@@ -166,16 +169,16 @@ aff_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__
             float sum = 0.f;
             uint32_t v[2][32];
             tmem_ld32(taddr0 + (uint32_t)(acc * kAffN), v[0]);
-            if (kWrite) {                                            // the warp's last store has been read
-                if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-                __syncwarp();
-            }
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                tmem_wait_ld(v[c]);
-                uint32_t (&x)[32] = v[c];
-                if (c == 0) {
-                    tmem_ld32(taddr0 + (uint32_t)(acc * kAffN + 32), v[1]);
+            for (int c = 0; c < kCols / 32; ++c) {
+                if (kWrite && (c & 1) == 0) {                        // the buffer's last store has been read
+                    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kBufs - 1) : "memory");
+                    __syncwarp();
+                }
+                tmem_wait_ld(v[c & 1]);
+                uint32_t (&x)[32] = v[c & 1];
+                if (c < kCols / 32 - 1) {
+                    tmem_ld32(taddr0 + (uint32_t)(acc * kAffN + (c + 1) * 32), v[(c + 1) & 1]);
                 } else {                                             // the accumulator is in registers: the next tile may have it
                     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                     __syncwarp();
@@ -199,7 +202,7 @@ aff_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__
                     }
                 } else {
                     const float4* cz = reinterpret_cast<const float4*>(P.z + col);
-                    const uint32_t rowaddr = store + (uint32_t)lane * 128u;
+                    const uint32_t rowaddr = store0 + (uint32_t)(buf * kAffStoreBytes) + (uint32_t)lane * 128u;
 #pragma unroll
                     for (int q = 0; q < 8; q += 2) {
                         uint32_t w[4];
@@ -212,25 +215,25 @@ aff_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__
                             asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w[2 * h]) : "f"(e0.y), "f"(e0.x));
                             asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w[2 * h + 1]) : "f"(e1.y), "f"(e1.x));
                         }
-                        // 16-byte chunk c * 4 + q / 2 of the row, at its place in the 128-byte swizzle
-                        const uint32_t chunk = (uint32_t)(c * 4 + q / 2) ^ (uint32_t)(lane & 7);
+                        // 16-byte chunk (c & 1) * 4 + q / 2 of the row, at its place in the 128-byte swizzle
+                        const uint32_t chunk = (uint32_t)((c & 1) * 4 + q / 2) ^ (uint32_t)(lane & 7);
                         asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(rowaddr + chunk * 16u), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]) : "memory");
+                    }
+                    if (c & 1) {                                     // 64 columns are complete (read while the next are evaluated)
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                        __syncwarp();
+                        if (lane == 0) {
+                            const int x0 = c0 + (c >> 1) * 64, y0 = row0 + quarter * 32;
+                            if (x0 < P.n && y0 < P.N)
+                                asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];"
+                                             ::"l"(reinterpret_cast<uint64_t>(&tmapC)), "r"(x0), "r"(y0), "r"(store0 + (uint32_t)(buf * kAffStoreBytes)) : "memory");
+                            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                        }
+                        if (++buf == kBufs) buf = 0;
                     }
                 }
             }
-            if (kWrite) {                                            // (read while the next tile is waited for and evaluated)
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                __syncwarp();
-                if (lane == 0) {
-                    const int y0 = row0 + quarter * 32;
-                    if (c0 < P.n && y0 < P.N)
-                        asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];"
-                                     ::"l"(reinterpret_cast<uint64_t>(&tmapC)), "r"(c0), "r"(y0), "r"(store) : "memory");
-                    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-                }
-            } else {
-                P.part[(long long)(c0 / kAffBlock) * P.npad + row] = sum;
-            }
+            if (!kWrite) P.part[(long long)(c0 / kAffBlock) * P.npad + row] = sum;
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
             return true;
         });
@@ -395,18 +398,22 @@ int build_affinity_tc(const __nv_bfloat16* E, int d, long long estride, const in
     int dev = 0, sms = 0;
     RDK_CUDA(cudaGetDevice(&dev));
     RDK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    RDK_CUDA(cudaFuncSetAttribute(aff_tc_kernel<kAffSums>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAffSmem));
-    RDK_CUDA(cudaFuncSetAttribute(aff_tc_kernel<kAffWrite>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAffSmem));
+    // the write: small CTAs where each has one tile, which it then starts the sooner; sixteen warps where they have many
+    auto sums_kernel = aff_tc_kernel<kAffSums, kAffEpiWarps>;
+    const bool few = (long long)(L.npad / kAffN) * (L.Npad / kAffM) <= sms;
+    auto write_kernel = few ? aff_tc_kernel<kAffWrite, kAffFewWarps> : aff_tc_kernel<kAffWrite, kAffEpiWarps>;
+    RDK_CUDA(cudaFuncSetAttribute(sums_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kAffSmem));
+    RDK_CUDA(cudaFuncSetAttribute(write_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kAffSmem));
     AffParams P;
     P.N = N; P.n = n; P.num_kb = (d + kAffK - 1) / kAffK; P.scale = scale; P.status = status; P.part = part; P.npad = L.npad; P.z = z;
     const long long tiles = (long long)(L.npad / kAffM) * (L.Npad / kAffN);       // of either pass
     if (tiles > 0x7fffffffLL) { set_error("rdk_build_affinity: too many tiles"); return RDK_ERR_UNSUPPORTED; }
     const unsigned grid = (unsigned)(tiles < sms ? tiles : sms);
     P.row_tiles = L.npad / kAffM; P.col_tiles = L.Npad / kAffN; P.row_inv = invk; P.col_inv = inv;
-    RDK_CUDA(launch_pdl(aff_tc_kernel<kAffSums>, grid, (unsigned)kAffThreads, (size_t)kAffSmem, s, keptA, tokB, out, P));
+    RDK_CUDA(launch_pdl(sums_kernel, grid, (unsigned)aff_threads(kAffEpiWarps), (size_t)kAffSmem, s, keptA, tokB, out, P));
     RDK_CUDA(launch_pdl(aff_norm_kernel, (unsigned)(L.npad / 32), 256u, 0, s, (const float*)part, (const float*)invk, z, L.blocks, L.npad));
     P.row_tiles = L.Npad / kAffM; P.col_tiles = L.npad / kAffN; P.row_inv = inv; P.col_inv = invk;
-    RDK_CUDA(launch_pdl(aff_tc_kernel<kAffWrite>, grid, (unsigned)kAffThreads, (size_t)kAffSmem, s, tokA, keptB, out, P));
+    RDK_CUDA(launch_pdl(write_kernel, grid, (unsigned)aff_threads(few ? kAffFewWarps : kAffEpiWarps), (size_t)kAffSmem, s, tokA, keptB, out, P));
     RDK_CUDA(launch_pdl(aff_finish_kernel, (unsigned)((n + wpb - 1) / wpb), 256u, 0, s, (const int32_t*)status, (const float*)invk, (const float*)z, Mt, ld, n, N));
     return RDK_OK;
 }
