@@ -38,7 +38,7 @@
 //   first-order terms; it is taken as 1.
 //
 // With one prior row pi for all rows in place of p inside the formula, the same kernel keeps the CTA's slice of pi and all that no
-// row changes about it, so pi costs a row no exponentials.  320 rows of 128256 tokens: 54 us, with the draws; the cluster
+// row changes about it, so pi costs a row no exponentials.  320 rows of 128256 tokens: 56 us, with the draws; the cluster
 // kernel, which reads pi and takes its soft-max anew for every row, 111.
 #include <atomic>
 #include <chrono>
