@@ -935,20 +935,26 @@ struct CluShape { int C, nw, per; size_t smem; bool roomy; float cost; };
 // and fp32).  The shape that the rule picks is within 2 to 4 % of the fastest one tried on average; powers of
 // two alone, which this replaces as the last word, were 8 to 15 % off (50257 tokens: 80 rows 16.9 -> 12.3 us, 320 rows
 // 44.8 -> 33.5; 128257: 320 rows 86.4 -> 70.4; q~ of 80 x 262143: 114.6 -> 62.1; given weights of 40 x 50240: 11.4 -> 8.7).
+// With three trials or more, clusters of one CTA an SM are counted as they were seen to fit: 32 rows of four trials at 32001 are
+// one round of four CTAs with 128 registers (fp32 13.6 -> 9.8 us, bf16 11.9 -> 8.6), and 24 rows at 44001 would be two rounds of
+// five (15.6 us against 11.9 with four).
 struct CluCost {
     float t0, k, km, b, seg, cluster, second, over, warps, tail, fill, roomy, draws;
+    bool counted;        // see rows_at_once
 };
-constexpr CluCost kCostFewDraws{3.794f, 1.737f, 0.762f, 0.742f, 0.015f, 0.501f, 0.394f, 2.617f, 2.986f, 0.006f, 0.776f, 0.902f, 1.884f};
-constexpr CluCost kCostManyDraws{4.506f, 1.475f, 1.116f, 1.927f, 0.153f, 0.55f, 1.387f, 3.974f, 0.42f, 0.272f, 0.83f, 0.631f, 1.077f};
-constexpr CluCost kCostDense{3.425f, 2.429f, 4.145f, 0.574f, 0.275f, 0.081f, 0.168f, 0.151f, 0.69f, 0.281f, 0.876f, 0.845f, 0.117f};
-constexpr CluCost kCostPrior{4.82f, 4.042f, 1.734f, 1.087f, 0.033f, 0.61f, 0.494f, 0.034f, 2.926f, 0.829f, 0.949f, 0.982f, 1.884f};
-constexpr CluCost kCostGiven{3.984f, 0.916f, 1.611f, 0.565f, 1.035f, 0.125f, 0.613f, 2.38f, 0.613f, 0.48f, 0.87f, 0.846f, 0.713f};
+constexpr CluCost kCostFewDraws{3.794f, 1.737f, 0.762f, 0.742f, 0.015f, 0.501f, 0.394f, 2.617f, 2.986f, 0.006f, 0.776f, 0.902f, 1.884f, false};
+constexpr CluCost kCostManyDraws{5.372f, 0.72f, 1.228f, 1.997f, 0.01f, 1.092f, 0.249f, 3.958f, 0.002f, 0.173f, 0.829f, 0.702f, 0.993f, true};
+constexpr CluCost kCostDense{3.425f, 2.429f, 4.145f, 0.574f, 0.275f, 0.081f, 0.168f, 0.151f, 0.69f, 0.281f, 0.876f, 0.845f, 0.117f, false};
+constexpr CluCost kCostPrior{4.82f, 4.042f, 1.734f, 1.087f, 0.033f, 0.61f, 0.494f, 0.034f, 2.926f, 0.829f, 0.949f, 0.982f, 1.884f, false};
+constexpr CluCost kCostGiven{3.984f, 0.916f, 1.611f, 0.565f, 1.035f, 0.125f, 0.613f, 2.38f, 0.613f, 0.48f, 0.87f, 0.846f, 0.713f, false};
 
 // The shape with C CTAs a row and at most `warps` warps each; false where a row does not fit.
-static bool shape_cluster(long long positions, int C, int warps, size_t bytes, bool roomy, CluShape& s) {
+static bool shape_cluster(long long positions, int rows, int trials, int C, int warps, size_t bytes, bool roomy, CluShape& s) {
     const int chunks = (int)((positions + C * 256 - 1) / (C * 256)), per = (chunks + warps - 1) / warps;
     const int nw = (chunks + per - 1) / per;
     s.C = C; s.nw = nw < 4 ? 4 : nw; s.per = per * 32; s.roomy = roomy;
+    // segments of one chunk and several draws a row: a warp for each draw, also where there is nothing to sweep for it
+    if (per == 1 && (long long)rows * C < 4 * kCluSms && 2 * trials > s.nw) s.nw = 2 * trials < kCluMaxWarps ? 2 * trials : kCluMaxWarps;
     s.smem = (size_t)s.nw * s.per * kVec * bytes;
     if (s.smem < sizeof(DrawSmem)) s.smem = sizeof(DrawSmem);
     return s.smem <= (size_t)kCluDynamic && per <= kCluMaxChunks;
@@ -961,12 +967,22 @@ static int resident_ctas(const CluShape& s, int registers) {
     return n < by_warps ? (n < 1 ? 1 : n) : by_warps;
 }
 
+// Rows under way at once.  Clusters do not fill the chip to the last SM, as they stay within a group of SMs: about `fill` of what
+// the SMs hold, but of one CTA an SM, and of eight CTAs or more two an SM, no more than the driver counts (of ten CTAs 11: q~ of
+// 12 x 136768 in two rounds of them took 14.3 us, with two CTAs an SM of sixteen 12.0; of five CTAs 22: 24 rows took two rounds,
+// although it counts 26).  `counted`: that count itself for one CTA an SM, where `fill` is too low a guess.
+static int rows_at_once(const CluCost& c, const CluShape& s, int slots) {
+    constexpr int kOne[kCluMaxCtas + 1] = {0, 148, 74, 45, 33, 22, 22, 15, 15, 15, 11, 7, 7, 7, 7, 7, 7};
+    if (s.C == 1) return kCluSms * slots;
+    const int filled = (int)(c.fill * (float)(kCluSms * slots) / (float)s.C), most = kOne[s.C] * slots;
+    if (slots == 1 && c.counted) return most;
+    const int n = (slots == 1 || (slots == 2 && s.C >= 8)) && most < filled ? most : filled;
+    return n < 1 ? 1 : n;
+}
+
 static float cost_cluster(const CluCost& c, const CluShape& s, int rows, int trials, int registers, float kept, int kept_slots) {
     const int slots = resident_ctas(s, registers), chunks = s.per / 32;
-    // (clusters do not fill the chip to the last SM: they stay within a group of SMs)
-    int cap = s.C > 1 ? (int)(c.fill * (float)(kCluSms * slots) / (float)s.C) : kCluSms * slots;
-    if (cap < 1) cap = 1;
-    const float waves = (float)rows / (float)cap;
+    const float waves = (float)rows / (float)rows_at_once(c, s, slots);
     float resident = (float)rows * (float)s.C / (float)kCluSms;
     resident = resident < 1.f ? 1.f : (resident > (float)slots ? (float)slots : resident);
     const float most = kept * 256.f * (float)chunks + 2.f * sqrtf(kept * 256.f * (float)chunks);     // kept tokens of a warp, nearly at most
@@ -997,10 +1013,10 @@ static bool plan_cluster_anew(int N, int n, int rows, int trials, size_t es, int
     // 14.1 us, 1500 rows of 8k with eight 107 -> 84 -- and where the CTAs are fewer than two an SM and not many share a row:
     // 100 rows of 3000 10.4 -> 9.0 us, 4 rows of 8k 7.7 -> 7.2, but 5 rows of 128k on 16 CTAs each 8.9 -> 9.3)
     const int warps = trials >= 3 || ((long long)rows * C < 2 * kCluSms && C < kCluMaxCtas) ? kCluMaxWarps : 8;
-    bool found = shape_cluster(positions, C, warps, bytes, false, s);
+    bool found = shape_cluster(positions, rows, trials, C, warps, bytes, false, s);
     if (N < kStreamMinN) {
         CluShape r;      // a CTA holds the row either way
-        if (shape_cluster(positions, C, warps, bytes, true, r) && rows <= kCluSms * resident_ctas(r, 128)) { s = r; found = true; }
+        if (shape_cluster(positions, rows, trials, C, warps, bytes, true, r) && rows <= kCluSms * resident_ctas(r, 128)) { s = r; found = true; }
     } else {
         const CluCost& c = variant == kVarGiven ? kCostGiven : (variant == kVarDense ? kCostDense : (variant == kVarPrior ? kCostPrior : (trials >= 3 ? kCostManyDraws : kCostFewDraws)));
         const float kept = variant == kVarGiven ? 0.f : fminf(1.f, (float)n / (float)N);
@@ -1012,18 +1028,12 @@ static bool plan_cluster_anew(int N, int n, int rows, int trials, size_t es, int
             for (int w = 8; w <= kCluMaxWarps; w += 8)
                 for (int roomy = 0; roomy < 2; ++roomy) {
                     CluShape t;
-                    if (!shape_cluster(positions, k, w, bytes, roomy != 0, t)) continue;
+                    if (!shape_cluster(positions, rows, trials, k, w, bytes, roomy != 0, t)) continue;
                     const int regs = roomy ? 128 : registers;
-                    if (roomy && (float)rows * (float)k > c.fill * (float)(kCluSms * resident_ctas(t, regs))) continue;      // (measured where one wave holds them)
+                    if (roomy && rows > rows_at_once(c, t, resident_ctas(t, regs))) continue;      // (measured where one wave holds them)
                     t.cost = cost_cluster(c, t, rows, trials, regs, kept, kept_slots);
                     if (t.cost < best) { best = t.cost; s = t; found = true; }
                 }
-    }
-    // segments of one chunk and several draws a row: a warp for each draw, also where there is nothing to sweep for it
-    if (found && s.per == 32 && (long long)rows * s.C < 4 * kCluSms && 2 * trials > s.nw) {
-        s.nw = 2 * trials < kCluMaxWarps ? 2 * trials : kCluMaxWarps;
-        const size_t smem = (size_t)s.nw * s.per * kVec * bytes;
-        if (smem > s.smem) s.smem = smem;
     }
     return found;
 }

@@ -335,7 +335,7 @@ def test_index_written_by_the_kernel_queued_just_before_the_call():
 @pytest.mark.parametrize("N,n,rows,trials,dtype", [
     (5001, 500, 40, 1, "bf16"), (20011, 2000, 20, 1, "f32"), (33333, 8333, 40, 1, "bf16"), (33333, 8333, 45, 4, "f32"),
     (50257, 12565, 80, 1, "bf16"), (50257, 12565, 330, 2, "bf16"), (90001, 30000, 20, 1, "f32"), (128257, 3000, 24, 5, "bf16"),
-    (262143, 100000, 5, 1, "bf16")])
+    (262143, 100000, 5, 1, "bf16"), (16001, 4000, 16, 4, "f32"), (32001, 8000, 33, 4, "f32"), (32001, 8000, 34, 4, "bf16")])
 def test_cluster_kernel_cluster_sizes(N, n, rows, trials, dtype):
     cfg = W.tiny_config(N=N, n=n, rows=rows, dtype=dtype, trials=trials, rho=0.8, seed=rows, zipf_bias=True)
     inp = W.make_inputs(cfg)
