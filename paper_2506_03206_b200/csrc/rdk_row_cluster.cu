@@ -969,7 +969,7 @@ static int resident_ctas(const CluShape& s, int registers) {
 
 // Rows under way at once.  Clusters do not fill the chip to the last SM, as they stay within a group of SMs: about `fill` of what
 // the SMs hold, but of one CTA an SM, and of eight CTAs or more two an SM, no more than the driver counts (of ten CTAs 11: q~ of
-// 12 x 136768 in two rounds of them took 14.3 us, with two CTAs an SM of sixteen 12.0; of five CTAs 22: 24 rows took two rounds,
+// 12 x 136768 in two rounds of them took 14.3 us, with two CTAs an SM of sixteen 10.0; of five CTAs 22: 24 rows took two rounds,
 // although it counts 26).  `counted`: that count itself for one CTA an SM, where `fill` is too low a guess.
 static int rows_at_once(const CluCost& c, const CluShape& s, int slots) {
     constexpr int kOne[kCluMaxCtas + 1] = {0, 148, 74, 45, 33, 22, 22, 15, 15, 15, 11, 7, 7, 7, 7, 7, 7};
