@@ -314,7 +314,8 @@ void rdk_test_set_spin_limit(uint32_t limit);
  * These calls take the cluster kernel (the one-CTA-per-row kernel where a row does not fit a cluster) and need no
  * workspace.  Given one (rdk_sample_and_verify_prior_ws; contents, alignment and sharing as in rdk_sample_and_verify), many
  * rows with one shared prior are served by the streaming kernels: rdk_sample_prior_workspace_bytes (host only, no CUDA
- * call) says how many bytes that takes, 0 where they would not serve.  A smaller or missing workspace is no error.
+ * call) says how many bytes that takes, 0 where they would not serve.  A smaller or missing workspace is no error,
+ * one that is not 256-byte aligned is (RDK_ERR_WORKSPACE_TOO_SMALL, as in rdk_sample_and_verify).
  * ------------------------------------------------------------------------------------------- */
 int rdk_sample_and_verify_prior(const rdk_problem* problem, const void* target, const void* prior,
                                 int64_t prior_row_stride, const void* drafter, const float* uniforms,

@@ -125,6 +125,13 @@ def lib() -> C.CDLL:
         L.rdk_sample_route.restype = C.c_int
         L.rdk_sample_route.argtypes = [C.POINTER(rdk_problem), C.c_int32, C.c_void_p, C.c_void_p, C.c_int32,
                                        C.c_void_p, C.c_size_t, C.POINTER(C.c_char_p)]
+        L.rdk_sample_and_verify_prior_ws.restype = C.c_int
+        L.rdk_sample_and_verify_prior_ws.argtypes = [C.POINTER(rdk_problem), C.c_void_p, C.c_void_p, C.c_int64, C.c_void_p,
+                                                     C.c_void_p, C.c_int32, C.POINTER(rdk_outputs), C.c_void_p, C.c_size_t,
+                                                     C.c_void_p]
+        L.rdk_sample_prior_workspace_bytes.restype = C.c_size_t
+        L.rdk_sample_prior_workspace_bytes.argtypes = [C.POINTER(rdk_problem), C.c_void_p, C.c_void_p, C.c_int64, C.c_void_p,
+                                                       C.c_int32]
         L.rdk_test_set_spin_limit.restype = None
         L.rdk_test_set_spin_limit.argtypes = [C.c_uint32]
         _lib = L

@@ -495,10 +495,10 @@ static int run_rows(const rdk_problem* pb, int mode, const void* target, const v
     auto cluster = [&]() -> cudaError_t {
         RowParams Q = P;
         uint32_t tag = 0;
-        if (Q.accepted_len && Q.accepted && ws) {                   // accepted_len is counted inside the kernel
+        if (Q.accepted_len && Q.accepted && ws && !(reinterpret_cast<uintptr_t>(ws) & 7u)) {       // accepted_len is counted inside the kernel
             if (mode == RDK_MODE_LINEAR && ws_bytes >= stream_workspace_bytes(P.rows, pb->batch, trials))
                 Q.arrivals = stream_workspace_arrivals(ws, P.rows);
-            else if (mode == RDK_MODE_PRECOMPUTED_W && !(reinterpret_cast<uintptr_t>(ws) & 7u) && ws_bytes / 8 >= (size_t)pb->batch * trials)
+            else if (mode == RDK_MODE_PRECOMPUTED_W && ws_bytes / 8 >= (size_t)pb->batch * trials)
                 Q.arrivals = static_cast<unsigned long long*>(ws);
             if (Q.arrivals) tag = next_tag();
         }
@@ -593,6 +593,10 @@ extern "C" int rdk_sample_and_verify_prior_ws(const rdk_problem* problem, const 
     if (out->accepted_len && !out->accepted) {
         set_error("rdk_sample_and_verify_prior: accepted_len needs the accepted output");
         return RDK_ERR_INVALID_ARG;
+    }
+    if (reinterpret_cast<uintptr_t>(ws) & 255u) {
+        set_error("rdk_sample_and_verify_prior_ws: the workspace is not 256-byte aligned");
+        return RDK_ERR_WORKSPACE_TOO_SMALL;
     }
     st = check_arch();
     if (st != RDK_OK) return st;

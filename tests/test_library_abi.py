@@ -202,3 +202,20 @@ def test_embedding_dimensions_beyond_the_limit_are_refused_by_every_route(B):
                 a = B.rdk_affinity(1 << 20, layout, 0, 64)
                 st = L.rdk_build_affinity(dummy, dtype, d, 0, dummy, 8, 64, 0.1, C.byref(a), dummy, dummy, 1 << 40, None)
                 assert st == B.RDK_ERR_UNSUPPORTED, (layout, dtype, d, st)
+
+
+@pytest.mark.skipif("__import__('torch').cuda.is_available()", reason="host logic, with addresses that no device may see")
+@pytest.mark.parametrize("dtype,stride", [(0, 0), (1, 0), (1, 4096)])
+def test_a_workspace_off_its_alignment_is_refused_with_a_prior(B, dtype, stride):
+    """The counters of accepted_len in it are 64-bit atomics: what rdk_sample_and_verify refuses, the call with a prior refuses as well,
+    whichever kernel would serve it.  A missing one and one that is too small are none of that."""
+    L, dummy = B.lib(), C.c_void_p(1 << 20)
+    pb = B.rdk_problem()
+    pb.N, pb.n, pb.batch, pb.positions, pb.kept_index = 4096, 512, 2, 3, 1 << 20
+    pb.target_dtype = pb.drafter_dtype = dtype
+    out = B.rdk_outputs()
+    out.accepted, out.accepted_len = 1 << 20, 1 << 20
+    for ws, size, refused in ((4, 1 << 20, True), (8, 1 << 20, True), (128, 64, True), (256, 1 << 20, False), (256, 8, False), (None, 0, False)):
+        st = L.rdk_sample_and_verify_prior_ws(C.byref(pb), dummy, dummy, stride, dummy, dummy, 1, C.byref(out),
+                                              None if ws is None else (1 << 21) + ws, size, None)
+        assert (st == B.RDK_ERR_WORKSPACE_TOO_SMALL) == refused and st != B.RDK_OK, (ws, st)
