@@ -159,6 +159,19 @@ long long prior_stride(const at::Tensor& prior, PyObject* o, const at::Tensor& t
     return rows2d(o, "prior").stride(0);
 }
 
+// A workspace of a call's own from torch's allocator, which hands the memory out again in the order of the stream.  The call that
+// takes it can do without: none (an undefined tensor) where the memory is not to be had, and while the stream is captured,
+// where the allocator may have to be kept out of it.
+at::Tensor own_workspace(size_t bytes, const at::Tensor& like, const c10::cuda::CUDAStream& current) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (!bytes || cudaStreamIsCapturing(current.stream(), &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) return at::Tensor();
+    try {
+        return at::empty({(int64_t)bytes}, like.options().dtype(at::kByte));
+    } catch (const c10::OutOfMemoryError&) {
+        return at::Tensor();
+    }
+}
+
 // (buffer, N, n, target, prior, drafter, uniforms, batch, positions, kind, out) -> status
 PyObject* sample_prior(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded([&]() -> PyObject* {
@@ -174,15 +187,11 @@ PyObject* sample_prior(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const void *z = pointer<void>(target), *pr = pointer<void>(prior), *y = pointer<void>(drafter);
         const float* up = pointer<float>(u);
         const c10::cuda::CUDAStream current = c10::cuda::getCurrentCUDAStream();
-        // A workspace of this call's own from torch's allocator, which hands the memory out again in the order of the stream;
-        // none while the stream is captured, where the allocator may have to be kept out of it.
-        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-        const size_t ws_bytes = rdk_sample_prior_workspace_bytes(&pb, z, pr, stride, y, (int32_t)trials);
-        at::Tensor ws;
-        if (ws_bytes && cudaStreamIsCapturing(current.stream(), &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone)
-            ws = at::empty({(int64_t)ws_bytes}, target.options().dtype(at::kByte));
-        void *wsp = ws.defined() ? pointer<void>(ws) : nullptr, *s = current.stream();
-        return PyLong_FromLong(unlocked([&] { return rdk_sample_and_verify_prior_ws(&pb, z, pr, stride, y, up, (int32_t)trials, &o, wsp, wsp ? ws_bytes : 0, s); }));
+        void* s = current.stream();
+        const at::Tensor ws = own_workspace(rdk_sample_prior_workspace_bytes(&pb, z, pr, stride, y, (int32_t)trials), target, current);
+        void* wsp = ws.defined() ? pointer<void>(ws) : nullptr;
+        const size_t ws_bytes = wsp ? (size_t)ws.numel() : 0;
+        return PyLong_FromLong(unlocked([&] { return rdk_sample_and_verify_prior_ws(&pb, z, pr, stride, y, up, (int32_t)trials, &o, wsp, ws_bytes, s); }));
     });
 }
 

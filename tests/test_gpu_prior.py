@@ -1,0 +1,69 @@
+"""The calls with one prior row for all rows that the streaming kernels serve: workspace, capture, several draws and positions, odd
+sizes, a wait that gives up, precision."""
+import numpy as np
+import pytest
+import torch
+
+import parity_util as PU
+import workloads as W
+from oracle import rdk_oracle as O
+
+pytestmark = pytest.mark.gpu
+
+OUTPUTS = ("draft_token", "out_token", "accepted", "accept_prob", "alpha", "theta", "S", "residual_mass", "accepted_len")
+
+
+def _rdk():
+    import paper_2506_03206_b200 as rdk
+    return rdk
+
+
+def _device_inputs(N, n, batch, positions, trials, seed):
+    """Random inputs made on the device, where no row is compared with the checker."""
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    rows = batch * positions
+    z = (torch.randn(rows, N, generator=g, device="cuda") * 2).to(torch.bfloat16)
+    y = (torch.randn(rows, n, generator=g, device="cuda") * 2).to(torch.bfloat16)
+    prior = (torch.randn(N, generator=g, device="cuda") * 2).to(torch.bfloat16)
+    u = torch.randint(0, 1 << 24, (rows, trials, 4), generator=g, device="cuda").float() / (1 << 24)
+    ids = torch.sort(torch.randperm(N, generator=g, device="cuda")[:n]).values.to(torch.int32)
+    return z, prior, y, u, ids
+
+
+def _wanted(rdk, idx, z, prior, y, batch, positions, trials):
+    """Bytes of workspace with which the streaming kernels serve (0: they do not)."""
+    B = rdk.binding
+    pb = B.make_problem(idx, z, y, batch, positions)
+    return B.lib().rdk_sample_prior_workspace_bytes(B.C.byref(pb), z.data_ptr(), prior.data_ptr(), 0, y.data_ptr(), trials)
+
+
+def test_no_memory_for_a_workspace_is_no_error():
+    """The call needs no workspace; where the allocator has none to give, the cluster kernel serves."""
+    rdk = _rdk()
+    N, n, rows = 16384, 2000, 5000
+    z, prior, y, u, ids = _device_inputs(N, n, rows, 1, 1, 3)
+    idx = rdk.rdk_prepare_ids(ids, N)
+    assert _wanted(rdk, idx, z, prior, y, rows, 1, 1) > 24 << 20
+    want = rdk.rdk_sample_and_verify_prior(idx, z, prior, y, u, rows, 1)
+    out = rdk.binding.alloc_outputs(rows, rows, 1, "cuda")
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    total = torch.cuda.get_device_properties(0).total_memory
+    try:
+        torch.cuda.set_per_process_memory_fraction((torch.cuda.memory_reserved() + (4 << 20)) / total)
+        held, size = [], 1 << 28                         # what is left over in the allocator's blocks
+        while size > 1 << 21:
+            try:
+                held.append(torch.empty(size, dtype=torch.uint8, device="cuda"))
+            except torch.cuda.OutOfMemoryError:
+                size >>= 1
+        rdk.rdk_sample_and_verify_prior(idx, z, prior, y, u, rows, 1, out=out)
+    finally:
+        held = None
+        torch.cuda.set_per_process_memory_fraction(1.0)
+    torch.cuda.synchronize()
+    rdk.binding.check_status_word(out)
+    for k in ("alpha", "theta", "S", "residual_mass"):
+        assert float((out[k] - want[k]).abs().max()) < 1e-5, k
+    # a draw on the other side of a boundary: prefix sums 1e-7 apart, some 2 n interval ends (as in assert_ok_at_scale)
+    assert int((out["draft_token"] != want["draft_token"]).sum()) <= 2 + 6e-7 * n * rows
