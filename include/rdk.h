@@ -316,6 +316,9 @@ void rdk_test_set_spin_limit(uint32_t limit);
  * rows with one shared prior are served by the streaming kernels: rdk_sample_prior_workspace_bytes (host only, no CUDA
  * call) says how many bytes that takes, 0 where they would not serve.  A smaller or missing workspace is no error,
  * one that is not 256-byte aligned is (RDK_ERR_WORKSPACE_TOO_SMALL, as in rdk_sample_and_verify).
+ * The streaming kernels' CTAs wait for one another: with a workspace a call whose grid does not become resident in time (other
+ * streams holding the SMs for a quarter of a second) ends in RDK_ERR_TIMEOUT in out->status_word, as in
+ * rdk_sample_and_verify.  A call without one has no such wait.
  * ------------------------------------------------------------------------------------------- */
 int rdk_sample_and_verify_prior(const rdk_problem* problem, const void* target, const void* prior,
                                 int64_t prior_row_stride, const void* drafter, const float* uniforms,

@@ -424,14 +424,22 @@ def rdk_redistribute_linear_prior(index: KeptIndex, target: torch.Tensor, prior:
 
 def rdk_sample_and_verify_prior(index: KeptIndex, target: torch.Tensor, prior: torch.Tensor, drafter: torch.Tensor,
                                 uniforms: torch.Tensor, batch: int, positions: int, drafter_kind: int = RDK_LOGITS,
-                                out: Optional[Dict[str, torch.Tensor]] = None) -> Dict[str, torch.Tensor]:
+                                out: Optional[Dict[str, torch.Tensor]] = None,
+                                ws: Optional[torch.Tensor] = None) -> Dict[str, torch.Tensor]:
     """The linear mode with a separate prior inside Eq. rdk-taylor; verification against softmax(target).  A [N]
-    prior is one row shared by all rows, a [rows, N] prior has a row for each."""
+    prior is one row shared by all rows, a [rows, N] prior has a row for each.
+
+    Many rows with one shared prior are about twice as fast with a workspace (sample_workspace(problem, RDK_MODE_LINEAR, ...)
+    gives one that is large enough).  Without `ws` the call allocates its own where it serves, except while the stream is
+    captured: a call that is to go into a graph as it runs outside of one needs `ws`.  With an empty tensor the call
+    does without."""
     if out is None:
         rows = batch * positions
         out = alloc_outputs(rows, batch, uniforms.numel() // (rows * 4), target.device)
     status = (_host or host()).sample_prior(index.buffer, index.N, index.n, target, prior, drafter, uniforms, batch, positions,
-                                            drafter_kind, out)
+                                            drafter_kind, out, ws)
     if status:
         _check(status, "rdk_sample_and_verify_prior")
+    if ws is not None:
+        out["_ws"] = ws    # keep the workspace alive until the stream has consumed it
     return out

@@ -172,10 +172,10 @@ at::Tensor own_workspace(size_t bytes, const at::Tensor& like, const c10::cuda::
     }
 }
 
-// (buffer, N, n, target, prior, drafter, uniforms, batch, positions, kind, out) -> status
+// (buffer, N, n, target, prior, drafter, uniforms, batch, positions, kind, out[, ws or None]) -> status
 PyObject* sample_prior(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded([&]() -> PyObject* {
-        arity(n, 11);
+        if (n != 11) arity(n, 12);
         const at::Tensor& target = rows2d(a[3], "target");
         const at::Tensor& prior = tensor(a[4], "prior");
         const at::Tensor& drafter = rows2d(a[5], "drafter");
@@ -188,9 +188,11 @@ PyObject* sample_prior(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const float* up = pointer<float>(u);
         const c10::cuda::CUDAStream current = c10::cuda::getCurrentCUDAStream();
         void* s = current.stream();
-        const at::Tensor ws = own_workspace(rdk_sample_prior_workspace_bytes(&pb, z, pr, stride, y, (int32_t)trials), target, current);
-        void* wsp = ws.defined() ? pointer<void>(ws) : nullptr;
-        const size_t ws_bytes = wsp ? (size_t)ws.numel() : 0;
+        at::Tensor ws;
+        if (n == 12 && a[11] != Py_None) ws = tensor(a[11], "ws");
+        else ws = own_workspace(rdk_sample_prior_workspace_bytes(&pb, z, pr, stride, y, (int32_t)trials), target, current);
+        void* wsp = ws.defined() && ws.numel() ? pointer<void>(ws) : nullptr;
+        const size_t ws_bytes = wsp ? ws.nbytes() : 0;
         return PyLong_FromLong(unlocked([&] { return rdk_sample_and_verify_prior_ws(&pb, z, pr, stride, y, up, (int32_t)trials, &o, wsp, ws_bytes, s); }));
     });
 }

@@ -67,3 +67,58 @@ def test_no_memory_for_a_workspace_is_no_error():
         assert float((out[k] - want[k]).abs().max()) < 1e-5, k
     # a draw on the other side of a boundary: prefix sums 1e-7 apart, some 2 n interval ends (as in assert_ok_at_scale)
     assert int((out["draft_token"] != want["draft_token"]).sum()) <= 2 + 6e-7 * n * rows
+
+
+def test_a_workspace_of_the_callers_also_under_capture():
+    """With `ws` the call is the same in a graph as outside of one, bit for bit and with new inputs in the same buffers; without, a captured
+    call takes the cluster kernel, as does one with a workspace that is too small.  The streaming kernels leave a record of each
+    row at the start of the workspace."""
+    rdk = _rdk()
+    B = rdk.binding
+    N, n, batch, positions, trials = 50264, 9000, 40, 5, 2
+    sets = [_device_inputs(N, n, batch, positions, trials, 70 + k) for k in range(3)]
+    ids = sets[0][4]
+    idx = rdk.rdk_prepare_ids(ids, N)
+    buf = [t.clone() for t in sets[0][:4]]
+    z, prior, y, u = buf
+    need = _wanted(rdk, idx, z, prior, y, batch, positions, trials)
+    assert need > 0
+    ws = B.sample_workspace(B.make_problem(idx, z, y, batch, positions), B.RDK_MODE_LINEAR, trials, "cuda")
+    assert ws.numel() >= need
+    head = 4160 * batch * positions
+
+    def call(out, ws):
+        return rdk.rdk_sample_and_verify_prior(idx, z, prior, y, u, batch, positions, out=out, ws=ws)
+
+    def outs():
+        return B.alloc_outputs(batch * positions, batch, trials, "cuda")
+
+    for given, streams in ((ws, True), (ws[: need // 2], False), (ws[:0], False)):
+        ws.fill_(0xA5)
+        call(outs(), given)
+        torch.cuda.synchronize()
+        assert bool((ws[:head] != 0xA5).any()) == streams, given.numel()
+    captured, plain = outs(), outs()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call(captured, ws)
+    for inputs in sets + sets[:1]:
+        for b, t in zip(buf, inputs):
+            b.copy_(t)
+        ws.fill_(0xA5)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert bool((ws[:head] != 0xA5).any())
+        call(plain, ws)
+        torch.cuda.synchronize()
+        B.check_status_word(captured)
+        for k in OUTPUTS:
+            assert torch.equal(captured[k], plain[k]), k
+    without, graph = outs(), torch.cuda.CUDAGraph()
+    call(without, ws[:0])
+    with torch.cuda.graph(graph):
+        call(captured, None)
+    graph.replay()
+    torch.cuda.synchronize()
+    for k in OUTPUTS:
+        assert torch.equal(captured[k], without[k]), k
