@@ -951,11 +951,11 @@ rdk_draw_kernel(const RowParams P, const int nseg, const int Lw) {
 #pragma unroll
         for (int k = 0; k < K; ++k)
             if (k < per && s0 + k < nseg) cdf[s0 + k] = before + run[k];
-    } else if (warp == 3) {   // alpha = sum over the segments of sum min(p, q~)
-        float alpha_l = 0.f;
-        for (int s = lane; s < nseg; s += 32) alpha_l += __ldcg(reinterpret_cast<const float4*>(rec + 16) + s).y;
-        alpha_l = warp_sum(alpha_l);
-        if (lane == 0) alpha_s = alpha_l;
+    } else if (warp == 3) {   // alpha = sum over the segments of sum min(p, q~), in fp64 as the others
+        double alpha_l = 0.0;
+        for (int s = lane; s < nseg; s += 32) alpha_l += (double)__ldcg(reinterpret_cast<const float4*>(rec + 16) + s).y;
+        alpha_l = warp_sum_d(alpha_l);
+        if (lane == 0) alpha_s = (float)alpha_l;
     }
     __syncthreads();
     const double S_d = cdfW[nseg - 1], R_d = cdfR[nseg - 1], Pt_d = cdfP[nseg - 1];

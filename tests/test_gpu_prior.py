@@ -122,3 +122,27 @@ def test_a_workspace_of_the_callers_also_under_capture():
     torch.cuda.synchronize()
     for k in OUTPUTS:
         assert torch.equal(captured[k], without[k]), k
+
+
+@pytest.mark.parametrize("shared_prior", [False, True])
+def test_alpha_is_the_records_sum_rounded_once(shared_prior):
+    """The draw kernel adds the segments' shares of alpha up in fp64, as it does those of the weights: the result is the sum of the
+    row's records (16 scalars, then four sums a segment, the second of min(p, q~)) rounded to fp32 once."""
+    rdk = _rdk()
+    B = rdk.binding
+    N, n, rows = 131072, 600, 300
+    z, prior, y, u, ids = _device_inputs(N, n, rows, 1, 1, 11)
+    idx = rdk.rdk_prepare_ids(ids, N)
+    ws = B.sample_workspace(B.make_problem(idx, z, y, rows, 1), B.RDK_MODE_LINEAR, 1, "cuda")
+    if shared_prior:
+        assert _wanted(rdk, idx, z, prior, y, rows, 1, 1) > 0
+        out = rdk.rdk_sample_and_verify_prior(idx, z, prior, y, u, rows, 1, ws=ws)
+    else:
+        assert rdk.rdk_sample_route(idx, B.RDK_MODE_LINEAR, z, y, rows, 1, 1, ws)[0] == B.RDK_ROUTE_STREAM_KERNEL
+        out = rdk.rdk_sample_and_verify(idx, B.RDK_MODE_LINEAR, z, y, None, u, rows, 1, ws=ws)
+    torch.cuda.synchronize()
+    B.check_status_word(out)
+    geo = rdk.rdk_stream_geometry(N, n)
+    record = ws[: 4160 * rows].view(rows, 4160)[:, 64:].contiguous().view(torch.float32).view(rows, 256, 4)
+    sums = record[:, : geo["ctas_per_row"] * geo["warps_per_cta"], 1].double().sum(1)
+    assert torch.equal(out["alpha"], sums.float())
