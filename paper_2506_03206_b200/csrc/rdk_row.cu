@@ -437,6 +437,7 @@ static int validate_problem(const rdk_problem* pb, const char* who, bool need_in
 // 600 x 16 of 32768 208 / 243, 160 x 16 of 128256 274 / 169; given weights, 160 x 32 of 50257 70 / 73, of 128257 145 / 154, x 16
 // 64 / 49 and 139 / 96.  Rows on 16-byte boundaries are quicker in the row kernel: given, 100 x 16 of 32768 18 / 21, of 128256
 // 50 / 60, of 262144 149 / 89, 40 x 64 of 262144 102 / 136, 40 x 32 of 32768 21 / 17.
+static const char* const kFewRows = "few rows: one cluster each is faster";
 static bool many_draws(const RowParams& P, int mode, size_t es) {
     if (P.N < kStreamMinN || P.trials < 16) return false;
     const long long draws = (long long)P.rows * P.trials;
@@ -445,6 +446,16 @@ static bool many_draws(const RowParams& P, int mode, size_t es) {
     if (P.trials >= 256 && P.N > 65536) return true;         // (4 rows x 256 of 262143: 194 / 310)
     if (!aligned) return draws >= 5120;
     return P.trials >= 64 ? draws >= 2560 : draws >= (P.N <= 131072 ? 1600 : 5120);
+}
+
+// Why the streaming kernels do not serve a linear call with draws (a static string), or NULL where they do: what the calls
+// go by and the host-only queries answer.  Calls whose draws outweigh the sweep do not take the cluster kernel, however
+// few their rows.
+static const char* not_streaming(const RowParams& P, const rdk_problem* pb, const void* ws, size_t ws_bytes) {
+    if (pb->flags & RDK_FLAG_ROW_KERNEL) return "RDK_FLAG_ROW_KERNEL is set";
+    if (const char* no = stream_ineligible(P, pb->target_dtype, pb->drafter_dtype, pb->drafter_kind, pb->batch, ws, ws_bytes)) return no;
+    if (many_draws(P, RDK_MODE_LINEAR, pb->target_dtype == RDK_F32 ? 4 : 2)) return P.prior ? "many draws with a prior" : nullptr;
+    return stream_few_rows(P, pb->target_dtype, pb->drafter_dtype, pb->drafter_kind) ? kFewRows : nullptr;
 }
 
 // what the host-only queries look at
@@ -508,14 +519,14 @@ static int run_rows(const rdk_problem* pb, int mode, const void* target, const v
         return r;
     };
     if (!(pb->flags & RDK_FLAG_ROW_KERNEL)) {
-        const bool streams = mode == RDK_MODE_LINEAR && trials > 0 && (!prior || ws);     // (a prior's call may come without a workspace)
+        const char* no = mode == RDK_MODE_LINEAR && trials > 0 ? not_streaming(P, pb, ws, ws_bytes) : "";
         const bool many = many_draws(P, mode, pb->target_dtype == RDK_F32 ? 4 : 2);
-        if (!many && (!streams || stream_few_rows(P, pb->target_dtype, pb->drafter_dtype, pb->drafter_kind))) e = cluster();
-        if (e == cudaErrorNotSupported && streams) {
-            e = launch_stream_linear(P, pb->target_dtype, pb->drafter_dtype, pb->drafter_kind, pb->batch, ws, ws_bytes, s);
+        if (no && !many) e = cluster();
+        if (e == cudaErrorNotSupported && (!no || no == kFewRows)) {
+            e = launch_stream_linear(P, pb->target_dtype, pb->drafter_dtype, pb->drafter_kind, pb->batch, ws, s);
             counted = e == cudaSuccess;
         }
-        if (e == cudaErrorNotSupported && !many) e = cluster();
+        if (e == cudaErrorNotSupported && !no && !many) e = cluster();
         if (counted) return RDK_OK;                                 // the kernel also wrote accepted_len
     }
     if (e == cudaErrorNotSupported)
@@ -574,10 +585,7 @@ extern "C" size_t rdk_sample_prior_workspace_bytes(const rdk_problem* problem, c
     if (!prior || prior_row_stride != 0 || trials < 1 || validate_problem(problem, "rdk_sample_prior_workspace_bytes", true) != RDK_OK) return 0;
     const RowParams P = linear_rows(problem, target, drafter, trials, prior);
     const size_t bytes = stream_workspace_bytes(P.rows, problem->batch, trials);
-    const bool streams = !(problem->flags & RDK_FLAG_ROW_KERNEL) && !many_draws(P, RDK_MODE_LINEAR, problem->target_dtype == RDK_F32 ? 4 : 2) &&
-                         !stream_few_rows(P, problem->target_dtype, problem->drafter_dtype, problem->drafter_kind) &&
-                         !stream_ineligible(P, problem->target_dtype, problem->drafter_dtype, problem->drafter_kind, problem->batch, reinterpret_cast<const void*>(uintptr_t(256)), bytes);
-    return streams ? bytes : 0;
+    return not_streaming(P, problem, reinterpret_cast<const void*>(uintptr_t(256)), bytes) ? 0 : bytes;
 }
 
 extern "C" int rdk_sample_and_verify_prior_ws(const rdk_problem* problem, const void* target, const void* prior,
@@ -614,11 +622,7 @@ extern "C" int rdk_sample_route(const rdk_problem* problem, int32_t mode, const 
         set_error("RDK_FLAG_W_AS_GIVEN applies to RDK_MODE_PRECOMPUTED_W only");
         return -RDK_ERR_INVALID_ARG;
     }
-    if (problem->flags & RDK_FLAG_ROW_KERNEL) { if (why) *why = "RDK_FLAG_ROW_KERNEL is set"; return RDK_ROUTE_ROW_KERNEL; }
-    const RowParams P = linear_rows(problem, target, drafter, trials, nullptr);
-    const char* no = stream_ineligible(P, problem->target_dtype, problem->drafter_dtype, problem->drafter_kind,
-                                       problem->batch, ws, ws_bytes);
-    if (!no && stream_few_rows(P, problem->target_dtype, problem->drafter_dtype, problem->drafter_kind)) no = "few rows: one cluster each is faster";
+    const char* no = not_streaming(linear_rows(problem, target, drafter, trials, nullptr), problem, ws, ws_bytes);
     if (no) { if (why) *why = no; return RDK_ROUTE_ROW_KERNEL; }
     return RDK_ROUTE_STREAM_KERNEL;
 }

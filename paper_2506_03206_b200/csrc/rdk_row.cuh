@@ -131,9 +131,9 @@ __device__ __forceinline__ int pick_in_segment(const float (&x)[kVec], float rem
 }
 
 
-// Launches the streaming kernel for the linear path when the problem qualifies; returns
-// cudaErrorNotSupported (and launches nothing) when the one-CTA-per-row kernel has to be used.
-cudaError_t launch_stream_linear(RowParams P, int tz, int ty, int kind, int batch, void* ws, size_t ws_bytes, cudaStream_t s);
+// Launches the streaming kernels for a problem that qualifies (see stream_ineligible); returns
+// cudaErrorNotSupported (and launches nothing) where their grid does not fit the SMs at hand.
+cudaError_t launch_stream_linear(RowParams P, int tz, int ty, int kind, int batch, void* ws, cudaStream_t s);
 size_t stream_workspace_bytes(int rows, int batch, int trials);
 unsigned long long* stream_workspace_arrivals(void* ws, int rows);     // one word per (sequence, trial) in that workspace
 // Why a problem cannot take the streaming kernel (a static string), or NULL when it can.  Host only.

@@ -1312,9 +1312,8 @@ bool stream_few_rows(const RowParams& P, int tz, int ty, int kind) {
 void set_stream_spin_limit(unsigned limit) { g_spin_limit.store(limit); }
 unsigned stream_spin_limit() { return g_spin_limit.load(); }
 
-cudaError_t launch_stream_linear(RowParams P, int tz, int ty, int kind, int batch, void* ws, size_t ws_bytes, cudaStream_t s) {
+cudaError_t launch_stream_linear(RowParams P, int tz, int ty, int kind, int batch, void* ws, cudaStream_t s) {
     const size_t es = tz == RDK_F32 ? 4 : 2, ys = ty == RDK_F32 ? 4 : 2;
-    if (stream_ineligible(P, tz, ty, kind, batch, ws, ws_bytes)) return cudaErrorNotSupported;
     StreamGeo g;
     if (!plan_stream(P.N, P.n, es, ys, fast_types(tz, ty, kind), P.prior != nullptr, g)) return cudaErrorNotSupported;
     g.G = 0;

@@ -603,3 +603,21 @@ def test_route_of_few_rows(N, n, rows, trials, streams):
     ws = B.sample_workspace(B.make_problem(idx, z, y, rows, 1), B.RDK_MODE_LINEAR, trials, "cuda")
     route, why = rdk.rdk_sample_route(idx, B.RDK_MODE_LINEAR, z, y, rows, 1, trials, ws)
     assert (route == B.RDK_ROUTE_STREAM_KERNEL) == streams and ("few rows" in why) == (not streams), (route, why)
+
+
+@pytest.mark.parametrize("N,rows,trials", [(4096, 640, 16), (4096, 279, 59), (4960, 434, 25), (32768, 4, 1), (65536, 400, 2), (8192, 150, 4)])
+def test_route_query_names_the_kernel_that_runs(N, rows, trials):
+    """Draws that outweigh the sweep beside few rows among them.  The streaming kernels leave a record of each row at the start of the
+    workspace; the cluster kernel and the one-CTA-per-row kernel leave nothing there."""
+    rdk = _rdk()
+    B = rdk.binding
+    n = N // 4
+    g = torch.Generator(device="cuda").manual_seed(N)
+    idx = rdk.rdk_prepare_ids(torch.arange(n, dtype=torch.int32, device="cuda") * 4, N)
+    z, y = (torch.randn(rows, k, generator=g, device="cuda").to(torch.bfloat16) for k in (N, n))
+    ws = B.sample_workspace(B.make_problem(idx, z, y, rows, 1), B.RDK_MODE_LINEAR, trials, "cuda").fill_(0xA5)
+    route, why = rdk.rdk_sample_route(idx, B.RDK_MODE_LINEAR, z, y, rows, 1, trials, ws)
+    out = rdk.rdk_sample_and_verify(idx, B.RDK_MODE_LINEAR, z, y, None, torch.rand(rows, trials, 4, generator=g, device="cuda"), rows, 1, ws=ws)
+    torch.cuda.synchronize()
+    B.check_status_word(out)
+    assert (route == B.RDK_ROUTE_STREAM_KERNEL) == bool((ws[: 4160 * rows] != 0xA5).any()), (route, why)
