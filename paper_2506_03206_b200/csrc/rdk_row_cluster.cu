@@ -1110,12 +1110,29 @@ static cudaError_t launch_kind_c(const RowParams& P, const CluGeo& g, const CluS
     return kind == RDK_LOGITS ? launch_variant<TZ, TY, RDK_LOGITS>(P, g, sh, variant, s) : launch_variant<TZ, TY, RDK_PROBS>(P, g, sh, variant, s);
 }
 
-// What the rule above expects of a linear call of 16-byte aligned rows, in us (INFINITY where no shape fits), times what it was
-// low by on average for calls of that kind.
+// What a linear call of 16-byte aligned rows is expected to take, in us (INFINITY where no shape fits), to be compared with the streaming
+// kernels' time: the rule above for the shape that it picks, without its draws (whose term there is fitted to few of them), and those
+// anew.  For each round of sixteen trials the turns of the one CTA's warps: a draw each where a segment is one chunk, else two
+// chunks at a time, and then a pick each unless every chunk is still in its warp's registers (of several waves of clusters one and
+// a half are in their draws at once); and what the draws of an SM's CTAs take of one another.
 float cluster_rows_cost(const RowParams& P, size_t es) {
     CluShape sh;
-    if (P.N < kStreamMinN || !plan_cluster(P.N, P.n, P.rows, P.trials, es, P.prior ? kVarPrior : kVarSparse, P.prior != nullptr, 0, sh)) return INFINITY;
-    return sh.cost * (P.prior ? 1.18f : (P.trials == 2 ? 1.14f : 1.06f));
+    const int variant = P.prior ? kVarPrior : kVarSparse;
+    if (P.N < kStreamMinN || !plan_cluster(P.N, P.n, P.rows, P.trials, es, variant, P.prior != nullptr, 0, sh)) return INFINITY;
+    const CluCost& c = P.prior ? kCostPrior : (P.trials >= 3 ? kCostManyDraws : kCostFewDraws);
+    const int registers = sh.roomy ? 128 : (P.prior ? 80 : 64), nch = sh.per / 32;
+    const float sweep = cost_cluster(c, sh, P.rows, 0, registers, fminf(1.f, (float)P.n / (float)P.N), P.prior ? 256 : 384);
+    const float turn = nch == 1 ? 1.6f : 0.94f;
+    auto round = [&](int trials) -> float {
+        const int draws = 2 * trials, items = draws * nch, each = (draws + sh.nw - 1) / sh.nw;
+        if (nch == 1) return turn * (float)each;
+        return turn * (float)((items + 2 * sh.nw - 1) / (2 * sh.nw)) + (items > 2 * sh.nw ? 1.94f * (float)each : 0.f);
+    };
+    const int last = P.trials % kCluRound;
+    const float rounds = (float)(P.trials / kCluRound) * round(kCluRound) + (last ? round(last) : 0.f) - turn;      // (one turn is in the sweep's time)
+    const float waves = (float)P.rows / (float)rows_at_once(c, sh, resident_ctas(sh, registers));
+    const float crowd = (float)P.rows * (float)P.trials / (float)kCluSms - 3.f;
+    return sweep + (waves > 1.f ? fminf(waves + c.tail, 1.5f) : 1.f) * rounds + (crowd > 0.f ? 0.33f * sqrtf((float)nch) * crowd : 0.f);
 }
 
 cudaError_t launch_cluster_rows(RowParams P, int mode, int tz, int ty, int kind, uint32_t tag, unsigned spin_limit, cudaStream_t s) {

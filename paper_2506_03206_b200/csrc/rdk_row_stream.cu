@@ -1272,41 +1272,47 @@ const char* stream_ineligible(const RowParams& P, int tz, int ty, int kind, int 
     return nullptr;
 }
 
+// A rule of thumb for the time of a call through these two kernels, in us: one row a group, a further one for each that a group
+// takes in turn (by its vectors a lane and the steps of its kept tokens, three times as long each where the pass is not unrolled), a
+// prior's slice, and the draws, whose CTAs are five to an SM at first.  A fit to 3200 calls, 6.5 % off (standard deviation).
+static float stream_rows_cost(const RowParams& P, const StreamGeo& g, size_t es, bool unrolled) {
+    const int groups = 148 / g.C, per_group = (P.rows + groups - 1) / groups;
+    const float nv = (float)g.nv, steps = (float)P.n * (float)g.Lw / (64.f * (float)P.N), draws = (float)P.rows * (float)P.trials;
+    float t = 12.9f + 0.8f * (nv - 4.f) - (es == 4 ? 1.2f : 0.f) + (g.C > 8 ? 1.6f : 0.f) + (P.prior ? 4.f : 0.f);
+    const float row = (es == 4 ? 0.39f : 0.48f) * nv - 0.63f + (unrolled ? 0.11f * steps : 0.1f + 0.3f * steps) + (P.prior ? 0.34f : 0.f);
+    if (per_group > 1) t += 0.6f + (row > 0.2f ? row : 0.2f) * (float)(per_group - 1);
+    if (draws >= 120.f) t += 0.74f;
+    if (draws > 740.f) t += 3.5f + (es == 4 ? 2.3f : (P.prior ? 4.8f : 3.3f)) * (draws / 740.f - 1.f);
+    return t;
+}
+
 // Whether the rows are better served by one cluster launch each than by setting up the streaming grid and a second kernel
-// for the draws (the streaming kernels pay off when a group of CTAs has several rows to stream): where the cluster kernel's
-// rule of thumb expects less time than this one.  12.3 us for one row a group, 1.8 more for the second kernel once it has a CTA
-// for nearly every SM, 1.9 for every further row of a group of four 16-byte vectors a lane (1.3 times that without the
-// unrolled pass), 3 where the draws take a second wave of CTAs, 4.7 for a prior's slice.  Measured, streaming / cluster, a quarter of
-// the tokens kept, us:  4608 bf16: 11.3 / 6.2 for 4 rows, 14.8 / 9.6 for 256, four draws a row 13.2 / 6.7 for 64; 8192: 15.1 / 10.5 for
-// 256, 16.4 / 16.5 for 320; 65536: 16.8 / 12.0 for 64, 20.0 / 21.3 for 128; 128256: 13.4 / 8.7 for 4, 17.3 / 15.5 for 32,
-// 20.3 / 21.8 for 64; with a prior 128256: 16.6 / 13.4 for 4, 21.6 / 24.7 for 32.  Over 540 such calls the faster kernel is
-// missed by 1.8 % on average; limits on the number of rows alone missed it by 6 %.
-// Calls that such limits gave to the cluster kernel stay there (its sums are the more exact by half): one or two draws and up
-// to 3200000 / N rows, 192 at most (24, or 96 in other types, above 32768 tokens; 56 for groups of sixteen CTAs).  It visits kept
-// tokens beyond a warp's 384 register slots in memory, twice: with more of them (a warp of the largest cluster has n / 128) fewer
-// rows, and few beyond twice as many.  Rows of 16385 to 49152 tokens, and those that take a group of sixteen CTAs, keep the limits
-// both ways, as the route query has told them.
+// for the draws (the streaming kernels pay off when a group of CTAs has several rows to stream, and with draws in numbers, which a cluster
+// makes in one of its CTAs): where the cluster kernel's rule of thumb expects less time than this one's.  Measured, streaming /
+// cluster, a quarter of the tokens kept, us.  bf16, one draw a row: 4608 tokens 11.2 / 6.2 for 4 rows, 17.1 / 16.4 for 512; 32000 12.2 / 6.7 for
+// 4, 15.3 / 12.8 for 96, 17.0 / 18.1 for 192; 128256 13.1 / 8.7 for 4, 16.4 / 15.5 for 32, 19.3 / 21.8 for 64; 262144 14.6 / 9.6 for 4, 21.2 / 23.4
+// for 32.  32000, four draws 12.3 / 6.8 for 4 rows, 15.4 / 17.0 for 96; fp32 12.0 / 6.6 and 15.5 / 17.1.  100032 x 4 rows: four draws 13.2 / 9.8,
+// eight 13.0 / 13.1, 32 13.4 / 30.1.  With a prior 128256 x 4 rows 16.9 / 10.3, x 32 21.7 / 21.6, x 64 25.0 / 33.0; 200000 x 1 17.4 / 11.5, x 24
+// 22.8 / 26.0.  Over 3755 such calls (4096 to 400000 tokens, 1 to 3700 rows, 1 to 32 draws each) the faster kernel is missed by 0.7 % on
+// average and by more than a tenth in 3 % of them, and so it is over 1201 drawn ones that no constant was fitted to.
+// Calls that limits on the number of rows gave to the cluster kernel before there was this rule stay there (its sums are the more
+// exact by half): one or two draws and up to 3200000 / N rows, 192 at most (24, or 96 in other types, above 32768 tokens; 56 for groups of
+// sixteen CTAs); with more kept tokens than a warp's 384 register slots (a warp of the largest cluster has n / 128), which it
+// visits in memory, twice, up to 24 rows, and 4 with twice as many.
 bool stream_few_rows(const RowParams& P, int tz, int ty, int kind) {
     const size_t es = tz == RDK_F32 ? 4 : 2;
     const bool fast = fast_types(tz, ty, kind);
-    StreamSegs sg;
-    if (P.trials < 1 || !stream_segments(P.N, es, sg)) return false;
-    const bool sixteen = sg.C == kMaxGroup;                  // 9 groups of 16 CTAs
-    if (!P.prior) {
-        int most = !fast ? 96 : (sixteen ? 56 : 24);
+    StreamGeo g;
+    if (P.trials < 1 || !plan_stream(P.N, P.n, es, ty == RDK_F32 ? 4 : 2, fast, P.prior != nullptr, g)) return false;
+    if (!P.prior && P.trials <= 2) {
+        int most = !fast ? 96 : (g.C == kMaxGroup ? 56 : 24);
         if (P.N <= 32768) { const int small = 3200000 / P.N; most = most > small ? most : (small < 192 ? small : 192); }
         const int kept = P.n / 128;
         if (kept > 384 && most > 24) most = 24;
         if (kept > 768) most = 4;
-        if (P.trials <= 2 && P.rows <= most) return true;
-        if ((P.N > 16384 && P.N <= 49152) || sixteen) return false;
+        if (P.rows <= most) return true;
     }
-    const int groups = 148 / sg.C, per_group = (P.rows + groups - 1) / groups;
-    const long long draws = (long long)P.rows * P.trials;
-    const float row = 1.87f * (float)sg.nv / 4.f * (fast && sg.nv == kFastNit ? 1.f : (es == 4 ? 0.85f : 1.3f));
-    const float t = 12.3f + (per_group > 1 ? 1.8f + row * (float)(per_group - 1) : (draws >= 120 ? 1.8f : 0.f)) + (draws > 740 && draws <= 8 * 148 ? 3.f : 0.f) +
-                    (P.prior ? 4.7f : 0.f) + (sg.C > 8 ? 0.9f : 0.f);
-    return cluster_rows_cost(P, es) < 0.97f * t;
+    return cluster_rows_cost(P, es) < stream_rows_cost(P, g, es, fast && fast_steps(g, g.nv) > 0);
 }
 
 void set_stream_spin_limit(unsigned limit) { g_spin_limit.store(limit); }

@@ -323,16 +323,19 @@ def test_a_wait_that_runs_out_reports_a_timeout_and_leaves_the_device_usable():
     word says RDK_ERR_TIMEOUT.  With the default limit restored the same call is correct again."""
     rdk = _rdk()
     B = rdk.binding
-    cfg = W.tiny_config(N=40000, n=7000, rows=64, dtype="bf16", trials=1, kept_rule="zipf", zipf_bias=True,
+    cfg = W.tiny_config(N=40000, n=7000, rows=64, dtype="bf16", trials=16, kept_rule="zipf", zipf_bias=True,
                         rho=0.8, seed=77)
     inp = W.make_inputs(cfg)
     kid = inp["kept_ids"].cuda()
     idx = rdk.rdk_prepare_ids(kid, cfg.N)
     dev = {k: inp[k].cuda() for k in ("target", "drafter", "uniforms")}
+    ws = B.sample_workspace(B.make_problem(idx, dev["target"], dev["drafter"], cfg.batch, cfg.positions), B.RDK_MODE_LINEAR, cfg.trials, "cuda")
+    route, why = rdk.rdk_sample_route(idx, B.RDK_MODE_LINEAR, dev["target"], dev["drafter"], cfg.batch, cfg.positions, cfg.trials, ws)
+    assert route == B.RDK_ROUTE_STREAM_KERNEL, why
     try:
         rdk.rdk_test_set_spin_limit(1)
         out = rdk.rdk_sample_and_verify(idx, B.RDK_MODE_LINEAR, dev["target"], dev["drafter"], None, dev["uniforms"],
-                                        cfg.batch, cfg.positions)
+                                        cfg.batch, cfg.positions, ws=ws)
         torch.cuda.synchronize()
         assert int(out["status_word"].item()) == B.RDK_ERR_TIMEOUT
         with pytest.raises(B.RdkError):
@@ -351,7 +354,7 @@ def test_row_kernel_flag_and_route_query():
     one-CTA-per-row kernel; rdk_sample_route names the kernel either call takes and why."""
     rdk = _rdk()
     B = rdk.binding
-    cfg = W.tiny_config(N=20000, n=3000, rows=6, dtype="bf16", trials=4, rho=0.6, seed=91)
+    cfg = W.tiny_config(N=20000, n=3000, rows=6, dtype="bf16", trials=64, rho=0.6, seed=91)
     inp = W.make_inputs(cfg)
     kid = inp["kept_ids"].cuda()
     idx = rdk.rdk_prepare_ids(kid, cfg.N)
@@ -383,7 +386,7 @@ def test_strided_rows_through_the_streaming_kernels():
     not a multiple of 8, so the drafter rows start at varying 16-byte phases)."""
     rdk = _rdk()
     B = rdk.binding
-    cfg = W.tiny_config(N=24576, n=5001, rows=40, dtype="bf16", trials=3, kept_rule="zipf", zipf_bias=True,
+    cfg = W.tiny_config(N=24576, n=5001, rows=600, dtype="bf16", trials=3, kept_rule="zipf", zipf_bias=True,
                         rho=0.7, seed=57)
     inp = W.make_inputs(cfg)
     tw = torch.zeros(cfg.rows, cfg.N + 24, dtype=torch.bfloat16)
@@ -397,7 +400,7 @@ def test_strided_rows_through_the_streaming_kernels():
     route, why = rdk.rdk_sample_route(idx, B.RDK_MODE_LINEAR, z, y, cfg.batch, cfg.positions, cfg.trials, out["_ws"])
     assert route == B.RDK_ROUTE_STREAM_KERNEL, why
     B.check_status_word(out)
-    PU.compare_sampling(inp, out, range(cfg.rows), "linear").assert_ok()
+    PU.compare_sampling(inp, out, range(0, cfg.rows, 7), "linear").assert_ok()
 
 
 @pytest.mark.parametrize("name,nrows", [("C2", 320), ("C3", 128), ("C4", 128)])
@@ -591,15 +594,28 @@ def test_linear_with_a_separate_prior(dtype, N, n, kind):
     PU.compare_sampling(inp, a, range(cfg.rows), "linear").assert_ok()
 
 
-@pytest.mark.parametrize("N,n,rows,trials,streams", [(32768, 8192, 97, 1, False), (32768, 8192, 98, 1, True), (32768, 8192, 4, 3, True),
-                                                     (262144, 49152, 40, 1, False), (262144, 65536, 40, 1, True), (262144, 65536, 24, 1, False),
-                                                     (262144, 131072, 24, 1, True), (262144, 131072, 4, 1, False)])
-def test_route_of_few_rows(N, n, rows, trials, streams):
-    """The query names the kernel that runs: with few rows the cluster kernel, fewer of them where many tokens are kept."""
+# Beside each: what the streaming kernels / the cluster kernel take, in us, where both were measured.
+@pytest.mark.parametrize("N,n,rows,trials,streams", [
+    (32768, 8192, 97, 1, False), (32768, 8192, 98, 1, False), (32768, 8192, 400, 1, True),                  # 15.3 / 12.8 at 96 rows of 32000, 21.9 / 27.5 at 384
+    (32768, 8192, 4, 3, False), (32768, 8192, 4, 64, True), (16384, 4096, 4, 3, False), (65536, 16384, 4, 3, False),    # four draws: 12.3 / 6.8; 12.3 / 6.6; 12.8 / 7.8
+    (262144, 49152, 40, 1, False), (262144, 65536, 40, 1, True), (262144, 65536, 24, 1, False),
+    (262144, 131072, 24, 1, True), (262144, 131072, 4, 1, False),
+    (49152, 12288, 4, 4, False), (20032, 5008, 8, 4, False), (32000, 8000, 32, 4, False),                   # 12.8 / 6.9, 12.1 / 6.6, 12.9 / 8.5
+    (65536, 16384, 64, 1, False), (128256, 32064, 64, 1, True), (32000, 8000, 192, 4, True),                # 15.7 / 11.9, 19.3 / 21.8, 21.1 / 25.8
+    (100032, 25008, 4, 32, True), (128256, 32064, 8, 16, True), (100032, 25008, 4, 4, False)])              # 13.4 / 30.1, 13.6 / 25.4, 13.2 / 9.8
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_route_of_few_rows(N, n, rows, trials, streams, dtype):
+    """The query names the kernel that is the faster: with few rows the cluster kernel, fewer of them where many tokens are kept,
+    and with many draws of them the streaming ones."""
     rdk = _rdk()
     B = rdk.binding
+    if dtype == "f32" and N > 200000:
+        pytest.skip("fp32 rows of that size do not fit the streaming kernels")
+    if dtype == "f32" and trials <= 2 and N > 32768 and rows <= 96:
+        streams = False
+    dt = {"bf16": torch.bfloat16, "f32": torch.float32}[dtype]
     idx = rdk.rdk_prepare_ids(torch.arange(n, dtype=torch.int32, device="cuda") * (N // n), N)
-    z, y = (torch.zeros(rows, k, dtype=torch.bfloat16, device="cuda") for k in (N, n))
+    z, y = (torch.zeros(rows, k, dtype=dt, device="cuda") for k in (N, n))
     ws = B.sample_workspace(B.make_problem(idx, z, y, rows, 1), B.RDK_MODE_LINEAR, trials, "cuda")
     route, why = rdk.rdk_sample_route(idx, B.RDK_MODE_LINEAR, z, y, rows, 1, trials, ws)
     assert (route == B.RDK_ROUTE_STREAM_KERNEL) == streams and ("few rows" in why) == (not streams), (route, why)

@@ -146,3 +146,14 @@ def test_alpha_is_the_records_sum_rounded_once(shared_prior):
     record = ws[: 4160 * rows].view(rows, 4160)[:, 64:].contiguous().view(torch.float32).view(rows, 256, 4)
     sums = record[:, : geo["ctas_per_row"] * geo["warps_per_cta"], 1].double().sum(1)
     assert torch.equal(out["alpha"], sums.float())
+
+
+# Beside each: what the streaming kernels / the cluster kernel take, in us
+@pytest.mark.parametrize("N,n,rows,trials,streams", [
+    (200000, 8000, 1, 1, False), (262144, 65536, 6, 1, False), (100032, 25008, 8, 2, False), (16384, 4096, 96, 1, False),       # 16.8 / 10.1, 19.4 / 12.3, 17.3 / 10.7, 17.5 / 11.0
+    (128256, 32064, 4, 1, False), (128256, 32064, 64, 1, True), (200000, 50000, 48, 1, True), (128256, 32064, 8, 16, True)])   # 16.9 / 10.3, 25.0 / 33.0, 25.8 / 36.9, 18.3 / 26.1
+def test_route_of_few_rows_with_a_prior(N, n, rows, trials, streams):
+    rdk = _rdk()
+    z, prior, y, u, ids = _device_inputs(N, n, rows, 1, trials, N)
+    idx = rdk.rdk_prepare_ids(ids, N)
+    assert (_wanted(rdk, idx, z, prior, y, rows, 1, trials) > 0) == streams
