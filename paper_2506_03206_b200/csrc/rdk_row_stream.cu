@@ -299,9 +299,12 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
     uint32_t l_eph = 1, l_st_a = dsm_a, l_fb = full_a, l_eb = empty_a;    // a fresh stage counts as released
     unsigned char* l_st_p = dsm;
     // one row: one bulk copy of the CTA's slice of the target row and one per warp of the matching drafter values,
-    // into the stage the streaming warps have released
-    auto load_row = [&]() {
+    // into the stage the streaming warps have released.  Once a wait has given up, a stage may be released with its last copies still
+    // under way, and its barrier must not be armed on top of them: false, and no copies.  (`first`: before the CTA's
+    // first barrier, where nothing can have given up and `fail` is not set yet.)
+    auto load_row = [&](bool first) -> bool {
         mbar_wait(l_eb, l_eph, &fail, spin_limit);
+        const int gave_up = first ? 0 : ld_volatile_s32(&fail);
         // the few elements a 16-byte copy cannot cover go by plain stores: a slice that ends inside a
         // vector, and the very end of the drafter buffer
         const uintptr_t b0 = reinterpret_cast<uintptr_t>(ny), b1 = b0 + kbytes;
@@ -316,6 +319,7 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
             for (int k = 0; k < nt; ++k) reinterpret_cast<TY*>(l_st_p + l_yw_off + (t0 - a0))[k] = reinterpret_cast<const TY*>(t0)[k];
         }
         const uint32_t total = zbytes + __reduce_add_sync(0xffffffffu, ybytes);
+        if (__any_sync(0xffffffffu, gave_up)) return false;
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the stage was last touched by plain loads and stores
         if (lane == 0) {
             if (total == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(l_fb) : "memory");
@@ -333,6 +337,7 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
         nz += (long long)g.G * P.target_stride; ny += (long long)g.G * P.drafter_stride;
         l_st_a += stage; l_st_p += stage; l_fb += 8u; l_eb += 8u;
         if (++l_s == g.NS) { l_s = 0; l_eph ^= 1u; l_st_a = dsm_a; l_st_p = dsm; l_fb = full_a; l_eb = empty_a; }
+        return true;
     };
     // The load warp sets up the ring by itself and starts the first rows' copies right away, so that HBM's first
     // answer travels while the rest of the CTA is still setting up: it initialises the ring's barriers, gives the
@@ -362,7 +367,7 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
         asm volatile("griddepcontrol.wait;" ::: "memory");     // the inputs may be the previous kernel's outputs
         // (the few elements of the prior's slice that a 16-byte copy cannot cover)
         if (PRI && lane < lenc - lenc_v) reinterpret_cast<TZ*>(dsm + off_cache)[lenc_v + lane] = static_cast<const TZ*>(P.prior)[j0c + lenc_v + lane];
-        for (int k = 0; k < pre_rows; ++k) load_row();
+        for (int k = 0; k < pre_rows; ++k) load_row(true);
     }
 
     if (NST == 0 && warp < kSW) {          // the route with runtime loops keeps the offsets in shared memory
@@ -398,6 +403,8 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
         }
     }
 
+    // all warps have come to the end of their work (the load warp waits in a place of its own)
+    auto barrier_all = [] { asm volatile("barrier.sync 0;" ::: "memory"); };
     if (warp < kSW) {
         // ================================ streaming warps ============================================
         const int r0 = w_r0, kcp = w_kcp, kcs = w_kcs;
@@ -857,32 +864,29 @@ rdk_stream_kernel(const RowParams P, const StreamGeo g) {
     } else {
         // ================================ load warp =====================================================
         // the first row went out during the set-up; one row per stage as the streaming warps release them
-        for (int it = pre_rows; it < rows_g; ++it) load_row();
+        int issued = pre_rows;
+        while (issued < rows_g && load_row(false)) ++issued;
+        barrier_all();
         if (ld_volatile_s32(&fail)) {
-            // A wait gave up somewhere, so nobody may have waited for the last copies: let them land before
-            // the CTA leaves (bounded as well, on a count of its own).
-            for (int k = 0; k < g.NS && k < rows_g; ++k) {
-                const int last_it = ((rows_g - 1 - k) / g.NS) * g.NS + k;        // last row that used stage k
-                const uint32_t bar = full_a + 8u * (uint32_t)k, parity = (uint32_t)((last_it / g.NS) & 1);
+            // A wait gave up somewhere (no warp has one left that still could), so nobody may have waited for the last copies: let them
+            // land before the CTA leaves (bounded as well, on a count of its own).
+            auto land = [&](uint32_t bar, uint32_t parity) {
                 uint32_t done = 0;
                 for (unsigned spins = 0; !done && spins < (1u << 16); ++spins) {
                     asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
                                  : "=r"(done) : "r"(bar), "r"(parity) : "memory");
                     if (!done) __nanosleep(100);
                 }
+            };
+            for (int k = 0; k < g.NS && k < issued; ++k) {
+                const int last_it = ((issued - 1 - k) / g.NS) * g.NS + k;        // last row that used stage k
+                land(full_a + 8u * (uint32_t)k, (uint32_t)((last_it / g.NS) & 1));
             }
-            if (PRI) {
-                uint32_t done = 0;
-                for (unsigned spins = 0; !done && spins < (1u << 16); ++spins) {
-                    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n selp.u32 %0, 1, 0, p;\n}"
-                                 : "=r"(done) : "r"(smem_u32(&prbar)) : "memory");
-                    if (!done) __nanosleep(100);
-                }
-            }
+            if (PRI) land(smem_u32(&prbar), 0u);
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
+    if (warp != kWLoad) barrier_all();
     if (kTmem && warp == 0) {               // every path ends here, also after a wait that gave up
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base_s), "r"(kTmemCols) : "memory");

@@ -157,3 +157,32 @@ def test_route_of_few_rows_with_a_prior(N, n, rows, trials, streams):
     z, prior, y, u, ids = _device_inputs(N, n, rows, 1, trials, N)
     idx = rdk.rdk_prepare_ids(ids, N)
     assert (_wanted(rdk, idx, z, prior, y, rows, 1, trials) > 0) == streams
+
+
+@pytest.mark.parametrize("N,n,rows,trials", [(50264, 9000, 200, 2), (128256, 32064, 8, 16), (16384, 4000, 700, 1)])
+def test_a_wait_that_runs_out_with_a_prior(N, n, rows, trials):
+    """With the limit of the device-side waits at one failed try, the waits for the exchange (and now and then for the copies, those of the
+    prior's slice among them) run out; every warp still reaches the end of the kernel, which takes up its copies, and the status word says
+    so.  With the default limit restored the same call on the same workspace is right again.  Groups of several rows and of one."""
+    rdk = _rdk()
+    B = rdk.binding
+    z, prior, y, u, ids = _device_inputs(N, n, rows, 1, trials, 5)
+    idx = rdk.rdk_prepare_ids(ids, N)
+    assert _wanted(rdk, idx, z, prior, y, rows, 1, trials) > 0
+    ws = B.sample_workspace(B.make_problem(idx, z, y, rows, 1), B.RDK_MODE_LINEAR, trials, "cuda")
+    want = rdk.rdk_sample_and_verify_prior(idx, z, prior, y, u, rows, 1, ws=ws)
+    torch.cuda.synchronize()
+    B.check_status_word(want)
+    try:
+        rdk.rdk_test_set_spin_limit(1)
+        for _ in range(5):
+            out = rdk.rdk_sample_and_verify_prior(idx, z, prior, y, u, rows, 1, ws=ws)
+            torch.cuda.synchronize()
+            assert int(out["status_word"].item()) == B.RDK_ERR_TIMEOUT
+    finally:
+        rdk.rdk_test_set_spin_limit(0)
+    out = rdk.rdk_sample_and_verify_prior(idx, z, prior, y, u, rows, 1, ws=ws)
+    torch.cuda.synchronize()
+    B.check_status_word(out)
+    for k in OUTPUTS:
+        assert torch.equal(out[k], want[k]), k
