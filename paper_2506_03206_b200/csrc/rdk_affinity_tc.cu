@@ -239,12 +239,12 @@ aff_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__
         });
         if (kWrite && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     }
-    // after a wait that gave up, copies may still be on their way into shared memory: let them land (bounded as well)
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    // after a wait that gave up (none can any more), copies may still be on their way into shared memory: let them land (bounded as well)
     if (abort_s && warp == 0)
         for (int s = 0; s < kAffStages; ++s)
             for (unsigned spins = 0; spins < (1u << 12); ++spins) __nanosleep(100);
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
     if (warp == 1) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem_base) : "memory");

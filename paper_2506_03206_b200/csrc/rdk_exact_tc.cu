@@ -271,10 +271,10 @@ exact_tc_kernel(const __grid_constant__ CUtensorMap tmapV, const __grid_constant
         }
     }
 
-    // after a wait that gave up, copies may still be on their way into shared memory: let them land
-    if (abort_s && warp == 0) for (int k = 0; k < 10000; ++k) __nanosleep(100);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    // after a wait that gave up (none can any more), copies may still be on their way into shared memory: let them land
+    if (abort_s && warp == 0) for (int k = 0; k < 10000; ++k) __nanosleep(100);
     if (sum_row0_s >= 0 && !abort_s)
         for (int c = threadIdx.x; c < kTcMaxRows; c += kTcThreads) {
             const float v = (tc_sums[0][c] + tc_sums[1][c]) + (tc_sums[2][c] + tc_sums[3][c]);
