@@ -364,13 +364,15 @@ def test_cluster_kernel_cluster_sizes(N, n, rows, trials, dtype):
 
 
 # One prior row for all rows through the streaming kernels, and the same shapes without it: groups of unequal length and of one
-# row; kept tokens per segment from none to all of them (segments that outgrow the cached slots), one to six steps of 64 slots
-@pytest.mark.parametrize("N,n,rows,kept", [
-    (16384, 900, 450, "random"), (65536, 8000, 190, "random"), (65536, 11000, 149, "highest"), (65536, 13000, 131, "random"),
-    (65536, 20000, 160, "lowest"), (131072, 7000, 90, "highest"), (131064, 34000, 83, "random"), (262144, 4000, 70, "random")])
+# row; kept tokens per segment from none to all of them (segments that outgrow the cached slots), one to six steps of 64 slots;
+# sequences of one position, of several and of more than the accept bits; draw kernels of 256 and of 128 threads (beyond 1184 draws)
+@pytest.mark.parametrize("N,n,batch,positions,kept", [
+    (16384, 900, 90, 5, "random"), (65536, 8000, 38, 5, "random"), (65536, 11000, 149, 1, "highest"), (65536, 13000, 131, 1, "random"),
+    (65536, 20000, 20, 8, "lowest"), (131072, 7000, 3, 30, "highest"), (131064, 34000, 83, 1, "random"), (262144, 4000, 14, 5, "random")])
 @pytest.mark.parametrize("shared_prior", [False, True])
-def test_stream_kernel_shared_prior(N, n, rows, kept, shared_prior):
-    cfg = W.tiny_config(N=N, n=n, rows=rows, dtype="bf16", trials=1, rho=0.7, seed=n, zipf_bias=True)
+def test_stream_kernel_shared_prior(N, n, batch, positions, kept, shared_prior):
+    rows, trials = batch * positions, 3
+    cfg = W.tiny_config(N=N, n=n, rows=rows, dtype="bf16", trials=trials, rho=0.7, seed=n, zipf_bias=True).with_rows(batch, positions)
     g = torch.Generator().manual_seed(n)
     ids = {"random": torch.sort(torch.randperm(N, generator=g)[:n]).values, "lowest": torch.arange(n), "highest": torch.arange(N - n, N)}[kept]
     inp = W.make_inputs(cfg)
@@ -387,15 +389,18 @@ def test_stream_kernel_shared_prior(N, n, rows, kept, shared_prior):
         prior = (torch.randn(N, generator=g) * 2).to(torch.bfloat16)
         prior[5] = -float("inf")
         pb = B.make_problem(idx, z, y, cfg.batch, cfg.positions)
-        wanted = B.lib().rdk_sample_prior_workspace_bytes(B.C.byref(pb), z.data_ptr(), prior.cuda().data_ptr(), 0, y.data_ptr(), 1)
+        wanted = B.lib().rdk_sample_prior_workspace_bytes(B.C.byref(pb), z.data_ptr(), prior.cuda().data_ptr(), 0, y.data_ptr(), trials)
         assert wanted > 0                                # the streaming kernels serve
         out = rdk.rdk_sample_and_verify_prior(idx, z, prior.cuda(), y, u, cfg.batch, cfg.positions)
     else:
         out = rdk.rdk_sample_and_verify(idx, B.RDK_MODE_LINEAR, z, y, None, u, cfg.batch, cfg.positions)
+        route, why = rdk.rdk_sample_route(idx, B.RDK_MODE_LINEAR, z, y, batch, positions, trials, out["_ws"])
+        assert route == B.RDK_ROUTE_STREAM_KERNEL, why
     torch.cuda.synchronize()
     B.check_status_word(out)
     some = sorted({0, 1, rows // 2, rows - 2, rows - 1})
     PU.compare_sampling(inp, out, some, "linear", prior=prior).assert_ok()
+    PU.compare_accepted_len(out, batch, positions, trials)
     # every row against the one-CTA-per-row or the cluster kernel
     if shared_prior:
         ref = rdk.rdk_sample_and_verify_prior(idx, z, prior.cuda().expand(rows, N).contiguous(), y, u, cfg.batch, cfg.positions)
@@ -404,4 +409,5 @@ def test_stream_kernel_shared_prior(N, n, rows, kept, shared_prior):
     torch.cuda.synchronize()
     for k in ("alpha", "theta", "S", "residual_mass"):
         assert float((out[k] - ref[k]).abs().max()) < 1e-5, k
-    assert int((out["draft_token"] != ref["draft_token"]).sum()) <= max(2, rows // 20)
+    # a draw on the other side of a boundary: prefix sums 1e-7 apart, some 2 n interval ends (as in assert_ok_at_scale)
+    assert int((out["draft_token"] != ref["draft_token"]).sum()) <= 2 + 6e-7 * n * rows * trials

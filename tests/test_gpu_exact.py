@@ -346,12 +346,16 @@ def test_bf16_row_sums_take_one_addition_per_cta(N, rows):
     assert float(((S.double() / ref - 1) ** 2).mean().sqrt()) <= 2.0 ** -24 * (k / 3) ** 0.5
 
 
-@pytest.mark.parametrize("N,n,rows", [(2000, 300, 5), (9473, 200, 17), (19000, 130, 33), (20011, 1001, 20), (32768, 520, 250), (40001, 64, 1)])
+@pytest.mark.parametrize("N,n,rows", [(18945, 300, 5), (56833, 200, 17), (19000, 130, 33), (20011, 1001, 20), (32768, 520, 250), (40001, 64, 1)])
 def test_panels_lower_than_the_instruction(N, n, rows):
-    """Up to 256 rows a CTA takes fewer tokens than the instruction has rows, so that every round of panels is full (32 to 128 tokens,
-    the last panel ragged): every entry of w against a float64 product of the same bf16 operands, and its row sums."""
+    """Up to 256 rows a CTA takes fewer tokens than the instruction has rows where the panels of two CTAs do not fit one round, so that
+    every round is full (72 to 112 tokens here, the last panel ragged): every entry of w against a float64 product of the same
+    bf16 operands, and its row sums."""
     rdk = _rdk()
     B = rdk.binding
+    ctas = torch.cuda.get_device_properties(0).multi_processor_count // 2 * 2
+    rounds = -(-(-(-N // 256)) // (ctas // 2))
+    assert rounds > 1 and -(-(-(-N // (rounds * ctas))) // 8) * 8 < 128 and N % (-(-(-(-N // (rounds * ctas))) // 8) * 8)
     g = torch.Generator(device="cuda").manual_seed(N)
     idx = rdk.rdk_prepare_ids(torch.arange(n, dtype=torch.int32).cuda(), N)
     ld = (n + 7) // 8 * 8

@@ -18,7 +18,8 @@ def _rdk():
     return rdk
 
 
-def _run_linear(cfg, inp, rows=None, check_qtilde=True, kept_override=None):
+def _run_linear(cfg, inp, rows=None, check_qtilde=True, kept_override=None, streams=False):
+    """streams: the test is one of the streaming kernels, so they have to be what serves."""
     rdk = _rdk()
     B = rdk.binding
     dev = "cuda"
@@ -30,6 +31,9 @@ def _run_linear(cfg, inp, rows=None, check_qtilde=True, kept_override=None):
                                     cfg.positions, kind)
     torch.cuda.synchronize()
     B.check_status_word(out)
+    if streams:
+        route, why = rdk.rdk_sample_route(idx, B.RDK_MODE_LINEAR, target, drafter, cfg.batch, cfg.positions, cfg.trials, out["_ws"], kind)
+        assert route == B.RDK_ROUTE_STREAM_KERNEL, why
     rows = list(range(cfg.rows)) if rows is None else rows
     kappa = kid.cpu().numpy()
     tally = PU.compare_sampling(inp, out, rows, "linear", kept_ids=kappa)
@@ -46,6 +50,11 @@ def _run_linear(cfg, inp, rows=None, check_qtilde=True, kept_override=None):
         PU.compare_qtilde(qt, refs, cfg.dtype == "bf16")
     tally.record(cfg.name)
     return tally
+
+
+def _assert_streams(rdk, idx, dev, cfg, ws):
+    route, why = rdk.rdk_sample_route(idx, rdk.binding.RDK_MODE_LINEAR, dev["target"], dev["drafter"], cfg.batch, cfg.positions, cfg.trials, ws)
+    assert route == rdk.binding.RDK_ROUTE_STREAM_KERNEL, why
 
 
 def test_config1_tiny_rdk_linear():
@@ -70,9 +79,10 @@ def test_probability_drafter_linear():
 
 def test_zipf_pruned_mid_size_spans_several_tiles():
     # several 4096-token tiles plus a ragged tail, Zipf-ranked kept ids, correlated logits
-    cfg = W.tiny_config(N=3 * 4096 + 1032, n=3300, rows=6, dtype="bf16", trials=4, kept_rule="zipf",
-                        zipf_bias=True, rho=0.8, seed=11)
-    _run_linear(cfg, W.make_inputs(cfg)).assert_ok()
+    for trials, streams in ((4, False), (64, True)):
+        cfg = W.tiny_config(N=3 * 4096 + 1032, n=3300, rows=6, dtype="bf16", trials=trials, kept_rule="zipf",
+                            zipf_bias=True, rho=0.8, seed=11)
+        _run_linear(cfg, W.make_inputs(cfg), streams=streams).assert_ok()
 
 
 def test_unsorted_and_out_of_vocabulary_ids():
@@ -151,21 +161,21 @@ def test_identical_distributions_fall_back_to_p_for_the_residual():
 
 
 def test_groups_of_three_and_two_ctas():
-    # 40000 bf16 logits -> three CTAs share a row; 12000 fp32 logits -> two
-    cfg = W.tiny_config(N=40000, n=9000, rows=5, dtype="bf16", trials=4, kept_rule="zipf", zipf_bias=True,
+    # 40000 bf16 logits -> three CTAs share a row; 12000 fp32 logits -> two (with draws in numbers, else few rows take the cluster kernel)
+    cfg = W.tiny_config(N=40000, n=9000, rows=5, dtype="bf16", trials=64, kept_rule="zipf", zipf_bias=True,
                         rho=0.7, seed=41)
-    _run_linear(cfg, W.make_inputs(cfg), check_qtilde=False).assert_ok()
-    cfg = W.tiny_config(N=12000, n=1500, rows=5, dtype="f32", trials=16, rho=0.5, seed=42)
-    _run_linear(cfg, W.make_inputs(cfg), check_qtilde=False).assert_ok()
+    _run_linear(cfg, W.make_inputs(cfg), check_qtilde=False, streams=True).assert_ok()
+    cfg = W.tiny_config(N=12000, n=1500, rows=5, dtype="f32", trials=64, rho=0.5, seed=42)
+    _run_linear(cfg, W.make_inputs(cfg), check_qtilde=False, streams=True).assert_ok()
 
 
 def test_kept_ids_crowded_into_one_slice():
     # every kept id lies in the first part of the vocabulary: the kept-token caches of the first warps
     # overflow and the rest of their kept tokens take the uncached route
-    cfg = W.tiny_config(N=70000, n=6000, rows=4, dtype="bf16", trials=8, rho=0.8, seed=43)
+    cfg = W.tiny_config(N=70000, n=6000, rows=4, dtype="bf16", trials=32, rho=0.8, seed=43)
     inp = W.make_inputs(cfg)
     ids = torch.arange(cfg.n, dtype=torch.int32) + 100
-    _run_linear(cfg, inp, kept_override=ids, check_qtilde=False).assert_ok()
+    _run_linear(cfg, inp, kept_override=ids, check_qtilde=False, streams=True).assert_ok()
     # the same ids in a scrambled order (rank -> drafter index table in use: generic row kernel)
     g = torch.Generator().manual_seed(4)
     _run_linear(cfg, inp, kept_override=ids[torch.randperm(cfg.n, generator=g)], check_qtilde=False).assert_ok()
@@ -173,10 +183,11 @@ def test_kept_ids_crowded_into_one_slice():
 
 def test_stream_kernel_probs_and_full_vocab():
     # n = N (nothing pruned) and a probability drafter through the streaming kernels
-    cfg = W.tiny_config(N=8192, n=8192, rows=3, dtype="bf16", trials=8, rho=0.9, seed=44)
-    _run_linear(cfg, W.make_inputs(cfg), check_qtilde=False).assert_ok()
-    cfg = W.tiny_config(N=20000, n=4000, rows=3, dtype="bf16", trials=8, drafter_kind="probs", rho=0.8, seed=45)
-    _run_linear(cfg, W.make_inputs(cfg), check_qtilde=False).assert_ok()
+    cfg = W.tiny_config(N=8192, n=8192, rows=3, dtype="bf16", trials=64, rho=0.9, seed=44)
+    _run_linear(cfg, W.make_inputs(cfg), check_qtilde=False, streams=True).assert_ok()
+    for dtype in ("bf16", "f32"):
+        cfg = W.tiny_config(N=20000, n=4000, rows=3, dtype=dtype, trials=64, drafter_kind="probs", rho=0.8, seed=45)
+        _run_linear(cfg, W.make_inputs(cfg), check_qtilde=False, streams=True).assert_ok()
 
 
 def test_many_rows_per_group_every_row_checked():
@@ -184,43 +195,43 @@ def test_many_rows_per_group_every_row_checked():
     phases all wrap several times.  Every row is compared with the checker."""
     cfg = W.tiny_config(N=40000, n=7000, rows=1500, dtype="bf16", trials=1, kept_rule="zipf", zipf_bias=True,
                         rho=0.8, seed=51)
-    _run_linear(cfg, W.make_inputs(cfg), check_qtilde=False).assert_ok()
+    _run_linear(cfg, W.make_inputs(cfg), check_qtilde=False, streams=True).assert_ok()
 
 
 def test_drafter_values_far_below_their_neighbours():
     """The streaming kernels scale a warp's exponentials by the first value of the warp's range (kept
     drafter values, target logits) and fall back to the maximum when that value lies far below it: make
     many such values very small (and some -inf) so that both routes run."""
-    cfg = W.tiny_config(N=30000, n=6000, rows=6, dtype="bf16", trials=4, kept_rule="zipf", zipf_bias=True,
+    cfg = W.tiny_config(N=30000, n=6000, rows=6, dtype="bf16", trials=64, kept_rule="zipf", zipf_bias=True,
                         rho=0.8, seed=61)
     inp = W.make_inputs(cfg)
     y = inp["drafter"].clone()
     y[:, ::7] = -250.0
     y[:, 5::31] = float("-inf")
     inp["drafter"] = y
-    _run_linear(cfg, inp, check_qtilde=False).assert_ok()
+    _run_linear(cfg, inp, check_qtilde=False, streams=True).assert_ok()
     # the same for the target logits, whose scale is the first logit of each 1024-token segment
     z = inp["target"].clone()
     z[:, ::1024] = -300.0
     z[:, 2048] = float("-inf")
     z[:, 5000:5003] = float("-inf")
     inp["target"] = z
-    _run_linear(cfg, inp, check_qtilde=False).assert_ok()
+    _run_linear(cfg, inp, check_qtilde=False, streams=True).assert_ok()
 
 
 def test_vocabulary_beyond_sixteen_full_groups():
     # N = 300000: segments of five vectors per lane (the generic sweep), fifteen CTAs per row
-    cfg = W.tiny_config(N=300000, n=2500, rows=3, dtype="bf16", trials=4, kept_rule="zipf", zipf_bias=True,
+    cfg = W.tiny_config(N=300000, n=2500, rows=3, dtype="bf16", trials=16, kept_rule="zipf", zipf_bias=True,
                         rho=0.8, seed=71)
     assert _rdk().rdk_stream_geometry(cfg.N, cfg.n)["segment_tokens"] == 1280
-    _run_linear(cfg, W.make_inputs(cfg), check_qtilde=False).assert_ok()
+    _run_linear(cfg, W.make_inputs(cfg), check_qtilde=False, streams=True).assert_ok()
 
 
 def test_few_rows_fewer_than_the_pipeline_depth():
     # one and two rows: the deferred second visits all happen after the row loop
     for rows in (1, 2):
-        cfg = W.tiny_config(N=20000, n=3000, rows=rows, dtype="bf16", trials=8, rho=0.6, seed=52 + rows)
-        _run_linear(cfg, W.make_inputs(cfg), check_qtilde=False).assert_ok()
+        cfg = W.tiny_config(N=20000, n=3000, rows=rows, dtype="bf16", trials=64, rho=0.6, seed=52 + rows)
+        _run_linear(cfg, W.make_inputs(cfg), check_qtilde=False, streams=True).assert_ok()
 
 
 def test_calls_back_to_back_share_one_workspace():
@@ -229,7 +240,7 @@ def test_calls_back_to_back_share_one_workspace():
     second kernel is still reading the workspace, and must not disturb it."""
     rdk = _rdk()
     B = rdk.binding
-    cfgs = [W.tiny_config(N=36000, n=7000, rows=60, dtype="bf16", trials=2, kept_rule="zipf", zipf_bias=True,
+    cfgs = [W.tiny_config(N=36000, n=7000, rows=60, dtype="bf16", trials=8, kept_rule="zipf", zipf_bias=True,
                           rho=0.8, seed=80 + i) for i in range(5)]
     inps = [W.make_inputs(c) for c in cfgs]
     kid = inps[0]["kept_ids"].to("cuda")          # one kept set for all five calls
@@ -244,6 +255,7 @@ def test_calls_back_to_back_share_one_workspace():
         ws = o["_ws"]
         outs.append(o)
     torch.cuda.synchronize()
+    _assert_streams(rdk, idx, dev[0], cfgs[0], ws)
     for c, inp, o in zip(cfgs, inps, outs):
         B.check_status_word(o)
         PU.compare_sampling(inp, o, range(c.rows), "linear", kept_ids=kid.cpu().numpy()).assert_ok()
@@ -256,7 +268,7 @@ def test_replayed_graph_with_new_inputs_in_the_same_buffers():
     tells one launch's records in the workspace from the previous launch's must live on the device."""
     rdk = _rdk()
     B = rdk.binding
-    cfgs = [W.tiny_config(N=36000, n=7000, rows=60, dtype="bf16", trials=2, kept_rule="zipf", zipf_bias=True,
+    cfgs = [W.tiny_config(N=36000, n=7000, rows=60, dtype="bf16", trials=8, kept_rule="zipf", zipf_bias=True,
                           rho=0.8, seed=90 + i) for i in range(4)]
     inps = [W.make_inputs(c) for c in cfgs]
     c0 = cfgs[0]
@@ -268,6 +280,7 @@ def test_replayed_graph_with_new_inputs_in_the_same_buffers():
                                     c0.batch, c0.positions, 0)
     ws = out["_ws"]
     torch.cuda.synchronize()
+    _assert_streams(rdk, idx, buf, c0, ws)
     graph = torch.cuda.CUDAGraph()
     with torch.cuda.graph(graph):
         rdk.rdk_sample_and_verify(idx, B.RDK_MODE_LINEAR, buf["target"], buf["drafter"], None, buf["uniforms"],
@@ -290,7 +303,7 @@ def test_inputs_written_by_the_kernel_queued_just_before_the_call():
     kernels that overwrite the same input buffers with new rows; every call is checked against the checker."""
     rdk = _rdk()
     B = rdk.binding
-    cfgs = [W.tiny_config(N=36000, n=7000, rows=48, dtype="bf16", trials=1, kept_rule="zipf", zipf_bias=True,
+    cfgs = [W.tiny_config(N=36000, n=7000, rows=48, dtype="bf16", trials=8, kept_rule="zipf", zipf_bias=True,
                           rho=0.8, seed=300 + i) for i in range(30)]
     inps = [W.make_inputs(c) for c in cfgs]
     c0 = cfgs[0]
@@ -308,6 +321,7 @@ def test_inputs_written_by_the_kernel_queued_just_before_the_call():
         ws = o["_ws"]
         outs.append(o)
     torch.cuda.synchronize()
+    _assert_streams(rdk, idx, buf, c0, ws)
     tally = PU.Tally()
     for c, inp, o in zip(cfgs, inps, outs):
         B.check_status_word(o)
@@ -330,8 +344,7 @@ def test_a_wait_that_runs_out_reports_a_timeout_and_leaves_the_device_usable():
     idx = rdk.rdk_prepare_ids(kid, cfg.N)
     dev = {k: inp[k].cuda() for k in ("target", "drafter", "uniforms")}
     ws = B.sample_workspace(B.make_problem(idx, dev["target"], dev["drafter"], cfg.batch, cfg.positions), B.RDK_MODE_LINEAR, cfg.trials, "cuda")
-    route, why = rdk.rdk_sample_route(idx, B.RDK_MODE_LINEAR, dev["target"], dev["drafter"], cfg.batch, cfg.positions, cfg.trials, ws)
-    assert route == B.RDK_ROUTE_STREAM_KERNEL, why
+    _assert_streams(rdk, idx, dev, cfg, ws)
     try:
         rdk.rdk_test_set_spin_limit(1)
         out = rdk.rdk_sample_and_verify(idx, B.RDK_MODE_LINEAR, dev["target"], dev["drafter"], None, dev["uniforms"],

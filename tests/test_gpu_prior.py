@@ -186,3 +186,67 @@ def test_a_wait_that_runs_out_with_a_prior(N, n, rows, trials):
     B.check_status_word(out)
     for k in OUTPUTS:
         assert torch.equal(out[k], want[k]), k
+
+
+# Rows padded to 64 elements, so that any N has them on 16-byte boundaries: the prior's slice and the target's end inside a vector
+@pytest.mark.parametrize("N,n,batch,positions,trials", [(50257, 12566, 30, 5, 3), (24583, 2000, 120, 4, 1), (65543, 9000, 3, 40, 4), (131071, 20002, 12, 7, 16)])
+def test_shared_prior_of_any_size(N, n, batch, positions, trials):
+    rdk = _rdk()
+    B = rdk.binding
+    rows = batch * positions
+    cfg = W.tiny_config(N=N, n=n, rows=rows, dtype="bf16", trials=trials, rho=0.8, seed=N, zipf_bias=True).with_rows(batch, positions)
+    inp = W.make_inputs(cfg)
+    idx = rdk.rdk_prepare_ids(inp["kept_ids"].cuda(), N)
+    wide = torch.full((rows, -(-N // 64) * 64), 50.0, dtype=torch.bfloat16, device="cuda")       # (what lies beyond N must not count)
+    wide[:, :N] = inp["target"].cuda()
+    z, y, u = wide[:, :N], inp["drafter"].cuda(), inp["uniforms"].cuda()
+    g = torch.Generator().manual_seed(N)
+    prior = (inp["target"][0].float() * 0.8 + torch.randn(N, generator=g)).to(torch.bfloat16)
+    prior_dev = torch.full((N + 8,), 50.0, dtype=torch.bfloat16, device="cuda")[:N].copy_(prior)
+    assert _wanted(rdk, idx, z, prior_dev, y, batch, positions, trials) > 0
+    out = rdk.rdk_sample_and_verify_prior(idx, z, prior_dev, y, u, batch, positions)
+    ref = rdk.rdk_sample_and_verify_prior(idx, z, prior_dev.expand(rows, N).contiguous(), y, u, batch, positions)
+    torch.cuda.synchronize()
+    for o in (out, ref):
+        B.check_status_word(o)
+        PU.compare_accepted_len(o, batch, positions, trials)
+    PU.compare_sampling(inp, out, sorted({0, 1, rows // 2, rows - 2, rows - 1}), "linear", prior=prior).assert_ok()
+    for k in ("alpha", "theta", "S", "residual_mass"):
+        assert float((out[k] - ref[k]).abs().max()) < 1e-5, k
+    assert int((out["draft_token"] != ref["draft_token"]).sum()) <= 2 + 6e-7 * n * rows * trials
+
+
+@pytest.mark.parametrize("shift", [0.0, 12.0, 30.0, -30.0])
+def test_shared_prior_above_and_below_the_target(shift):
+    """theta pi / N is the smaller of the two nearly everywhere, or for half of the tokens, or hardly anywhere: the second visit takes
+    away what it is above p, where the smallest difference of a lane's logits says that there is any."""
+    rdk = _rdk()
+    B = rdk.binding
+    N, n, rows, trials = 37003, 5000, 160, 2
+    cfg = W.tiny_config(N=N, n=n, rows=rows, dtype="bf16", trials=trials, rho=0.7, seed=31)
+    inp = W.make_inputs(cfg)
+    g = torch.Generator().manual_seed(3)
+    prior = torch.randn(N, generator=g)
+    prior[: N // 2] += shift
+    prior[11] = -float("inf")
+    inp["target"][:, 13] = -float("inf")
+    inp["target"][7, N // 2:] = -float("inf")            # every token of a segment where there is none of the target
+    prior = prior.to(torch.bfloat16)
+    idx = rdk.rdk_prepare_ids(inp["kept_ids"].cuda(), N)
+    wide = torch.zeros(rows, -(-N // 64) * 64, dtype=torch.bfloat16, device="cuda")
+    wide[:, :N] = inp["target"].cuda()
+    z, y, u = wide[:, :N], inp["drafter"].cuda(), inp["uniforms"].cuda()
+    assert _wanted(rdk, idx, z, prior.cuda(), y, rows, 1, trials) > 0
+    out = rdk.rdk_sample_and_verify_prior(idx, z, prior.cuda(), y, u, rows, 1)
+    torch.cuda.synchronize()
+    B.check_status_word(out)
+    PU.compare_sampling(inp, out, sorted({0, 1, 7, *range(8, rows, 13)}), "linear", prior=prior).assert_ok()
+    # tokens that are not kept and lie below theta pi / N, all rows: the share of alpha that the test is about
+    p, pi = torch.softmax(z.double(), 1), torch.softmax(prior.cuda().double(), 0)
+    q = torch.zeros_like(p)
+    q[:, inp["kept_ids"].cuda().long()] = torch.softmax(y.double(), 1)
+    theta = (pi * q).sum(1, keepdim=True)
+    w = (N * q + theta * pi) / (N + pi)
+    w = w / w.sum(1, keepdim=True)
+    assert bool(((theta * pi / N > p) & (q == 0)).any())
+    assert float((out["alpha"].double() - torch.minimum(p, w).sum(1)).abs().max()) < 1e-5
