@@ -338,8 +338,12 @@ def bench_workload(ctx: Ctx, name: str, steps: int, warmup: int, prior: bool, he
             B.rdk_sample_and_verify_prior(index, s["target"], shared_prior, s["drafter"], s["uniforms"],
                                           cfg.batch, cfg.positions, kind, out=out_list[i % nsets])
         kernel_fn = lambda i: step(i, outs_nolen)
-        launches_per_step = 2              # stream kernel, draw kernel
-        kernels = "rdk_stream_kernel + rdk_draw_kernel (shared prior)"
+        launches_per_step = 2              # stream kernel, draw kernel; or cluster row kernel, accepted length
+        s0 = sets[0]
+        pb = B.make_problem(index, s0["target"], s0["drafter"], cfg.batch, cfg.positions, kind)
+        streams = B.lib().rdk_sample_prior_workspace_bytes(B.C.byref(pb), s0["target"].data_ptr(), shared_prior.data_ptr(), 0,
+                                                           s0["drafter"].data_ptr(), trials) > 0
+        kernels = ("rdk_stream_kernel + rdk_draw_kernel" if streams else "rdk_cluster_kernel") + " (shared prior; reported by the library)"
     else:
         route, why = B.rdk_sample_route(index, B.RDK_MODE_LINEAR, sets[0]["target"], sets[0]["drafter"], cfg.batch,
                                         cfg.positions, trials, ws, kind)

@@ -356,7 +356,7 @@ int launch_exact_tc(const __nv_bfloat16* A, long long lda, const __nv_bfloat16* 
     const int stage_bytes = kVocBytes + P.T * P.R * kBK;
     // Up to 256 rows the call is the read of Mt, and a last round with few panels reads it with few SMs.  So the panels are made
     // lower than the instruction, as low as leaves every round full; the rest of the instruction's rows are idle (whole calls with
-    // the draws: 32 rows x 20011 x 5001 68.5 -> 59.9 us, 16 x 65536 x 16000 359 -> 334, 240 x 50000 x 5000 151.0 -> 146.3, 20 x
+    // the draws: 32 rows x 20011 x 5001 68.5 -> 59.9 us, 16 x 65536 x 16000 359 -> 334, 240 x 50000 x 5000 151 -> 144 to 149, 20 x
     // 32768 x 8192 104.1 -> 102.8).  Not where one round holds all panels: more of them, each with the operand to fetch, were
     // slower (16 x 8192 x 2000 24.6 -> 25.3).
     P.voc = kVoc;

@@ -931,9 +931,9 @@ struct CluShape { int C, nw, per; size_t smem; bool roomy; float cost; };
 // chain (k; km where waves follow one another), b for each 256-position chunk of a warp, what the number of warps and CTAs of a row adds
 // to the exchange and to the prefix sums, a second pass over the chunks for the draws (unless there is but one), more
 // rounds of draws, kept tokens beyond a warp's registers (visited in memory, twice) and the warps that share the SM.
-// The constants are a fit to measured calls: 30 to 40 shapes each of 350 problems (N from 5001 to 262143, 1 to 1000 rows, bf16
-// and fp32).  The shape that the rule picks is within 2 to 4 % of the fastest one tried on average; powers of
-// two alone, which this replaces as the last word, were 8 to 15 % off (50257 tokens: 80 rows 16.9 -> 12.3 us, 320 rows
+// The constants are a fit to measured calls: 539 problems (N from 4992 to 262143, 1 to 1000 rows, bf16 and fp32), some 39 shapes of each.
+// The shape that the rule picks is within 1 to 4 % of the fastest one tried on average (a prior 0.7 %, one draw a row 3.9 %); powers of
+// two alone, which this replaces as the last word, were 8 to 20 % off (50257 tokens: 80 rows 16.9 -> 12.3 us, 320 rows
 // 44.8 -> 33.5; 128257: 320 rows 86.4 -> 70.4; q~ of 80 x 262143: 114.6 -> 62.1; given weights of 40 x 50240: 11.4 -> 8.7).
 // With three trials or more, clusters of one CTA an SM are counted as they were seen to fit: 32 rows of four trials at 32001 are
 // one round of four CTAs with 128 registers (fp32 13.6 -> 9.8 us, bf16 11.9 -> 8.6), and 24 rows at 44001 would be two rounds of

@@ -1,8 +1,8 @@
 // Streaming form of the linear-time path (Eq. rdk-taylor + Algorithm 4 steps 4-8) for N >= 4096
-// and kept ids in ascending order: one persistent kernel, one launch per call.
+// and kept ids in ascending order: a persistent kernel that streams the rows, and a kernel that draws.
 //
 // The grid is G groups of C CTAs, one CTA per SM.  Group g takes rows g, g + G, ...; within a row,
-// streaming warp w of CTA c owns the contiguous token range ("segment") s = 16 c + w.  A CTA has 20
+// streaming warp w of CTA c owns the contiguous token range ("segment") s = 16 c + w.  A CTA has 19
 // warps and no block-wide barrier in its row loop:
 //   load warp      : per row, one bulk copy (TMA) of the CTA's slice of the target logits and one per
 //                    streaming warp of the matching contiguous run of drafter values, into a ring of
@@ -12,18 +12,16 @@
 //                    pairs are cached.  Second visit B(row), NB - 1 rows later: sum min(p, q~) over
 //                    the cached pairs, when the row's scalars are known.
 //   publish warp   : folds the CTA's 16 warp records of a row into one and publishes it in global
-//                    memory as five 64-bit words, each a value paired with a per-call tag (so every
-//                    word validates itself and no fence is needed); NB rows later, writes the row's
-//                    per-segment sums and raises the CTA's flag for that row.
+//                    memory as five 64-bit words (seven with a prior), each a value paired with a per-call tag (so
+//                    every word validates itself and no fence is needed); NB rows later, writes the row's
+//                    per-segment sums for the draw kernel.
 //   collect warp   : polls the C records of a row and leaves the row scalars and every warp's scale
 //                    factors in shared memory for the second visits.
-//   draw warp      : CTA c of a group turns rows c, c + C, ... of the group into draws once all C
-//                    flags of the row are up: prefix sums over the segments, locate the segment of the
-//                    draft draw, re-read that one segment (still in L2), pick the token, run the
-//                    rejection test, on rejection the same for the residual draw, write the outputs
-//                    and count the accepted prefix of the sequence.
+// The draw kernel has a CTA for each row and trial: prefix sums over the segments, locate the segments of
+// the draft and of the residual draw, read these again (they are still in L2), pick the tokens, run the rejection
+// test, write the outputs and count the accepted prefix of the sequence.
 // The exchange of a row costs about two first visits of latency; with the second visit trailing by
-// NB - 1 rows and the exchange and the draws in warps of their own, both are off the streaming
+// NB - 1 rows and the exchange in warps of its own, it is off the streaming
 // warps' critical path.  Everything that depends only on (N, n, kept ids, element size) -- which
 // kept slots belong to which segment and where their target logits sit in the CTA's slice -- is
 // tabulated once by rdk_prepare_ids and read from the kept-id index.
@@ -39,7 +37,9 @@
 //
 // With one prior row pi for all rows in place of p inside the formula, the same kernel keeps the CTA's slice of pi and all that no
 // row changes about it, so pi costs a row no exponentials.  320 rows of 128256 tokens: 56 us, with the draws; the cluster
-// kernel, which reads pi and takes its soft-max anew for every row, 111.
+// kernel, which reads pi and takes its soft-max anew for every row, 111.  What bounds it is what bounds the kernel without a prior: 60 % of
+// the issue slots are taken (30.5 M warp instructions, where 22.8 M serve the same rows without one), the special-function unit is at
+// 41 %, HBM at 25 %; and the pair cache leaves five live rows in place of six to hide the exchange behind.
 #include <atomic>
 #include <chrono>
 
@@ -58,7 +58,7 @@ constexpr int kMaxChunks = 128;          // 256-token chunks per segment
 constexpr int kMaxNB = 8;                // most rows whose records and caches are alive at once (StreamGeo::NB)
 constexpr int kTmemCols = 512;           // tensor memory columns of an SM (128 lanes x 512 columns x 32 bits)
 constexpr int kTmemWarpCols = kTmemCols / (kSW / 4);   // columns of a streaming warp: four warps share a 32-lane quarter
-constexpr int kXrecBytes = 64;           // one published CTA record: five (value, tag) words, padded
+constexpr int kXrecBytes = 64;           // one published CTA record: five (value, tag) words (seven with a prior), padded
 constexpr int kRecFloats = 16 + 4 * kMaxSeg;   // one row's record: 16 scalars, then per segment the sums of w, min(p, q~),
                                          // max(0, p - q~) and p
 constexpr int kFastNit = 64 / kSW;       // 16-byte vectors per lane in a segment of the common length
@@ -1078,7 +1078,7 @@ static size_t stream_smem(const StreamGeo& g, size_t es, bool offsets_in_smem, b
     return (size_t)g.NS * stage + (prior ? slice : 0) + (offsets_in_smem ? (size_t)kSW * g.ycap * (8 * g.NB + 2) : 0) + (size_t)g.NS * 16;
 }
 
-constexpr size_t kStreamSmemBudget = 212 * 1024;    // dynamic shared memory a CTA may ask for: 227 KB less the static part (14.2 KB)
+constexpr size_t kStreamSmemBudget = 212 * 1024;    // dynamic shared memory a CTA may ask for: 227 KB less the static part (14.4 KB)
 
 // Stage count, live rows and cache capacity for a vocabulary of N tokens with n kept ids; false when
 // the shapes do not fit shared memory.
