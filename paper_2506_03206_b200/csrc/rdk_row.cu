@@ -437,7 +437,6 @@ static int validate_problem(const rdk_problem* pb, const char* who, bool need_in
 // 600 x 16 of 32768 208 / 243, 160 x 16 of 128256 274 / 169; given weights, 160 x 32 of 50257 70 / 73, of 128257 145 / 154, x 16
 // 64 / 49 and 139 / 96.  Rows on 16-byte boundaries are quicker in the row kernel: given, 100 x 16 of 32768 18 / 21, of 128256
 // 50 / 60, of 262144 149 / 89, 40 x 64 of 262144 102 / 136, 40 x 32 of 32768 21 / 17.
-static const char* const kFewRows = "few rows: one cluster each is faster";
 static bool many_draws(const RowParams& P, int mode, size_t es) {
     if (P.N < kStreamMinN || P.trials < 16) return false;
     const long long draws = (long long)P.rows * P.trials;
@@ -448,13 +447,16 @@ static bool many_draws(const RowParams& P, int mode, size_t es) {
     return P.trials >= 64 ? draws >= 2560 : draws >= (P.N <= 131072 ? 1600 : 5120);
 }
 
+static const char* const kFewRows = "few rows: one cluster each is faster";
+
 // Why the streaming kernels do not serve a linear call with draws (a static string), or NULL where they do: what the calls
 // go by and the host-only queries answer.  Calls whose draws outweigh the sweep do not take the cluster kernel, however
-// few their rows.
+// few their rows: the draw kernel has a CTA for each (with a prior, streaming / one CTA per row, us: 640 rows x 16 trials of 16384 tokens
+// 89 / 125, 160 x 64 of 32000 85 / 105, of 65536 90 / 170, of 128256 102 / 297, 40 x 256 of 262144 172 / 564).
 static const char* not_streaming(const RowParams& P, const rdk_problem* pb, const void* ws, size_t ws_bytes) {
     if (pb->flags & RDK_FLAG_ROW_KERNEL) return "RDK_FLAG_ROW_KERNEL is set";
     if (const char* no = stream_ineligible(P, pb->target_dtype, pb->drafter_dtype, pb->drafter_kind, pb->batch, ws, ws_bytes)) return no;
-    if (many_draws(P, RDK_MODE_LINEAR, pb->target_dtype == RDK_F32 ? 4 : 2)) return P.prior ? "many draws with a prior" : nullptr;
+    if (many_draws(P, RDK_MODE_LINEAR, pb->target_dtype == RDK_F32 ? 4 : 2)) return nullptr;
     return stream_few_rows(P, pb->target_dtype, pb->drafter_dtype, pb->drafter_kind) ? kFewRows : nullptr;
 }
 

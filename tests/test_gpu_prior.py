@@ -19,7 +19,7 @@ def _rdk():
 
 
 def _device_inputs(N, n, batch, positions, trials, seed):
-    """Random inputs made on the device, where no row is compared with the checker."""
+    """Random inputs made on the device, where no row is compared with the oracle."""
     g = torch.Generator(device="cuda").manual_seed(seed)
     rows = batch * positions
     z = (torch.randn(rows, N, generator=g, device="cuda") * 2).to(torch.bfloat16)
@@ -151,7 +151,8 @@ def test_alpha_is_the_records_sum_rounded_once(shared_prior):
 # Beside each: what the streaming kernels / the cluster kernel take, in us
 @pytest.mark.parametrize("N,n,rows,trials,streams", [
     (200000, 8000, 1, 1, False), (262144, 65536, 6, 1, False), (100032, 25008, 8, 2, False), (16384, 4096, 96, 1, False),       # 16.8 / 10.1, 19.4 / 12.3, 17.3 / 10.7, 17.5 / 11.0
-    (128256, 32064, 4, 1, False), (128256, 32064, 64, 1, True), (200000, 50000, 48, 1, True), (128256, 32064, 8, 16, True)])   # 16.9 / 10.3, 25.0 / 33.0, 25.8 / 36.9, 18.3 / 26.1
+    (128256, 32064, 4, 1, False), (128256, 32064, 64, 1, True), (200000, 50000, 48, 1, True), (128256, 32064, 8, 16, True),    # 16.9 / 10.3, 25.0 / 33.0, 25.8 / 36.9, 18.3 / 26.1
+    (32000, 4000, 160, 64, True), (16384, 2048, 640, 16, True)])                                                            # beside one CTA per row: 85 / 105, 89 / 125
 def test_route_of_few_rows_with_a_prior(N, n, rows, trials, streams):
     rdk = _rdk()
     z, prior, y, u, ids = _device_inputs(N, n, rows, 1, trials, N)
